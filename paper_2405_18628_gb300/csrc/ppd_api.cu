@@ -358,8 +358,8 @@ ppd_status enqueue_attention_any(const void *q, const void *kc, const void *vc, 
 }
 
 // Blocks of the fused step's narrow argmax grid (0: use the wide grid).  When
-// the attention grid's slices do not fill whole rounds, the CTAs of the last,
-// partial round that hold one slice fewer -- grid - (n_units mod grid) of
+// the attention grid's jobs do not fill whole rounds, the CTAs of the last,
+// partial round that hold one job fewer -- grid - (jobs mod grid) of
 // them -- have a slice's time to spare; the argmax blocks take as many SMs
 // (at most half of them), the CTAs dispatched last, which are those, wait for
 // them, and nothing on the critical path does.  Each block's share of the
@@ -369,11 +369,15 @@ ppd_status enqueue_attention_any(const void *q, const void *kc, const void *vc, 
 int narrow_argmax_grid(int L, int B, int H, int T, int D, int V, int S_max)
 {
     if (attention_splits(L, B, H, T, S_max)) return 0;
-    const int T_pad = (T + 31) & ~31;
-    const long long n_qb = T_pad > 64 ? (T + 127) / 128 : 1;
-    const long long n_units = (long long)L * B * H * n_qb;
-    const long long grid = n_units < split_grid() ? n_units : split_grid();
-    const long long r = n_units % grid;
+    AttnParams p{};
+    p.T_pad = (T + 31) & ~31;
+    p.n_qb = p.T_pad > 64 ? (T + 127) / 128 : 1;
+    // two groups of CTAs with queues of their own: none is known to have time to spare
+    if (p.n_qb == 3) return 0;
+    p.n_units = (int)((long long)L * B * H) * p.n_qb;
+    const long long n_jobs = ppd::whole_jobs(p);
+    const long long grid = ppd::attention_grid(p, split_grid());
+    const long long r = n_jobs % grid;
     if (r == 0) return 0;
     long long g = grid - r;
     if (g > num_sms() / 2) g = num_sms() / 2;

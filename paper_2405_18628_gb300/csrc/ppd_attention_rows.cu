@@ -4,32 +4,58 @@
 // the cached prefix, its tree ancestors and itself).
 //
 // With more than 64 tree tokens the queries fill the tensor core's M side, so
-// this kernel keeps one query per TMEM lane (queries zero-padded to 128).  A
-// unit is a (layer, sequence, head) slice and a block of 128 of its query rows;
-// its tiles are the KV prefix and then the tree's keys, 128 per tile:
+// this kernel keeps one query per TMEM lane (queries zero-padded to 128).  Per
+// block of 128 queries and tile of 128 keys:
 //
 //   S  = Q * K_tile^T          tcgen05.mma, M = 128 queries, N = 128 keys, K = D
-//   P  = exp2(S*scale*log2e - m)   two softmax warps per 32 query rows, each
-//                              thread owning one query row and 64 of the 128
-//                              keys; P is split into bf16 hi + lo and written
-//                              back to TMEM over the scores it came from
+//   P  = exp2(S*scale*log2e - m)   four softmax warps, one query row per thread;
+//                              P is split into bf16 hi + lo and written back to
+//                              TMEM over the scores it came from
 //   O += P_hi * V + P_lo * V   tcgen05.mma with A read from TMEM, M = 128
 //                              queries, N = D, two products per 16 keys
 //
-// A row's running maximum and row sum are registers of its two threads; they
-// exchange partial maxima through shared memory only on the exact path (a
-// unit's first tile, or a score more than 2^16 above the running maximum --
-// decided per tile by a vote over the softmax warps) and partial sums at the
-// end of a unit.  The tree mask is a 64-bit ancestor bitset per thread, built
-// from the parent array in registers.  Three score buffers in TMEM let two PV
-// products and the next S product queue in the tensor pipe; the single O
-// accumulator of a finished unit is read back after the next unit's first
-// tile, and that unit's first PV product waits for the readback.  The unit
-// walk (with the work split), the fused step's side warp and the merge of a
-// cut unit's partial states are those of the kernel for trees of up to 64
-// tokens (ppd_attention.cu), and so are the warp roles (352 threads), except
-// that the producer queues each V tile two tiles behind its K tile, the order
-// in which the MMA issuer consumes them.
+// A CTA runs two such streams, each with its own scores, output accumulator and
+// softmax warps (warps 0-3 and 4-7), and the tensor core alternates between
+// them: PV and the next S of one stream execute while the other stream's
+// softmax runs.  The bound is the tensor pipe, 3 x 512 cycles per block and
+// tile (D = 128), or HBM for trees of up to 128 tokens.  One stream with three
+// score buffers, issued from one lane's branch, kept the pipe 43 % busy: the
+// softmax and its hand-offs took longer than the pipe's work for a tile, and
+// the issue of a tcgen05.mma ~100 cycles.  Steps of 32 x 32 slices, D = 128:
+// 285 tokens over 1500 keys 541 -> 458 us; 96 tokens over 4096 keys (40 x 40
+// slices) 628 -> 575 us, 0.92 of the measured copy rate; eight ragged sequences
+// of up to 16384 keys with 128 tokens (4 x 32 slices each) 1046 -> 935 us.
+// Measured on the way: probabilities handed over in one piece per tile, 5 %
+// slower on 285 tokens; the softmax unrolled over a tile with its scores in
+// registers, 606 us there (instruction fetch).  What the streams work on:
+//
+//   a pair job     two blocks of 128 queries of one (layer, sequence, head)
+//                  slice, one per stream; every K and V tile is loaded once and
+//                  read by both
+//   a single job   one block; its tiles go to the streams in turn, and the two
+//                  partial softmax states are merged at the job's end (a row's
+//                  two accumulators sit in the same TMEM lane)
+//
+// Trees of 65-128 tokens are single jobs, 129-256 pair jobs, 385-512 two pair
+// jobs a slice; 257-384 tokens are a pair and a single job, done by two groups
+// of CTAs side by side so that the second reader of a slice finds it in L2.
+//
+// A thread owns a whole query row: the running maximum and the row sum are
+// registers and no vote or exchange is needed.  The maximum is lazy: it moves
+// only when a score exceeds it by more than 2^16, and the warp then rescales
+// its rows of O (the PV product of the tile before is complete by then: the
+// tensor pipe executes one thread's products in order, and the wait for S(i)
+// covers everything issued before it).  The tree mask is a 128-bit ancestor
+// bitset per tile and thread, built from the parent array in registers.
+//
+// The K and V tiles share one ring of shared-memory slots, loaded in the order
+// the products consume them: K0 V0 K1 V1 ... for pair jobs, K0 K1 V0 K2 V1 ...
+// for single jobs (an SM's copies land roughly in issue order, so a tile
+// queued ahead of its turn would hold back the one needed first).
+//
+// The work split, the fused step's side warp and the merge of a cut unit's
+// partial states are those of the kernel for trees of up to 64 tokens
+// (ppd_attention.cu), and so are the warp roles (352 threads).
 #include "ppd_attention_common.cuh"
 
 #include <cmath>
@@ -40,47 +66,129 @@ template <int D_>
 struct RowsLayout {
     static constexpr int D = D_;
     static constexpr int KT = 128;                         // keys per tile
-    static constexpr int M = 128;                          // query rows per unit (zero-padded)
+    static constexpr int M = 128;                          // query rows per block (zero-padded)
     static constexpr int DCH = D / 64;                     // 64-column groups along D
     static constexpr uint32_t GROUP_BYTES = 128 * 128;     // 128 rows of 64 bf16
     static constexpr uint32_t TILE_BYTES = KT * D * 2;
     static constexpr uint32_t Q_BYTES = M * D * 2;
-    static constexpr int QS = 2;                           // Q buffers
-    static constexpr int KS = (D == 64) ? 4 : 2;           // K tile ring
-    static constexpr int VS = (D == 64) ? 4 : 3;           // V tile ring
+    static constexpr int QS = 2;                           // Q slots: one per stream, or two jobs' deep
+    static constexpr int RS = (D == 64) ? 10 : 5;          // slots of the K/V tile ring
 
     static constexpr uint32_t OFF_Q = 0;
-    static constexpr uint32_t OFF_K = OFF_Q + QS * Q_BYTES;
-    static constexpr uint32_t OFF_V = OFF_K + KS * TILE_BYTES;
-    static constexpr uint32_t OFF_BAR = OFF_V + VS * TILE_BYTES;
+    static constexpr uint32_t OFF_R = OFF_Q + QS * Q_BYTES;
+    static constexpr uint32_t OFF_BAR = OFF_R + RS * TILE_BYTES;
     static constexpr int B_QFULL = 0;
     static constexpr int B_QEMPTY = B_QFULL + QS;
-    static constexpr int B_KFULL = B_QEMPTY + QS;
-    static constexpr int B_KEMPTY = B_KFULL + KS;
-    static constexpr int B_VFULL = B_KEMPTY + KS;
-    static constexpr int B_VEMPTY = B_VFULL + VS;
-    // Score tiles in TMEM: P is written over S, so S(g + NSB) waits for PV(g);
-    // three buffers keep two PV products and one S product in the tensor pipe.
-    static constexpr int NSB = 3;
-    static constexpr int B_SFULL = B_VEMPTY + VS;   // [NSB] scores of tile g in TMEM
-    static constexpr int B_PFULL = B_SFULL + NSB;   // [NSB] probabilities of tile g in TMEM (8 warps)
-    static constexpr int B_PDONE = B_PFULL + NSB;   // [NSB] PV product of tile g complete
-    static constexpr int B_OFREE = B_PDONE + NSB;   // a unit's output read back from TMEM (8 warps)
-    static constexpr int B_DRAIN = B_OFREE + 1;
+    static constexpr int B_FULL = B_QEMPTY + QS;    // [RS] tile landed
+    static constexpr int B_EMPTY = B_FULL + RS;     // [RS] every product that reads the slot is done
+    static constexpr int B_SFULL = B_EMPTY + RS;    // [2] scores of the stream's tile in TMEM
+    static constexpr int B_PFULL = B_SFULL + 2;     // [2][2] its probabilities, keys 0-63 and 64-127, in TMEM (4 warps)
+    static constexpr int B_DONE = B_PFULL + 4;      // [2] the stream's last PV product of a job complete
+    static constexpr int B_OFREE = B_DONE + 2;      // [2] a job's output read back from TMEM (8 arrivals)
+    static constexpr int B_DRAIN = B_OFREE + 2;
     static constexpr int NBAR = B_DRAIN + 1;
     static constexpr uint32_t OFF_TMEMPTR = OFF_BAR + NBAR * 8;
     static constexpr uint32_t OFF_ABORT = OFF_TMEMPTR + 4;
-    static constexpr uint32_t OFF_XM = (OFF_ABORT + 4 + 15) & ~15u;   // [2][M] partial row maxima
-    static constexpr uint32_t OFF_XL = OFF_XM + 2 * M * 4;            // [2][M] partial row sums
-    static constexpr uint32_t OFF_RANGE = OFF_XL + 2 * M * 4;        // WorkRange
+    static constexpr uint32_t OFF_X = (OFF_ABORT + 4 + 15) & ~15u;   // [2][M] (maximum, sum) per stream and row
+    static constexpr uint32_t OFF_RANGE = OFF_X + 2 * M * 8;         // WorkRange
     static constexpr uint32_t SMEM_BYTES = OFF_RANGE + ((sizeof(WorkRange) + 15) & ~15u);
-    // TMEM columns: S0 | S1 | S2 (128 each; P is written over S) | O (D)
-    static constexpr uint32_t T_S = 0, T_O = NSB * 128, TMEM_COLS = 512;
-    static_assert(NSB * 128 + D <= 512, "TMEM budget");
+    // TMEM columns: S_A | S_B (128 each; P is written over S) | O_A | O_B (D each)
+    static constexpr uint32_t T_S = 0, T_O = 256, TMEM_COLS = 512;
 
     static_assert(SMEM_BYTES <= 232448, "shared memory budget");
-    static_assert((OFF_K | OFF_V | Q_BYTES) % 1024 == 0, "1024-byte aligned operand tiles");
+    static_assert((OFF_R | Q_BYTES | TILE_BYTES) % 1024 == 0, "1024-byte aligned operand tiles");
 };
+
+// One job of a CTA: tiles [j0, j1) of a block of 128 queries (qb), or of the
+// two blocks qb and qb + 1 (pair).
+struct RowsJob {
+    UnitInfo ui;   // n_tiles: the job's tiles, the tree tiles past its last query left out
+    int j0, j1;
+    bool pair;
+};
+
+// Walks a CTA's jobs in order (every role walks the same sequence).  Whole
+// jobs round-robin: single jobs (n_qb 1), pair jobs (n_qb 2, or 4 with two a
+// slice); with n_qb 3 the first p.pair_grid CTAs take the slices' pairs and
+// the others their third blocks.  SPLIT: single jobs, the CTA's range of tiles.
+template <bool SPLIT>
+struct RowsIter {
+    SegIter<SPLIT> seg;
+    int x, step, n, per;
+    bool pair;
+    PPD_DEV RowsIter(const AttnParams &p, const WorkRange &w) : seg(w)
+    {
+        const int c = (int)blockIdx.x, G = (int)gridDim.x;
+        pair = !SPLIT && p.n_qb >= 2 && (p.n_qb != 3 || c < p.pair_grid);
+        x = c;
+        step = G;
+        if (p.n_qb == 3) {
+            x = pair ? c : c - p.pair_grid;
+            step = pair ? p.pair_grid : G - p.pair_grid;
+        }
+        per = p.n_qb == 4 ? 2 : 1;
+        n = p.n_units / p.n_qb * per;
+    }
+    PPD_DEV bool next(const AttnParams &p, RowsJob &j)
+    {
+        if (SPLIT) {
+            Seg s;
+            if (!seg.next(p, s)) return false;
+            j.ui = s.ui;
+            j.j0 = s.j0;
+            j.j1 = s.j1;
+            j.pair = false;
+            return true;
+        }
+        if (x >= n) return false;
+        const int slice = per == 2 ? x >> 1 : x;
+        const int qb = pair ? (per == 2 ? 2 * (x & 1) : 0) : p.n_qb - 1;
+        j.ui = unit_info(p, slice * p.n_qb + qb);
+        // a query's ancestors come before it: no tree tile past the job's last block
+        j.ui.n_tiles = j.ui.n_pref + qb + (pair ? 2 : 1);
+        j.j0 = 0;
+        j.j1 = j.ui.n_tiles;
+        j.pair = pair;
+        x += step;
+        return true;
+    }
+};
+
+// Position in the ring of tiles: slot and the parity of its current phase.
+template <int RS>
+struct RingPos {
+    int slot = 0;
+    uint32_t phase = 0;
+    PPD_DEV void advance()
+    {
+        if (++slot == RS) {
+            slot = 0;
+            phase ^= 1u;
+        }
+    }
+};
+
+// prefetch_first_tiles for whole jobs: this CTA's first `n` prefix tiles.
+template <bool SPLIT>
+PPD_DEV void rows_prefetch(const AttnParams &p, int lane, const CUtensorMap *kc, const CUtensorMap *vc,
+                           int dch, int n)
+{
+    if (SPLIT) {
+        prefetch_first_tiles<SPLIT>(p, lane, kc, vc, dch, n);
+        return;
+    }
+    const WorkRange none{};
+    const RowsIter<SPLIT> it(p, none);
+    if (lane != 0 || it.x >= it.n) return;
+    const int lbh = it.per == 2 ? it.x >> 1 : it.x;
+    const int P = min(max(ld_relaxed_gpu_s32(p.prefix_len + (lbh / p.H) % p.B), 0), p.S_max);
+    for (int j = 0; j < min(n, (P + 127) >> 7); ++j) {
+        for (int c = 0; c < dch; ++c) {
+            tma_prefetch_l2_3d(kc, c * 64, j * 128, lbh);
+            tma_prefetch_l2_3d(vc, c * 64, j * 128, lbh);
+        }
+    }
+}
 
 template <int D, bool SPLIT>
 __global__ void __launch_bounds__(352, 1)
@@ -91,6 +199,7 @@ tree_attention_rows_kernel(const __grid_constant__ CUtensorMap map_q,
                            const __grid_constant__ CUtensorMap map_vt, const AttnParams p)
 {
     using Lay = RowsLayout<D>;
+    using Pos = RingPos<Lay::RS>;
     extern __shared__ __align__(1024) uint8_t smem[];
     if (smem_addr(smem) & 1023u) {
         if (threadIdx.x == 0 && p.dev_status)
@@ -101,17 +210,19 @@ tree_attention_rows_kernel(const __grid_constant__ CUtensorMap map_q,
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + Lay::OFF_BAR);
     uint32_t *tmem_ptr = reinterpret_cast<uint32_t *>(smem + Lay::OFF_TMEMPTR);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + Lay::OFF_ABORT);
-    float *xm = reinterpret_cast<float *>(smem + Lay::OFF_XM);
-    float *xl = reinterpret_cast<float *>(smem + Lay::OFF_XL);
+    float2 *xs = reinterpret_cast<float2 *>(smem + Lay::OFF_X);
 
-    const int warp = threadIdx.x >> 5;
+    const int warp = warp_uniform((int)threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     const int T = p.T;
 
     if (threadIdx.x == 0) {
-        for (int i = 0; i < Lay::NBAR; ++i)
-            mbar_init(bars + i, ((i >= Lay::B_PFULL && i < Lay::B_PFULL + Lay::NSB) || i == Lay::B_OFREE)
-                                    ? 8u : 1u);
+        for (int i = 0; i < Lay::NBAR; ++i) {
+            uint32_t count = 1;
+            if (i >= Lay::B_PFULL && i < Lay::B_PFULL + 4) count = 4;
+            if (i >= Lay::B_OFREE && i < Lay::B_OFREE + 2) count = 8;
+            mbar_init(bars + i, count);
+        }
         *abort_flag = 0;
         mbar_fence_init();
     }
@@ -131,7 +242,7 @@ tree_attention_rows_kernel(const __grid_constant__ CUtensorMap map_q,
     // grid: everything above overlapped it, nothing below reads before it is done
     // (the first K/V tiles are only asked of L2 before)
     if (p.pdl_wait) {
-        if (warp == 8) prefetch_first_tiles<SPLIT>(p, lane, &map_kc, &map_vc, Lay::DCH, 3);
+        if (warp == 8) rows_prefetch<SPLIT>(p, lane, &map_kc, &map_vc, Lay::DCH, 3);
         asm volatile("griddepcontrol.wait;" ::: "memory");
     }
     WorkRange *wr_s = reinterpret_cast<WorkRange *>(smem + Lay::OFF_RANGE);
@@ -156,344 +267,508 @@ tree_attention_rows_kernel(const __grid_constant__ CUtensorMap map_q,
         if (p.fused) fused_side_warp<false>(p, wr, lane, abort_flag);
     } else if (warp == 8) {
         // ------------------------------------------------------------ TMA producer
-        // One queue of copies in the order the MMA issuer consumes them -- S(g)
-        // then PV(g - 2) -- so each tile's V follows the K tile two tiles later:
-        // Q(unit), K(g), V(g - 2), K(g + 1), V(g - 1), ...  An SM's copies land
-        // roughly in issue order, so a V tile queued ahead of its turn would
-        // hold back the K tile the next score product waits for, and vice versa.
         if (lane == 0) {
-            const uint64_t pol = l2_policy_evict_first();
-            constexpr int LAG = 2;
-            int v_row[LAG + 1], v_lbh[LAG + 1];
-            bool v_tree[LAG + 1];
-            int g = 0, gv = 0, k = 0;
-            auto load_v = [&]() {   // V tile gv (its coordinates queued when K(gv) was loaded)
-                const int i = gv % (LAG + 1);
-                const int vs = gv % Lay::VS;
-                if (gv >= Lay::VS)
-                    mbar_wait(bars + Lay::B_VEMPTY + vs, ((gv / Lay::VS) - 1) & 1, abort_flag);
+            // slices read by more than one CTA stay in L2 for the second reader
+            const uint64_t pol = p.n_qb > 2 ? l2_policy_evict_normal() : l2_policy_evict_first();
+            Pos pos;
+            int n_tiles = 0, n_q0 = 0, n_q1 = 0;   // copies issued: ring tiles, Q blocks per slot
+            auto load = [&](const CUtensorMap *map, int row, int lbh) {
+                // a fresh barrier counts as past its odd phase: the first round never waits
+                mbar_wait(bars + Lay::B_EMPTY + pos.slot, pos.phase ^ 1u, abort_flag);
                 if (!*abort_flag) {
-                    mbar_arrive_expect_tx(bars + Lay::B_VFULL + vs, Lay::TILE_BYTES);
+                    uint64_t *full = bars + Lay::B_FULL + pos.slot;
+                    mbar_arrive_expect_tx(full, Lay::TILE_BYTES);
 #pragma unroll
                     for (int c = 0; c < Lay::DCH; ++c)
-                        tma_load_3d(smem + Lay::OFF_V + vs * Lay::TILE_BYTES + c * Lay::GROUP_BYTES,
-                                    v_tree[i] ? &map_vt : &map_vc, bars + Lay::B_VFULL + vs, c * 64,
-                                    v_row[i], v_lbh[i], pol);
+                        tma_load_3d(smem + Lay::OFF_R + pos.slot * Lay::TILE_BYTES + c * Lay::GROUP_BYTES, map,
+                                    full, c * 64, row, lbh, pol);
+                    ++n_tiles;
                 }
-                ++gv;
+                pos.advance();
             };
-            SegIter<SPLIT> it(wr);
-            for (Seg sg; it.next(p, sg); ++k) {
-                const UnitInfo &ui = sg.ui;
-                const int qs = k % Lay::QS;
-                if (k >= Lay::QS)
-                    mbar_wait(bars + Lay::B_QEMPTY + qs, ((k / Lay::QS) - 1) & 1, abort_flag);
+            auto load_q = [&](int qs, uint32_t parity, int qb, int lbh) {
+                mbar_wait(bars + Lay::B_QEMPTY + qs, parity ^ 1u, abort_flag);
                 if (!*abort_flag) {
                     // rows T..127 of the box lie beyond the tensor and arrive as zeros
                     mbar_arrive_expect_tx(bars + Lay::B_QFULL + qs, Lay::Q_BYTES);
 #pragma unroll
                     for (int c = 0; c < Lay::DCH; ++c)
-                        tma_load_3d(smem + Lay::OFF_Q + qs * Lay::Q_BYTES + c * Lay::GROUP_BYTES,
-                                    &map_q, bars + Lay::B_QFULL + qs, c * 64, ui.qb * Lay::M,
-                                    ui.lbh, pol);
+                        tma_load_3d(smem + Lay::OFF_Q + qs * Lay::Q_BYTES + c * Lay::GROUP_BYTES, &map_q,
+                                    bars + Lay::B_QFULL + qs, c * 64, qb * Lay::M, lbh, pol);
+                    n_q0 += qs == 0;
+                    n_q1 += qs == 1;
                 }
-                for (int j = sg.j0; j < sg.j1; ++j, ++g) {
+            };
+            // V tiles of a single job trail their K tiles by two: their coordinates
+            int v_row[2] = {0, 0}, v_lbh[2] = {0, 0};
+            bool v_tree[2] = {false, false};
+            int g = 0, k = 0;
+            RowsIter<SPLIT> it(p, wr);
+            for (RowsJob jb; it.next(p, jb); ++k) {
+                const UnitInfo &ui = jb.ui;
+                if (!jb.pair) load_q(k & 1, (uint32_t)(k >> 1) & 1u, ui.qb, ui.lbh);
+                for (int j = jb.j0; j < jb.j1; ++j, ++g) {
                     const bool tree = (j >= ui.n_pref);
                     const int row = (tree ? j - ui.n_pref : j) * Lay::KT;
-                    const int ks = g % Lay::KS;
-                    if (g >= Lay::KS)
-                        mbar_wait(bars + Lay::B_KEMPTY + ks, ((g / Lay::KS) - 1) & 1, abort_flag);
-                    if (!*abort_flag) {
-                        mbar_arrive_expect_tx(bars + Lay::B_KFULL + ks, Lay::TILE_BYTES);
-#pragma unroll
-                        for (int c = 0; c < Lay::DCH; ++c)
-                            tma_load_3d(smem + Lay::OFF_K + ks * Lay::TILE_BYTES + c * Lay::GROUP_BYTES,
-                                        tree ? &map_kt : &map_kc, bars + Lay::B_KFULL + ks, c * 64,
-                                        row, ui.lbh, pol);
+                    if (jb.pair) {
+                        load(tree ? &map_kt : &map_kc, row, ui.lbh);
+                        load(tree ? &map_vt : &map_vc, row, ui.lbh);
+                        // the Q slots are free once the job before has its last scores:
+                        // its first tiles are queued ahead of that wait
+                        if (j == jb.j0) {
+                            load_q(0, (uint32_t)k & 1u, ui.qb, ui.lbh);
+                            load_q(1, (uint32_t)k & 1u, ui.qb + 1, ui.lbh);
+                        }
+                        continue;
                     }
-                    const int i = g % (LAG + 1);
-                    v_row[i] = row;
-                    v_lbh[i] = ui.lbh;
-                    v_tree[i] = tree;
-                    if (g >= LAG) load_v();
+                    if (g & 1) {
+                        if (g >= 2) load(v_tree[1] ? &map_vt : &map_vc, v_row[1], v_lbh[1]);
+                        v_row[1] = row;
+                        v_lbh[1] = ui.lbh;
+                        v_tree[1] = tree;
+                    } else {
+                        if (g >= 2) load(v_tree[0] ? &map_vt : &map_vc, v_row[0], v_lbh[0]);
+                        v_row[0] = row;
+                        v_lbh[0] = ui.lbh;
+                        v_tree[0] = tree;
+                    }
+                    load(tree ? &map_kt : &map_kc, row, ui.lbh);
                 }
             }
-            while (gv < g) load_v();
+            if (!it.pair) {
+                for (int e = max(0, g - 2); e < g; ++e)
+                    load((e & 1 ? v_tree[1] : v_tree[0]) ? &map_vt : &map_vc, e & 1 ? v_row[1] : v_row[0],
+                         e & 1 ? v_lbh[1] : v_lbh[0]);
+            }
             if (*abort_flag) {
                 // let every copy already issued land before the CTA can exit
-                for (int i = max(0, g - Lay::KS); i < g; ++i)
-                    mbar_wait_drain(bars + Lay::B_KFULL + i % Lay::KS, (i / Lay::KS) & 1);
-                for (int i = max(0, k - Lay::QS); i < k; ++i)
-                    mbar_wait_drain(bars + Lay::B_QFULL + i % Lay::QS, (i / Lay::QS) & 1);
-                for (int i = max(0, gv - Lay::VS); i < gv; ++i)
-                    mbar_wait_drain(bars + Lay::B_VFULL + i % Lay::VS, (i / Lay::VS) & 1);
+                for (int i = max(0, n_tiles - Lay::RS); i < n_tiles; ++i)
+                    mbar_wait_drain(bars + Lay::B_FULL + i % Lay::RS, (i / Lay::RS) & 1);
+                if (n_q0 > 0) mbar_wait_drain(bars + Lay::B_QFULL + 0, (n_q0 - 1) & 1);
+                if (n_q1 > 0) mbar_wait_drain(bars + Lay::B_QFULL + 1, (n_q1 - 1) & 1);
             }
         }
     } else if (warp == 9) {
         // ------------------------------------------------------------ MMA issuer
-        if (lane == 0) {
-            const uint32_t idesc_qk = make_idesc_bf16(128, 128, 0, 0);
-            const uint32_t idesc_pv = make_idesc_bf16(128, D, 0, 1);
-            const uint32_t sq = smem_addr(smem + Lay::OFF_Q);
-            const uint32_t sk = smem_addr(smem + Lay::OFF_K);
-            const uint32_t sv = smem_addr(smem + Lay::OFF_V);
+        // the whole warp walks the jobs and waits; one elected lane issues
+        const uint32_t idesc_qk = make_idesc_bf16(128, 128, 0, 0);
+        const uint32_t idesc_pv = make_idesc_bf16(128, D, 0, 1);
+        const uint32_t tmem = warp_uniform(tmem_base);
+        const uint64_t dq0 = make_smem_desc(warp_uniform(smem_addr(smem + Lay::OFF_Q)), 16, 1024);
+        const uint64_t dk0 = make_smem_desc(warp_uniform(smem_addr(smem + Lay::OFF_R)), 16, 1024);
+        const uint64_t dv0 = make_smem_desc(warp_uniform(smem_addr(smem + Lay::OFF_R)), Lay::GROUP_BYTES, 1024);
+        using a_t = kind_t<0>;
+        using b_t = kind_t<1>;
 
-            // O += P_hi V + P_lo V for tile gp.  Per 32 keys the probability columns
-            // hold 8 columns of hi pairs for keys 0..15, 8 for keys 16..31, then the
-            // lo pairs in the same order.
-            // A unit's first PV product overwrites O: unit k >= 1 waits until the
-            // softmax warps have read unit k-1's output back.
-            const uint32_t t_o = tmem_base + Lay::T_O;
-            auto issue_pv = [&](int gp, bool first, int kp) {
-                const int pb = gp % Lay::NSB;
-                mbar_wait(bars + Lay::B_PFULL + pb, (gp / Lay::NSB) & 1, abort_flag);
-                if (first && kp >= 1) mbar_wait(bars + Lay::B_OFREE, (kp - 1) & 1, abort_flag);
-                const int vs = gp % Lay::VS;
-                mbar_wait(bars + Lay::B_VFULL + vs, (gp / Lay::VS) & 1, abort_flag);
+        Pos pos;                                  // next ring slot to consume
+        Pos p_v[2];                               // pair jobs: the V tile of a stream's pending tile
+        bool pend[2] = {false, false};            // a tile's PV product is still to be issued
+        bool p_first[2] = {false, false}, p_last[2] = {false, false};   // the tile's place in its job
+        bool p_frees[2] = {false, false};         // its PV product is the last reader of the V tile
+        int p_job[2] = {0, 0}, of_seen[2] = {0, 0};
+        uint32_t p_par[2] = {0, 0};
+        bool dead = false;                        // the CTA gave up: keep the control flow, issue nothing
+        bool v_seen = false;                      // the next PV product's V tile is known to have landed
+
+        // O_s += P_hi V + P_lo V for stream s's pending tile, as its halves of 64 keys
+        // arrive.  Per 32 keys the probability columns hold 8 columns of hi pairs for
+        // keys 0..15, 8 for keys 16..31, then the lo pairs in the same order.  A job's
+        // first PV product overwrites O: it waits until the softmax warps have read back
+        // the outputs of every job before.
+        auto issue_pv = [&](auto s_c, bool pair) {
+            constexpr int s = decltype(s_c)::value;
+            const Pos v = pair ? p_v[s] : pos;
+            if (!pair) pos.advance();
+            if (!v_seen) mbar_wait(bars + Lay::B_FULL + v.slot, v.phase, abort_flag);
+            if (p_first[s])
+                for (; of_seen[s] < p_job[s]; ++of_seen[s])
+                    mbar_wait(bars + Lay::B_OFREE + s, (uint32_t)of_seen[s] & 1u, abort_flag);
+#pragma unroll
+            for (int half = 0; half < 2; ++half) {
+                mbar_wait(bars + Lay::B_PFULL + 2 * s + half, p_par[s], abort_flag);
                 tc_fence_after();
-                if (!*abort_flag) {
-                    const uint32_t a0 = tmem_base + Lay::T_S + (uint32_t)pb * 128u;
-                    const uint64_t b0 = make_smem_desc(sv + vs * Lay::TILE_BYTES, Lay::GROUP_BYTES, 1024);
+                if (elect_one()) {
+                    if (!dead) {
+                        const uint32_t t_o = tmem + Lay::T_O + s * D;
+                        const uint32_t a0 = tmem + Lay::T_S + s * 128u;
+                        const uint64_t b0 = desc_advance(dv0, v.slot * Lay::TILE_BYTES);
 #pragma unroll
-                    for (int kk = 0; kk < Lay::KT / 16; ++kk) {
-                        const uint64_t b = desc_advance(b0, kk * 2048);
-                        const uint32_t a_hi = a0 + 32u * (kk >> 1) + 8u * (kk & 1);
-                        umma_bf16_ta(t_o, a_hi, b, idesc_pv, (first && kk == 0) ? 0u : 1u);
-                        umma_bf16_ta(t_o, a_hi + 16u, b, idesc_pv, 1u);
-                    }
-                }
-                umma_commit(bars + Lay::B_PDONE + pb);
-                umma_commit(bars + Lay::B_VEMPTY + vs);
-            };
-
-            // Tiles are issued as S(g), PV(g-2), across unit boundaries: the scores
-            // of the tile after next are queued in the tensor pipe before the PV
-            // product that has to wait for the softmax of the current tile, so the
-            // softmax warps find S(g+1) ready when they finish tile g.  (S(g) reuses
-            // the buffer of tile g-3, whose PV product was issued one tile earlier.)
-            int g = 0, k = 0;
-            int lag_g[2] = {-1, -1}, lag_k[2] = {0, 0};   // tiles g-2 and g-1 awaiting PV
-            bool lag_first[2] = {false, false};
-            SegIter<SPLIT> it(wr);
-            for (Seg sg; it.next(p, sg); ++k) {
-                const int qs = k % Lay::QS;
-                mbar_wait(bars + Lay::B_QFULL + qs, (k / Lay::QS) & 1, abort_flag);
-                for (int j = sg.j0; j < sg.j1; ++j, ++g) {
-                    const int ks = g % Lay::KS;
-                    const int sb = g % Lay::NSB;
-                    mbar_wait(bars + Lay::B_KFULL + ks, (g / Lay::KS) & 1, abort_flag);
-                    // P(g - NSB) lives in this S buffer until its PV product is done
-                    if (g >= Lay::NSB)
-                        mbar_wait(bars + Lay::B_PDONE + sb, ((g - Lay::NSB) / Lay::NSB) & 1, abort_flag);
-                    tc_fence_after();
-                    if (!*abort_flag) {
-                        const uint64_t a0 = make_smem_desc(sq + qs * Lay::Q_BYTES, 16, 1024);
-                        const uint64_t b0 = make_smem_desc(sk + ks * Lay::TILE_BYTES, 16, 1024);
-                        const uint32_t d_s = tmem_base + Lay::T_S + sb * 128u;
-#pragma unroll
-                        for (int kk = 0; kk < D / 16; ++kk) {
-                            const uint32_t off = (kk >> 2) * Lay::GROUP_BYTES + (kk & 3) * 32;
-                            umma_bf16(d_s, desc_advance(a0, off), desc_advance(b0, off), idesc_qk,
-                                      kk > 0 ? 1u : 0u);
+                        for (int kk = 4 * half; kk < 4 * half + 4; ++kk) {
+                            const uint64_t b = desc_advance(b0, kk * 2048);
+                            const uint32_t a_hi = a0 + 32u * (kk >> 1) + 8u * (kk & 1);
+                            umma_bf16_ta(t_o, a_hi, b, idesc_pv, (p_first[s] && kk == 0) ? 0u : 1u);
+                            umma_bf16_ta(t_o, a_hi + 16u, b, idesc_pv, 1u);
                         }
                     }
-                    umma_commit(bars + Lay::B_SFULL + sb);
-                    umma_commit(bars + Lay::B_KEMPTY + ks);
-                    if (j == sg.j1 - 1) umma_commit(bars + Lay::B_QEMPTY + qs);
-                    if (lag_g[0] >= 0) issue_pv(lag_g[0], lag_first[0], lag_k[0]);
-                    lag_g[0] = lag_g[1];
-                    lag_first[0] = lag_first[1];
-                    lag_k[0] = lag_k[1];
-                    lag_g[1] = g;
-                    lag_first[1] = (j == sg.j0);
-                    lag_k[1] = k;
+                    if (half == 1) {
+                        if (p_frees[s]) umma_commit(bars + Lay::B_EMPTY + v.slot);
+                        if (p_last[s]) umma_commit(bars + Lay::B_DONE + s);
+                    }
+                }
+                __syncwarp();
+            }
+            p_par[s] ^= 1u;
+            pend[s] = false;
+        };
+
+        // S_s = Q K^T of one tile, after the stream's pending PV product (which reads
+        // the probabilities that the new scores replace: one thread's products execute
+        // in the order they are issued).  k_done: no later product reads the K tile;
+        // q_done: the job's last scores from Q slot qs.
+        auto issue_s = [&](auto s_c, int qs, const Pos &kp, const Pos &next_v, bool first, bool last, bool k_done, bool v_done,
+                           bool q_done, int job) {
+            constexpr int s = decltype(s_c)::value;
+            mbar_wait(bars + Lay::B_FULL + kp.slot, kp.phase, abort_flag);
+            // look for the next PV product's V tile now, while the tensor pipe still has
+            // queued work, and not right before that product
+            v_seen = mbar_test(bars + Lay::B_FULL + next_v.slot, next_v.phase);
+            tc_fence_after();
+            if (elect_one()) {
+                if (!dead) {
+                    const uint64_t a0 = desc_advance(dq0, qs * Lay::Q_BYTES);
+                    const uint64_t b0 = desc_advance(dk0, kp.slot * Lay::TILE_BYTES);
+                    const uint32_t d_s = tmem + Lay::T_S + s * 128u;
+#pragma unroll
+                    for (int kk = 0; kk < D / 16; ++kk) {
+                        const uint32_t off = (kk >> 2) * Lay::GROUP_BYTES + (kk & 3) * 32;
+                        umma_bf16(d_s, desc_advance(a0, off), desc_advance(b0, off), idesc_qk, kk > 0 ? 1u : 0u);
+                    }
+                }
+                umma_commit(bars + Lay::B_SFULL + s);
+                if (k_done) umma_commit(bars + Lay::B_EMPTY + kp.slot);
+                if (q_done) umma_commit(bars + Lay::B_QEMPTY + qs);
+            }
+            __syncwarp();
+            pend[s] = true;
+            p_first[s] = first;
+            p_last[s] = last;
+            p_frees[s] = v_done;
+            p_job[s] = job;
+        };
+
+        int g = 0, k = 0;
+        RowsIter<SPLIT> it(p, wr);
+        const bool pair = it.pair;
+        for (RowsJob jb;; ++k) {
+            const int n = warp_uniform(it.next(p, jb) ? jb.j1 - jb.j0 : 0);
+            if (n == 0) break;
+            if (!pair) {
+                const int qs = k & 1;
+                for (int j = 0; j < n; ++j, ++g) {
+                    auto tile = [&](auto s_c) {
+                        if (pend[decltype(s_c)::value]) issue_pv(s_c, false);
+                        if (j == 0) {
+                            mbar_wait(bars + Lay::B_QFULL + qs, (uint32_t)(k >> 1) & 1u, abort_flag);
+                            dead = warp_uniform(*abort_flag) != 0;
+                        }
+                        const Pos kp = pos;
+                        pos.advance();
+                        // a stream's last tile of the job is one of the job's last two
+                        issue_s(s_c, qs, kp, pos, j < 2, j + 2 >= n, true, true, j == n - 1, k);
+                    };
+                    if (g & 1) tile(b_t{});
+                    else tile(a_t{});
+                }
+            } else {
+                // K0 V0 K1 V1 ...; the job's last tile holds no key that a query of its first
+                // block may see (n >= 2), so stream A stops one tile earlier
+                for (int j = 0; j < n; ++j) {
+                    const bool first = j == 0, last = j == n - 1;
+                    const Pos kp = pos;
+                    pos.advance();
+                    const Pos vp = pos;
+                    pos.advance();
+                    if (pend[0]) issue_pv(a_t{}, true);
+                    if (!last) {
+                        if (first) {
+                            mbar_wait(bars + Lay::B_QFULL + 0, (uint32_t)k & 1u, abort_flag);
+                            dead = warp_uniform(*abort_flag) != 0;
+                        }
+                        issue_s(a_t{}, 0, kp, p_v[1], first, j == n - 2, false, false, j == n - 2, k);
+                        p_v[0] = vp;
+                    }
+                    if (pend[1]) issue_pv(b_t{}, true);
+                    if (first) mbar_wait(bars + Lay::B_QFULL + 1, (uint32_t)k & 1u, abort_flag);
+                    issue_s(b_t{}, 1, kp, p_v[0], first, last, true, true, last, k);
+                    p_v[1] = vp;
                 }
             }
-            for (int x = 0; x < 2; ++x)
-                if (lag_g[x] >= 0) issue_pv(lag_g[x], lag_first[x], lag_k[x]);
-            umma_commit(bars + Lay::B_DRAIN);
-            mbar_wait_drain(bars + Lay::B_DRAIN, 0);
         }
+        v_seen = false;
+        if (pair || !(g & 1)) {
+            if (pend[0]) issue_pv(a_t{}, pair);
+            if (pend[1]) issue_pv(b_t{}, pair);
+        } else {
+            if (pend[1]) issue_pv(b_t{}, false);
+            if (pend[0]) issue_pv(a_t{}, false);
+        }
+        if (elect_one()) umma_commit(bars + Lay::B_DRAIN);
+        __syncwarp();
+        mbar_wait_drain(bars + Lay::B_DRAIN, 0);
     } else {
         // ------------------------------------------------------------ softmax warps
-        const int qd = warp & 3;                 // TMEM lane quadrant of this warp
-        const int h = warp >> 2;                 // key half: keys [64h, 64h + 64) of a tile
-        const int q = qd * 32 + lane;            // query row (tree token) of this thread
-        const uint32_t lane_off = (uint32_t)(qd * 32) << 16;
+        const int s = warp >> 2;                 // stream
+        const int q = (warp & 3) * 32 + lane;    // query row of the block, and TMEM lane
+        const uint32_t lane_off = (uint32_t)((warp & 3) * 32) << 16;
+        const uint32_t t_s = tmem_base + lane_off + Lay::T_S + s * 128u;
+        const uint32_t t_os = tmem_base + lane_off + Lay::T_O + s * D;
         const float sl2 = p.scale_log2;
+        const uint64_t sl2x2 = pack2(sl2, sl2);
         const bool vec_out = (reinterpret_cast<uintptr_t>(p.out) & 15u) == 0;
         const bool out32 = (reinterpret_cast<uintptr_t>(p.out) & 31u) == 0;
+        constexpr int NW = kMaxTree / 32;
 
-        float m = -INFINITY;    // running maximum of the row (log2 units), same in both threads
-        float l = 0.f;          // this thread's share of the row sum
-        // anc[t] bit i: tree node 128t + 64h + i is an ancestor of (or is) this
-        // thread's query; tmask: the word of the current tree tile
-        uint64_t anc[kMaxTree / 128] = {};
-        uint64_t tmask = 0;
+        float m = -INFINITY;    // running maximum of the row (log2 units)
+        float l = 0.f;          // its row sum
+        // bit i of anc[w]: tree node 32w + i is an ancestor of (or is) this thread's query
+        // (indexed at run time, so it stays out of the registers)
+        uint32_t anc[NW] = {};
         int cur_key = -1;
-        int g = 0;
-        // a finished segment whose output still sits in TMEM; a partial one (a
-        // unit cut by the work split) goes to its slot instead of the output
-        // pend_f: bit 0 a segment is pending, bit 1 it is partial, bit 2 it was
-        // the range's first segment; pend_m, pend_l its row's maximum and sum
-        int pend_f = 0, pend_u = 0, pend_g = 0;
-        float pend_m = 0.f, pend_l = 0.f;
+        int g = 0;              // tiles of the CTA's jobs so far
+        uint32_t s_par = 0, d_par = 0;   // phase parities: scores; bit x: stream x's jobs done
 
-
-        // Probabilities of this thread's 64 keys from its raw scores s against the
-        // maximum mx (exponents clamped at 64), split into bf16 hi + lo and stored
-        // over the scores in TMEM; `lt` gets their sum and `maxd` the largest
-        // unclamped exponent.
-        auto emit = [&](auto kind_c, const uint32_t (&s)[4][16], float mx, int n_valid,
-                        uint32_t t_s, float &lt, float &maxd) {
-            constexpr int KIND = decltype(kind_c)::value;
-            float lt4[4] = {0.f, 0.f, 0.f, 0.f};
-            float md2[2] = {-INFINITY, -INFINITY};
+        // Probabilities of 32 keys from their raw scores r against the maximum, split
+        // into bf16 hi (truncated) + lo and stored over the scores.
+        auto emit = [&](auto bits_c, const uint32_t (&r)[32], uint32_t bits, uint64_t negm, uint32_t t_dst,
+                        uint64_t (&sum)[2]) {
+            constexpr bool BITS = decltype(bits_c)::value != 0;
+            uint32_t w[32];
 #pragma unroll
-            for (int c = 0; c < 2; ++c) {
-                uint32_t wh[16], wl[16];
-#pragma unroll
-                for (int e = 0; e < 32; e += 2) {
-                    float pv[2];
-                    uint32_t hb[2];
-#pragma unroll
-                    for (int x = 0; x < 2; ++x) {
-                        const int i = 32 * c + e + x;          // key 64h + i of the tile
-                        float d = fmaf(__uint_as_float(s[i >> 4][i & 15]), sl2, -mx);
-                        if (KIND == kMaskRows) d = (64 * h + i < n_valid) ? d : -INFINITY;
-                        if (KIND == kMaskTree) d = ((tmask >> i) & 1ull) ? d : -INFINITY;
-                        md2[x] = fmaxf(md2[x], d);
-                        pv[x] = ex2(fminf(d, 64.f));
-                        lt4[(e >> 1) & 3] += pv[x];
-                        hb[x] = __float_as_uint(pv[x]) & 0xFFFF0000u;
-                    }
-                    wh[e >> 1] = __byte_perm(hb[0], hb[1], 0x7632);
-                    const __nv_bfloat162 lo = __floats2bfloat162_rn(pv[0] - __uint_as_float(hb[0]),
-                                                                    pv[1] - __uint_as_float(hb[1]));
-                    wl[e >> 1] = *reinterpret_cast<const uint32_t *>(&lo);
+            for (int e = 0; e < 32; e += 2) {
+                const uint64_t d = fma2(pack2(__uint_as_float(r[e]), __uint_as_float(r[e + 1])), sl2x2, negm);
+                float d0, d1;
+                unpack2(d, d0, d1);
+                if (BITS) {
+                    d0 = ((bits >> e) & 1u) ? d0 : -INFINITY;
+                    d1 = ((bits >> (e + 1)) & 1u) ? d1 : -INFINITY;
                 }
-                tmem_st16(t_s + 32u * c, wh);
-                tmem_st16(t_s + 32u * c + 16u, wl);
+                const float p0 = ex2(d0), p1 = ex2(d1);
+                const uint64_t pp = pack2(p0, p1);
+                sum[(e >> 1) & 1] = add2(sum[(e >> 1) & 1], pp);
+                const uint32_t u0 = __float_as_uint(p0), u1 = __float_as_uint(p1);
+                w[e >> 1] = __byte_perm(u0, u1, 0x7632);
+                // minus the hi parts
+                const uint64_t nh = pack2(__uint_as_float((u0 & 0xFFFF0000u) ^ 0x80000000u),
+                                          __uint_as_float((u1 & 0xFFFF0000u) ^ 0x80000000u));
+                float l0, l1;
+                unpack2(add2(pp, nh), l0, l1);
+                const __nv_bfloat162 lo = __floats2bfloat162_rn(l0, l1);
+                w[16 + (e >> 1)] = *reinterpret_cast<const uint32_t *>(&lo);
             }
-            lt = (lt4[0] + lt4[1]) + (lt4[2] + lt4[3]);
-            maxd = fmaxf(md2[0], md2[1]);
+            tmem_st32(t_dst, w);
         };
 
-        // Largest visible scaled score among this thread's 64 keys.
-        auto part_max = [&](auto kind_c, const uint32_t (&s)[4][16], int n_valid) {
-            constexpr int KIND = decltype(kind_c)::value;
-            float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+        // Largest of 32 raw scores (the visible ones) and mx.
+        auto chunk_max = [&](auto bits_c, const uint32_t (&r)[32], uint32_t bits, float mx) {
+            constexpr bool BITS = decltype(bits_c)::value != 0;
+            float a = mx, b = -INFINITY;
 #pragma unroll
-            for (int i = 0; i < 64; ++i) {
-                const float v = __uint_as_float(s[i >> 4][i & 15]) * sl2;
-                bool vis = true;
-                if (KIND == kMaskRows) vis = 64 * h + i < n_valid;
-                if (KIND == kMaskTree) vis = ((tmask >> i) & 1ull) != 0;
-                mx[i & 3] = fmaxf(mx[i & 3], vis ? v : -INFINITY);
+            for (int e = 0; e < 32; e += 4) {
+                float v[4];
+#pragma unroll
+                for (int x = 0; x < 4; ++x) {
+                    v[x] = __uint_as_float(r[e + x]);
+                    if (BITS) v[x] = ((bits >> (e + x)) & 1u) ? v[x] : -INFINITY;
+                }
+                a = max3(a, v[0], v[1]);
+                b = max3(b, v[2], v[3]);
             }
-            return fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
+            return fmaxf(a, b);
         };
 
-        // Output of a finished unit: this thread's half of the row of O times 1 / l;
-        // then O is free for the next unit's first PV product.
-        auto read_back = [&](int lbh_out, int qb_out, int g_last, float linv) {
-            mbar_wait(bars + Lay::B_PDONE + g_last % Lay::NSB, (g_last / Lay::NSB) & 1, abort_flag);
-            tc_fence_after();
-            const uint32_t t_o = tmem_base + lane_off + Lay::T_O + (uint32_t)h * (D / 2);
-            const int qg = qb_out * Lay::M + q;
-            float *orow = p.out + ((size_t)lbh_out * T + qg) * D + h * (D / 2);
-            // the half row in two round trips to TMEM, then full-sector stores
-            uint32_t r[2][16];
-#pragma unroll
-            for (int c2 = 0; c2 < D / 32; c2 += 2) {
-#pragma unroll
-                for (int ch = 0; ch < 2; ++ch) tmem_ld16(t_o + (c2 + ch) * 16, r[ch]);
-                tmem_wait_ld();
-                if (qg >= T) continue;
-#pragma unroll
-                for (int ch = 0; ch < 2; ++ch) {
-                    if (out32) {
-#pragma unroll
-                        for (int e = 0; e < 16; e += 8)
-                            st_global_v8(orow + (c2 + ch) * 16 + e, r[ch] + e, linv);
-                    } else if (vec_out) {
-#pragma unroll
-                        for (int e = 0; e < 16; e += 4)
-                            *reinterpret_cast<float4 *>(orow + (c2 + ch) * 16 + e) =
-                                make_float4(__uint_as_float(r[ch][e]) * linv, __uint_as_float(r[ch][e + 1]) * linv,
-                                            __uint_as_float(r[ch][e + 2]) * linv,
-                                            __uint_as_float(r[ch][e + 3]) * linv);
-                    } else {
-#pragma unroll
-                        for (int e = 0; e < 16; ++e) orow[(c2 + ch) * 16 + e] = __uint_as_float(r[ch][e]) * linv;
-                    }
-                }
-            }
+        // Half of a tile's probabilities (and any rescaled O) are in TMEM.
+        auto p_ready = [&](int half) {
+            tmem_wait_st();
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(bars + Lay::B_OFREE);
+            if (lane == 0) mbar_arrive(bars + Lay::B_PFULL + 2 * s + half);
         };
 
-        // Partial state of a cut unit into slot `slot`: this thread's half of the
-        // row of O unnormalised, and (h == 0) the row's maximum and sum; then O
-        // is free.  Slots are 256-byte aligned rows of D floats.
-        const size_t slot_floats = split_slot_floats(D);
-        auto write_partial = [&](int slot, int qb_out, int g_last, float rm, float rl) {
-            mbar_wait(bars + Lay::B_PDONE + g_last % Lay::NSB, (g_last / Lay::NSB) & 1, abort_flag);
+        // One tile of the stream: scores in TMEM to probabilities in TMEM.
+        auto softmax_tile = [&](auto bits_c, const uint32_t (&bits)[4], bool first) {
+            constexpr bool BITS = decltype(bits_c)::value != 0;
+            uint32_t r[4][32];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) tmem_ld32(t_s + 32 * c, r[c]);
+            float mx = -INFINITY;
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                tmem_wait_ld32(r[c]);
+                mx = chunk_max(bits_c, r[c], bits[c], mx);
+            }
+            mx *= sl2;   // sl2 > 0
+            const bool up = mx > m + 16.f || (first && mx > m);
+            float alpha = 1.f;
+            if (up) {
+                alpha = ex2(m - mx);   // 0 from -inf
+                m = mx;
+            }
+            if (!first && __any_sync(0xffffffffu, up)) {
+                // rescale this row of O: the PV product of the stream's tile before is
+                // complete (it was issued before these scores' product)
+                tc_fence_after();
+#pragma unroll 1
+                for (int ch = 0; ch < D / 16; ++ch) {
+                    uint32_t o[16];
+                    tmem_ld16(t_os + ch * 16, o);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
+                    tmem_st16(t_os + ch * 16, o);
+                }
+                l *= alpha;
+            }
+            const uint64_t negm = pack2(-m, -m);
+            uint64_t sum[2] = {0ull, 0ull};
+            // the scores are read again, half a tile at a time in one rolled loop: unrolled
+            // over the tile, the code of eight warps at different places did not fit the
+            // instruction caches
+#pragma unroll 1
+            for (int half = 0; half < 2; ++half) {
+                const uint32_t t_h = t_s + 64u * (uint32_t)half;
+                uint32_t ra[32], rb[32];
+                tmem_ld32(t_h, ra);
+                tmem_ld32(t_h + 32, rb);
+                const uint32_t b0 = BITS && half ? bits[2] : bits[0], b1 = BITS && half ? bits[3] : bits[1];
+                tmem_wait_ld32(ra);
+                tmem_wait_ld32(rb);
+                emit(bits_c, ra, b0, negm, t_h, sum);
+                emit(bits_c, rb, b1, negm, t_h + 32, sum);
+                p_ready(half);
+            }
+            float l0, l1;
+            unpack2(add2(sum[0], sum[1]), l0, l1);
+            l += l0 + l1;
+        };
+
+        // 32 output values of row `orow` at `scale`.
+        auto store32 = [&](float *dst, const uint32_t (&r)[32], float scale) {
+            if (out32) {
+#pragma unroll
+                for (int e = 0; e < 32; e += 8) st_global_v8(dst + e, r + e, scale);
+            } else if (vec_out) {
+#pragma unroll
+                for (int e = 0; e < 32; e += 4)
+                    *reinterpret_cast<float4 *>(dst + e) =
+                        make_float4(__uint_as_float(r[e]) * scale, __uint_as_float(r[e + 1]) * scale,
+                                    __uint_as_float(r[e + 2]) * scale, __uint_as_float(r[e + 3]) * scale);
+            } else {
+#pragma unroll
+                for (int e = 0; e < 32; ++e) dst[e] = __uint_as_float(r[e]) * scale;
+            }
+        };
+
+        auto wait_done = [&](int st) {
+            mbar_wait(bars + Lay::B_DONE + st, (d_par >> st) & 1u, abort_flag);
+            d_par ^= 1u << st;
+        };
+        auto o_free = [&](int st, uint32_t n) {   // this warp has read stream st's output (n arrivals)
+            if (lane == 0) mbar_arrive_n(bars + Lay::B_OFREE + st, n);
+        };
+
+        // End of a pair job: this stream's block of 128 rows.
+        auto finish_pair = [&](const RowsJob &jb) {
+            const int qg = (jb.ui.qb + s) * Lay::M + q;
+            if (qg < T && p.lse) p.lse[(size_t)jb.ui.lbh * T + qg] = (m + lg2(l)) * 0.69314718055994530942f;
+            const float linv = rcp(l);
+            float *orow = p.out + ((size_t)jb.ui.lbh * T + qg) * D;
+            wait_done(s);
             tc_fence_after();
-            const uint32_t t_o = tmem_base + lane_off + Lay::T_O + (uint32_t)h * (D / 2);
-            float *base = p.split_part + (size_t)slot * slot_floats;
-            float *orow = base + (size_t)q * D + h * (D / 2);
-            const bool live = qb_out * Lay::M + q < T;
-            uint32_t r[2][16];
 #pragma unroll
-            for (int c2 = 0; c2 < D / 32; c2 += 2) {
-#pragma unroll
-                for (int ch = 0; ch < 2; ++ch) tmem_ld16(t_o + (c2 + ch) * 16, r[ch]);
-                tmem_wait_ld();
-                if (live) {
-#pragma unroll
-                    for (int ch = 0; ch < 2; ++ch)
-#pragma unroll
-                        for (int e = 0; e < 16; e += 8)
-                            st_global_v8(orow + (c2 + ch) * 16 + e, r[ch] + e, 1.f);
+            for (int c = 0; c < D; c += 64) {
+                uint32_t r0[32], r1[32];
+                tmem_ld32(t_os + c, r0);
+                tmem_ld32(t_os + c + 32, r1);
+                tmem_wait_ld32(r0);
+                tmem_wait_ld32(r1);
+                if (c + 64 == D) {
+                    tc_fence_before();
+                    __syncwarp();
+                    o_free(s, 2);
+                }
+                if (qg < T) {
+                    store32(orow + c, r0, linv);
+                    store32(orow + c + 32, r1, linv);
                 }
             }
-            if (h == 0 && live) {
-                base[(size_t)kSplitRows * D + q] = rm;
-                base[(size_t)kSplitRows * D + kSplitRows + q] = rl;
+        };
+
+        // End of a single job: the row's two partial states (one per stream) merged;
+        // this thread writes half of the row, stream A's the first D / 2 columns.  `st0`:
+        // the stream of the job's first tile, `both`: the other one had tiles too.
+        auto finish_single = [&](const RowsJob &jb, int st0, bool both, int slot) {
+            named_bar_sync(1, 256);   // the job before is done with the exchange
+            xs[s * Lay::M + q] = make_float2(m, l);
+            named_bar_sync(1, 256);
+            const float2 xo = xs[(s ^ 1) * Lay::M + q];
+            const float mt = fmaxf(m, xo.x);
+            // a stream without tiles, or whose tiles hide every key from this row, has
+            // weight 0; its accumulator may hold anything then
+            const float w_own = m == -INFINITY ? 0.f : ex2(m - mt);
+            const float w_oth = xo.x == -INFINITY ? 0.f : ex2(xo.x - mt);
+            const float lt = w_own * l + w_oth * xo.y;
+            const int qg = jb.ui.qb * Lay::M + q;
+            const bool whole = !SPLIT || (jb.j0 == 0 && jb.j1 == jb.ui.n_tiles);
+            const float inv = whole ? rcp(lt) : 1.f;
+            float *dst;
+            if (whole) {
+                if (s == 0 && qg < T && p.lse)
+                    p.lse[(size_t)jb.ui.lbh * T + qg] = (mt + lg2(lt)) * 0.69314718055994530942f;
+                dst = p.out + ((size_t)jb.ui.lbh * T + qg) * D;
+            } else {
+                // a part of a cut unit: the unnormalised row, its maximum and its sum
+                float *base = p.split_part + (size_t)slot * split_slot_floats(D);
+                if (s == 0 && qg < T) {
+                    base[(size_t)kSplitRows * D + q] = mt;
+                    base[(size_t)kSplitRows * D + kSplitRows + q] = lt;
+                }
+                dst = base + (size_t)q * D;
             }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bars + Lay::B_OFREE);
+            dst += s * (D / 2);
+            const float fa = (s == 0 ? w_own : w_oth) * inv, fb = (s == 0 ? w_oth : w_own) * inv;
+            const bool has_a = both || st0 == 0, has_b = both || st0 == 1;
+            if (has_a) wait_done(0);
+            if (has_b) wait_done(1);
+            tc_fence_after();
+            const uint32_t t_o = tmem_base + lane_off + Lay::T_O + (uint32_t)s * (D / 2);
+#pragma unroll
+            for (int c = 0; c < D / 2; c += 32) {
+                uint32_t r0[32], r1[32];
+                tmem_ld32(t_o + c, r0);
+                tmem_ld32(t_o + D + c, r1);
+                tmem_wait_ld32(r0);
+                tmem_wait_ld32(r1);
+                if (c + 32 == D / 2) {
+                    tc_fence_before();
+                    __syncwarp();
+                    o_free(0, 1);
+                    o_free(1, 1);
+                }
+                if (qg < T) {
+#pragma unroll
+                    for (int e = 0; e < 32; ++e) {
+                        const float a = fa != 0.f ? __uint_as_float(r0[e]) * fa : 0.f;
+                        r0[e] = __float_as_uint(fb != 0.f ? fmaf(__uint_as_float(r1[e]), fb, a) : a);
+                    }
+                    store32(dst + c, r0, 1.f);
+                }
+            }
         };
 
-        // The pending segment: a whole unit's output, or a part's state (counted
-        // in at the end of the range).
-        auto flush_pending = [&]() {
-            const int lbh_o = pend_u / p.n_qb, qb_o = pend_u - lbh_o * p.n_qb;
-            if (!SPLIT || !(pend_f & 2)) read_back(lbh_o, qb_o, pend_g, rcp(pend_l));
-            else write_partial(2 * (int)blockIdx.x + ((pend_f & 4) ? 0 : 1), qb_o, pend_g, pend_m, pend_l);
-        };
-
+        RowsIter<SPLIT> it(p, wr);
         int k = 0;
-        SegIter<SPLIT> it(wr);
-        for (Seg sg; it.next(p, sg); ++k) {
-            const UnitInfo &ui = sg.ui;
-            const int qg = ui.qb * Lay::M + q;   // this thread's tree token
-            if (ui.b * p.n_qb + ui.qb != cur_key) {
-                // ancestors of node qg among tree nodes 128t + [64h, 64h + 64)
+        for (RowsJob jb; it.next(p, jb); ++k) {
+            const UnitInfo &ui = jb.ui;
+            const int qb = ui.qb + (jb.pair ? s : 0);
+            const int qg = qb * Lay::M + q;   // this thread's tree token
+            if (ui.b * p.n_qb + qb != cur_key) {
 #pragma unroll
-                for (int t = 0; t < kMaxTree / 128; ++t) anc[t] = 0;
+                for (int w = 0; w < NW; ++w) anc[w] = 0;
                 if (qg < T) {
                     bool bad = false;
                     int a = qg;
                     while (true) {
-                        if (((a >> 6) & 1) == h) {
-#pragma unroll
-                            for (int t = 0; t < kMaxTree / 128; ++t)
-                                if ((a >> 7) == t) anc[t] |= 1ull << (a & 63);
-                        }
+                        anc[a >> 5] |= 1u << (a & 31);
                         const int pa = __ldg(p.parent + (size_t)ui.b * T + a);
                         if (a == 0) {
                             bad = (pa != -1);
@@ -505,131 +780,79 @@ tree_attention_rows_kernel(const __grid_constant__ CUtensorMap map_q,
                         }
                         a = pa;
                     }
-                    if (bad && h == 0 && p.dev_status) p.dev_status[ui.b] = kErrTree;
+                    if (bad && p.dev_status) p.dev_status[ui.b] = kErrTree;
                 }
-                if (qg == 0 && h == 0 && p.dev_status && (ui.P_raw < 0 || ui.P_raw > p.S_max))
+                if (qg == 0 && p.dev_status && (ui.P_raw < 0 || ui.P_raw > p.S_max))
                     p.dev_status[ui.b] = kErrCapacity;
-                cur_key = ui.b * p.n_qb + ui.qb;
+                cur_key = ui.b * p.n_qb + qb;
             }
 
-            for (int j = sg.j0; j < sg.j1; ++j, ++g) {
+            const int n = jb.j1 - jb.j0;
+            const int st0 = g & 1;   // single job: the stream of its first tile
+            // this stream's tiles of the job: all of a pair's, every other one of a single's
+            // (stream A's queries see nothing of a pair's last tree tile)
+            const int n_s = jb.pair && s == 0 ? n - 1 : n;
+            for (int i = jb.pair ? 0 : (s ^ st0); i < n_s; i += jb.pair ? 1 : 2) {
+                const int j = jb.j0 + i;
                 const bool tree = (j >= ui.n_pref);
                 const int n_valid = tree ? T : min(Lay::KT, ui.P - j * Lay::KT);
-                if (tree) {
-#pragma unroll
-                    for (int t = 0; t < kMaxTree / 128; ++t)
-                        if (j - ui.n_pref == t) tmask = anc[t];
-                }
-                const int kind = tree ? kMaskTree : (n_valid < Lay::KT ? kMaskRows : kMaskNone);
-                const int sb = g % Lay::NSB;
-                mbar_wait(bars + Lay::B_SFULL + sb, (g / Lay::NSB) & 1, abort_flag);
+                const bool first = i < (jb.pair ? 1 : 2);
+                mbar_wait(bars + Lay::B_SFULL + s, s_par, abort_flag);
+                s_par ^= 1u;
                 tc_fence_after();
-                const uint32_t t_s = tmem_base + lane_off + Lay::T_S + (uint32_t)sb * 128u +
-                                     (uint32_t)h * 64u;
-                uint32_t s[4][16];
+                if (!tree && n_valid == Lay::KT) {
+                    const uint32_t all[4] = {~0u, ~0u, ~0u, ~0u};
+                    softmax_tile(kind_t<0>{}, all, first);
+                } else {
+                    uint32_t bits[4];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) tmem_ld16(t_s + 16u * i, s[i]);
-                tmem_wait_ld();
-
-                float lt = 0.f;
-                bool exact = (j == sg.j0);
-                if (!exact) {
-                    // optimistic pass against the current maximum
-                    float maxd = -INFINITY;
-                    if (kind == kMaskNone) emit(kind_t<kMaskNone>{}, s, m, n_valid, t_s, lt, maxd);
-                    else if (kind == kMaskRows) emit(kind_t<kMaskRows>{}, s, m, n_valid, t_s, lt, maxd);
-                    else emit(kind_t<kMaskTree>{}, s, m, n_valid, t_s, lt, maxd);
-                    exact = named_bar_or(1, 256, maxd > 16.f);
-                }
-                if (exact) {
-                    float pm;
-                    if (kind == kMaskNone) pm = part_max(kind_t<kMaskNone>{}, s, n_valid);
-                    else if (kind == kMaskRows) pm = part_max(kind_t<kMaskRows>{}, s, n_valid);
-                    else pm = part_max(kind_t<kMaskTree>{}, s, n_valid);
-                    xm[h * Lay::M + q] = pm;
-                    named_bar_sync(1, 256);
-                    const float mn = fmaxf(m, fmaxf(xm[q], xm[Lay::M + q]));
-                    const float alpha = (mn == m) ? 1.f : ex2(m - mn);
-                    if (j > sg.j0) {
-                        if (__any_sync(0xffffffffu, alpha != 1.f)) {
-                            // rescale this thread's half of the row of O once the PV
-                            // product of the previous tile has landed
-                            mbar_wait(bars + Lay::B_PDONE + (g - 1) % Lay::NSB,
-                                      ((g - 1) / Lay::NSB) & 1, abort_flag);
-                            tc_fence_after();
-                            const uint32_t t_o = tmem_base + lane_off + Lay::T_O + (uint32_t)h * (D / 2);
+                    for (int c = 0; c < 4; ++c) {
+                        const int left = n_valid - 32 * c;
+                        bits[c] = left >= 32 ? ~0u : (left > 0 ? (1u << left) - 1u : 0u);
+                        if (tree) bits[c] = anc[4 * (j - ui.n_pref) + c];
+                    }
+                    // V rows of invisible keys in a partial prefix tile may be NaN: zero them
+                    // (a pair's tile once, by stream A, whose PV product comes first)
+                    if (!tree && (!jb.pair || s == 0)) {
+                        const int e = g + i;
+                        int pos;   // the V tile's place in the ring order
+                        if (jb.pair) pos = 2 * e + 1;
+                        else pos = (SPLIT && e == wr.n_tiles - 1) ? 2 * e + 1 : 2 * e + 2;
+                        const int vs = pos % Lay::RS;
+                        mbar_wait(bars + Lay::B_FULL + vs, (uint32_t)(pos / Lay::RS) & 1u, abort_flag);
+                        if (q >= n_valid) {
+                            const uint32_t vrow = smem_addr(smem + Lay::OFF_R + vs * Lay::TILE_BYTES) + q * 128u;
 #pragma unroll
-                            for (int ch = 0; ch < D / 32; ++ch) {
-                                uint32_t r[16];
-                                tmem_ld16(t_o + ch * 16, r);
-                                tmem_wait_ld();
+                            for (int c = 0; c < Lay::DCH; ++c)
 #pragma unroll
-                                for (int e = 0; e < 16; ++e)
-                                    r[e] = __float_as_uint(__uint_as_float(r[e]) * alpha);
-                                tmem_st16(t_o + ch * 16, r);
-                            }
+                                for (int x = 0; x < 8; ++x)
+                                    st_shared_v4(vrow + c * Lay::GROUP_BYTES + x * 16, 0u, 0u, 0u, 0u);
                         }
-                        l *= alpha;
+                        fence_proxy_async_smem();
                     }
-                    m = mn;
-                    tmem_wait_st();   // optimistic probabilities are overwritten below
-                    float unused;
-                    if (kind == kMaskNone) emit(kind_t<kMaskNone>{}, s, m, n_valid, t_s, lt, unused);
-                    else if (kind == kMaskRows) emit(kind_t<kMaskRows>{}, s, m, n_valid, t_s, lt, unused);
-                    else emit(kind_t<kMaskTree>{}, s, m, n_valid, t_s, lt, unused);
-                }
-                l += lt;
-
-                // V rows of invisible keys in a partial prefix tile may be NaN: zero them
-                if (kind == kMaskRows && h == 0) {
-                    const int vs = g % Lay::VS;
-                    mbar_wait(bars + Lay::B_VFULL + vs, (g / Lay::VS) & 1, abort_flag);
-                    if (q >= n_valid) {
-                        const uint32_t vrow = smem_addr(smem + Lay::OFF_V + vs * Lay::TILE_BYTES) + q * 128u;
-#pragma unroll
-                        for (int c = 0; c < Lay::DCH; ++c)
-#pragma unroll
-                            for (int x = 0; x < 8; ++x)
-                                st_shared_v4(vrow + c * Lay::GROUP_BYTES + x * 16, 0u, 0u, 0u, 0u);
-                    }
-                }
-                tmem_wait_st();
-                fence_proxy_async_smem();
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(bars + Lay::B_PFULL + sb);
-
-                // the previous segment's output, once this segment's first tile is on its way
-                if (j == sg.j0 && pend_f) {
-                    flush_pending();
-                    pend_f = 0;
-                }
-
-                if (j == sg.j1 - 1) {
-                    // ------------------------------------------ segment end: row sum, LSE
-                    xl[h * Lay::M + q] = l;
-                    named_bar_sync(1, 256);
-                    const float L = xl[q] + xl[Lay::M + q];
-                    if ((!SPLIT || seg_whole(sg)) && h == 0 && qg < T && p.lse)
-                        p.lse[(size_t)ui.lbh * T + qg] = (m + lg2(L)) * 0.69314718055994530942f;
-                    pend_u = sg.u;
-                    pend_g = g;
-                    pend_m = m;
-                    pend_l = L;
-                    pend_f = 1;
-                    if (SPLIT && !seg_whole(sg)) {
-                        // a part: slot 2c for the tail range's first segment, 2c + 1 for its last
-                        pend_f |= 2 | (sg.u == wr.u_first ? 4 : 0);
-                        // the part holding the unit's first tile records it for the merge
-                        if (sg.j0 == 0 && threadIdx.x == 0)
-                            p.split_rec[blockIdx.x] = SplitRecord{seg_unit_origin(wr, it, sg), wr.n_tail, sg.u, ui.n_tiles};
-                    }
-                    m = -INFINITY;
-                    l = 0.f;
+                    softmax_tile(kind_t<1>{}, bits, first);
                 }
             }
+            g += n;
+
+            if (jb.pair) {
+                finish_pair(jb);
+            } else {
+                int slot = 0;
+                if (SPLIT && !(jb.j0 == 0 && jb.j1 == ui.n_tiles)) {
+                    // a part: slot 2c for the range's first segment, 2c + 1 for its last
+                    const int u = ui.lbh * p.n_qb + ui.qb;
+                    slot = 2 * (int)blockIdx.x + (u == wr.u_first ? 0 : 1);
+                    // the part holding the unit's first tile records it for the merge
+                    if (jb.j0 == 0 && threadIdx.x == 0)
+                        p.split_rec[blockIdx.x] =
+                            SplitRecord{wr.x_first + (wr.n_tiles - it.seg.left) - jb.j1, wr.n_tail, u, ui.n_tiles};
+                }
+                finish_single(jb, st0, n >= 2, slot);
+            }
+            m = -INFINITY;
+            l = 0.f;
         }
-        if (pend_f) flush_pending();
     }
 
     tc_fence_before();
@@ -645,13 +868,31 @@ tree_attention_rows_kernel(const __grid_constant__ CUtensorMap map_q,
 }
 
 template <int D>
-static cudaError_t launch_rows_t(const AttnMaps &m, const AttnParams &p, int num_sms,
+static cudaError_t launch_rows_t(const AttnMaps &m, const AttnParams &p0, int num_sms,
                                  bool programmatic, cudaStream_t stream)
 {
     static std::atomic<uint64_t> configured[2] = {{0}, {0}};
-    if (p.split)
+    if (p0.split)
         return launch_attention_grid(tree_attention_rows_kernel<D, true>, RowsLayout<D>::SMEM_BYTES, 352,
-                                     configured[1], m, p, num_sms, programmatic, stream);
+                                     configured[1], m, p0, num_sms, programmatic, stream);
+    AttnParams p = p0;
+    if (p.n_qb == 3) {
+        // the split of the CTAs with the shortest longest queue, a pair counted as 2 n + 4
+        // and a single block as n + 4.5 tiles of 128 x 128 with n prefix tiles (S_max
+        // standing in for the device-side prefix lengths): three and three tree tiles, and
+        // the end of a job, which only a pair's other stream overlaps
+        const long long n = p.n_units / 3, grid = attention_grid(p, num_sms), np = (p.S_max + 127) / 128;
+        long long best = -1;
+        for (long long g = 1; g < grid; ++g) {
+            const long long pairs = (4 * np + 8) * ((n + g - 1) / g);
+            const long long singles = (2 * np + 9) * ((n + grid - g - 1) / (grid - g));
+            const long long t = pairs > singles ? pairs : singles;
+            if (best < 0 || t <= best) {
+                best = t;
+                p.pair_grid = (int)g;
+            }
+        }
+    }
     return launch_attention_grid(tree_attention_rows_kernel<D, false>, RowsLayout<D>::SMEM_BYTES, 352,
                                  configured[0], m, p, num_sms, programmatic, stream);
 }

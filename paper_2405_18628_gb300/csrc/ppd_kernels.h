@@ -82,6 +82,7 @@ struct AttnParams {
     int L, B, H, T, T_pad, S_max, n_units;
     int n_qb;                   // query blocks of 128 per (layer, sequence, head) slice
     int n_tt;                   // tree-key tiles of 128 per slice
+    int pair_grid;              // query-row kernel, n_qb 3: CTAs that take the slices' pairs of blocks
     float scale_log2;           // softmax scale * log2(e)
     // Work split: split != 0 shares the units left after the full round-robin
     // rounds out by their key tiles (B <= kSplitMaxB); units cut by a range
@@ -112,7 +113,17 @@ struct SplitRecord {
     int u, n_tiles;
 };
 
-// CTAs of an attention launch: one per SM, at most one per unit (with the
+// Jobs of a launch without the work split: its units, except that the
+// query-row kernel takes two blocks of queries of a slice as one job (n_qb 2 to
+// 4: one, two -- a pair and a single block -- and two jobs a slice).
+inline long long whole_jobs(const AttnParams &p)
+{
+    if (p.T_pad <= 64 || p.n_qb == 1) return p.n_units;
+    const long long slices = p.n_units / p.n_qb;
+    return p.n_qb == 2 ? slices : 2 * slices;
+}
+
+// CTAs of an attention launch: one per SM, at most one per job (with the
 // work split: at most one per tile, and kSplitMaxGrid).
 inline int attention_grid(const AttnParams &p, int num_sms)
 {
@@ -122,7 +133,8 @@ inline int attention_grid(const AttnParams &p, int num_sms)
         grid = grid < kSplitMaxGrid ? grid : kSplitMaxGrid;
         grid = grid < max_tiles ? grid : max_tiles;
     } else {
-        grid = grid < p.n_units ? grid : p.n_units;
+        const long long jobs = whole_jobs(p);
+        grid = grid < jobs ? grid : jobs;
     }
     return (int)grid;
 }

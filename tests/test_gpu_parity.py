@@ -189,6 +189,33 @@ def test_attention_trees_over_128_tokens(cuda_device, T, P, D):
                                atol=1e-3)
 
 
+@pytest.mark.parametrize("T,D,P", [
+    (65, 128, [0, 128]),       # one block of queries: a job of one tile, its other stream idle
+    (128, 64, [127, 1]),
+    (129, 128, [0, 129]),      # pairs; the second block holds one query
+    (256, 64, [257, 128]),
+    (257, 64, [130, 0]),       # pairs and single third blocks side by side
+    (384, 128, [1, 140]),
+    (385, 64, [129, 0]),       # two pairs a slice
+    (512, 64, [0, 200]),
+])
+def test_attention_rows_many_jobs(cuda_device, T, D, P):
+    """More jobs than SMs in every form of the query-row kernel (single blocks,
+    pairs, both), at the edges of its blocks and key tiles."""
+    w = W.Workload("jobs", L=4, B=2, H=44, D=D, P=max(P), T=T, V=16, n_cand=(T + 3) // 4,
+                   max_depth=6, chains="fill3", match_rate=0.5, seed=T)
+    pl = np.asarray(P, np.int32)
+    s = W.make_step_inputs(w, prefix_len=pl)
+    t = tensors(w, prefix_len=pl)
+    out, lse, st = run_attention({k: v.to(cuda_device) for k, v in t.items()}, pl, s.parent,
+                                 cuda_device)
+    ref, ref_lse, _, ref_st = oracle.tree_attention(t["q"], t["k_cache"], t["v_cache"], t["k_tree"],
+                                                    t["v_tree"], pl, s.parent)
+    assert (st.cpu().numpy() == 0).all() and (ref_st == 0).all()
+    assert_attn_close(out.cpu().numpy().reshape(ref.shape), ref, f"T={T} D={D}")
+    np.testing.assert_allclose(lse.cpu().numpy().reshape(ref_lse.shape), ref_lse, rtol=0, atol=1e-3)
+
+
 def test_attention_peaked_scores_and_scale(cuda_device):
     """Large scores force the running-max rescale path on later tiles."""
     w = W.scaled(W.WORKLOADS["vicuna7b"], L=1, H=2, P=1000)
