@@ -179,6 +179,20 @@ PPD_DEV void prefetch_first_tiles(const AttnParams &p, int lane, const CUtensorM
     }
 }
 
+// Position in a ring of tile slots: slot and the parity of its current phase.
+template <int RS>
+struct RingPos {
+    int slot = 0;
+    uint32_t phase = 0;
+    PPD_DEV void advance()
+    {
+        if (++slot == RS) {
+            slot = 0;
+            phase ^= 1u;
+        }
+    }
+};
+
 // One stretch of a unit's tiles [j0, j1) processed by this CTA.
 struct Seg {
     UnitInfo ui;

@@ -84,7 +84,7 @@ struct RowsLayout {
     static constexpr int B_SFULL = B_EMPTY + RS;    // [2] scores of the stream's tile in TMEM
     static constexpr int B_PFULL = B_SFULL + 2;     // [2][2] its probabilities, keys 0-63 and 64-127, in TMEM (4 warps)
     static constexpr int B_DONE = B_PFULL + 4;      // [2] the stream's last PV product of a job complete
-    static constexpr int B_OFREE = B_DONE + 2;      // [2] a job's output read back from TMEM (8 arrivals)
+    static constexpr int B_OFREE = B_DONE + 2;      // [2] a stream's output of a job read back from TMEM (8 arrivals)
     static constexpr int B_DRAIN = B_OFREE + 2;
     static constexpr int NBAR = B_DRAIN + 1;
     static constexpr uint32_t OFF_TMEMPTR = OFF_BAR + NBAR * 8;
@@ -151,20 +151,6 @@ struct RowsIter {
         j.pair = pair;
         x += step;
         return true;
-    }
-};
-
-// Position in the ring of tiles: slot and the parity of its current phase.
-template <int RS>
-struct RingPos {
-    int slot = 0;
-    uint32_t phase = 0;
-    PPD_DEV void advance()
-    {
-        if (++slot == RS) {
-            slot = 0;
-            phase ^= 1u;
-        }
     }
 };
 
@@ -365,7 +351,7 @@ tree_attention_rows_kernel(const __grid_constant__ CUtensorMap map_q,
         bool pend[2] = {false, false};            // a tile's PV product is still to be issued
         bool p_first[2] = {false, false}, p_last[2] = {false, false};   // the tile's place in its job
         bool p_frees[2] = {false, false};         // its PV product is the last reader of the V tile
-        int p_job[2] = {0, 0}, of_seen[2] = {0, 0};
+        int p_job[2] = {-1, -1};                  // its job, counting those with tiles of the stream
         uint32_t p_par[2] = {0, 0};
         bool dead = false;                        // the CTA gave up: keep the control flow, issue nothing
         bool v_seen = false;                      // the next PV product's V tile is known to have landed
@@ -374,15 +360,15 @@ tree_attention_rows_kernel(const __grid_constant__ CUtensorMap map_q,
         // arrive.  Per 32 keys the probability columns hold 8 columns of hi pairs for
         // keys 0..15, 8 for keys 16..31, then the lo pairs in the same order.  A job's
         // first PV product overwrites O: it waits until the softmax warps have read back
-        // the outputs of every job before.
+        // the output of the stream's job before (one phase of the barrier for each job
+        // with tiles of the stream, so the wait is never more than one phase behind).
         auto issue_pv = [&](auto s_c, bool pair) {
             constexpr int s = decltype(s_c)::value;
             const Pos v = pair ? p_v[s] : pos;
             if (!pair) pos.advance();
             if (!v_seen) mbar_wait(bars + Lay::B_FULL + v.slot, v.phase, abort_flag);
-            if (p_first[s])
-                for (; of_seen[s] < p_job[s]; ++of_seen[s])
-                    mbar_wait(bars + Lay::B_OFREE + s, (uint32_t)of_seen[s] & 1u, abort_flag);
+            if (p_first[s] && p_job[s] >= 1)
+                mbar_wait(bars + Lay::B_OFREE + s, (uint32_t)(p_job[s] - 1) & 1u, abort_flag);
 #pragma unroll
             for (int half = 0; half < 2; ++half) {
                 mbar_wait(bars + Lay::B_PFULL + 2 * s + half, p_par[s], abort_flag);
@@ -416,7 +402,7 @@ tree_attention_rows_kernel(const __grid_constant__ CUtensorMap map_q,
         // in the order they are issued).  k_done: no later product reads the K tile;
         // q_done: the job's last scores from Q slot qs.
         auto issue_s = [&](auto s_c, int qs, const Pos &kp, const Pos &next_v, bool first, bool last, bool k_done, bool v_done,
-                           bool q_done, int job) {
+                           bool q_done) {
             constexpr int s = decltype(s_c)::value;
             mbar_wait(bars + Lay::B_FULL + kp.slot, kp.phase, abort_flag);
             // look for the next PV product's V tile now, while the tensor pipe still has
@@ -443,7 +429,7 @@ tree_attention_rows_kernel(const __grid_constant__ CUtensorMap map_q,
             p_first[s] = first;
             p_last[s] = last;
             p_frees[s] = v_done;
-            p_job[s] = job;
+            if (first) ++p_job[s];
         };
 
         int g = 0, k = 0;
@@ -464,7 +450,7 @@ tree_attention_rows_kernel(const __grid_constant__ CUtensorMap map_q,
                         const Pos kp = pos;
                         pos.advance();
                         // a stream's last tile of the job is one of the job's last two
-                        issue_s(s_c, qs, kp, pos, j < 2, j + 2 >= n, true, true, j == n - 1, k);
+                        issue_s(s_c, qs, kp, pos, j < 2, j + 2 >= n, true, true, j == n - 1);
                     };
                     if (g & 1) tile(b_t{});
                     else tile(a_t{});
@@ -484,12 +470,12 @@ tree_attention_rows_kernel(const __grid_constant__ CUtensorMap map_q,
                             mbar_wait(bars + Lay::B_QFULL + 0, (uint32_t)k & 1u, abort_flag);
                             dead = warp_uniform(*abort_flag) != 0;
                         }
-                        issue_s(a_t{}, 0, kp, p_v[1], first, j == n - 2, false, false, j == n - 2, k);
+                        issue_s(a_t{}, 0, kp, p_v[1], first, j == n - 2, false, false, j == n - 2);
                         p_v[0] = vp;
                     }
                     if (pend[1]) issue_pv(b_t{}, true);
                     if (first) mbar_wait(bars + Lay::B_QFULL + 1, (uint32_t)k & 1u, abort_flag);
-                    issue_s(b_t{}, 1, kp, p_v[0], first, last, true, true, last, k);
+                    issue_s(b_t{}, 1, kp, p_v[0], first, last, true, true, last);
                     p_v[1] = vp;
                 }
             }
@@ -528,7 +514,7 @@ tree_attention_rows_kernel(const __grid_constant__ CUtensorMap map_q,
         uint32_t s_par = 0, d_par = 0;   // phase parities: scores; bit x: stream x's jobs done
 
         // Probabilities of 32 keys from their raw scores r against the maximum, split
-        // into bf16 hi (truncated) + lo and stored over the scores.
+        // into bf16 hi + lo and stored over the scores.
         auto emit = [&](auto bits_c, const uint32_t (&r)[32], uint32_t bits, uint64_t negm, uint32_t t_dst,
                         uint64_t (&sum)[2]) {
             constexpr bool BITS = decltype(bits_c)::value != 0;
@@ -545,15 +531,7 @@ tree_attention_rows_kernel(const __grid_constant__ CUtensorMap map_q,
                 const float p0 = ex2(d0), p1 = ex2(d1);
                 const uint64_t pp = pack2(p0, p1);
                 sum[(e >> 1) & 1] = add2(sum[(e >> 1) & 1], pp);
-                const uint32_t u0 = __float_as_uint(p0), u1 = __float_as_uint(p1);
-                w[e >> 1] = __byte_perm(u0, u1, 0x7632);
-                // minus the hi parts
-                const uint64_t nh = pack2(__uint_as_float((u0 & 0xFFFF0000u) ^ 0x80000000u),
-                                          __uint_as_float((u1 & 0xFFFF0000u) ^ 0x80000000u));
-                float l0, l1;
-                unpack2(add2(pp, nh), l0, l1);
-                const __nv_bfloat162 lo = __floats2bfloat162_rn(l0, l1);
-                w[16 + (e >> 1)] = *reinterpret_cast<const uint32_t *>(&lo);
+                split_bf16x2(pp, p0, p1, w[e >> 1], w[16 + (e >> 1)]);
             }
             tmem_st32(t_dst, w);
         };
@@ -733,16 +711,16 @@ tree_attention_rows_kernel(const __grid_constant__ CUtensorMap map_q,
             const uint32_t t_o = tmem_base + lane_off + Lay::T_O + (uint32_t)s * (D / 2);
 #pragma unroll
             for (int c = 0; c < D / 2; c += 32) {
-                uint32_t r0[32], r1[32];
-                tmem_ld32(t_o + c, r0);
-                tmem_ld32(t_o + D + c, r1);
+                uint32_t r0[32] = {}, r1[32] = {};
+                if (has_a) tmem_ld32(t_o + c, r0);
+                if (has_b) tmem_ld32(t_o + D + c, r1);
                 tmem_wait_ld32(r0);
                 tmem_wait_ld32(r1);
                 if (c + 32 == D / 2) {
                     tc_fence_before();
                     __syncwarp();
-                    o_free(0, 1);
-                    o_free(1, 1);
+                    if (has_a) o_free(0, 1);
+                    if (has_b) o_free(1, 1);
                 }
                 if (qg < T) {
 #pragma unroll

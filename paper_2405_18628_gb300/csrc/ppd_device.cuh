@@ -370,6 +370,24 @@ PPD_DEV void tmem_st16(uint32_t taddr, const uint32_t (&r)[16])
         : "memory");
 }
 
+// The same with 8 columns.
+PPD_DEV void tmem_ld8(uint32_t taddr, uint32_t (&r)[8])
+{
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]),
+          "=r"(r[6]), "=r"(r[7])
+        : "r"(taddr));
+}
+
+PPD_DEV void tmem_st8(uint32_t taddr, const uint32_t (&r)[8])
+{
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(taddr),
+        "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
+        : "memory");
+}
+
 // The same with 32 columns.
 PPD_DEV void tmem_ld32(uint32_t taddr, uint32_t (&r)[32])
 {
@@ -424,6 +442,18 @@ PPD_DEV uint64_t add2(uint64_t a, uint64_t b)
     uint64_t d;
     asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
     return d;
+}
+
+// The pair pp = (p0, p1) as bf16 hi + lo: hi the nearest bf16, lo the nearest to
+// what is left, together within 2^-18 of each value (hi truncated: 2^-17).
+PPD_DEV void split_bf16x2(uint64_t pp, float p0, float p1, uint32_t &hi, uint32_t &lo)
+{
+    const __nv_bfloat162 h = __floats2bfloat162_rn(p0, p1);
+    hi = *reinterpret_cast<const uint32_t *>(&h);
+    float l0, l1;
+    unpack2(fma2(pack2(__uint_as_float(hi << 16), __uint_as_float(hi & 0xFFFF0000u)), pack2(-1.f, -1.f), pp), l0, l1);
+    const __nv_bfloat162 l = __floats2bfloat162_rn(l0, l1);
+    lo = *reinterpret_cast<const uint32_t *>(&l);
 }
 
 // ---------------------------------------------------------------- descriptors
