@@ -216,6 +216,31 @@ def test_attention_rows_many_jobs(cuda_device, T, D, P):
     np.testing.assert_allclose(lse.cpu().numpy().reshape(ref_lse.shape), ref_lse, rtol=0, atol=1e-3)
 
 
+@pytest.mark.parametrize("T,D", [(1, 64), (32, 64), (33, 64), (64, 64), (32, 128), (33, 128), (64, 128)])
+def test_attention_first_key_far_from_the_maximum(cuda_device, T, D):
+    """Trees of up to 64 tokens: a slice starts from its first key's scores as
+    the running maxima.  Single keys 40 times larger than the rest put those
+    far above or far below the true ones, in the first tile and in later ones;
+    more slices than SMs, prefixes that are empty, end inside a tile, and span
+    tiles, and another tree for every sequence."""
+    pl = np.asarray([0, 129, 300], np.int32)
+    w = W.Workload("first", L=1, B=3, H=60, D=D, P=300, T=T, V=16, n_cand=(T + 3) // 4,
+                   max_depth=6, chains="fill3", match_rate=0.5, seed=T + D)
+    s = W.make_step_inputs(w, prefix_len=pl)
+    t = tensors(w, prefix_len=pl)
+    t["k_cache"][:, :, :20, 0] *= 40
+    t["k_cache"][:, :, 20:40, 5] *= 40
+    t["k_cache"][:, :, 40:, 128] *= 40
+    t["k_tree"][:, :, ::2, 0] *= 40
+    out, lse, st = run_attention({k: v.to(cuda_device) for k, v in t.items()}, pl, s.parent,
+                                 cuda_device)
+    ref, ref_lse, _, ref_st = oracle.tree_attention(t["q"], t["k_cache"], t["v_cache"], t["k_tree"],
+                                                    t["v_tree"], pl, s.parent)
+    assert (st.cpu().numpy() == 0).all() and (ref_st == 0).all()
+    assert_attn_close(out.cpu().numpy().reshape(ref.shape), ref, f"T={T} D={D}")
+    np.testing.assert_allclose(lse.cpu().numpy().reshape(ref_lse.shape), ref_lse, rtol=0, atol=1e-3)
+
+
 def test_attention_peaked_scores_and_scale(cuda_device):
     """Large scores force the running-max rescale path on later tiles."""
     w = W.scaled(W.WORKLOADS["vicuna7b"], L=1, H=2, P=1000)
