@@ -241,47 +241,48 @@ bool attn_dims_ok(int L, int B, int H, int T, int D, int S_max, ppd_dtype dt)
     return true;
 }
 
+// How an attention launch shares its work out: whole units round-robin, one
+// cluster of CTAs per unit (cluster > 1), or equal ranges of all key tiles
+// (split; needs a workspace and a batch of at most kSplitMaxB).  Only launches
+// with fewer units than SMs can gain from either: with more, the last round's
+// idle SMs cost less than the merge (measured on the Vicuna-7B/13B and
+// MobileLlama shapes).  Counted in tiles of 128 keys, S_max standing in for the
+// (device-side) prefix lengths: whole units take t_u tiles; a cluster of c takes
+// its share and about kClusterCostTiles for the merge through distributed
+// shared memory; the work split takes its share of all tiles, which is smaller,
+// and about kSplitCostTiles for the range planning and the merge grid.
+struct AttnPlan {
+    int split, cluster;
+};
+constexpr long long kClusterCostTiles = 2, kSplitCostTiles = 6;
+
+AttnPlan plan_attention(int L, int B, int H, int T, int S_max, bool workspace, bool clusters)
+{
+    AttnPlan plan{0, 1};
+    const int n_tt = T > 64 ? (T + 127) / 128 : 1;
+    const long long units = (long long)L * B * H * n_tt, sms = split_grid();
+    if (units >= sms) return plan;
+    const long long t_u = (S_max + 127) / 128 + n_tt;
+    long long best = t_u;
+    for (int c = 2; clusters && c <= ppd::kMaxCluster && c <= t_u && units * c <= sms; ++c) {
+        const long long cost = (t_u + c - 1) / c + kClusterCostTiles;
+        if (cost < best && units <= ppd::max_attention_clusters(c)) {
+            best = cost;
+            plan.cluster = c;
+        }
+    }
+    if (workspace && B <= ppd::kSplitMaxB && (units * t_u + sms - 1) / sms + kSplitCostTiles < best) plan = {1, 1};
+    return plan;
+}
+
 // Enqueue the attention of all L*B*H slices (bf16 operands).
-// Does sharing the launch's key tiles over all SMs (the work split) beat one
-// whole slice per SM?  Only launches with fewer slices than SMs can gain (with
-// more, the last round's idle SMs cost less than the merge; measured on the
-// Vicuna-7B/13B and MobileLlama shapes).  Counted in tiles of 128 keys, with
-// S_max standing in for the (device-side) prefix lengths: one round of whole
-// slices takes t_u tiles; the split takes its share of all tiles plus about
-// kSplitCostTiles for the range planning and the merge grid.
-constexpr long long kSplitCostTiles = 6;
-
-bool split_pays(const AttnParams &p, int sms)
-{
-    if (p.n_units >= sms) return false;
-    const long long t_u = (p.S_max + 127) / 128 + p.n_tt;
-    const long long share = ((long long)p.n_units * t_u + sms - 1) / sms;
-    return share + kSplitCostTiles < t_u;
-}
-
-// Whether an attention launch of these sizes, given a workspace, shares its key
-// tiles out (the work split): a batch of at most kSplitMaxB and a launch that
-// gains from it.
-bool attention_splits(int L, int B, int H, int T, int S_max)
-{
-    if (B > ppd::kSplitMaxB) return false;
-    AttnParams p{};
-    const int T_pad = (T + 31) & ~31;
-    p.S_max = S_max;
-    p.n_qb = T_pad > 64 ? (T + 127) / 128 : 1;
-    p.n_tt = p.n_qb;
-    p.n_units = (int)((long long)L * B * H) * p.n_qb;
-    return split_pays(p, split_grid());
-}
-
-// With a workspace of the full layout and attention_splits(...), the key tiles
-// are shared evenly over the CTAs (see ppd_attention_common.cuh).
+// set_status: every sequence's dev_status is written (else only raised).
 ppd_status enqueue_attention(const void *q, const void *kc, const void *vc, const void *kt,
                              const void *vt, const int32_t *prefix_len, const int32_t *parent,
                              int L, int B, int H, int T, int D, int S_max, float scale, float *out,
                              float *lse, int32_t *dev_status, uint8_t *ws, const WsLayout *wl,
                              const ppd::FusedStep *fused, bool programmatic, bool chained,
-                             cudaStream_t stream)
+                             bool set_status, cudaStream_t stream)
 {
     const int T_pad = (T + 31) & ~31;
     const uint64_t lbh = (uint64_t)L * B * H;
@@ -312,7 +313,11 @@ ppd_status enqueue_attention(const void *q, const void *kc, const void *vc, cons
     p.n_units = (int)lbh * p.n_qb;
     const float sc = scale > 0.f ? scale : 1.0f / std::sqrt((float)D);
     p.scale_log2 = sc * 1.4426950408889634f;
-    if (ws && wl && attention_splits(L, B, H, T, S_max)) {
+    ppd::plan_rows(p, split_grid());
+    const AttnPlan plan = plan_attention(L, B, H, T, S_max, ws && wl, !(fused && fused->in_grid));
+    p.cluster = plan.cluster;
+    p.set_status = set_status;
+    if (plan.split) {
         p.split = 1;
         p.split_rec = reinterpret_cast<ppd::SplitRecord *>(ws + wl->split_rec);
         p.split_part = reinterpret_cast<float *>(ws + wl->split_part);
@@ -324,7 +329,12 @@ ppd_status enqueue_attention(const void *q, const void *kc, const void *vc, cons
                                                   stream));
 }
 
-// fp32 operands: round to bf16 copies in the workspace first.
+// fp32 operands: round to bf16 copies in the workspace first (of the caches the
+// rows below each prefix): by five grids, as the fused step counts them, or
+// (chained) by one in the chain of programmatic launches.  chained: the call is a
+// link of such a chain and its attention grid waits for whatever precedes it
+// itself.  A fused step's bf16 attention grid overlaps the argmax grid before it
+// -- when there is one: it only reads caller inputs before its end phase.
 ppd_status enqueue_attention_any(const void *q, const void *kc, const void *vc, const void *kt,
                                  const void *vt, const int32_t *prefix_len, const int32_t *parent,
                                  int L, int B, int H, int T, int D, int S_max, ppd_dtype dt,
@@ -332,14 +342,10 @@ ppd_status enqueue_attention_any(const void *q, const void *kc, const void *vc, 
                                  uint8_t *ws, const WsLayout &wl, const ppd::FusedStep *fused,
                                  cudaStream_t stream, bool chained = false)
 {
-    // With bf16 operands the attention grid only reads caller inputs before its end
-    // phase, so it may overlap the preceding (argmax) grid -- when there is one.
-    // `chained`: the grid follows a status reset launched as a programmatic
-    // dependent, and waits for it (and so for whatever preceded it) itself.
     if (dt == PPD_BF16)
         return enqueue_attention(q, kc, vc, kt, vt, prefix_len, parent, L, B, H, T, D, S_max, scale,
                                  out, lse, dev_status, ws, ws ? &wl : nullptr, fused,
-                                 fused != nullptr && !fused->in_grid, chained, stream);
+                                 fused != nullptr && !fused->in_grid, chained, chained, stream);
     const int64_t lbh = (int64_t)L * B * H;
     const int64_t n_t = lbh * T * D, n_c = lbh * (int64_t)S_max * D;
     uint16_t *bq = reinterpret_cast<uint16_t *>(ws + wl.conv);
@@ -347,14 +353,29 @@ ppd_status enqueue_attention_any(const void *q, const void *kc, const void *vc, 
     uint16_t *bvt = bkt + n_t;
     uint16_t *bkc = bvt + n_t;
     uint16_t *bvc = bkc + n_c;
-    if (ppd::launch_round_bf16((const float *)q, bq, n_t, stream) != cudaSuccess ||
-        ppd::launch_round_bf16((const float *)kt, bkt, n_t, stream) != cudaSuccess ||
-        ppd::launch_round_bf16((const float *)vt, bvt, n_t, stream) != cudaSuccess ||
-        ppd::launch_round_bf16((const float *)kc, bkc, n_c, stream) != cudaSuccess ||
-        ppd::launch_round_bf16((const float *)vc, bvc, n_c, stream) != cudaSuccess)
-        return cuda_failed();
+    ppd::RoundArgs r{};
+    const void *src[5] = {q, kt, vt, kc, vc};
+    uint16_t *dst[5] = {bq, bkt, bvt, bkc, bvc};
+    r.prefix_len = prefix_len;
+    r.B = B;
+    r.H = H;
+    r.D = D;
+    for (int i = 0; i < 5; ++i) r.t[i] = {(const float *)src[i], dst[i], i < 3 ? T : S_max, i >= 3};
+    if (chained) {
+        r.n = 5;
+        const cudaError_t e = ppd::launch_round_bf16(r, lbh, true, stream);
+        if (e != cudaSuccess) return cuda_status(e);
+    } else {
+        for (int i = 0; i < 5; ++i) {
+            ppd::RoundArgs one = r;
+            one.t[0] = r.t[i];
+            one.n = 1;
+            const cudaError_t e = ppd::launch_round_bf16(one, lbh, false, stream);
+            if (e != cudaSuccess) return cuda_status(e);
+        }
+    }
     return enqueue_attention(bq, bkc, bvc, bkt, bvt, prefix_len, parent, L, B, H, T, D, S_max,
-                             scale, out, lse, dev_status, ws, &wl, fused, false, false, stream);
+                             scale, out, lse, dev_status, ws, &wl, fused, false, chained, chained, stream);
 }
 
 // Blocks of the fused step's narrow argmax grid (0: use the wide grid).  When
@@ -364,17 +385,20 @@ ppd_status enqueue_attention_any(const void *q, const void *kc, const void *vc, 
 // (at most half of them), the CTAs dispatched last, which are those, wait for
 // them, and nothing on the critical path does.  Each block's share of the
 // logits must then be at most half a slice's K/V bytes (S_max standing in for
-// the device-side prefix lengths).  The work split (fewer slices than SMs)
-// leaves no CTA with time to spare.
+// the device-side prefix lengths).  Either split (fewer slices than SMs) leaves
+// no CTA with time to spare.
 int narrow_argmax_grid(int L, int B, int H, int T, int D, int V, int S_max)
 {
-    if (attention_splits(L, B, H, T, S_max)) return 0;
+    const AttnPlan plan = plan_attention(L, B, H, T, S_max, true, true);
+    if (plan.split || plan.cluster > 1) return 0;
     AttnParams p{};
     p.T_pad = (T + 31) & ~31;
     p.n_qb = p.T_pad > 64 ? (T + 127) / 128 : 1;
-    // two groups of CTAs with queues of their own: none is known to have time to spare
-    if (p.n_qb == 3) return 0;
     p.n_units = (int)((long long)L * B * H) * p.n_qb;
+    p.S_max = S_max;
+    ppd::plan_rows(p, split_grid());
+    // two groups of CTAs with queues of their own: none is known to have time to spare
+    if (p.pairs && p.n_qb == 3) return 0;
     const long long n_jobs = ppd::whole_jobs(p);
     const long long grid = ppd::attention_grid(p, split_grid());
     const long long r = n_jobs % grid;
@@ -558,7 +582,7 @@ int ppd_verify_step_launches(int L, int B, int H, int T, int D, int V, int S_max
     const int form = ppd_verify_step_form(L, B, H, T, D, V, S_max, dt);
     if (form < 0) return -1;
     const int round = dt == PPD_F32 ? 5 : 0;   // fp32 -> bf16 copies of Q, K/V tree, K/V cache
-    const int attn = attention_splits(L, B, H, T, S_max) ? 2 : 1;   // + the merge grid
+    const int attn = plan_attention(L, B, H, T, S_max, true, form != kFormSide).split ? 2 : 1;   // + the merge grid
     if (form == kFormTwoGrids) return 1 + round + attn;
     if (form == kFormSide) return 1 + round + attn;   // the status reset, then one grid
     // partial maxima, combine (or statistics), acceptance, attention, compaction
@@ -617,13 +641,10 @@ ppd_status ppd_tree_attention(const void *q, const void *k_cache, const void *v_
     const bool ws_ok = workspace && ws_bytes >= wl.total && aligned(workspace, kAlign);
     if (dt == PPD_F32 && !ws_ok) return PPD_ERR_INVALID_ARG;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    // dev_status is reset by a one-block grid launched as a programmatic
-    // dependent (it waits for the preceding grid before writing); the attention
-    // grid is its programmatic dependent in turn, so a sequence of calls (one
-    // per layer, as a model runs them) launches each grid while the previous
-    // one still runs and only the setup that reads no input runs early
-    if (ppd::launch_zero_status(dev_status, B, s) != cudaSuccess) return cuda_failed();
-    // a bf16 call without a full workspace runs unsplit
+    // one link of a chain of programmatic launches (one call per layer, as a model
+    // runs them): the grid starts while the previous one still runs, does the setup
+    // that reads no input, and waits for it; its spare warps write dev_status
+    // (a bf16 call without a full workspace has no work split)
     return enqueue_attention_any(q, k_cache, v_cache, k_tree, v_tree, prefix_len, parent, L, B, H,
                                  T, D, S_max, dt, scale, out, lse, dev_status,
                                  ws_ok ? static_cast<uint8_t *>(workspace) : nullptr, wl, nullptr, s,

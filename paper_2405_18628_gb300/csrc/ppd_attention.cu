@@ -117,7 +117,8 @@ struct AttnLayout {
     static_assert(NC == 8 || NC == 16 || NC == 32, "query columns of a softmax thread");
 };
 
-template <int D, int TP, int NWG, bool SPLIT>
+// MODE: whole units round-robin (0), the work split (1), the cluster split (2).
+template <int D, int TP, int NWG, int MODE>
 __global__ void __launch_bounds__((4 * NWG + 3) * 32, 1)
 tree_attention_kernel(const __grid_constant__ CUtensorMap map_q,
                       const __grid_constant__ CUtensorMap map_kc,
@@ -128,6 +129,7 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap map_q,
     using Lay = AttnLayout<D, TP, NWG>;
     using KPos = RingPos<Lay::KS>;
     using VPos = RingPos<Lay::VS>;
+    constexpr bool SPLIT = MODE == 1, RANGE = MODE != 0;
     constexpr int NC = Lay::NC;
     using Cols = uint32_t[Lay::NC];   // a softmax thread's scores of one tile
     extern __shared__ __align__(1024) uint8_t smem[];
@@ -174,7 +176,7 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap map_q,
     // grid: everything above overlapped it, nothing below reads before it is done
     // (the first K/V tiles are only asked of L2 before)
     if (p.pdl_wait) {
-        if (warp == Lay::SW) prefetch_first_tiles<SPLIT>(p, lane, &map_kc, &map_vc, Lay::DCH, 3);
+        if (warp == Lay::SW) prefetch_first_tiles<RANGE>(p, lane, &map_kc, &map_vc, Lay::DCH, 3);
         asm volatile("griddepcontrol.wait;" ::: "memory");
     }
     WorkRange *wr_s = reinterpret_cast<WorkRange *>(smem + Lay::OFF_RANGE);
@@ -197,6 +199,7 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap map_q,
     if (warp == Lay::SW + 2) {
         // ------------------------------------------------------------ fused-step side work
         if (p.fused) fused_side_warp<true>(p, wr, lane, abort_flag);
+        else if (p.set_status) status_warp(p, lane);
     } else if (warp == Lay::SW) {
         // ------------------------------------------------------------ TMA producer
         if (lane == 0) {
@@ -204,7 +207,7 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap map_q,
             KPos kp;
             VPos vp;
             int g = 0, k = 0;
-            SegIter<SPLIT> it(wr);
+            SegIter<RANGE> it(wr);
             for (Seg sg; it.next(p, sg); ++k) {
                 const UnitInfo &ui = sg.ui;
                 const int u = sg.u;
@@ -304,7 +307,7 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap map_q,
         int g = 0, k = 0;
         bool prev_first = false;
         uint32_t prev_to = 0;
-        SegIter<SPLIT> it(wr);
+        SegIter<RANGE> it(wr);
         for (Seg sg;; ++k) {
             const int n = warp_uniform(it.next(p, sg) ? sg.j1 - sg.j0 : 0);
             if (n == 0) break;
@@ -530,7 +533,7 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap map_q,
         };
 
         int k = 0;
-        SegIter<SPLIT> it(wr);
+        SegIter<RANGE> it(wr);
         for (Seg sg; it.next(p, sg); ++k) {
             const UnitInfo &ui = sg.ui;
             const int u = sg.u;
@@ -559,16 +562,6 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap map_q,
                     // lane collects its key's bit of each set
                     uint64_t anc = 0;
                     int a = lane < NC && q0 + lane < T ? q0 + lane : -1;
-                    bool bad = false;
-#pragma unroll
-                    for (int x = 0; x < TP / 32; ++x) {
-                        const int i = lane + 32 * x;
-                        if (i < T) bad |= i == 0 ? par[x] != -1 : (par[x] < 0 || par[x] >= i);
-                    }
-                    if (wg == 0 && wq == 0 && p.dev_status) {
-                        if (bad) p.dev_status[ui.b] = kErrTree;
-                        if (lane == 0 && (ui.P_raw < 0 || ui.P_raw > p.S_max)) p.dev_status[ui.b] = kErrCapacity;
-                    }
                     while (__any_sync(0xffffffffu, a >= 0)) {
                         if (a >= 0) anc |= 1ull << a;
                         const int i = a < 0 ? 0 : a;
@@ -666,7 +659,7 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap map_q,
                 if (t < NC) {
                     const float l = red[t] + red[NC + t] + red[2 * NC + t] + red[3 * NC + t];
                     const float m = -nm[t];
-                    if (!SPLIT || seg_whole(sg)) {
+                    if (!RANGE || (SPLIT && seg_whole(sg))) {
                         if (p.lse && q0 + t < T) p.lse[(size_t)u * T + q0 + t] = (m + lg2(l)) * 0.69314718055994530942f;
                         linv[ob * TP + t] = rcp(l);
                     } else {
@@ -688,18 +681,41 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap map_q,
                 }
             }
         }
-        if (pend_f) {
+        if (MODE == 2) {
+            // this CTA's part of the unit for the cluster: O rows over the K ring (every
+            // copy has landed and every product that reads it is done), maxima and sums
+            // where the segment's end left them
+            if (pend_f) {
+                float *st = reinterpret_cast<float *>(smem + Lay::OFF_K);
+                read_o(0, pend_g, [&](int e, float v) { st[(q0 + e) * D + t] = v; });
+            } else if (t < NC) {
+                pmx[t] = -INFINITY;
+                linv[t] = 0.f;
+            }
+        } else if (pend_f) {
             named_bar_sync(1 + wg, 128);   // the row sums are in shared memory
             flush_pending();
         }
     }
 
+    if (MODE == 2) {
+        __syncwarp();
+        cluster_sync();
+        if (warp < Lay::SW) {
+            const int u = (int)blockIdx.x / p.cluster;
+            cluster_merge(p, smem_addr(smem) + Lay::OFF_K, D * 4, smem_addr(smem) + Lay::OFF_PMX,
+                          smem_addr(smem) + Lay::OFF_LINV, 4, D, (int)blockIdx.x - u * p.cluster, T, (size_t)u * T,
+                          threadIdx.x, Lay::SW * 32);
+        }
+        __syncwarp();
+        cluster_sync();   // no CTA leaves while a peer reads its shared memory
+    }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     if (*abort_flag && threadIdx.x == 0) {
         for (int b = 0; b < p.B; ++b) {
-            if (p.dev_status) p.dev_status[b] = kErrTimeout;
+            if (p.dev_status) atomicMax(p.dev_status + b, (int)kErrTimeout);
             if (p.fused) atomicMax(p.fs.status + b, (int)kErrTimeout);
         }
     }
@@ -750,12 +766,51 @@ static cudaError_t launch_tree_attention_t(const AttnMaps &m, const AttnParams &
                                            bool programmatic, cudaStream_t stream)
 {
     using Lay = AttnLayout<D, TP, NWG>;
-    static std::atomic<uint64_t> configured[2] = {{0}, {0}};
+    static std::atomic<uint64_t> configured[3] = {{0}, {0}, {0}};
+    if (p.cluster > 1)
+        return launch_attention_grid(tree_attention_kernel<D, TP, NWG, 2>, Lay::SMEM_BYTES, Lay::THREADS,
+                                     configured[2], m, p, num_sms, programmatic, stream);
     if (p.split)
-        return launch_attention_grid(tree_attention_kernel<D, TP, NWG, true>, Lay::SMEM_BYTES, Lay::THREADS,
+        return launch_attention_grid(tree_attention_kernel<D, TP, NWG, 1>, Lay::SMEM_BYTES, Lay::THREADS,
                                      configured[1], m, p, num_sms, programmatic, stream);
-    return launch_attention_grid(tree_attention_kernel<D, TP, NWG, false>, Lay::SMEM_BYTES, Lay::THREADS,
+    return launch_attention_grid(tree_attention_kernel<D, TP, NWG, 0>, Lay::SMEM_BYTES, Lay::THREADS,
                                  configured[0], m, p, num_sms, programmatic, stream);
+}
+
+// Asked of one attention kernel for all of them: each takes a whole SM, so the
+// answer only depends on how the device groups its SMs.
+int max_attention_clusters(int size)
+{
+    static std::atomic<int> cache[64][kMaxCluster + 1];   // the answer + 1
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return 0;
+    }
+    if (dev < 0 || dev >= 64 || size < 1 || size > kMaxCluster) return 0;
+    int got = cache[dev][size].load(std::memory_order_relaxed);
+    if (got > 0) return got - 1;
+    using Lay = AttnLayout<128, 64, 2>;
+    auto kern = tree_attention_kernel<128, 64, 2, 2>;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)size);
+    cfg.blockDim = dim3(Lay::THREADS);
+    cfg.dynamicSmemBytes = Lay::SMEM_BYTES;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)size;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Lay::SMEM_BYTES) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) {
+        (void)cudaGetLastError();
+        n = 0;
+    }
+    cache[dev][size].store(n + 1, std::memory_order_relaxed);
+    return n;
 }
 
 cudaError_t launch_tree_attention(const AttnMaps &m, const AttnParams &p, int D, int num_sms,

@@ -76,8 +76,8 @@ PPD_DEV WorkRange plan_range(const AttnParams &p, int lane)
     w.u_first = p.n_units;
     w.u_last = -1;
     w.n_tiles = 0;
-    w.rr_units = p.split ? 0 : p.n_units;   // units taken whole, round-robin
-    if (!p.split) return w;
+    w.rr_units = p.split || p.cluster > 1 ? 0 : p.n_units;   // units taken whole, round-robin
+    if (w.rr_units > 0) return w;
     const unsigned full = 0xffffffffu;
     const int per_b = p.H * p.n_qb;
     auto nt_of = [&](int b) {
@@ -85,6 +85,14 @@ PPD_DEV WorkRange plan_range(const AttnParams &p, int lane)
                           p.S_max);
         return ((P + 127) >> 7) + p.n_tt;
     };
+    if (p.cluster > 1) {
+        // the cluster's unit, this CTA's share of its tiles
+        w.u_first = w.u_last = c / p.cluster;
+        const int r = c - w.u_first * p.cluster, nt = nt_of(w.u_first / per_b % p.B);
+        w.j_first = r * nt / p.cluster;
+        w.n_tiles = (r + 1) * nt / p.cluster - w.j_first;
+        return w;
+    }
     const int w0 = lane < p.B ? per_b * nt_of(lane) : 0;
     const int w1 = lane + 32 < p.B ? per_b * nt_of(lane + 32) : 0;
     int s0 = w0, s1 = w1;   // inclusive prefix sums over b
@@ -335,6 +343,78 @@ static __device__ __forceinline__ void split_merge_chunk(const float *split_part
         for (int x = 0; x < 8; ++x) dst[x] = acc[x] * inv;
     }
     if (c0 == 0 && lse) lse[out_row0 + r] = (M + lg2(Ls)) * 0.69314718055994530942f;
+}
+
+// The end of a cluster split: every CTA of the cluster has left its partial state
+// in its shared memory -- unnormalised O rows at `o` (`pitch` bytes apart), each
+// row's maximum at `m` and sum at `l` (`ml_pitch` bytes apart; maximum -inf: no key seen, the
+// row of O may hold anything) -- and all threads have passed a cluster_sync().
+// CTA `rank` merges its share of the n_rows rows, four columns per thread at a
+// time, every CTA's values loaded before any is used.
+PPD_DEV void cluster_merge(const AttnParams &p, uint32_t o, uint32_t pitch, uint32_t m, uint32_t l, uint32_t ml_pitch,
+                           int D, int rank, int n_rows, size_t out_row0, int tid, int n_threads)
+{
+    const int n = p.cluster, per_row = D / 4;
+    const int r0 = rank * n_rows / n, r1 = (rank + 1) * n_rows / n;
+    const bool vec_out = (reinterpret_cast<uintptr_t>(p.out) & 15u) == 0;
+    for (int i = tid; i < (r1 - r0) * per_row; i += n_threads) {
+        const int row = r0 + i / per_row, c4 = i % per_row;
+        float mc[kMaxCluster], lc[kMaxCluster];
+        float4 v[kMaxCluster];
+#pragma unroll
+        for (int c = 0; c < kMaxCluster; ++c) {
+            mc[c] = -INFINITY;
+            if (c < n) {
+                mc[c] = ld_cluster_f32(cluster_map(m + row * ml_pitch, c));
+                lc[c] = ld_cluster_f32(cluster_map(l + row * ml_pitch, c));
+                v[c] = ld_cluster_v4(cluster_map(o + row * pitch + c4 * 16, c));
+            }
+        }
+        float M = -INFINITY, Ls = 0.f;
+#pragma unroll
+        for (int c = 0; c < kMaxCluster; ++c) M = fmaxf(M, mc[c]);
+        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int c = 0; c < kMaxCluster; ++c) {
+            if (c >= n || mc[c] == -INFINITY) continue;
+            const float w = ex2(mc[c] - M);
+            Ls = fmaf(w, lc[c], Ls);
+            acc.x = fmaf(w, v[c].x, acc.x);
+            acc.y = fmaf(w, v[c].y, acc.y);
+            acc.z = fmaf(w, v[c].z, acc.z);
+            acc.w = fmaf(w, v[c].w, acc.w);
+        }
+        const float inv = 1.f / Ls;
+        float *dst = p.out + (out_row0 + row) * D + c4 * 4;
+        if (vec_out) {
+            *reinterpret_cast<float4 *>(dst) = make_float4(acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv);
+        } else {
+            dst[0] = acc.x * inv;
+            dst[1] = acc.y * inv;
+            dst[2] = acc.z * inv;
+            dst[3] = acc.w * inv;
+        }
+        if (c4 == 0 && p.lse) p.lse[out_row0 + row] = (M + lg2(Ls)) * 0.69314718055994530942f;
+    }
+}
+
+// The statuses of an attention call that is not part of a fused step, by one
+// spare warp per CTA: sequence b by CTA b mod grid, a malformed tree before a
+// prefix length outside the cache.  Every status gets its one plain store here,
+// at the start of the grid; only a CTA whose waits ran out, seconds later,
+// raises it again (atomicMax).
+PPD_DEV void status_warp(const AttnParams &p, int lane)
+{
+    for (int b = blockIdx.x; b < p.B; b += gridDim.x) {
+        bool bad = false;
+        for (int i = lane; i < p.T; i += 32) {
+            const int pa = __ldg(p.parent + (size_t)b * p.T + i);
+            bad |= i == 0 ? pa != -1 : (pa < 0 || pa >= i);
+        }
+        bad = __any_sync(0xffffffffu, bad);
+        const int P = __ldg(p.prefix_len + b);
+        if (lane == 0) p.dev_status[b] = bad ? kErrTree : (P < 0 || P > p.S_max ? kErrCapacity : kOk);
+    }
 }
 
 PPD_DEV void st_shared_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
@@ -707,8 +787,15 @@ cudaError_t launch_attention_grid(Kern kern, uint32_t smem, int threads,
     cfg.blockDim = dim3((unsigned)threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
-    cudaLaunchAttribute attr[2];
+    cudaLaunchAttribute attr[3];
     unsigned n_attr = 0;
+    if (p.cluster > 1) {
+        attr[n_attr].id = cudaLaunchAttributeClusterDimension;
+        attr[n_attr].val.clusterDim.x = (unsigned)p.cluster;
+        attr[n_attr].val.clusterDim.y = 1;
+        attr[n_attr].val.clusterDim.z = 1;
+        ++n_attr;
+    }
     if (programmatic) {
         attr[n_attr].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[n_attr].val.programmaticStreamSerializationAllowed = 1;

@@ -39,6 +39,7 @@
 // Trees of 65-128 tokens are single jobs, 129-256 pair jobs, 385-512 two pair
 // jobs a slice; 257-384 tokens are a pair and a single job, done by two groups
 // of CTAs side by side so that the second reader of a slice finds it in L2.
+// Launches with few slices take single jobs throughout (plan_rows).
 //
 // A thread owns a whole query row: the running maximum and the row sum are
 // registers and no vote or exchange is needed.  The maximum is lazy: it moves
@@ -94,6 +95,10 @@ struct RowsLayout {
     static constexpr uint32_t SMEM_BYTES = OFF_RANGE + ((sizeof(WorkRange) + 15) & ~15u);
     // TMEM columns: S_A | S_B (128 each; P is written over S) | O_A | O_B (D each)
     static constexpr uint32_t T_S = 0, T_O = 256, TMEM_COLS = 512;
+    // floats between the rows of a partial state in shared memory: lanes hold
+    // neighbouring rows, so their 16-byte stores spread over the banks
+    static constexpr int C_PITCH = D + 4;
+    static_assert(M * C_PITCH * 4 <= RS * TILE_BYTES, "a partial state fits over the ring");
 
     static_assert(SMEM_BYTES <= 232448, "shared memory budget");
     static_assert((OFF_R | Q_BYTES | TILE_BYTES) % 1024 == 0, "1024-byte aligned operand tiles");
@@ -110,28 +115,32 @@ struct RowsJob {
 // Walks a CTA's jobs in order (every role walks the same sequence).  Whole
 // jobs round-robin: single jobs (n_qb 1), pair jobs (n_qb 2, or 4 with two a
 // slice); with n_qb 3 the first p.pair_grid CTAs take the slices' pairs and
-// the others their third blocks.  SPLIT: single jobs, the CTA's range of tiles.
-template <bool SPLIT>
+// the others their third blocks.  RANGE (either split): single jobs, the CTA's range
+// of tiles.
+template <bool RANGE>
 struct RowsIter {
-    SegIter<SPLIT> seg;
+    SegIter<RANGE> seg;
     int x, step, n, per;
     bool pair;
     PPD_DEV RowsIter(const AttnParams &p, const WorkRange &w) : seg(w)
     {
         const int c = (int)blockIdx.x, G = (int)gridDim.x;
-        pair = !SPLIT && p.n_qb >= 2 && (p.n_qb != 3 || c < p.pair_grid);
+        pair = !RANGE && p.pairs && (p.n_qb != 3 || c < p.pair_grid);
         x = c;
         step = G;
-        if (p.n_qb == 3) {
-            x = pair ? c : c - p.pair_grid;
-            step = pair ? p.pair_grid : G - p.pair_grid;
+        per = p.n_qb;   // jobs a slice
+        if (p.pairs) {
+            per = p.n_qb == 4 ? 2 : 1;
+            if (p.n_qb == 3) {
+                x = pair ? c : c - p.pair_grid;
+                step = pair ? p.pair_grid : G - p.pair_grid;
+            }
         }
-        per = p.n_qb == 4 ? 2 : 1;
         n = p.n_units / p.n_qb * per;
     }
     PPD_DEV bool next(const AttnParams &p, RowsJob &j)
     {
-        if (SPLIT) {
+        if (RANGE) {
             Seg s;
             if (!seg.next(p, s)) return false;
             j.ui = s.ui;
@@ -141,8 +150,8 @@ struct RowsIter {
             return true;
         }
         if (x >= n) return false;
-        const int slice = per == 2 ? x >> 1 : x;
-        const int qb = pair ? (per == 2 ? 2 * (x & 1) : 0) : p.n_qb - 1;
+        const int slice = x / per, i = x - slice * per;
+        const int qb = pair ? 2 * i : (p.pairs ? p.n_qb - 1 : i);
         j.ui = unit_info(p, slice * p.n_qb + qb);
         // a query's ancestors come before it: no tree tile past the job's last block
         j.ui.n_tiles = j.ui.n_pref + qb + (pair ? 2 : 1);
@@ -155,18 +164,18 @@ struct RowsIter {
 };
 
 // prefetch_first_tiles for whole jobs: this CTA's first `n` prefix tiles.
-template <bool SPLIT>
+template <bool RANGE>
 PPD_DEV void rows_prefetch(const AttnParams &p, int lane, const CUtensorMap *kc, const CUtensorMap *vc,
                            int dch, int n)
 {
-    if (SPLIT) {
-        prefetch_first_tiles<SPLIT>(p, lane, kc, vc, dch, n);
+    if (RANGE) {
+        prefetch_first_tiles<RANGE>(p, lane, kc, vc, dch, n);
         return;
     }
     const WorkRange none{};
-    const RowsIter<SPLIT> it(p, none);
+    const RowsIter<RANGE> it(p, none);
     if (lane != 0 || it.x >= it.n) return;
-    const int lbh = it.per == 2 ? it.x >> 1 : it.x;
+    const int lbh = it.x / it.per;
     const int P = min(max(ld_relaxed_gpu_s32(p.prefix_len + (lbh / p.H) % p.B), 0), p.S_max);
     for (int j = 0; j < min(n, (P + 127) >> 7); ++j) {
         for (int c = 0; c < dch; ++c) {
@@ -176,7 +185,8 @@ PPD_DEV void rows_prefetch(const AttnParams &p, int lane, const CUtensorMap *kc,
     }
 }
 
-template <int D, bool SPLIT>
+// MODE: whole jobs (0), the work split (1), the cluster split (2).
+template <int D, int MODE>
 __global__ void __launch_bounds__(352, 1)
 tree_attention_rows_kernel(const __grid_constant__ CUtensorMap map_q,
                            const __grid_constant__ CUtensorMap map_kc,
@@ -186,6 +196,7 @@ tree_attention_rows_kernel(const __grid_constant__ CUtensorMap map_q,
 {
     using Lay = RowsLayout<D>;
     using Pos = RingPos<Lay::RS>;
+    constexpr bool SPLIT = MODE == 1, RANGE = MODE != 0;
     extern __shared__ __align__(1024) uint8_t smem[];
     if (smem_addr(smem) & 1023u) {
         if (threadIdx.x == 0 && p.dev_status)
@@ -197,6 +208,7 @@ tree_attention_rows_kernel(const __grid_constant__ CUtensorMap map_q,
     uint32_t *tmem_ptr = reinterpret_cast<uint32_t *>(smem + Lay::OFF_TMEMPTR);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + Lay::OFF_ABORT);
     float2 *xs = reinterpret_cast<float2 *>(smem + Lay::OFF_X);
+    float2 *cs = reinterpret_cast<float2 *>(smem);   // cluster split: [M] over the Q slots, free by then
 
     const int warp = warp_uniform((int)threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
@@ -228,7 +240,7 @@ tree_attention_rows_kernel(const __grid_constant__ CUtensorMap map_q,
     // grid: everything above overlapped it, nothing below reads before it is done
     // (the first K/V tiles are only asked of L2 before)
     if (p.pdl_wait) {
-        if (warp == 8) rows_prefetch<SPLIT>(p, lane, &map_kc, &map_vc, Lay::DCH, 3);
+        if (warp == 8) rows_prefetch<RANGE>(p, lane, &map_kc, &map_vc, Lay::DCH, 3);
         asm volatile("griddepcontrol.wait;" ::: "memory");
     }
     WorkRange *wr_s = reinterpret_cast<WorkRange *>(smem + Lay::OFF_RANGE);
@@ -251,6 +263,7 @@ tree_attention_rows_kernel(const __grid_constant__ CUtensorMap map_q,
     if (warp == 10) {
         // ------------------------------------------------------------ fused-step side work
         if (p.fused) fused_side_warp<false>(p, wr, lane, abort_flag);
+        else if (p.set_status) status_warp(p, lane);
     } else if (warp == 8) {
         // ------------------------------------------------------------ TMA producer
         if (lane == 0) {
@@ -289,7 +302,7 @@ tree_attention_rows_kernel(const __grid_constant__ CUtensorMap map_q,
             int v_row[2] = {0, 0}, v_lbh[2] = {0, 0};
             bool v_tree[2] = {false, false};
             int g = 0, k = 0;
-            RowsIter<SPLIT> it(p, wr);
+            RowsIter<RANGE> it(p, wr);
             for (RowsJob jb; it.next(p, jb); ++k) {
                 const UnitInfo &ui = jb.ui;
                 if (!jb.pair) load_q(k & 1, (uint32_t)(k >> 1) & 1u, ui.qb, ui.lbh);
@@ -433,7 +446,7 @@ tree_attention_rows_kernel(const __grid_constant__ CUtensorMap map_q,
         };
 
         int g = 0, k = 0;
-        RowsIter<SPLIT> it(p, wr);
+        RowsIter<RANGE> it(p, wr);
         const bool pair = it.pair;
         for (RowsJob jb;; ++k) {
             const int n = warp_uniform(it.next(p, jb) ? jb.j1 - jb.j0 : 0);
@@ -686,13 +699,18 @@ tree_attention_rows_kernel(const __grid_constant__ CUtensorMap map_q,
             const float w_oth = xo.x == -INFINITY ? 0.f : ex2(xo.x - mt);
             const float lt = w_own * l + w_oth * xo.y;
             const int qg = jb.ui.qb * Lay::M + q;
-            const bool whole = !SPLIT || (jb.j0 == 0 && jb.j1 == jb.ui.n_tiles);
+            const bool whole = !RANGE || (SPLIT && jb.j0 == 0 && jb.j1 == jb.ui.n_tiles);
             const float inv = whole ? rcp(lt) : 1.f;
             float *dst;
             if (whole) {
                 if (s == 0 && qg < T && p.lse)
                     p.lse[(size_t)jb.ui.lbh * T + qg] = (mt + lg2(lt)) * 0.69314718055994530942f;
                 dst = p.out + ((size_t)jb.ui.lbh * T + qg) * D;
+            } else if (MODE == 2) {
+                // this CTA's part for the cluster: rows over the ring (every copy has landed,
+                // and the waits below cover every product that reads it)
+                if (s == 0) cs[q] = make_float2(mt, lt);
+                dst = reinterpret_cast<float *>(smem + Lay::OFF_R) + q * Lay::C_PITCH;
             } else {
                 // a part of a cut unit: the unnormalised row, its maximum and its sum
                 float *base = p.split_part + (size_t)slot * split_slot_floats(D);
@@ -703,6 +721,7 @@ tree_attention_rows_kernel(const __grid_constant__ CUtensorMap map_q,
                 dst = base + (size_t)q * D;
             }
             dst += s * (D / 2);
+            const bool live = qg < T;
             const float fa = (s == 0 ? w_own : w_oth) * inv, fb = (s == 0 ? w_oth : w_own) * inv;
             const bool has_a = both || st0 == 0, has_b = both || st0 == 1;
             if (has_a) wait_done(0);
@@ -722,18 +741,24 @@ tree_attention_rows_kernel(const __grid_constant__ CUtensorMap map_q,
                     if (has_a) o_free(0, 1);
                     if (has_b) o_free(1, 1);
                 }
-                if (qg < T) {
+                if (live) {
 #pragma unroll
                     for (int e = 0; e < 32; ++e) {
                         const float a = fa != 0.f ? __uint_as_float(r0[e]) * fa : 0.f;
                         r0[e] = __float_as_uint(fb != 0.f ? fmaf(__uint_as_float(r1[e]), fb, a) : a);
                     }
-                    store32(dst + c, r0, 1.f);
+                    if (MODE == 2) {
+#pragma unroll
+                        for (int e = 0; e < 32; e += 4)
+                            st_shared_v4(smem_addr(dst + c + e), r0[e], r0[e + 1], r0[e + 2], r0[e + 3]);
+                    } else {
+                        store32(dst + c, r0, 1.f);
+                    }
                 }
             }
         };
 
-        RowsIter<SPLIT> it(p, wr);
+        RowsIter<RANGE> it(p, wr);
         int k = 0;
         for (RowsJob jb; it.next(p, jb); ++k) {
             const UnitInfo &ui = jb.ui;
@@ -743,25 +768,14 @@ tree_attention_rows_kernel(const __grid_constant__ CUtensorMap map_q,
 #pragma unroll
                 for (int w = 0; w < NW; ++w) anc[w] = 0;
                 if (qg < T) {
-                    bool bad = false;
                     int a = qg;
                     while (true) {
                         anc[a >> 5] |= 1u << (a & 31);
                         const int pa = __ldg(p.parent + (size_t)ui.b * T + a);
-                        if (a == 0) {
-                            bad = (pa != -1);
-                            break;
-                        }
-                        if (pa < 0 || pa >= a) {
-                            bad = true;
-                            break;
-                        }
+                        if (pa < 0 || pa >= a) break;   // the root, or a malformed tree
                         a = pa;
                     }
-                    if (bad && p.dev_status) p.dev_status[ui.b] = kErrTree;
                 }
-                if (qg == 0 && p.dev_status && (ui.P_raw < 0 || ui.P_raw > p.S_max))
-                    p.dev_status[ui.b] = kErrCapacity;
                 cur_key = ui.b * p.n_qb + qb;
             }
 
@@ -795,7 +809,7 @@ tree_attention_rows_kernel(const __grid_constant__ CUtensorMap map_q,
                         const int e = g + i;
                         int pos;   // the V tile's place in the ring order
                         if (jb.pair) pos = 2 * e + 1;
-                        else pos = (SPLIT && e == wr.n_tiles - 1) ? 2 * e + 1 : 2 * e + 2;
+                        else pos = (RANGE && e == wr.n_tiles - 1) ? 2 * e + 1 : 2 * e + 2;
                         const int vs = pos % Lay::RS;
                         mbar_wait(bars + Lay::B_FULL + vs, (uint32_t)(pos / Lay::RS) & 1u, abort_flag);
                         if (q >= n_valid) {
@@ -831,14 +845,28 @@ tree_attention_rows_kernel(const __grid_constant__ CUtensorMap map_q,
             m = -INFINITY;
             l = 0.f;
         }
+        if (MODE == 2 && wr.n_tiles == 0 && s == 0) cs[q] = make_float2(-INFINITY, 0.f);
     }
 
+    if (MODE == 2) {
+        __syncwarp();
+        cluster_sync();
+        if (warp < 8) {
+            const int u = (int)blockIdx.x / p.cluster;
+            const int lbh = u / p.n_qb, qb = u - lbh * p.n_qb;
+            cluster_merge(p, smem_addr(smem) + Lay::OFF_R, Lay::C_PITCH * 4, smem_addr(cs), smem_addr(cs) + 4, 8, D,
+                          (int)blockIdx.x - u * p.cluster, min(Lay::M, T - qb * Lay::M),
+                          (size_t)lbh * T + (size_t)qb * Lay::M, threadIdx.x, 256);
+        }
+        __syncwarp();
+        cluster_sync();   // no CTA leaves while a peer reads its shared memory
+    }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     if (*abort_flag && threadIdx.x == 0) {
         for (int b = 0; b < p.B; ++b) {
-            if (p.dev_status) p.dev_status[b] = kErrTimeout;
+            if (p.dev_status) atomicMax(p.dev_status + b, (int)kErrTimeout);
             if (p.fused) atomicMax(p.fs.status + b, (int)kErrTimeout);
         }
     }
@@ -846,32 +874,17 @@ tree_attention_rows_kernel(const __grid_constant__ CUtensorMap map_q,
 }
 
 template <int D>
-static cudaError_t launch_rows_t(const AttnMaps &m, const AttnParams &p0, int num_sms,
+static cudaError_t launch_rows_t(const AttnMaps &m, const AttnParams &p, int num_sms,
                                  bool programmatic, cudaStream_t stream)
 {
-    static std::atomic<uint64_t> configured[2] = {{0}, {0}};
-    if (p0.split)
-        return launch_attention_grid(tree_attention_rows_kernel<D, true>, RowsLayout<D>::SMEM_BYTES, 352,
-                                     configured[1], m, p0, num_sms, programmatic, stream);
-    AttnParams p = p0;
-    if (p.n_qb == 3) {
-        // the split of the CTAs with the shortest longest queue, a pair counted as 2 n + 4
-        // and a single block as n + 4.5 tiles of 128 x 128 with n prefix tiles (S_max
-        // standing in for the device-side prefix lengths): three and three tree tiles, and
-        // the end of a job, which only a pair's other stream overlaps
-        const long long n = p.n_units / 3, grid = attention_grid(p, num_sms), np = (p.S_max + 127) / 128;
-        long long best = -1;
-        for (long long g = 1; g < grid; ++g) {
-            const long long pairs = (4 * np + 8) * ((n + g - 1) / g);
-            const long long singles = (2 * np + 9) * ((n + grid - g - 1) / (grid - g));
-            const long long t = pairs > singles ? pairs : singles;
-            if (best < 0 || t <= best) {
-                best = t;
-                p.pair_grid = (int)g;
-            }
-        }
-    }
-    return launch_attention_grid(tree_attention_rows_kernel<D, false>, RowsLayout<D>::SMEM_BYTES, 352,
+    static std::atomic<uint64_t> configured[3] = {{0}, {0}, {0}};
+    if (p.cluster > 1)
+        return launch_attention_grid(tree_attention_rows_kernel<D, 2>, RowsLayout<D>::SMEM_BYTES, 352,
+                                     configured[2], m, p, num_sms, programmatic, stream);
+    if (p.split)
+        return launch_attention_grid(tree_attention_rows_kernel<D, 1>, RowsLayout<D>::SMEM_BYTES, 352,
+                                     configured[1], m, p, num_sms, programmatic, stream);
+    return launch_attention_grid(tree_attention_rows_kernel<D, 0>, RowsLayout<D>::SMEM_BYTES, 352,
                                  configured[0], m, p, num_sms, programmatic, stream);
 }
 

@@ -189,6 +189,41 @@ PPD_DEV void st_global_v8(float *dst, const uint32_t *v, float scale)
                  : "memory");
 }
 
+// ---------------------------------------------------------------- clusters
+
+// Barrier over every thread of the cluster: what a thread wrote (to its own
+// shared memory, for peers to read) before its arrival is seen by every thread
+// after its wait.
+PPD_DEV void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// The address of the same shared-memory location in the cluster's CTA `rank`.
+PPD_DEV uint32_t cluster_map(uint32_t saddr, uint32_t rank)
+{
+    uint32_t a;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(saddr), "r"(rank));
+    return a;
+}
+
+PPD_DEV float ld_cluster_f32(uint32_t a)
+{
+    float v;
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+    return v;
+}
+
+PPD_DEV float4 ld_cluster_v4(uint32_t a)
+{
+    float4 v;
+    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                 : "r"(a)
+                 : "memory");
+    return v;
+}
+
 // ---------------------------------------------------------------- TMA
 
 PPD_DEV void tma_prefetch_map(const CUtensorMap *map)

@@ -82,7 +82,8 @@ struct AttnParams {
     int L, B, H, T, T_pad, S_max, n_units;
     int n_qb;                   // query blocks of 128 per (layer, sequence, head) slice
     int n_tt;                   // tree-key tiles of 128 per slice
-    int pair_grid;              // query-row kernel, n_qb 3: CTAs that take the slices' pairs of blocks
+    int pairs;                  // query-row kernel: two blocks of queries of a slice are one job
+    int pair_grid;              // with n_qb 3: the CTAs that take the slices' pairs
     float scale_log2;           // softmax scale * log2(e)
     // Work split: split != 0 shares the units left after the full round-robin
     // rounds out by their key tiles (B <= kSplitMaxB); units cut by a range
@@ -91,6 +92,11 @@ struct AttnParams {
     int split;
     float *split_part;          // [2 * grid][kSplitRows * (D + 2)] partial states
     struct SplitRecord *split_rec;   // [grid]
+    // Cluster split: cluster > 1 gives every unit a cluster of that many CTAs, each an
+    // equal share of its tiles; their partial states are merged through distributed
+    // shared memory.
+    int cluster;
+    int set_status;             // the attention grid writes every sequence's dev_status itself
     int fused;                  // run the end phase below
     FusedStep fs;
     // Launched as a programmatic dependent of the preceding grid (a chain of
@@ -105,6 +111,13 @@ constexpr int kSplitMaxB = 64;
 constexpr int kSplitMaxGrid = 256;
 constexpr int kSplitRows = 128;
 
+// CTAs of a cluster at most (the portable size).
+constexpr int kMaxCluster = 8;
+
+// Clusters of `size` attention CTAs (one per SM) the current device can hold at
+// once; 0 when it cannot be asked.
+int max_attention_clusters(int size);
+
 // The unit a CTA has to have merged: it holds the unit's first tile and its
 // range ends inside the unit (u = -1: none).  off: the unit's tile 0 among
 // the tail's tiles; n_tail: the tail's tile count.
@@ -113,14 +126,49 @@ struct SplitRecord {
     int u, n_tiles;
 };
 
-// Jobs of a launch without the work split: its units, except that the
-// query-row kernel takes two blocks of queries of a slice as one job (n_qb 2 to
-// 4: one, two -- a pair and a single block -- and two jobs a slice).
+// Jobs of a launch without a split: its units, or with p.pairs (n_qb 2 to 4)
+// one, two -- a pair and a single block -- and two jobs a slice.
 inline long long whole_jobs(const AttnParams &p)
 {
-    if (p.T_pad <= 64 || p.n_qb == 1) return p.n_units;
+    if (!p.pairs) return p.n_units;
     const long long slices = p.n_units / p.n_qb;
     return p.n_qb == 2 ? slices : 2 * slices;
+}
+
+// Whether the query-row kernel's whole jobs are pairs of query blocks, and for
+// n_qb 3 the split of the CTAs between pairs and single blocks: the choice with
+// the shortest longest queue.  A pair counts as 2 n + 4 and a single block next
+// to it as n + 4.5 tiles of 128 x 128 with n prefix tiles (S_max standing in for
+// the device-side prefix lengths): three tree tiles each, and the end of a job,
+// which only a pair's other stream overlaps.  Without pairs every block streams
+// its keys itself: 15 % more a tile (L2), but twice the jobs, so it is the
+// choice for launches with few slices (16 x 32 calls of 32 slices, 285 tokens
+// over 1500 keys: pairs 36.6 us a call, single blocks 30.1).
+inline void plan_rows(AttnParams &p, int num_sms)
+{
+    p.pairs = 0;
+    if (p.T_pad <= 64 || p.n_qb < 2) return;
+    const long long S = p.n_units / p.n_qb, G = num_sms, n = (p.S_max + 127) / 128;
+    const long long single_all = (23 * (2 * n + 9)) * ((p.n_units + G - 1) / G);   // in 1/40 tiles
+    long long best = -1;
+    int grid = 0;
+    if (p.n_qb == 3) {
+        const long long Gp = G < 2 * S ? G : 2 * S;
+        for (long long g = 1; g < Gp; ++g) {
+            const long long a = (4 * n + 8) * ((S + g - 1) / g), b = (2 * n + 9) * ((S + Gp - g - 1) / (Gp - g));
+            const long long t = a > b ? a : b;
+            if (best < 0 || t <= best) {
+                best = t;
+                grid = (int)g;
+            }
+        }
+    } else {
+        const long long jobs = p.n_qb == 2 ? S : 2 * S;
+        best = (4 * n + 8) * ((jobs + G - 1) / G);
+    }
+    if (best < 0 || 20 * best > single_all) return;
+    p.pairs = 1;
+    p.pair_grid = grid;
 }
 
 // CTAs of an attention launch: one per SM, at most one per job (with the
@@ -128,6 +176,7 @@ inline long long whole_jobs(const AttnParams &p)
 inline int attention_grid(const AttnParams &p, int num_sms)
 {
     long long grid = num_sms;
+    if (p.cluster > 1) return p.n_units * p.cluster;
     if (p.split) {
         const long long max_tiles = (long long)p.n_units * ((p.S_max + 127) / 128 + p.n_tt);
         grid = grid < kSplitMaxGrid ? grid : kSplitMaxGrid;
@@ -231,7 +280,20 @@ cudaError_t launch_next_tree(const float *logits, const int32_t *parent, const i
                              int32_t *next_parent, int32_t *next_cand, int32_t *next_state,
                              int32_t *status, cudaStream_t stream);
 
-cudaError_t launch_round_bf16(const float *src, uint16_t *dst, int64_t n, cudaStream_t stream);
+// fp32 -> bf16 copies (round to nearest even) of n tensors [lbh][rows][D]; of a
+// `cache` tensor only the rows below the sequence's prefix length.  chained: as
+// a programmatic dependent of the stream's previous grid.
+struct RoundArgs {
+    struct Tensor {
+        const float *src;
+        uint16_t *dst;
+        int rows;
+        int cache;
+    } t[5];
+    const int32_t *prefix_len;
+    int n, B, H, D;
+};
+cudaError_t launch_round_bf16(const RoundArgs &r, int64_t lbh, bool chained, cudaStream_t stream);
 
 // Zero `n` status words once the preceding grid has completed, as a
 // programmatic dependent launch that lets the next grid launch at once.

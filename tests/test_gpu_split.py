@@ -140,3 +140,28 @@ def test_split_status_per_call(cuda_device):
     out, _, st = _attend(t_dev, pl, parent, cuda_device, ws)
     assert (st == 0).all(), st
     assert_attn_close(out.reshape(ref.shape), ref, "clean call after a failed one")
+
+
+@pytest.mark.parametrize("H,T,D,prefix,S_max", [
+    (40, 64, 64, [2000, 2048], 2048),     # 80 slices: the work split of the key-row kernel
+    (38, 96, 128, [1900, 1500], 4096),    # 76 slices: clusters of 2
+    (40, 100, 64, [4000, 10], 4096),      # 80 slices: the work split of the query-row kernel
+    (20, 33, 64, [1000, 127], 1024),      # 40 slices: clusters of 3
+    (14, 17, 128, [700, 0], 1024),        # 28: clusters of 5, one of a single tile
+    (10, 128, 64, [900, 513], 1024),      # 20: clusters of 6, query-row kernel
+    (7, 300, 64, [400, 129], 600),        # 14 slices of three query blocks
+    (1, 64, 128, [1, 900], 4096),         # clusters of 8 with more CTAs than tiles
+])
+def test_split_sizes(cuda_device, H, T, D, prefix, S_max):
+    """Clusters of every size, and the work split where no cluster size fits."""
+    L, B = 1, 2
+    t, pl, parent = _case(L, B, H, T, D, prefix, S_max, seed=H + T)
+    t_dev = {k: v.to(cuda_device) for k, v in t.items()}
+    ref, ref_lse, _, _ = oracle.tree_attention(t["q"], t["k_cache"], t["v_cache"], t["k_tree"],
+                                               t["v_tree"], pl, parent)
+    ws = ppd.workspace(L, B, H, T, D, 1, S_max, device=cuda_device)
+    for w in (ws, None):
+        out, lse, st = _attend(t_dev, pl, parent, cuda_device, w)
+        assert (st == 0).all(), st
+        assert_attn_close(out.reshape(ref.shape), ref, "split" if w is not None else "no workspace")
+        np.testing.assert_allclose(lse.reshape(ref_lse.shape), ref_lse, rtol=0, atol=1e-3)
