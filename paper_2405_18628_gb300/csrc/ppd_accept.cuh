@@ -145,8 +145,8 @@ PPD_DEV AcceptResult accept_warp_pass(TopLoad top, Pass pass, const int32_t *par
     for (int k = 0; k < nw; ++k) {
         const int i = lane + 32 * k;
         if (i < T) {
-            const int pa = __ldg(par + i);
-            const int tk = __ldg(tok + i);
+            const int pa = __ldcg(par + i);
+            const int tk = __ldcg(tok + i);
             s_par[i] = pa;
             if (i == 0)
                 bad |= (pa != -1) || tk < 0 || tk >= V;
@@ -165,7 +165,7 @@ PPD_DEV AcceptResult accept_warp_pass(TopLoad top, Pass pass, const int32_t *par
             if (i == 0) {
                 ok = true;
             } else {
-                const int tk = __ldg(tok + i);
+                const int tk = __ldcg(tok + i);
                 ok = tk >= 0 && pass(i, s_par[i], tk);
             }
         }
@@ -252,8 +252,8 @@ PPD_DEV AcceptResult accept_warp_small(const int (&top)[2], Pass pass, const int
         pa[k] = -1;
         tk[k] = -1;
         if (i < T) {
-            pa[k] = __ldg(par + i);
-            tk[k] = __ldg(tok + i);
+            pa[k] = __ldcg(par + i);
+            tk[k] = __ldcg(tok + i);
             if (i == 0)
                 bad |= (pa[k] != -1) || tk[k] < 0 || tk[k] >= V;
             else

@@ -658,15 +658,8 @@ ppd_status ppd_node_argmax(const float *logits, int B, int T, int V, int32_t *ar
     if ((double)B * T * V > 9.0e15 || (double)B * T * 64 > 2147483647.0) return PPD_ERR_INVALID_ARG;
     const WsLayout wl = workspace_layout(1, B, 1, T, 1, V, 0, PPD_BF16);
     if (!workspace || ws_bytes < wl.total || !aligned(workspace, kAlign)) return PPD_ERR_INVALID_ARG;
-    uint8_t *ws = static_cast<uint8_t *>(workspace);
-    cudaStream_t s = static_cast<cudaStream_t>(stream);
-    float *pv = reinterpret_cast<float *>(ws + wl.part_val);
-    int32_t *pi = reinterpret_cast<int32_t *>(ws + wl.part_idx);
-    const int64_t rows = (int64_t)B * T;
-    if (ppd::launch_argmax_partials(logits, rows, V, wl.splits, pv, pi, nullptr, 1.f, nullptr, 0, s) !=
-        cudaSuccess)
-        return cuda_failed();
-    return cuda_status(ppd::launch_argmax_combine(pv, pi, rows, wl.splits, argmax_out, s));
+    return cuda_status(ppd::launch_node_argmax(logits, (int64_t)B * T, V, 1.f, argmax_out, nullptr, nullptr,
+                                               static_cast<cudaStream_t>(stream)));
 }
 
 ppd_status ppd_accept_path(const int32_t *argmax, const int32_t *cand_tokens,
@@ -754,17 +747,8 @@ ppd_status ppd_node_stats(const float *logits, int B, int T, int V, float temper
     if ((double)B * T * V > 9.0e15 || (double)B * T * 64 > 2147483647.0) return PPD_ERR_INVALID_ARG;
     const WsLayout wl = workspace_layout(1, B, 1, T, 1, V, 0, PPD_BF16);
     if (!workspace || ws_bytes < wl.total || !aligned(workspace, kAlign)) return PPD_ERR_INVALID_ARG;
-    uint8_t *ws = static_cast<uint8_t *>(workspace);
-    cudaStream_t s = static_cast<cudaStream_t>(stream);
-    float *pv = reinterpret_cast<float *>(ws + wl.part_val);
-    int32_t *pi = reinterpret_cast<int32_t *>(ws + wl.part_idx);
-    float *pst = reinterpret_cast<float *>(ws + wl.part_stats);
-    const int64_t rows = (int64_t)B * T;
-    if (ppd::launch_argmax_partials(logits, rows, V, wl.splits, pv, pi, pst, temperature, nullptr, 0,
-                                    s) != cudaSuccess)
-        return cuda_failed();
-    return cuda_status(ppd::launch_node_stats_combine(pv, pi, pst, rows, wl.splits, argmax_out,
-                                                      lse_out, entropy_out, s));
+    return cuda_status(ppd::launch_node_argmax(logits, (int64_t)B * T, V, temperature, argmax_out, lse_out,
+                                               entropy_out, static_cast<cudaStream_t>(stream)));
 }
 
 ppd_status ppd_typical_accept(const float *logits, const float *lse, const float *entropy,
@@ -786,20 +770,17 @@ ppd_status ppd_typical_accept(const float *logits, const float *lse, const float
                                                   epsilon, delta, static_cast<cudaStream_t>(stream)));
 }
 
-// topk [B][n_states][K] int32, kstate [B] int32, then the partial lists
-// (values fp32, indices int32) [B][n_states][kNextMaxSplit][K] each, then the
-// chain rows' log-sum-exps fp32 [B][n_states][kNextMaxEpt].
-static size_t next_part_bytes(int B, int n_states, int K)
+// topk [B][n_states][K] int32, kstate [B] int32, then the chain rows'
+// log-sum-exps fp32 [B][n_states][kNextMaxEpt].
+static size_t next_lse_offset(int B, int n_states, int K)
 {
-    return align_up((size_t)B * n_states * ppd::kNextMaxSplit * K * sizeof(int32_t));
+    return align_up(align_up((size_t)B * n_states * K * sizeof(int32_t)) + (size_t)B * sizeof(int32_t));
 }
 
 size_t ppd_next_tree_workspace_bytes(int B, int n_states, int K)
 {
     if (B < 1 || n_states < 1 || K < 1) return 0;
-    return align_up(align_up((size_t)B * n_states * K * sizeof(int32_t)) + (size_t)B * sizeof(int32_t)) +
-           2 * next_part_bytes(B, n_states, K) +
-           align_up((size_t)B * n_states * ppd::kNextMaxEpt * sizeof(float));
+    return next_lse_offset(B, n_states, K) + align_up((size_t)B * n_states * ppd::kNextMaxEpt * sizeof(float));
 }
 
 ppd_status ppd_next_tree_ept(const float *logits, const int32_t *parent,
@@ -823,14 +804,10 @@ ppd_status ppd_next_tree_ept(const float *logits, const int32_t *parent,
     int32_t *topk = static_cast<int32_t *>(workspace);
     int32_t *kstate = reinterpret_cast<int32_t *>(static_cast<char *>(workspace) +
                                                   align_up((size_t)B * n_states * K * sizeof(int32_t)));
-    char *parts = static_cast<char *>(workspace) +
-                  align_up(align_up((size_t)B * n_states * K * sizeof(int32_t)) + (size_t)B * sizeof(int32_t));
-    float *part_val = reinterpret_cast<float *>(parts);
-    int32_t *part_idx = reinterpret_cast<int32_t *>(parts + next_part_bytes(B, n_states, K));
-    float *lse = reinterpret_cast<float *>(parts + 2 * next_part_bytes(B, n_states, K));
+    float *lse = reinterpret_cast<float *>(static_cast<char *>(workspace) + next_lse_offset(B, n_states, K));
     return cuda_status(ppd::launch_next_tree(
         logits, parent, cand_tokens, path, accept_len, next_token, B, T, V, n_states, T_next,
-        tmpl_parent, tmpl_rank, K, n_ept, ept_mean, topk, kstate, part_val, part_idx, lse, num_sms(),
+        tmpl_parent, tmpl_rank, K, n_ept, ept_mean, topk, kstate, lse, num_sms(),
         next_parent, next_cand, next_state, dev_status, static_cast<cudaStream_t>(stream)));
 }
 

@@ -31,6 +31,11 @@ PPD_DEV uint64_t global_timer()
     return t;
 }
 
+// Programmatic launches: let the stream's next programmatic grid start; wait for
+// the previous grid to complete (and be visible).
+PPD_DEV void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+PPD_DEV void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // ---------------------------------------------------------------- mbarrier
 
 PPD_DEV void mbar_init(uint64_t *bar, uint32_t count)
@@ -211,6 +216,13 @@ PPD_DEV float ld_cluster_f32(uint32_t a)
 {
     float v;
     asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+    return v;
+}
+
+PPD_DEV unsigned long long ld_cluster_u64(uint32_t a)
+{
+    unsigned long long v;
+    asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(v) : "r"(a) : "memory");
     return v;
 }
 

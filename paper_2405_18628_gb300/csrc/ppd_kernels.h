@@ -203,6 +203,32 @@ cudaError_t launch_tree_attention(const AttnMaps &m, const AttnParams &p, int D,
 cudaError_t launch_tree_attention_rows(const AttnMaps &m, const AttnParams &p, int D, int num_sms,
                                        bool programmatic, cudaStream_t stream);
 
+// A kernel launch as a programmatic dependent of the stream's previous grid (it
+// may start before that grid completes; the kernel waits with pdl_wait()), in
+// clusters of `cluster` (1 1 1: none).
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_chained(void (*kern)(KArgs...), dim3 grid, dim3 block, dim3 cluster,
+                                  cudaStream_t stream, Args... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.numAttrs = 1;
+    if (cluster.x * cluster.y * cluster.z > 1) {
+        attr[1].id = cudaLaunchAttributeClusterDimension;
+        attr[1].val.clusterDim.x = cluster.x;
+        attr[1].val.clusterDim.y = cluster.y;
+        attr[1].val.clusterDim.z = cluster.z;
+        cfg.numAttrs = 2;
+    }
+    cfg.attrs = attr;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
+}
+
 // Splits per node row of the argmax: about 512 blocks over all rows, chunks of
 // at least 2048 logits, at most 64 splits.
 inline int argmax_split_count(int64_t rows, int V)
@@ -249,6 +275,11 @@ struct AcceptArgs {
 cudaError_t launch_accept_path(const int32_t *argmax, const AcceptArgs &a, int B,
                                cudaStream_t stream);
 
+// Node argmax in one grid, a cluster of CTAs per row; with lse_out also the
+// natural-log log-sum-exp and entropy of softmax(row / temperature).
+cudaError_t launch_node_argmax(const float *logits, int64_t rows, int V, float temperature,
+                               int32_t *argmax_out, float *lse_out, float *ent_out, cudaStream_t stream);
+
 // argmax, natural-log log-sum-exp and entropy per row from stats partials.
 cudaError_t launch_node_stats_combine(const float *part_val, const int32_t *part_idx,
                                       const float *part_stats, int64_t rows, int splits,
@@ -269,16 +300,15 @@ cudaError_t launch_kv_compact(void *k_cache, void *v_cache, const void *k_tree,
 // Next-step candidate tree: at most this many guesses per depth.
 constexpr int kNextMaxK = 16;
 constexpr int kNextMaxEpt = 128;
-constexpr int kNextMaxSplit = 16;   // blocks sharing one row's columns
+constexpr int kNextMaxSplit = 8;    // CTAs (a cluster) sharing one row's columns
 
 cudaError_t launch_next_tree(const float *logits, const int32_t *parent, const int32_t *cand,
                              const int32_t *path, const int32_t *accept_len,
                              const int32_t *next_token, int B, int T, int V, int n_states,
                              int T_next, const int32_t *tmpl_parent, const int32_t *tmpl_rank, int K,
-                             int n_ept, int ept_mean, int32_t *topk, int32_t *kstate,
-                             float *part_val, int32_t *part_idx, float *lse, int num_sms,
-                             int32_t *next_parent, int32_t *next_cand, int32_t *next_state,
-                             int32_t *status, cudaStream_t stream);
+                             int n_ept, int ept_mean, int32_t *topk, int32_t *kstate, float *lse,
+                             int num_sms, int32_t *next_parent, int32_t *next_cand,
+                             int32_t *next_state, int32_t *status, cudaStream_t stream);
 
 // fp32 -> bf16 copies (round to nearest even) of n tensors [lbh][rows][D]; of a
 // `cache` tensor only the rows below the sequence's prefix length.  chained: as

@@ -13,16 +13,20 @@
 // lowest-index prompt child by a shared-memory minimum, one node per thread;
 // the end node's prompt children ranked by ballots; each chain walked through
 // those links).  The probability mode then takes each chain row's log-sum-exp
-// (next_lse_kernel, one block a row).  next_topk_kernel shares each row's
-// columns among up to kNextMaxSplit blocks: every thread keeps its own top-K
-// of the averaged logits (or of sum_j exp(x_j - lse_j), the probability mean
-// without its 1/n_ept, which no ranking sees) over a strided slice of its
-// block's columns, read four 16-byte loads per row at a time; each warp takes
-// the best K of its lanes (K rounds of a shuffle maximum, the winning lane
-// popping its head) and one warp the best K of the warps, a partial list.
-// next_topk_merge_kernel, one warp per (sequence, position), takes the best K
-// of the partial lists, and next_assemble_kernel, one warp per sequence, fills
-// the state's template with the root token and the guesses.
+// (next_lse_kernel, one block a row).  next_topk_kernel ranks the averaged
+// logits (or sum_j exp(x_j - lse_j), the probability mean without its 1/n_ept,
+// which no ranking sees) of each row with a cluster of up to kNextMaxSplit CTAs
+// and next_assemble_kernel, one block per sequence, fills the state's template
+// with the root token and the guesses.
+//
+// All of it is latency: the rows of four sequences with four chains each are 6
+// MB, about a microsecond of HBM, behind dependent loads (which rows?) and the
+// selection.  Selecting costs three block barriers a batch of 8192 columns,
+// whatever the values: every warp's K-th largest lane maximum (K rounds of one
+// redux) is a lower bound of the K-th best, the largest of those bounds leaves
+// a few dozen candidates, and a candidate's place is the number of better ones.
+// Insertion into per-thread lists, with the merges of lists in grids of their
+// own, took 48.2 us there (one box; 14.1 now).
 #include "ppd.h"
 #include "ppd_accept.cuh"
 #include "ppd_device.cuh"
@@ -35,17 +39,15 @@ namespace ppd {
 constexpr int kTopkThreads = 512;                  // one tree node per thread (T <= 512)
 constexpr int kTopkWarps = kTopkThreads / 32;
 constexpr int kBatch = 4;                          // 16-byte loads in flight per row and thread
+constexpr int kEach = 4 * kBatch;                  // columns per thread and batch
 constexpr float kLog2e = 1.4426950408889634f;
 static_assert(kMaxTree <= kTopkThreads, "find_chains takes one tree node per thread");
 
-// The kernels of one call form a chain of programmatic launches: each lets
-// the next one launch at its entry, and the next does its setup from the
-// call's inputs (the chains, the template) before it waits for the previous
-// grid to complete and reads what that grid wrote.  The first kernel of a
-// call is launched in plain stream order, so the call's inputs are complete
-// before any of its kernels start.
-PPD_DEV void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-PPD_DEV void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// A call's kernels form a chain of programmatic launches, and so do calls one
+// after the other: each kernel waits for the previous grid before it reads an
+// input.  The kernels in front of next_assemble_kernel let it start only once
+// their own wait is over, so it may read the call's inputs (the template) ahead
+// of its wait for their results.
 
 // Running log-sum-exp of a row: maximum m, sum s of exp(x - m) over the finite
 // entries, and whether a NaN or +inf was seen.  -inf entries add nothing and
@@ -89,54 +91,16 @@ PPD_DEV void lse_warp(LseAcc &a)
     }
 }
 
-// The K-th entry of a best-K list: the one a new entry must beat.
-struct TopkEdge {
-    float v;
-    int i;
-};
-
-// Insert (x, v) into a best-K list (best first) that it is known to enter, and
-// return the list's new K-th entry.  Out of line: the score loops test each
-// candidate against the K-th entry inline and call this rarely (a few dozen
-// times per thread), so one copy of the insertion keeps their code within the
-// instruction cache.
-__device__ __noinline__ TopkEdge topk_insert_slow(float *hv, int *hi, int K, float x, int v)
+// An entry of a ranking as one integer, larger = earlier: NaN first, then the
+// larger value (-0 = +0), then the lower index (< 2^31).  Never 0.
+PPD_DEV uint32_t rank_key(float x)
 {
-    float cv = x;
-    int ci = v;
-    for (int r = 0; r < K; ++r) {
-        if (ranks_before(cv, ci, hv[r], hi[r])) {
-            const float sv = hv[r];
-            const int si = hi[r];
-            hv[r] = cv;
-            hi[r] = ci;
-            cv = sv;
-            ci = si;
-        }
-    }
-    return TopkEdge{hv[K - 1], hi[K - 1]};
+    if (x != x) return 0xFFFFFFFFu;
+    const uint32_t u = x == 0.f ? 0u : __float_as_uint(x);
+    return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
-
-PPD_DEV void topk_insert(float *hv, int *hi, TopkEdge &edge, int K, float x, int v)
-{
-    if (ranks_before(x, v, edge.v, edge.i)) edge = topk_insert_slow(hv, hi, K, x, v);
-}
-
-// The best entry over the lanes of a warp (value, index, and the lane holding it).
-PPD_DEV void warp_best(float &bv, int &bi, int &bl)
-{
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        const float ov = __shfl_xor_sync(0xffffffffu, bv, off);
-        const int oi = __shfl_xor_sync(0xffffffffu, bi, off);
-        const int ol = __shfl_xor_sync(0xffffffffu, bl, off);
-        if (ranks_before(ov, oi, bv, bi)) {
-            bv = ov;
-            bi = oi;
-            bl = ol;
-        }
-    }
-}
+PPD_DEV unsigned long long rank_entry(uint32_t key, int i) { return (unsigned long long)key << 32 | (uint32_t)~i; }
+PPD_DEV int entry_index(unsigned long long e) { return (int)~(uint32_t)e; }
 
 // The n_ept prompt chains below sequence b's accepted end node, for chain
 // position d (one block of kTopkThreads threads, T <= kTopkThreads): each
@@ -160,13 +124,13 @@ PPD_DEV void find_chains(ChainSmem &c, const int32_t *parent, const int32_t *can
     const int cap = n_states - 1;
     const int32_t *par = parent + (size_t)b * T;
     const int32_t *tok = cand + (size_t)b * T;
-    const int n = __ldg(accept_len + b);
-    const int e = (n >= 1 && n <= T) ? __ldg(path + (size_t)b * T + n - 1) : -1;
+    const int n = __ldcg(accept_len + b);
+    const int e = (n >= 1 && n <= T) ? __ldcg(path + (size_t)b * T + n - 1) : -1;
     for (int i = tid; i < T; i += kTopkThreads) c.fc[i] = INT_MAX;
     __syncthreads();
     bool head = false;
     if (tid < T) {
-        const int pa = __ldg(par + tid), tk = __ldg(tok + tid);
+        const int pa = __ldcg(par + tid), tk = __ldcg(tok + tid);
         if (tk == -1 && pa >= 0 && pa < tid) atomicMin(c.fc + pa, tid);
         head = tk == -1 && e >= 0 && e < T && pa == e && tid > e;
     }
@@ -223,6 +187,7 @@ next_lse_kernel(const float *__restrict__ logits, const int32_t *parent, const i
     __shared__ int s_b[kTopkWarps];
     const int b = blockIdx.x, d = blockIdx.y + 1, j = blockIdx.z;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    pdl_wait();
     pdl_release();
     find_chains(cs, parent, cand, path, accept_len, b, d, T, n_states, n_ept);
     if (d > cs.k) return;   // uniform over the block
@@ -266,314 +231,276 @@ next_lse_kernel(const float *__restrict__ logits, const int32_t *parent, const i
 }
 
 // Top-K (K <= kNextMaxK) of the averaged logits (ept_mean 0) or probabilities
-// (ept_mean 1) over columns [z * chunk, (z + 1) * chunk) at chain position d
-// (1-based) of sequence b, z = blockIdx.z, written to the partial lists
-// part_*[((b * (n_states - 1) + d - 1) * gridDim.z + z) * K ...] in ranking
-// order (NaN first, then larger value, then lower index).  The first block of
-// position 1 also writes the state k of its sequence to kstate[b].  vec: rows
-// may be read as float4 (chunk is then a multiple of 4).
+// (ept_mean 1) at chain position d (1-based) of sequence b, in ranking order,
+// into topk[(b * (n_states - 1) + d - 1) * K ...]: one cluster, CTA z taking
+// columns [z * chunk, (z + 1) * chunk).  Position 1 also writes the state k of
+// its sequence to kstate[b].  vec: rows may be read as float4 (chunk is then a
+// multiple of 4).
 __global__ void __launch_bounds__(kTopkThreads)
 next_topk_kernel(const float *__restrict__ logits, const int32_t *parent, const int32_t *cand,
                  const int32_t *path, const int32_t *accept_len, int T, int V, int n_states, int K,
-                 int n_ept, int ept_mean, int vec, int chunk, const float *lse, float *part_val,
-                 int32_t *part_idx, int32_t *kstate)
+                 int n_ept, int ept_mean, int vec, int chunk, const float *lse, int32_t *topk,
+                 int32_t *kstate)
 {
+    // a warp has at most K lanes above its own bound, so at most this many candidates
+    constexpr int kMaxCand = kTopkWarps * kNextMaxK * kEach;
     __shared__ ChainSmem cs;
     __shared__ float s_lse[kNextMaxEpt];
-    __shared__ float s_lv[kTopkWarps][kNextMaxK];
-    __shared__ int s_li[kTopkWarps][kNextMaxK];
+    __shared__ unsigned long long s_bound[kTopkWarps], s_list[2][kNextMaxK], s_cand[kMaxCand];
+    __shared__ int s_n;
     const int b = blockIdx.x;
     const int d = blockIdx.y + 1;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
+    pdl_wait();   // the inputs, the log-sum-exps, and the previous call's readers of topk and kstate
     pdl_release();
     find_chains(cs, parent, cand, path, accept_len, b, d, T, n_states, n_ept);
-    pdl_wait();   // the log-sum-exps, and the previous call's readers of kstate and the lists
     if (tid == 0 && d == 1 && blockIdx.z == 0) kstate[b] = cs.k;
-    if (d > cs.k) return;   // uniform over the block
+    if (d > cs.k) return;   // uniform over the cluster
     auto row = [&](int j) { return logits + ((size_t)b * T + cs.node[j]) * V; };
     const bool probs = ept_mean == 1 && n_ept > 1;
-    const int c0 = (int)blockIdx.z * chunk, c1 = min(V, c0 + chunk);   // this block's columns
+    const int c0 = (int)blockIdx.z * chunk, c1 = min(V, c0 + chunk);   // this CTA's columns
 
     // ---- probability mode: the chain rows' log-sum-exps (next_lse_kernel)
     if (probs) {
         for (int j = tid; j < n_ept; j += kTopkThreads)
             s_lse[j] = __ldcg(lse + ((size_t)b * (n_states - 1) + d - 1) * kNextMaxEpt + j);
-        __syncthreads();
     }
+    if (tid < kNextMaxK) s_list[0][tid] = 0;
+    if (tid == 0) s_n = 0;
+    __syncthreads();
 
-    // ---- this thread's best K over its columns, best first
-    float hv[kNextMaxK];
-    int hi[kNextMaxK];
-#pragma unroll
-    for (int r = 0; r < kNextMaxK; ++r) {
-        hv[r] = -INFINITY;
-        hi[r] = INT_MAX;
-    }
-    TopkEdge edge{-INFINITY, INT_MAX};
     const float n_f = (float)n_ept;
-    if (vec) {
-        const int e4 = c1 >> 2;
-        for (int base = (c0 >> 2) + tid; base < e4; base += kBatch * kTopkThreads) {
-            float4 sc[kBatch];
+    int cur = 0;   // the list of the batches before
+    const int step = vec ? kEach * kTopkThreads : kBatch * kTopkThreads;
+    for (int first = c0; first < c1; first += step) {
+        // ---- this thread's columns: element e is column col(e), ascending in e
+        const int base = first + (vec ? 4 * tid : tid);
+        auto col = [&](int e) { return base + (vec ? (e >> 2) * 4 * kTopkThreads + (e & 3) : e * kTopkThreads); };
+        float sc[kEach];
+        if (vec) {
+            float4 a[kBatch];
 #pragma unroll
-            for (int q = 0; q < kBatch; ++q) sc[q] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (probs) {
-                // sum_j p_j(v), chain order; a NaN lse_j makes every score NaN
-                for (int j = 0; j < n_ept; ++j) {
-                    const float4 *x4 = reinterpret_cast<const float4 *>(row(j));
-                    const float l = s_lse[j];
-                    float4 x[kBatch];
+            for (int q = 0; q < kBatch; ++q) a[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+            // the EPT average is summed in chain order, then divided once (IEEE); the
+            // probabilities are summed in chain order, a NaN lse_j making every score NaN
+            for (int j = 0; j < n_ept; ++j) {
+                const float *x = row(j);
+                float4 f[kBatch];
 #pragma unroll
-                    for (int q = 0; q < kBatch; ++q) x[q] = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-                    for (int q = 0; q < kBatch; ++q)
-                        if (base + q * kTopkThreads < e4) x[q] = __ldcs(x4 + base + q * kTopkThreads);
-#pragma unroll
-                    for (int q = 0; q < kBatch; ++q) {
-                        if (base + q * kTopkThreads < e4) {
-                            sc[q].x += exp2f((x[q].x - l) * kLog2e);
-                            sc[q].y += exp2f((x[q].y - l) * kLog2e);
-                            sc[q].z += exp2f((x[q].z - l) * kLog2e);
-                            sc[q].w += exp2f((x[q].w - l) * kLog2e);
-                        }
-                    }
+                for (int q = 0; q < kBatch; ++q) {
+                    f[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (col(4 * q) < c1) f[q] = __ldcs(reinterpret_cast<const float4 *>(x + col(4 * q)));
                 }
-            } else {
-                // the EPT average: summed in chain order, then one IEEE division
-                const float4 *x0 = reinterpret_cast<const float4 *>(row(0));
+                const float l = probs ? s_lse[j] : 0.f;
 #pragma unroll
-                for (int q = 0; q < kBatch; ++q)
-                    if (base + q * kTopkThreads < e4) sc[q] = __ldcs(x0 + base + q * kTopkThreads);
-                if (n_ept > 1) {
-                    for (int j = 1; j < n_ept; ++j) {
-                        const float4 *x4 = reinterpret_cast<const float4 *>(row(j));
-                        float4 x[kBatch];
-#pragma unroll
-                        for (int q = 0; q < kBatch; ++q) {
-                            x[q] = make_float4(0.f, 0.f, 0.f, 0.f);
-                            if (base + q * kTopkThreads < e4) x[q] = __ldcs(x4 + base + q * kTopkThreads);
-                        }
-#pragma unroll
-                        for (int q = 0; q < kBatch; ++q) {
-                            sc[q].x += x[q].x;
-                            sc[q].y += x[q].y;
-                            sc[q].z += x[q].z;
-                            sc[q].w += x[q].w;
-                        }
+                for (int q = 0; q < kBatch; ++q) {
+                    if (probs) {
+                        f[q].x = exp2f((f[q].x - l) * kLog2e);
+                        f[q].y = exp2f((f[q].y - l) * kLog2e);
+                        f[q].z = exp2f((f[q].z - l) * kLog2e);
+                        f[q].w = exp2f((f[q].w - l) * kLog2e);
                     }
-#pragma unroll
-                    for (int q = 0; q < kBatch; ++q) {
-                        sc[q].x = sc[q].x / n_f;
-                        sc[q].y = sc[q].y / n_f;
-                        sc[q].z = sc[q].z / n_f;
-                        sc[q].w = sc[q].w / n_f;
+                    if (j == 0) {
+                        a[q] = f[q];
+                    } else {
+                        a[q].x += f[q].x;
+                        a[q].y += f[q].y;
+                        a[q].z += f[q].z;
+                        a[q].w += f[q].w;
                     }
                 }
             }
 #pragma unroll
             for (int q = 0; q < kBatch; ++q) {
-                const int v4 = base + q * kTopkThreads;
-                if (v4 < e4) {
-                    topk_insert(hv, hi, edge, K, sc[q].x, 4 * v4);
-                    topk_insert(hv, hi, edge, K, sc[q].y, 4 * v4 + 1);
-                    topk_insert(hv, hi, edge, K, sc[q].z, 4 * v4 + 2);
-                    topk_insert(hv, hi, edge, K, sc[q].w, 4 * v4 + 3);
+                sc[4 * q] = a[q].x;
+                sc[4 * q + 1] = a[q].y;
+                sc[4 * q + 2] = a[q].z;
+                sc[4 * q + 3] = a[q].w;
+            }
+        } else {
+#pragma unroll
+            for (int e = 0; e < kEach; ++e) sc[e] = 0.f;
+            for (int j = 0; j < n_ept; ++j) {
+                const float *x = row(j);
+                const float l = probs ? s_lse[j] : 0.f;
+#pragma unroll
+                for (int e = 0; e < kBatch; ++e) {
+                    float f = col(e) < c1 ? __ldcs(x + col(e)) : 0.f;
+                    if (probs) f = exp2f((f - l) * kLog2e);
+                    sc[e] = j == 0 ? f : sc[e] + f;
                 }
             }
         }
-    } else {
-        for (int v = c0 + tid; v < c1; v += kTopkThreads) {
-            float xv;
-            if (probs) {
-                xv = 0.f;
-                for (int j = 0; j < n_ept; ++j) xv += exp2f((__ldcs(row(j) + v) - s_lse[j]) * kLog2e);
-            } else {
-                xv = __ldcs(row(0) + v);
-                if (n_ept > 1) {
-                    for (int j = 1; j < n_ept; ++j) xv += __ldcs(row(j) + v);
-                    xv = xv / n_f;
-                }
+        const bool mean = !probs && n_ept > 1;
+        uint32_t key[kEach];
+        uint32_t bk = 0;   // the thread's best
+        int bi = INT_MAX;
+#pragma unroll
+        for (int e = 0; e < kEach; ++e) {
+            const bool live = (vec || e < kBatch) && col(e) < c1;
+            key[e] = live ? rank_key(mean ? sc[e] / n_f : sc[e]) : 0u;
+            if (key[e] > bk) {
+                bk = key[e];
+                bi = col(e);
             }
-            topk_insert(hv, hi, edge, K, xv, v);
         }
-    }
 
-    // ---- each warp's best K (K rounds: the best head over the lanes, its lane
-    // pops it), then warp 0 takes the best K of the warps' lists
-    for (int r = 0; r < K; ++r) {
-        float bv = hv[0];
-        int bi = hi[0], bl = lane;
-        warp_best(bv, bi, bl);
-        if (lane == 0) {
-            s_lv[warp][r] = bv;
-            s_li[warp][r] = bi;
-        }
-        if (lane == bl) {
-            for (int q = 0; q + 1 < K; ++q) {
-                hv[q] = hv[q + 1];
-                hi[q] = hi[q + 1];
-            }
-            hv[K - 1] = -INFINITY;
-            hi[K - 1] = INT_MAX;
-        }
-    }
-    __syncthreads();
-    if (warp == 0) {
-        int ptr = 0;   // lane w: next entry of warp w's list
+        // ---- the warp's K-th best lane: at least K entries are as good
+        unsigned long long bound = 0;
         for (int r = 0; r < K; ++r) {
-            float bv = -INFINITY;
-            int bi = INT_MAX, bl = lane;
-            if (lane < kTopkWarps && ptr < K) {
-                bv = s_lv[lane][ptr];
-                bi = s_li[lane][ptr];
+            const uint32_t m = __reduce_max_sync(0xffffffffu, bk);
+            if (m == 0) {   // fewer than K lanes hold anything
+                bound = 0;
+                break;
             }
-            warp_best(bv, bi, bl);
-            if (lane == 0) {
-                const size_t o = (((size_t)b * (n_states - 1) + d - 1) * gridDim.z + blockIdx.z) * K + r;
-                part_val[o] = bv;
-                part_idx[o] = bi;
-            }
-            if (lane == bl) ++ptr;
+            const bool top = bk == m;
+            int i = bi;
+            if (__popc(__ballot_sync(0xffffffffu, top)) > 1) i = __reduce_min_sync(0xffffffffu, top ? bi : INT_MAX);
+            const bool win = top && bi == i;
+            if (r == K - 1) bound = __shfl_sync(0xffffffffu, rank_entry(m, bi), __ffs(__ballot_sync(0xffffffffu, win)) - 1);
+            if (win) bk = 0;
+        }
+        if (lane == 0) s_bound[warp] = bound;
+        __syncthreads();
+        // ---- the candidates: at least as good as every bound, better than the list's last
+        unsigned long long least = s_list[cur][K - 1] + 1;
+#pragma unroll
+        for (int w = 0; w < kTopkWarps; ++w) least = s_bound[w] > least ? s_bound[w] : least;
+        const uint32_t least_key = (uint32_t)(least >> 32);
+#pragma unroll
+        for (int e = 0; e < kEach; ++e) {
+            if (key[e] >= least_key && key[e] != 0 && rank_entry(key[e], col(e)) >= least)
+                s_cand[atomicAdd(&s_n, 1)] = rank_entry(key[e], col(e));
+        }
+        if (tid < kNextMaxK) s_list[cur ^ 1][tid] = 0;
+        __syncthreads();
+        // ---- each entry's place is the number of better ones
+        const int n = s_n;
+        for (int x = tid; x < n + K; x += kTopkThreads) {
+            const unsigned long long mine = x < n ? s_cand[x] : s_list[cur][x - n];
+            int place = 0;
+            for (int y = 0; y < n; ++y) place += s_cand[y] > mine;
+            for (int y = 0; y < K; ++y) place += s_list[cur][y] > mine;
+            if (mine != 0 && place < K) s_list[cur ^ 1][place] = mine;
+        }
+        __syncthreads();
+        if (tid == 0) s_n = 0;
+        cur ^= 1;
+    }
+
+    // ---- the cluster's lists: CTA 0 places every entry among all of them
+    if (cur == 1 && tid < K) s_list[0][tid] = s_list[1][tid];
+    __syncthreads();
+    cluster_sync();
+    if (blockIdx.z == 0) {
+        const int n = (int)gridDim.z * K;   // <= 128 entries
+        unsigned long long *all = s_cand;
+        if (tid < n) all[tid] = ld_cluster_u64(cluster_map(smem_addr(&s_list[0][0]) + (uint32_t)tid % K * 8, tid / K));
+        __syncthreads();
+        if (tid < n) {
+            const unsigned long long mine = all[tid];
+            int place = 0;
+            for (int y = 0; y < n; ++y) place += all[y] > mine;
+            if (mine != 0 && place < K)
+                topk[((size_t)b * (n_states - 1) + d - 1) * K + place] = entry_index(mine);
         }
     }
+    cluster_sync();   // no CTA leaves while CTA 0 reads its list
 }
 
-// One warp per (sequence b, chain position d <= its state): the best K of the
-// n_split partial lists, in ranking order, into topk[(b * (n_states - 1) + d -
-// 1) * K ...].  Lane z walks list z.
-__global__ void __launch_bounds__(32)
-next_topk_merge_kernel(const float *part_val, const int32_t *part_idx, int n_states, int K,
-                       int n_split, const int32_t *kstate, int32_t *topk)
-{
-    const int b = blockIdx.x, d = blockIdx.y + 1, lane = threadIdx.x;
-    pdl_release();
-    pdl_wait();   // the partial lists and the states
-    if (d > __ldcg(kstate + b)) return;   // uniform over the warp
-    const size_t base = ((size_t)b * (n_states - 1) + d - 1) * n_split;
-    int ptr = 0;
-    for (int r = 0; r < K; ++r) {
-        float bv = -INFINITY;
-        int bi = INT_MAX, bl = lane;
-        if (lane < n_split && ptr < K) {
-            bv = __ldcg(part_val + (base + lane) * K + ptr);
-            bi = __ldcg(part_idx + (base + lane) * K + ptr);
-        }
-        warp_best(bv, bi, bl);
-        if (lane == 0) topk[((size_t)b * (n_states - 1) + d - 1) * K + r] = bi;
-        if (lane == bl) ++ptr;
-    }
-}
+// One block per sequence: state, template checks, and the next tree.  The
+// templates (all states', when they fit) are in shared memory before the wait
+// for the states and guesses.
+constexpr int kAsmThreads = 256;
+constexpr int kAsmEntries = 4096;
 
-// One warp per sequence: state, template checks, and the next tree.
-__global__ void __launch_bounds__(128)
-next_assemble_kernel(const int32_t *parent, const int32_t *cand, const int32_t *path,
-                     const int32_t *accept_len, const int32_t *next_token, int B, int T,
+__global__ void __launch_bounds__(kAsmThreads)
+next_assemble_kernel(const int32_t *path, const int32_t *accept_len, const int32_t *next_token, int T,
                      int n_states, int T_next, const int32_t *tmpl_parent, const int32_t *tmpl_rank,
                      int K, const int32_t *topk, const int32_t *kstate, int32_t *next_parent,
-                     int32_t *next_cand, int32_t *next_state, int32_t *status)
+                     int32_t *next_cand, int32_t *next_state, int32_t *status, int early)
 {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int b = blockIdx.x * 4 + warp;
-    if (b >= B) return;
-    const int n = __ldg(accept_len + b);
-    const int nt = __ldg(next_token + b);
+    __shared__ int16_t s_par[kAsmEntries], s_rank[kAsmEntries];   // clamped: every valid value fits
+    const int b = blockIdx.x, tid = threadIdx.x;
+    const int total = n_states * T_next;
+    const bool all = early && total <= kAsmEntries;
+    auto clamp16 = [](int v) { return (int16_t)max(-2, min(v, 32767)); };
+    auto load = [&](int first, int n) {
+        for (int i = tid; i < n; i += kAsmThreads) {
+            s_par[i] = clamp16(__ldg(tmpl_parent + first + i));
+            s_rank[i] = clamp16(__ldg(tmpl_rank + first + i));
+        }
+    };
+    if (!early) pdl_wait();
+    pdl_release();
+    if (all) load(0, total);
+    if (early) pdl_wait();   // the states and the guesses (and, of a call's only grid, the inputs)
+    const int n = __ldcg(accept_len + b), nt = __ldcg(next_token + b);
     bool bad = !(n >= 1 && n <= T && nt >= 0);
-    pdl_wait();   // the states and the guesses
     int k = 0;
     if (!bad) {
-        const int e = __ldg(path + (size_t)b * T + n - 1);
+        const int e = __ldcg(path + (size_t)b * T + n - 1);
         bad = !(e >= 0 && e < T);
         if (!bad && n_states > 1) k = __ldcg(kstate + b);
     }
-    const int32_t *tp = tmpl_parent + (size_t)k * T_next;
-    const int32_t *tr = tmpl_rank + (size_t)k * T_next;
+    if (!all) load(k * T_next, T_next);
+    __syncthreads();
+    const int16_t *tp = s_par + (all ? k * T_next : 0), *tr = s_rank + (all ? k * T_next : 0);
     int32_t *np = next_parent + (size_t)b * T_next;
     int32_t *nc = next_cand + (size_t)b * T_next;
-    // template checks and each node's candidate depth (walk to the root)
-    for (int i = lane; i < T_next && !bad; i += 32) {
-        const int pi = __ldg(tp + i);
-        if (i == 0) {
-            bad |= pi != -1;
-            continue;
-        }
-        bad |= pi < 0 || pi >= i;
-        const int r = __ldg(tr + i);
-        if (r >= 0) bad |= r >= K;
+    // template checks: parents before their children, ranks below K
+    for (int i = tid; i < T_next && !bad; i += kAsmThreads) {
+        if (i == 0) bad |= tp[0] != -1;
+        else bad |= tp[i] < 0 || tp[i] >= i || tr[i] >= K;
     }
-    bad = __any_sync(0xffffffffu, bad);
+    bad = __syncthreads_or(bad);
+    // each candidate's depth: only candidates above it, at most k of them with itself
+    int tok[2] = {-1, -1};   // T_next <= 512: two nodes a thread
     if (!bad) {
-        for (int i = lane; i < T_next; i += 32) {
-            const int r = __ldg(tr + i);
-            int tokv = -1;
+#pragma unroll
+        for (int x = 0; x < 2; ++x) {
+            const int i = tid + x * kAsmThreads;
+            if (i >= T_next) continue;
             if (i == 0) {
-                tokv = nt;
-            } else if (r >= 0) {
-                int depth = 0, a = i;
+                tok[x] = nt;
+            } else if (tr[i] >= 0) {
+                int depth = 0;
                 bool ok = true;
-                while (a > 0) {
-                    ok &= __ldg(tr + a) >= 0;     // every node above a candidate is a candidate
+                for (int a = i; a > 0; a = tp[a]) {
+                    ok &= tr[a] >= 0;
                     ++depth;
-                    a = __ldg(tp + a);
                 }
-                if (!ok || depth > k) {
-                    tokv = INT_MIN;               // marks a bad template
-                } else {
-                    tokv = __ldcg(topk + ((size_t)b * (n_states - 1) + depth - 1) * K + r);
-                }
+                if (!ok || depth > k) bad = true;
+                else tok[x] = __ldcg(topk + ((size_t)b * (n_states - 1) + depth - 1) * K + tr[i]);
             }
-            nc[i] = tokv;
-            np[i] = __ldg(tp + i);
-        }
-        __syncwarp();
-        bool inv = false;
-        for (int i = lane; i < T_next; i += 32) inv |= nc[i] == INT_MIN;
-        bad = __any_sync(0xffffffffu, inv);
-    }
-    if (bad) {
-        for (int i = lane; i < T_next; i += 32) {
-            np[i] = -1;
-            nc[i] = -1;
         }
     }
-    if (lane == 0) {
+    bad = __syncthreads_or(bad);
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+        const int i = tid + x * kAsmThreads;
+        if (i >= T_next) continue;
+        np[i] = bad ? -1 : tp[i];
+        nc[i] = bad ? -1 : tok[x];
+    }
+    if (tid == 0) {
         next_state[b] = bad ? -1 : k;
         status[b] = bad ? kErrTree : kOk;
     }
-}
-
-// A kernel launch, as a programmatic dependent of the stream's previous grid
-// when `chained` (it may then start before that grid completes, and waits
-// for it with griddepcontrol.wait).
-template <typename... KArgs, typename... Args>
-static cudaError_t launch_chained(void (*kern)(KArgs...), dim3 grid, dim3 block, bool chained,
-                                  cudaStream_t stream, Args... args)
-{
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = block;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = chained ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
 }
 
 cudaError_t launch_next_tree(const float *logits, const int32_t *parent, const int32_t *cand,
                              const int32_t *path, const int32_t *accept_len,
                              const int32_t *next_token, int B, int T, int V, int n_states,
                              int T_next, const int32_t *tmpl_parent, const int32_t *tmpl_rank, int K,
-                             int n_ept, int ept_mean, int32_t *topk, int32_t *kstate,
-                             float *part_val, int32_t *part_idx, float *lse, int num_sms,
-                             int32_t *next_parent, int32_t *next_cand, int32_t *next_state,
-                             int32_t *status, cudaStream_t stream)
+                             int n_ept, int ept_mean, int32_t *topk, int32_t *kstate, float *lse,
+                             int num_sms, int32_t *next_parent, int32_t *next_cand,
+                             int32_t *next_state, int32_t *status, cudaStream_t stream)
 {
-    bool chained = false;   // the call's first kernel waits for the work before it
     if (n_states > 1) {
         const int vec = (V % 4 == 0) && ((reinterpret_cast<uintptr_t>(logits) & 15) == 0);
-        // each row shared by n_split blocks, about two blocks per SM in all
+        // each row shared by a cluster, about two CTAs per SM in all, no CTA without columns
         const long long rows = (long long)B * (n_states - 1);
         int n_split = (int)((2LL * num_sms + rows - 1) / rows);
         n_split = n_split < 1 ? 1 : (n_split > kNextMaxSplit ? kNextMaxSplit : n_split);
@@ -583,27 +510,20 @@ cudaError_t launch_next_tree(const float *logits, const int32_t *parent, const i
         const unsigned cap = (unsigned)(n_states - 1);
         cudaError_t e;
         if (ept_mean == 1 && n_ept > 1) {
-            e = launch_chained(next_lse_kernel, dim3((unsigned)B, cap, (unsigned)n_ept),
-                               dim3(kTopkThreads), chained, stream, logits, parent, cand, path,
-                               accept_len, T, V, n_states, n_ept, vec, lse);
+            e = launch_chained(next_lse_kernel, dim3((unsigned)B, cap, (unsigned)n_ept), dim3(kTopkThreads),
+                               dim3(1), stream, logits, parent, cand, path, accept_len, T, V, n_states,
+                               n_ept, vec, lse);
             if (e != cudaSuccess) return e;
-            chained = true;
         }
-        e = launch_chained(next_topk_kernel, dim3((unsigned)B, cap, (unsigned)n_split),
-                           dim3(kTopkThreads), chained, stream, logits, parent, cand, path,
-                           accept_len, T, V, n_states, K, n_ept, ept_mean, vec, chunk,
-                           (const float *)lse, part_val, part_idx, kstate);
+        e = launch_chained(next_topk_kernel, dim3((unsigned)B, cap, (unsigned)n_split), dim3(kTopkThreads),
+                           dim3(1, 1, (unsigned)n_split), stream, logits, parent, cand, path, accept_len, T,
+                           V, n_states, K, n_ept, ept_mean, vec, chunk, (const float *)lse, topk, kstate);
         if (e != cudaSuccess) return e;
-        e = launch_chained(next_topk_merge_kernel, dim3((unsigned)B, cap), dim3(32), true, stream,
-                           (const float *)part_val, (const int32_t *)part_idx, n_states, K, n_split,
-                           (const int32_t *)kstate, topk);
-        if (e != cudaSuccess) return e;
-        chained = true;
     }
-    return launch_chained(next_assemble_kernel, dim3((unsigned)((B + 3) / 4)), dim3(128), chained,
-                          stream, parent, cand, path, accept_len, next_token, B, T, n_states,
-                          T_next, tmpl_parent, tmpl_rank, K, (const int32_t *)topk,
-                          (const int32_t *)kstate, next_parent, next_cand, next_state, status);
+    return launch_chained(next_assemble_kernel, dim3((unsigned)B), dim3(kAsmThreads), dim3(1), stream, path,
+                          accept_len, next_token, T, n_states, T_next, tmpl_parent, tmpl_rank, K,
+                          (const int32_t *)topk, (const int32_t *)kstate, next_parent, next_cand,
+                          next_state, status, n_states > 1 ? 1 : 0);
 }
 
 }  // namespace ppd

@@ -4,8 +4,9 @@
 // Node argmax (paper Section 3 step (2): exact matching compares every guess
 // token with the model's top-1 token at its parent) streams the fp32 logits
 // with 16-byte loads, reduces (value, index) pairs with warp shuffles, and
-// splits long rows over several blocks whose partial results are combined by
-// the last block to finish.  Acceptance (Section 3 steps (2)-(3)) runs one
+// splits long rows over several blocks: a cluster, whose first CTA reads the
+// others' results, or in the fused step partial results that its side warps
+// combine.  Acceptance (Section 3 steps (2)-(3)) runs one
 // warp per sequence: ballots build the bitset of matching nodes, each lane
 // walks its nodes' root paths, and a warp max-reduction picks the deepest
 // accepted node.  Compaction (Section 3 step (3)) copies the accepted rows
@@ -17,7 +18,6 @@
 
 #include <climits>
 #include <cmath>
-#include <mutex>
 
 namespace ppd {
 
@@ -218,6 +218,102 @@ cudaError_t launch_argmax_narrow(const float *logits, int64_t rows, int V, int s
     return cudaGetLastError();
 }
 
+// Node argmax (and with kStats lse and entropy) in one grid: a cluster of CTAs
+// per row, CTA r scanning columns [r*chunk, (r+1)*chunk) as the partial kernel
+// does; the first CTA reads the others' results from their shared memory.
+// Latency-bound (64 rows of 32000: 8 MB).  With this grid in place of a partial
+// and a combine grid, the calls after a forward pass launched as a programmatic
+// chain and the next tree's two grids, those calls took 28.3 us instead of 53.5
+// (host-bound: 64 nodes, 1024 slices, four calls).
+template <bool kStats>
+__global__ void __launch_bounds__(256)
+node_argmax_kernel(const float *__restrict__ logits, int V, int chunk, int vec, int32_t *argmax_out,
+                   float stat_k, float *lse_out, float *ent_out, int n_cta)
+{
+    struct Best {
+        float v;
+        int i;
+        float m, s, t;
+    };
+    __shared__ Best s_b[8], s_all;
+    pdl_release();
+    pdl_wait();
+    const int64_t row = blockIdx.x / n_cta;
+    const int r = blockIdx.x % n_cta, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // the CTA's columns in eight spans, one per warp, multiples of four
+    const int span = ((chunk + 7) / 8 + 3) & ~3;
+    const int c1 = min(V, (r + 1) * chunk), lo = min(c1, r * chunk + warp * span), hi = min(c1, lo + span);
+    float bv;
+    int bi;
+    SoftStats st;
+    warp_logit_span<kStats, 8>(logits + row * (int64_t)V, lo, hi, vec != 0, stat_k, lane, bv, bi, st);
+    if (lane == 0) s_b[warp] = Best{bv, bi, st.m, st.s, st.t};
+    __syncthreads();
+    auto merge = [&](const Best &o) {
+        consider(o.v, o.i, bv, bi);
+        if (kStats) {
+            SoftStats x;
+            x.m = o.m;
+            x.s = o.s;
+            x.t = o.t;
+            stats_merge(st, x);
+        }
+    };
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < 8; ++w) merge(s_b[w]);
+        s_all = Best{bv, bi, st.m, st.s, st.t};
+    }
+    if (n_cta > 1) {
+        __syncthreads();
+        cluster_sync();
+        if (r == 0 && warp == 0) {
+            Best o{-INFINITY, INT_MAX, -INFINITY, 0.f, 0.f};
+            if (lane < n_cta) {
+                const uint32_t a = cluster_map(smem_addr(&s_all), lane);
+                o.v = ld_cluster_f32(a);
+                o.i = __float_as_int(ld_cluster_f32(a + 4));
+                if (kStats) {
+                    o.m = ld_cluster_f32(a + 8);
+                    o.s = ld_cluster_f32(a + 12);
+                    o.t = ld_cluster_f32(a + 16);
+                }
+            }
+            for (int c = 1; c < n_cta; ++c) {
+                Best x;
+                x.v = __shfl_sync(0xffffffffu, o.v, c);
+                x.i = __shfl_sync(0xffffffffu, o.i, c);
+                if (kStats) {
+                    x.m = __shfl_sync(0xffffffffu, o.m, c);
+                    x.s = __shfl_sync(0xffffffffu, o.s, c);
+                    x.t = __shfl_sync(0xffffffffu, o.t, c);
+                }
+                if (lane == 0) merge(x);
+            }
+        }
+        cluster_sync();   // no CTA leaves while the first reads its result
+    }
+    if (r == 0 && threadIdx.x == 0) {
+        argmax_out[row] = bi;
+        if (kStats) stats_finish(st, lse_out[row], ent_out[row]);
+    }
+}
+
+cudaError_t launch_node_argmax(const float *logits, int64_t rows, int V, float temperature,
+                               int32_t *argmax_out, float *lse_out, float *ent_out, cudaStream_t stream)
+{
+    const int vec = (V % 4 == 0) && ((reinterpret_cast<uintptr_t>(logits) & 15) == 0);
+    int n = argmax_split_count(rows, V);
+    if (n > 8) n = 8;   // the portable cluster size
+    const int chunk = (((V + n - 1) / n) + 3) & ~3;
+    n = (V + chunk - 1) / chunk;
+    const dim3 grid((unsigned)(rows * n));
+    if (lse_out)
+        return launch_chained(node_argmax_kernel<true>, grid, dim3(256), dim3((unsigned)n), stream, logits, V, chunk,
+                              vec, argmax_out, 1.4426950408889634f / temperature, lse_out, ent_out, n);
+    return launch_chained(node_argmax_kernel<false>, grid, dim3(256), dim3((unsigned)n), stream, logits, V, chunk,
+                          vec, argmax_out, 0.f, (float *)nullptr, (float *)nullptr, n);
+}
+
 cudaError_t launch_argmax_combine(const float *part_val, const int32_t *part_idx, int64_t rows,
                                   int splits, int32_t *argmax_out, cudaStream_t stream)
 {
@@ -228,30 +324,51 @@ cudaError_t launch_argmax_combine(const float *part_val, const int32_t *part_idx
 
 // ------------------------------------------------------------------ accept
 
+PPD_DEV void write_accept(const AcceptArgs &a, int b, const AcceptResult &r)
+{
+    a.accept_len[b] = r.n_acc;
+    a.next_token[b] = r.next_token;
+    a.new_prefix_len[b] = r.new_prefix_len;
+    a.dev_status[b] = r.status;
+}
+
+// (Grids of a programmatic chain start before the one that writes their inputs is
+// done, so what other grids write is read through L2.)
+// One warp per sequence; trees of up to 64 nodes in registers, whose walks cost
+// shuffles instead of dependent loads.
 __global__ void __launch_bounds__(128)
 accept_path_kernel(const int32_t *argmax, AcceptArgs a, int B)
 {
     __shared__ int s_par[4][kAcceptScratchInts];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int b = blockIdx.x * 4 + warp;
+    pdl_release();
+    pdl_wait();
     if (b >= B) return;
-    const int32_t *top = argmax + (size_t)b * a.T;
-    const AcceptResult r = accept_warp([&](int n) { return __ldg(top + n); }, a.parent + (size_t)b * a.T,
-                                       a.cand_tokens + (size_t)b * a.T, __ldg(a.prefix_len + b), a.T,
-                                       a.V, a.S_max, lane, s_par[warp], a.path + (size_t)b * a.T);
-    if (lane == 0) {
-        a.accept_len[b] = r.n_acc;
-        a.next_token[b] = r.next_token;
-        a.new_prefix_len[b] = r.new_prefix_len;
-        a.dev_status[b] = r.status;
+    const size_t o = (size_t)b * a.T;
+    const int32_t *top = argmax + o;
+    AcceptResult r;
+    if (a.T <= 64) {
+        int top_r[2], path_r[2];
+#pragma unroll
+        for (int k = 0; k < 2; ++k) top_r[k] = lane + 32 * k < a.T ? __ldcg(top + lane + 32 * k) : 0;
+        r = accept_warp_small(
+            top_r, [&](int, int pa, int tk) { return tk == node_value(top_r, pa); }, a.parent + o,
+            a.cand_tokens + o, __ldcg(a.prefix_len + b), a.T, a.V, a.S_max, lane, path_r);
+#pragma unroll
+        for (int k = 0; k < 2; ++k)
+            if (lane + 32 * k < a.T) a.path[o + lane + 32 * k] = path_r[k];
+    } else {
+        r = accept_warp([&](int n) { return __ldcg(top + n); }, a.parent + o, a.cand_tokens + o,
+                        __ldcg(a.prefix_len + b), a.T, a.V, a.S_max, lane, s_par[warp], a.path + o);
     }
+    if (lane == 0) write_accept(a, b, r);
 }
 
 cudaError_t launch_accept_path(const int32_t *argmax, const AcceptArgs &a, int B,
                                cudaStream_t stream)
 {
-    accept_path_kernel<<<(B + 3) / 4, 128, 0, stream>>>(argmax, a, B);
-    return cudaGetLastError();
+    return launch_chained(accept_path_kernel, dim3((unsigned)((B + 3) / 4)), dim3(128), dim3(1), stream, argmax, a, B);
 }
 
 // Node statistics: argmax, natural-log log-sum-exp and entropy of each row
@@ -286,20 +403,17 @@ typical_accept_kernel(const float *logits, const float *lse, const float *ent,
     __shared__ int s_par[4][kAcceptScratchInts];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int b = blockIdx.x * 4 + warp;
+    pdl_release();
+    pdl_wait();
     if (b >= B) return;
     const size_t o = (size_t)b * a.T;
     const int32_t *top = argmax + o;
     const AcceptResult r = accept_warp_typical(
-        [&](int n) { return __ldg(top + n); }, logits + o * a.V,
-        [&](int n) { return __ldg(lse + o + n); }, [&](int n) { return __ldg(ent + o + n); },
-        inv_temp, epsilon, delta, a.parent + o, a.cand_tokens + o, __ldg(a.prefix_len + b), a.T,
+        [&](int n) { return __ldcg(top + n); }, logits + o * a.V,
+        [&](int n) { return __ldcg(lse + o + n); }, [&](int n) { return __ldcg(ent + o + n); },
+        inv_temp, epsilon, delta, a.parent + o, a.cand_tokens + o, __ldcg(a.prefix_len + b), a.T,
         a.V, a.S_max, lane, s_par[warp], a.path + o);
-    if (lane == 0) {
-        a.accept_len[b] = r.n_acc;
-        a.next_token[b] = r.next_token;
-        a.new_prefix_len[b] = r.new_prefix_len;
-        a.dev_status[b] = r.status;
-    }
+    if (lane == 0) write_accept(a, b, r);
 }
 
 cudaError_t launch_typical_accept(const float *logits, const float *lse, const float *ent,
@@ -307,9 +421,8 @@ cudaError_t launch_typical_accept(const float *logits, const float *lse, const f
                                   float temperature, float epsilon, float delta,
                                   cudaStream_t stream)
 {
-    typical_accept_kernel<<<(B + 3) / 4, 128, 0, stream>>>(logits, lse, ent, argmax, a, B,
-                                                           1.0f / temperature, epsilon, delta);
-    return cudaGetLastError();
+    return launch_chained(typical_accept_kernel, dim3((unsigned)((B + 3) / 4)), dim3(128), dim3(1), stream, logits,
+                          lse, ent, argmax, a, B, 1.0f / temperature, epsilon, delta);
 }
 
 // ------------------------------------------------------------------ compaction
@@ -321,14 +434,16 @@ kv_compact_kernel(uint8_t *kc, uint8_t *vc, const uint8_t *__restrict__ kt,
                   int row_bytes)
 {
     const int chunks = row_bytes >> 4;
+    pdl_release();
+    pdl_wait();
     for (int64_t u = blockIdx.x; u < n_units; u += gridDim.x) {
         const int b = (int)((u / H) % B);
-        const int n = __ldg(accept_len + b);
-        const int P = __ldg(prefix_len + b);
+        const int n = __ldcg(accept_len + b);
+        const int P = __ldcg(prefix_len + b);
         if (n <= 0 || n > T || P < 0 || (long long)P + n > S_max) continue;
         for (int w = threadIdx.x; w < n * chunks; w += blockDim.x) {
             const int j = w / chunks, c = w - j * chunks;
-            const int src = __ldg(path + (size_t)b * T + j);
+            const int src = __ldcg(path + (size_t)b * T + j);
             if (src < 0 || src >= T) continue;
             const size_t so = ((size_t)u * T + src) * row_bytes + (size_t)c * 16;
             const size_t dof = ((size_t)u * S_max + P + j) * row_bytes + (size_t)c * 16;
@@ -348,11 +463,10 @@ cudaError_t launch_kv_compact(void *k_cache, void *v_cache, const void *k_tree,
 {
     const int64_t n_units = (int64_t)L * B * H;
     const int grid = (int)(n_units < 4096 ? n_units : 4096);
-    kv_compact_kernel<<<grid, 128, 0, stream>>>(
-        static_cast<uint8_t *>(k_cache), static_cast<uint8_t *>(v_cache),
-        static_cast<const uint8_t *>(k_tree), static_cast<const uint8_t *>(v_tree), path,
-        accept_len, prefix_len, n_units, B, H, T, S_max, D * elem_bytes);
-    return cudaGetLastError();
+    return launch_chained(kv_compact_kernel, dim3((unsigned)grid), dim3(128), dim3(1), stream,
+                          static_cast<uint8_t *>(k_cache), static_cast<uint8_t *>(v_cache),
+                          static_cast<const uint8_t *>(k_tree), static_cast<const uint8_t *>(v_tree), path,
+                          accept_len, prefix_len, n_units, B, H, T, S_max, D * elem_bytes);
 }
 
 // ------------------------------------------------------------------ status reset
@@ -594,63 +708,21 @@ cudaError_t launch_selftest_umma(const CUtensorMap &ma, const CUtensorMap &mb, c
 }
 
 // ------------------------------------------------------------------ argmax without a workspace
-//
-// ppd_node_argmax_noalloc keeps its partial maxima in this fixed array instead of a
-// caller-provided workspace.  Every GPU that loads the library holds it until the
-// process exits.  Host code may not use the array's name as a device address: the
-// address is looked up once per device with cudaGetSymbolAddress, with that device
-// current, on the first call there.
-namespace {
-
-constexpr int64_t kNoAllocMaxPartials = 1 << 16;   // (row, split) pairs: 512 KiB in total
-
-static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocMaxPartials * 8];
-
-constexpr int kMaxDevices = 64;
-std::mutex g_noalloc_mutex;
-void *g_noalloc_addr[kMaxDevices] = {nullptr};
-
-// Device address of the scratch array on the current device (looked up once).
-cudaError_t noalloc_scratch(void **addr)
-{
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
-    std::lock_guard<std::mutex> lock(g_noalloc_mutex);
-    if (g_noalloc_addr[dev] == nullptr) {
-        void *p = nullptr;
-        e = cudaGetSymbolAddress(&p, g_noalloc_scratch);
-        if (e != cudaSuccess) return e;
-        g_noalloc_addr[dev] = p;
-    }
-    *addr = g_noalloc_addr[dev];
-    return cudaSuccess;
-}
-
-}  // namespace
 
 }  // namespace ppd
 
+// The same grid as ppd_node_argmax, which needs no scratch; requests of more than
+// 65,536 rows stay refused.
 extern "C" ppd_status ppd_node_argmax_noalloc(const float *logits, int B, int T, int V,
                                               int32_t *argmax_out, void *stream)
 {
+    constexpr int64_t kMaxRows = 1 << 16;
     if (!logits || !argmax_out || B < 1 || T < 1 || V < 1) return PPD_ERR_INVALID_ARG;
     if ((double)B * T * V > 9.0e15) return PPD_ERR_INVALID_ARG;
     const int64_t rows = (int64_t)B * T;
-    if (rows > ppd::kNoAllocMaxPartials) return PPD_ERR_UNSUPPORTED;   // B*T above the array's size
-    int splits = ppd::argmax_split_count(rows, V);
-    if (rows * splits > ppd::kNoAllocMaxPartials) splits = (int)(ppd::kNoAllocMaxPartials / rows);
-    void *scratch = nullptr;
-    if (ppd::noalloc_scratch(&scratch) != cudaSuccess) return PPD_ERR_CUDA;
-    float *pv = static_cast<float *>(scratch);
-    int32_t *pi = reinterpret_cast<int32_t *>(static_cast<unsigned char *>(scratch) +
-                                              ppd::kNoAllocMaxPartials * 4);
-    cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (ppd::launch_argmax_partials(logits, rows, V, splits, pv, pi, nullptr, 1.f, nullptr, 0, s) !=
-        cudaSuccess)
-        return PPD_ERR_CUDA;
-    return ppd::launch_argmax_combine(pv, pi, rows, splits, argmax_out, s) == cudaSuccess ? PPD_OK
-                                                                                          : PPD_ERR_CUDA;
+    if (rows > kMaxRows) return PPD_ERR_UNSUPPORTED;
+    return ppd::launch_node_argmax(logits, rows, V, 1.f, argmax_out, nullptr, nullptr,
+                                   static_cast<cudaStream_t>(stream)) == cudaSuccess
+               ? PPD_OK
+               : PPD_ERR_CUDA;
 }
-

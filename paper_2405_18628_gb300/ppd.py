@@ -177,7 +177,7 @@ def ppd_node_argmax(logits, argmax_out, workspace=None, stream=None):
 
 def ppd_node_argmax_noalloc(logits, argmax_out, stream=None):
     """Node argmax without a workspace: logits fp32 [B,T,V] -> argmax_out int32
-    [B,T], partial maxima kept in the library's fixed device array."""
+    [B,T] (the same grid as ppd_node_argmax, which needs no scratch)."""
     B, T, V = logits.shape
     x, am = _ptrs(logits, argmax_out)
     st = load().ppd_node_argmax_noalloc(x, B, T, V, am, _stream(stream))

@@ -311,3 +311,45 @@ def test_next_tree_small_vocab_split_rows(cuda_device, V, K):
         else:
             _compare(got, ref)
         assert (ref["next_state"] > 0).any()
+
+
+@pytest.mark.parametrize("B,V", [(7, 140000),      # several batches of columns in every CTA of a row
+                                 (7, 20001),       # the same with scalar loads, an odd last CTA
+                                 (160, 9000)])     # a row per CTA
+@pytest.mark.parametrize("n_ept", [1, 2])
+def test_next_tree_selection(cuda_device, B, V, n_ept):
+    """The selection on rows that crowd its candidates: sorted either way,
+    constant, all but a few entries -inf, NaNs and ties at the end, a few
+    values repeated everywhere."""
+    T, K = 7, 16
+    parent = np.tile(np.array([-1, 0, 1, 1, 2, 3, 0], np.int32), (B, 1))
+    cand = np.tile(np.array([3, 4, -1, -1, -1, -1, -1], np.int32), (B, 1))
+    path = np.tile(np.array([0, 1, -1, -1, -1, -1, -1], np.int32), (B, 1))
+    rng = np.random.default_rng(V + n_ept)
+    logits = rng.standard_normal((B, T, V)).astype(np.float32)
+    ramp = np.linspace(-3, 3, V).astype(np.float32)
+    for b in range(B):
+        for r in range(2, 6):
+            x = logits[b, r]
+            kind = b % 7
+            if kind == 0:
+                x[:] = ramp
+            elif kind == 1:
+                x[:] = ramp[::-1]
+            elif kind == 2:
+                x[:] = 0.5
+            elif kind == 3:
+                x[:] = -np.inf
+                x[[5, V // 2, V - 1]] = [-2.0, 1.0, 1.0]
+            elif kind == 4:
+                x[-40:] = 9.0
+                x[[V - 3, V // 3]] = np.nan
+            elif kind == 5:
+                x[:] = np.round(x)
+                x[x == 0] *= rng.choice([-1.0, 1.0])      # -0 and +0 rank alike
+    alen, nt = np.full(B, 2, np.int32), np.arange(B, dtype=np.int32)
+    tp, tr = W.make_tree_templates(3, 128, K, rng, n_ept=n_ept)
+    ref = oracle.next_tree(logits, parent, cand, path, alen, nt, tp, tr, K, n_ept=n_ept)
+    assert (ref["status"] == 0).all() and (ref["next_state"] == 2).all()
+    got = _run(cuda_device, logits, parent, cand, path, alen, nt, tp, tr, K, n_ept=n_ept)
+    _compare(got, ref)

@@ -300,6 +300,33 @@ def test_node_argmax_matches_oracle(cuda_device, B, T, V):
         np.testing.assert_array_equal(out.cpu().numpy(), oracle.node_argmax(x))
 
 
+@pytest.mark.parametrize("rows,V", [(1, 128256), (3, 300001), (700, 4100), (8, 2049), (130, 8193)])
+def test_node_argmax_cluster_sizes(cuda_device, rows, V):
+    """One to eight CTAs a row, spans that end inside a CTA's last warps, odd
+    vocabularies: ties across CTAs and warps go to the lower index."""
+    rng = np.random.default_rng(rows + V)
+    x = rng.standard_normal((1, rows, V)).astype(np.float32)
+    for r in range(0, rows, 2):
+        x[0, r, rng.integers(0, V, size=6)] = 30.0
+    x[0, rows - 1, V - 1] = np.nan
+    out = torch.empty((1, rows), dtype=torch.int32, device=cuda_device)
+    lse, ent = torch.empty((1, rows), device=cuda_device), torch.empty((1, rows), device=cuda_device)
+    ws = ppd.workspace(1, 1, 1, rows, 64, V, 1, device=cuda_device)
+    xd = torch.from_numpy(x).to(cuda_device)
+    ppd.ppd_node_argmax(xd, out, ws)
+    want = oracle.node_argmax(x)
+    np.testing.assert_array_equal(out.cpu().numpy(), want)
+    out.fill_(-5)
+    ppd.ppd_node_stats(xd, 0.7, out, lse, ent, ws)
+    np.testing.assert_array_equal(out.cpu().numpy(), want)
+    ref_lse, ref_ent = oracle.node_stats(x, 0.7)
+    fine = ~np.isnan(ref_lse)
+    assert (np.isnan(lse.cpu().numpy()) == ~fine).all()
+    # fp32 sums of up to 3e5 terms per row, in eight-way trees: about 1e-6 relative
+    np.testing.assert_allclose(lse.cpu().numpy()[fine], ref_lse[fine], rtol=4e-6, atol=2e-5)
+    np.testing.assert_allclose(ent.cpu().numpy()[fine], ref_ent[fine], rtol=4e-5, atol=4e-5)
+
+
 # ----------------------------------------------------------------------------- accept
 
 def _random_accept_case(rng, B, T, V, match=0.6):
