@@ -106,7 +106,8 @@ struct AttnLayout {
     static constexpr uint32_t OFF_PMX = OFF_LINV + OB * TP * 4;   // [OB][TP] maxima of a partial
     static constexpr uint32_t OFF_RED = OFF_PMX + OB * TP * 4;    // [NWG][4][NC] reduction scratch
     static constexpr uint32_t OFF_RANGE = (OFF_RED + NWG * 4 * NC * 4 + 15) & ~15u;   // WorkRange
-    static constexpr uint32_t SMEM_BYTES = OFF_RANGE + ((sizeof(WorkRange) + 15) & ~15u);
+    static constexpr uint32_t OFF_SEQ = OFF_RANGE + ((sizeof(WorkRange) + 15) & ~15u);   // order of the sequences
+    static constexpr uint32_t SMEM_BYTES = OFF_SEQ + kSplitMaxB;
     // TMEM columns: S0 | S1 | O0 (hi | lo) | O1 (hi | lo)
     static constexpr uint32_t T_S = 0, T_O = 2 * TP;
     static constexpr uint32_t TMEM_COLS = TP == 64 ? 512 : 256;
@@ -117,7 +118,8 @@ struct AttnLayout {
     static_assert(NC == 8 || NC == 16 || NC == 32, "query columns of a softmax thread");
 };
 
-// MODE: whole units round-robin (0), the work split (1), the cluster split (2).
+// MODE: whole units round-robin (0), the work split (1), the cluster split (2),
+// whole units with the longest sequences first (3).
 template <int D, int TP, int NWG, int MODE>
 __global__ void __launch_bounds__((4 * NWG + 3) * 32, 1)
 tree_attention_kernel(const __grid_constant__ CUtensorMap map_q,
@@ -129,7 +131,7 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap map_q,
     using Lay = AttnLayout<D, TP, NWG>;
     using KPos = RingPos<Lay::KS>;
     using VPos = RingPos<Lay::VS>;
-    constexpr bool SPLIT = MODE == 1, RANGE = MODE != 0;
+    constexpr bool SPLIT = MODE == 1, RANGE = MODE == 1 || MODE == 2, RAGGED = MODE == 3;
     constexpr int NC = Lay::NC;
     using Cols = uint32_t[Lay::NC];   // a softmax thread's scores of one tile
     extern __shared__ __align__(1024) uint8_t smem[];
@@ -181,7 +183,7 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap map_q,
     }
     WorkRange *wr_s = reinterpret_cast<WorkRange *>(smem + Lay::OFF_RANGE);
     if (warp == Lay::SW) {
-        const WorkRange w = plan_range(p, lane);   // whole units round-robin without p.split
+        const WorkRange w = plan_range(p, lane, RAGGED ? smem + Lay::OFF_SEQ : nullptr);   // whole units round-robin without p.split
         if (lane == 0) {
             *wr_s = w;
             if (SPLIT) p.split_rec[blockIdx.x].u = -1;   // no cut unit recorded yet
@@ -207,7 +209,7 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap map_q,
             KPos kp;
             VPos vp;
             int g = 0, k = 0;
-            SegIter<RANGE> it(wr);
+            SegIter<RANGE, RAGGED> it(wr);
             for (Seg sg; it.next(p, sg); ++k) {
                 const UnitInfo &ui = sg.ui;
                 const int u = sg.u;
@@ -307,7 +309,7 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap map_q,
         int g = 0, k = 0;
         bool prev_first = false;
         uint32_t prev_to = 0;
-        SegIter<RANGE> it(wr);
+        SegIter<RANGE, RAGGED> it(wr);
         for (Seg sg;; ++k) {
             const int n = warp_uniform(it.next(p, sg) ? sg.j1 - sg.j0 : 0);
             if (n == 0) break;
@@ -533,7 +535,7 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap map_q,
         };
 
         int k = 0;
-        SegIter<RANGE> it(wr);
+        SegIter<RANGE, RAGGED> it(wr);
         for (Seg sg; it.next(p, sg); ++k) {
             const UnitInfo &ui = sg.ui;
             const int u = sg.u;
@@ -677,7 +679,7 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap map_q,
                     pend_f |= 2 | (sg.u == wr.u_first ? 4 : 0);
                     // the part holding the unit's first tile records it for the merge
                     if (sg.j0 == 0 && threadIdx.x == 0)
-                        p.split_rec[blockIdx.x] = SplitRecord{seg_unit_origin(wr, it, sg), wr.n_tail, u, ui.n_tiles};
+                        p.split_rec[blockIdx.x] = SplitRecord{wr.x_first + (wr.n_tiles - it.left) - sg.j1, wr.n_tail, u, ui.n_tiles};
                 }
             }
         }
@@ -766,7 +768,10 @@ static cudaError_t launch_tree_attention_t(const AttnMaps &m, const AttnParams &
                                            bool programmatic, cudaStream_t stream)
 {
     using Lay = AttnLayout<D, TP, NWG>;
-    static std::atomic<uint64_t> configured[3] = {{0}, {0}, {0}};
+    static std::atomic<uint64_t> configured[4] = {{0}, {0}, {0}, {0}};
+    if (whole_ragged(p))
+        return launch_attention_grid(tree_attention_kernel<D, TP, NWG, 3>, Lay::SMEM_BYTES, Lay::THREADS,
+                                     configured[3], m, p, num_sms, programmatic, stream);
     if (p.cluster > 1)
         return launch_attention_grid(tree_attention_kernel<D, TP, NWG, 2>, Lay::SMEM_BYTES, Lay::THREADS,
                                      configured[2], m, p, num_sms, programmatic, stream);

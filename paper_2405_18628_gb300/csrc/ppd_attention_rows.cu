@@ -92,7 +92,8 @@ struct RowsLayout {
     static constexpr uint32_t OFF_ABORT = OFF_TMEMPTR + 4;
     static constexpr uint32_t OFF_X = (OFF_ABORT + 4 + 15) & ~15u;   // [2][M] (maximum, sum) per stream and row
     static constexpr uint32_t OFF_RANGE = OFF_X + 2 * M * 8;         // WorkRange
-    static constexpr uint32_t SMEM_BYTES = OFF_RANGE + ((sizeof(WorkRange) + 15) & ~15u);
+    static constexpr uint32_t OFF_SEQ = OFF_RANGE + ((sizeof(WorkRange) + 15) & ~15u);   // order of the sequences
+    static constexpr uint32_t SMEM_BYTES = OFF_SEQ + kSplitMaxB;
     // TMEM columns: S_A | S_B (128 each; P is written over S) | O_A | O_B (D each)
     static constexpr uint32_t T_S = 0, T_O = 256, TMEM_COLS = 512;
     // floats between the rows of a partial state in shared memory: lanes hold
@@ -117,9 +118,9 @@ struct RowsJob {
 // slice); with n_qb 3 the first p.pair_grid CTAs take the slices' pairs and
 // the others their third blocks.  RANGE (either split): single jobs, the CTA's range
 // of tiles.
-template <bool RANGE>
+template <bool RANGE, bool RAGGED = false>
 struct RowsIter {
-    SegIter<RANGE> seg;
+    SegIter<RANGE, RAGGED> seg;
     int x, step, n, per;
     bool pair;
     PPD_DEV RowsIter(const AttnParams &p, const WorkRange &w) : seg(w)
@@ -149,8 +150,11 @@ struct RowsIter {
             j.pair = false;
             return true;
         }
-        if (x >= n) return false;
-        const int slice = x / per, i = x - slice * per;
+        int job = x;
+        if (RAGGED && seg.seq) job = ragged_job(p, seg.seq, x, step, n, per);
+        if (job < 0 || job >= n) return false;
+        x += step;
+        const int slice = job / per, i = job - slice * per;
         const int qb = pair ? 2 * i : (p.pairs ? p.n_qb - 1 : i);
         j.ui = unit_info(p, slice * p.n_qb + qb);
         // a query's ancestors come before it: no tree tile past the job's last block
@@ -158,7 +162,6 @@ struct RowsIter {
         j.j0 = 0;
         j.j1 = j.ui.n_tiles;
         j.pair = pair;
-        x += step;
         return true;
     }
 };
@@ -185,7 +188,8 @@ PPD_DEV void rows_prefetch(const AttnParams &p, int lane, const CUtensorMap *kc,
     }
 }
 
-// MODE: whole jobs (0), the work split (1), the cluster split (2).
+// MODE: whole jobs round-robin (0), the work split (1), the cluster split (2),
+// whole jobs with the longest sequences first (3).
 template <int D, int MODE>
 __global__ void __launch_bounds__(352, 1)
 tree_attention_rows_kernel(const __grid_constant__ CUtensorMap map_q,
@@ -196,7 +200,7 @@ tree_attention_rows_kernel(const __grid_constant__ CUtensorMap map_q,
 {
     using Lay = RowsLayout<D>;
     using Pos = RingPos<Lay::RS>;
-    constexpr bool SPLIT = MODE == 1, RANGE = MODE != 0;
+    constexpr bool SPLIT = MODE == 1, RANGE = MODE == 1 || MODE == 2, RAGGED = MODE == 3;
     extern __shared__ __align__(1024) uint8_t smem[];
     if (smem_addr(smem) & 1023u) {
         if (threadIdx.x == 0 && p.dev_status)
@@ -245,7 +249,7 @@ tree_attention_rows_kernel(const __grid_constant__ CUtensorMap map_q,
     }
     WorkRange *wr_s = reinterpret_cast<WorkRange *>(smem + Lay::OFF_RANGE);
     if (warp == 8) {
-        const WorkRange w = plan_range(p, lane);   // whole units round-robin without p.split
+        const WorkRange w = plan_range(p, lane, RAGGED ? smem + Lay::OFF_SEQ : nullptr);   // whole units round-robin without p.split
         if (lane == 0) {
             *wr_s = w;
             if (SPLIT) p.split_rec[blockIdx.x].u = -1;   // no cut unit recorded yet
@@ -302,7 +306,7 @@ tree_attention_rows_kernel(const __grid_constant__ CUtensorMap map_q,
             int v_row[2] = {0, 0}, v_lbh[2] = {0, 0};
             bool v_tree[2] = {false, false};
             int g = 0, k = 0;
-            RowsIter<RANGE> it(p, wr);
+            RowsIter<RANGE, RAGGED> it(p, wr);
             for (RowsJob jb; it.next(p, jb); ++k) {
                 const UnitInfo &ui = jb.ui;
                 if (!jb.pair) load_q(k & 1, (uint32_t)(k >> 1) & 1u, ui.qb, ui.lbh);
@@ -446,7 +450,7 @@ tree_attention_rows_kernel(const __grid_constant__ CUtensorMap map_q,
         };
 
         int g = 0, k = 0;
-        RowsIter<RANGE> it(p, wr);
+        RowsIter<RANGE, RAGGED> it(p, wr);
         const bool pair = it.pair;
         for (RowsJob jb;; ++k) {
             const int n = warp_uniform(it.next(p, jb) ? jb.j1 - jb.j0 : 0);
@@ -758,7 +762,7 @@ tree_attention_rows_kernel(const __grid_constant__ CUtensorMap map_q,
             }
         };
 
-        RowsIter<RANGE> it(p, wr);
+        RowsIter<RANGE, RAGGED> it(p, wr);
         int k = 0;
         for (RowsJob jb; it.next(p, jb); ++k) {
             const UnitInfo &ui = jb.ui;
@@ -877,7 +881,10 @@ template <int D>
 static cudaError_t launch_rows_t(const AttnMaps &m, const AttnParams &p, int num_sms,
                                  bool programmatic, cudaStream_t stream)
 {
-    static std::atomic<uint64_t> configured[3] = {{0}, {0}, {0}};
+    static std::atomic<uint64_t> configured[4] = {{0}, {0}, {0}, {0}};
+    if (whole_ragged(p))
+        return launch_attention_grid(tree_attention_rows_kernel<D, 3>, RowsLayout<D>::SMEM_BYTES, 352,
+                                     configured[3], m, p, num_sms, programmatic, stream);
     if (p.cluster > 1)
         return launch_attention_grid(tree_attention_rows_kernel<D, 2>, RowsLayout<D>::SMEM_BYTES, 352,
                                      configured[2], m, p, num_sms, programmatic, stream);

@@ -171,6 +171,13 @@ inline void plan_rows(AttnParams &p, int num_sms)
     p.pair_grid = grid;
 }
 
+// Whether the launch takes whole jobs of several sequences, whose lengths (known
+// to the device alone) may differ.
+inline bool whole_ragged(const AttnParams &p)
+{
+    return p.B > 1 && p.B <= kSplitMaxB && !p.split && p.cluster <= 1;
+}
+
 // CTAs of an attention launch: one per SM, at most one per job (with the
 // work split: at most one per tile, and kSplitMaxGrid).
 inline int attention_grid(const AttnParams &p, int num_sms)
