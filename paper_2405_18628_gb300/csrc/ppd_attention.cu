@@ -369,6 +369,7 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap map_q,
         float *red = reinterpret_cast<float *>(smem + Lay::OFF_RED) + wg * 4 * NC;   // [4][NC]
         float *linv = reinterpret_cast<float *>(smem + Lay::OFF_LINV) + q0;       // [OB][TP]
         float *pmx = reinterpret_cast<float *>(smem + Lay::OFF_PMX) + q0;         // [OB][TP]
+        float2 *ml = reinterpret_cast<float2 *>(smem + Lay::OFF_PMX) + q0;        // cluster split: [TP] over pmx
 
         uint64_t lacc[NC / 2];   // this key row's share of every owned query's row sum, in pairs
 #pragma unroll
@@ -664,6 +665,8 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap map_q,
                     if (!RANGE || (SPLIT && seg_whole(sg))) {
                         if (p.lse && q0 + t < T) p.lse[(size_t)u * T + q0 + t] = (m + lg2(l)) * 0.69314718055994530942f;
                         linv[ob * TP + t] = rcp(l);
+                    } else if (MODE == 2) {
+                        ml[t] = make_float2(m, l);
                     } else {
                         linv[ob * TP + t] = l;
                         pmx[ob * TP + t] = m;
@@ -691,8 +694,7 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap map_q,
                 float *st = reinterpret_cast<float *>(smem + Lay::OFF_K);
                 read_o(0, pend_g, [&](int e, float v) { st[(q0 + e) * D + t] = v; });
             } else if (t < NC) {
-                pmx[t] = -INFINITY;
-                linv[t] = 0.f;
+                ml[t] = make_float2(-INFINITY, 0.f);
             }
         } else if (pend_f) {
             named_bar_sync(1 + wg, 128);   // the row sums are in shared memory
@@ -705,9 +707,8 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap map_q,
         cluster_sync();
         if (warp < Lay::SW) {
             const int u = (int)blockIdx.x / p.cluster;
-            cluster_merge(p, smem_addr(smem) + Lay::OFF_K, D * 4, smem_addr(smem) + Lay::OFF_PMX,
-                          smem_addr(smem) + Lay::OFF_LINV, 4, D, (int)blockIdx.x - u * p.cluster, T, (size_t)u * T,
-                          threadIdx.x, Lay::SW * 32);
+            cluster_merge<1>(p, smem_addr(smem) + Lay::OFF_K, D * 4, smem_addr(smem) + Lay::OFF_PMX,
+                          D, (int)blockIdx.x - u * p.cluster, T, (size_t)u * T, threadIdx.x, Lay::SW * 32);
         }
         __syncwarp();
         cluster_sync();   // no CTA leaves while a peer reads its shared memory

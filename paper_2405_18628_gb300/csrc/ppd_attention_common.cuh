@@ -81,6 +81,29 @@ PPD_DEV int ragged_job(const AttnParams &p, const uint8_t *seq, int i, int step,
 PPD_DEV long long split_start(int c, long long N, int G) { return (long long)c * N / G; }
 PPD_DEV int split_cta_of(long long x, long long N, int G) { return (int)(((x + 1) * G + N - 1) / N) - 1; }
 
+// This CTA's work where any thread can tell by itself: whole units round-robin,
+// or with the cluster split its share of its cluster's unit.  (Every role plans for
+// itself as soon as the inputs are there: no pass through shared memory.)
+template <bool kHint = false>
+PPD_DEV WorkRange plan_alone(const AttnParams &p)
+{
+    WorkRange w{};
+    w.u_first = p.n_units;
+    w.u_last = -1;
+    w.rr_units = p.n_units;
+    if (p.cluster > 1) {
+        const int c = (int)blockIdx.x;
+        w.rr_units = 0;
+        w.u_first = w.u_last = c / p.cluster;
+        const int32_t *P = p.prefix_len + w.u_first / (p.H * p.n_qb) % p.B;
+        const int nt = ((min(max(kHint ? ld_relaxed_gpu_s32(P) : __ldg(P), 0), p.S_max) + 127) >> 7) + p.n_tt;
+        const int r = c - w.u_first * p.cluster;
+        w.j_first = r * nt / p.cluster;
+        w.n_tiles = (r + 1) * nt / p.cluster - w.j_first;
+    }
+    return w;
+}
+
 // This CTA's work, computed by one whole warp (every lane gets the result).
 // The tiles of one layer's block of sequence b number H * n_qb * (n_pref(b) +
 // n_tt); lanes hold sequences b = lane and lane + 32.
@@ -91,13 +114,14 @@ PPD_DEV int split_cta_of(long long x, long long N, int G) { return (int)(((x + 1
 template <bool kHint = false>
 PPD_DEV WorkRange plan_range(const AttnParams &p, int lane, uint8_t *seq = nullptr)
 {
+    if (p.cluster > 1) return plan_alone<kHint>(p);
     WorkRange w{};
     const int G = (int)gridDim.x, c = (int)blockIdx.x;
     // no tail range unless one is found below
     w.u_first = p.n_units;
     w.u_last = -1;
     w.n_tiles = 0;
-    w.rr_units = p.split || p.cluster > 1 ? 0 : p.n_units;   // units taken whole, round-robin
+    w.rr_units = p.split ? 0 : p.n_units;   // units taken whole, round-robin
     w.seq = nullptr;
     const unsigned full = 0xffffffffu;
     const int per_b = p.H * p.n_qb;
@@ -122,14 +146,6 @@ PPD_DEV WorkRange plan_range(const AttnParams &p, int lane, uint8_t *seq = nullp
         if (lane < p.B) seq[r0] = (uint8_t)lane;
         if (lane + 32 < p.B) seq[r1] = (uint8_t)(lane + 32);
         w.seq = seq;
-        return w;
-    }
-    if (p.cluster > 1) {
-        // the cluster's unit, this CTA's share of its tiles
-        w.u_first = w.u_last = c / p.cluster;
-        const int r = c - w.u_first * p.cluster, nt = nt_of(w.u_first / per_b % p.B);
-        w.j_first = r * nt / p.cluster;
-        w.n_tiles = (r + 1) * nt / p.cluster - w.j_first;
         return w;
     }
     const int w0 = lane < p.B ? per_b * nt_of(lane) : 0;
@@ -382,54 +398,62 @@ static __device__ __forceinline__ void split_merge_chunk(const float *split_part
 
 // The end of a cluster split: every CTA of the cluster has left its partial state
 // in its shared memory -- unnormalised O rows at `o` (`pitch` bytes apart), each
-// row's maximum at `m` and sum at `l` (`ml_pitch` bytes apart; maximum -inf: no key seen, the
-// row of O may hold anything) -- and all threads have passed a cluster_sync().
-// CTA `rank` merges its share of the n_rows rows, four columns per thread at a
-// time, every CTA's values loaded before any is used.
-PPD_DEV void cluster_merge(const AttnParams &p, uint32_t o, uint32_t pitch, uint32_t m, uint32_t l, uint32_t ml_pitch,
-                           int D, int rank, int n_rows, size_t out_row0, int tid, int n_threads)
+// row's (maximum, sum) at `ml` (maximum -inf: no key seen, the row of O may hold
+// anything) -- and all threads have passed a cluster_sync().  CTA `rank` merges
+// its share of the n_rows rows, 4 X columns per thread at a time (four of each
+// X-th of the row, so that a warp reads whole lines), every CTA's values loaded
+// before any is used.  X = 2 pays with many rows (the query-row kernel: 16 calls
+// of 64 units, 200 tokens, 343 -> 326 us), X = 1 keeps more threads busy with few.
+template <int X>
+PPD_DEV void cluster_merge(const AttnParams &p, uint32_t o, uint32_t pitch, uint32_t ml, int D, int rank, int n_rows,
+                           size_t out_row0, int tid, int n_threads)
 {
-    const int n = p.cluster, per_row = D / 4;
+    const int n = p.cluster, per_row = D / (4 * X);
     const int r0 = rank * n_rows / n, r1 = (rank + 1) * n_rows / n;
     const bool vec_out = (reinterpret_cast<uintptr_t>(p.out) & 15u) == 0;
     for (int i = tid; i < (r1 - r0) * per_row; i += n_threads) {
-        const int row = r0 + i / per_row, c4 = i % per_row;
-        float mc[kMaxCluster], lc[kMaxCluster];
-        float4 v[kMaxCluster];
+        const int row = r0 + i / per_row, col = 4 * (i % per_row);   // and D / X further
+        float2 s[kMaxCluster];
+        float4 v[kMaxCluster][X];
 #pragma unroll
         for (int c = 0; c < kMaxCluster; ++c) {
-            mc[c] = -INFINITY;
+            s[c] = make_float2(-INFINITY, 0.f);
             if (c < n) {
-                mc[c] = ld_cluster_f32(cluster_map(m + row * ml_pitch, c));
-                lc[c] = ld_cluster_f32(cluster_map(l + row * ml_pitch, c));
-                v[c] = ld_cluster_v4(cluster_map(o + row * pitch + c4 * 16, c));
+                s[c] = ld_cluster_v2(cluster_map(ml + row * 8, c));
+                const uint32_t a = cluster_map(o + row * pitch + col * 4, c);
+#pragma unroll
+                for (int x = 0; x < X; ++x) v[c][x] = ld_cluster_v4(a + x * (4 * D / X));
             }
         }
         float M = -INFINITY, Ls = 0.f;
 #pragma unroll
-        for (int c = 0; c < kMaxCluster; ++c) M = fmaxf(M, mc[c]);
-        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int c = 0; c < kMaxCluster; ++c) M = fmaxf(M, s[c].x);
+        float acc[4 * X] = {};
 #pragma unroll
         for (int c = 0; c < kMaxCluster; ++c) {
-            if (c >= n || mc[c] == -INFINITY) continue;
-            const float w = ex2(mc[c] - M);
-            Ls = fmaf(w, lc[c], Ls);
-            acc.x = fmaf(w, v[c].x, acc.x);
-            acc.y = fmaf(w, v[c].y, acc.y);
-            acc.z = fmaf(w, v[c].z, acc.z);
-            acc.w = fmaf(w, v[c].w, acc.w);
+            if (c >= n || s[c].x == -INFINITY) continue;
+            const float w = ex2(s[c].x - M);
+            Ls = fmaf(w, s[c].y, Ls);
+#pragma unroll
+            for (int x = 0; x < X; ++x) {
+                acc[4 * x] = fmaf(w, v[c][x].x, acc[4 * x]);
+                acc[4 * x + 1] = fmaf(w, v[c][x].y, acc[4 * x + 1]);
+                acc[4 * x + 2] = fmaf(w, v[c][x].z, acc[4 * x + 2]);
+                acc[4 * x + 3] = fmaf(w, v[c][x].w, acc[4 * x + 3]);
+            }
         }
         const float inv = 1.f / Ls;
-        float *dst = p.out + (out_row0 + row) * D + c4 * 4;
+        float *dst = p.out + (out_row0 + row) * D + col;
         if (vec_out) {
-            *reinterpret_cast<float4 *>(dst) = make_float4(acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv);
+#pragma unroll
+            for (int x = 0; x < 4 * X; x += 4)
+                *reinterpret_cast<float4 *>(dst + x / 4 * (D / X)) =
+                    make_float4(acc[x] * inv, acc[x + 1] * inv, acc[x + 2] * inv, acc[x + 3] * inv);
         } else {
-            dst[0] = acc.x * inv;
-            dst[1] = acc.y * inv;
-            dst[2] = acc.z * inv;
-            dst[3] = acc.w * inv;
+#pragma unroll
+            for (int x = 0; x < 4 * X; ++x) dst[x / 4 * (D / X) + x % 4] = acc[x] * inv;
         }
-        if (c4 == 0 && p.lse) p.lse[out_row0 + row] = (M + lg2(Ls)) * 0.69314718055994530942f;
+        if (col == 0 && p.lse) p.lse[out_row0 + row] = (M + lg2(Ls)) * 0.69314718055994530942f;
     }
 }
 

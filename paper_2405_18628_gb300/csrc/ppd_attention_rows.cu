@@ -858,7 +858,7 @@ tree_attention_rows_kernel(const __grid_constant__ CUtensorMap map_q,
         if (warp < 8) {
             const int u = (int)blockIdx.x / p.cluster;
             const int lbh = u / p.n_qb, qb = u - lbh * p.n_qb;
-            cluster_merge(p, smem_addr(smem) + Lay::OFF_R, Lay::C_PITCH * 4, smem_addr(cs), smem_addr(cs) + 4, 8, D,
+            cluster_merge<2>(p, smem_addr(smem) + Lay::OFF_R, Lay::C_PITCH * 4, smem_addr(cs), D,
                           (int)blockIdx.x - u * p.cluster, min(Lay::M, T - qb * Lay::M),
                           (size_t)lbh * T + (size_t)qb * Lay::M, threadIdx.x, 256);
         }

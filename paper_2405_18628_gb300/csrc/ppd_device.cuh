@@ -226,6 +226,13 @@ PPD_DEV unsigned long long ld_cluster_u64(uint32_t a)
     return v;
 }
 
+PPD_DEV float2 ld_cluster_v2(uint32_t a)
+{
+    float2 v;
+    asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a) : "memory");
+    return v;
+}
+
 PPD_DEV float4 ld_cluster_v4(uint32_t a)
 {
     float4 v;
