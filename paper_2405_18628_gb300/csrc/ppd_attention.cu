@@ -94,8 +94,7 @@ struct AttnLayout {
     static constexpr int B_VFULL = B_KEMPTY + KS;
     static constexpr int B_VEMPTY = B_VFULL + VS;
     static constexpr int B_SFULL = B_VEMPTY + VS;
-    static constexpr int B_SFREE = B_SFULL + 2;
-    static constexpr int B_PFULL = B_SFREE + 2;
+    static constexpr int B_PFULL = B_SFULL + 2;   // also: the tile's scores are read
     static constexpr int B_PFREE = B_PFULL + PB;
     static constexpr int B_DRAIN = B_PFREE + PB;
     static constexpr int NBAR = B_DRAIN + 1;
@@ -154,9 +153,7 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap map_q,
     if (threadIdx.x == 0) {
         for (int i = 0; i < Lay::NBAR; ++i) {
             uint32_t count = 1;
-            if ((i >= Lay::B_SFREE && i < Lay::B_SFREE + 2) ||
-                (i >= Lay::B_PFULL && i < Lay::B_PFULL + Lay::PB))
-                count = Lay::SW;
+            if (i >= Lay::B_PFULL && i < Lay::B_PFULL + Lay::PB) count = Lay::SW;
             mbar_init(bars + i, count);
         }
         *abort_flag = 0;
@@ -318,8 +315,9 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap map_q,
             mbar_wait(bars + Lay::B_QFULL + qs, (k >> 1) & 1, abort_flag);
             for (int j = 0; j < n; ++j, ++g) {
                 const int sb = g & 1;
+                // (the score buffer is free: tile g - 2's PV product, issued before, waited
+                // for its probabilities)
                 mbar_wait(bars + Lay::B_KFULL + kp.slot, kp.phase, abort_flag);
-                mbar_wait(bars + Lay::B_SFREE + sb, ((g >> 1) & 1) ^ 1, abort_flag);
                 tc_fence_after();
                 const bool dead = warp_uniform(*abort_flag) != 0;
                 if (elect_one()) {
@@ -632,10 +630,7 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap map_q,
                 fence_proxy_async_smem();
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) {
-                    mbar_arrive(bars + Lay::B_PFULL + ps);
-                    mbar_arrive(bars + Lay::B_SFREE + sb);
-                }
+                if (lane == 0) mbar_arrive(bars + Lay::B_PFULL + ps);
 
                 // the previous segment's output, once this segment's first tile is on its way
                 if (first && pend_f) {
