@@ -56,7 +56,8 @@
 //
 // The work split, the fused step's side warp and the merge of a cut unit's
 // partial states are those of the kernel for trees of up to 64 tokens
-// (ppd_attention.cu), and so are the warp roles (352 threads).
+// (ppd_attention.cu).  Warp roles (384 threads): warps 0-7 softmax, 8 TMA producer,
+// 9 and 10 the streams' MMA issuers (9 owns TMEM), 11 the fused step's side work.
 #include "ppd_attention_common.cuh"
 
 #include <cmath>
@@ -87,7 +88,8 @@ struct RowsLayout {
     static constexpr int B_DONE = B_PFULL + 4;      // [2] the stream's last PV product of a job complete
     static constexpr int B_OFREE = B_DONE + 2;      // [2] a stream's output of a job read back from TMEM (8 arrivals)
     static constexpr int B_DRAIN = B_OFREE + 2;
-    static constexpr int NBAR = B_DRAIN + 1;
+    static constexpr int B_TURN = B_DRAIN + 1;      // [2] the other issuer is done with its turn
+    static constexpr int NBAR = B_TURN + 2;
     static constexpr uint32_t OFF_TMEMPTR = OFF_BAR + NBAR * 8;
     static constexpr uint32_t OFF_ABORT = OFF_TMEMPTR + 4;
     static constexpr uint32_t OFF_X = (OFF_ABORT + 4 + 15) & ~15u;   // [2][M] (maximum, sum) per stream and row
@@ -113,6 +115,13 @@ struct RowsJob {
     bool pair;
 };
 
+// Does this CTA take pair jobs (all its jobs are of one kind)?
+template <bool RANGE>
+PPD_DEV bool rows_pair_cta(const AttnParams &p)
+{
+    return !RANGE && p.pairs && (p.n_qb != 3 || (int)blockIdx.x < p.pair_grid);
+}
+
 // Walks a CTA's jobs in order (every role walks the same sequence).  Whole
 // jobs round-robin: single jobs (n_qb 1), pair jobs (n_qb 2, or 4 with two a
 // slice); with n_qb 3 the first p.pair_grid CTAs take the slices' pairs and
@@ -126,7 +135,7 @@ struct RowsIter {
     PPD_DEV RowsIter(const AttnParams &p, const WorkRange &w) : seg(w)
     {
         const int c = (int)blockIdx.x, G = (int)gridDim.x;
-        pair = !RANGE && p.pairs && (p.n_qb != 3 || c < p.pair_grid);
+        pair = rows_pair_cta<RANGE>(p);
         x = c;
         step = G;
         per = p.n_qb;   // jobs a slice
@@ -191,7 +200,7 @@ PPD_DEV void rows_prefetch(const AttnParams &p, int lane, const CUtensorMap *kc,
 // MODE: whole jobs round-robin (0), the work split (1), the cluster split (2),
 // whole jobs with the longest sequences first (3).
 template <int D, int MODE>
-__global__ void __launch_bounds__(352, 1)
+__global__ void __launch_bounds__(384, 1)
 tree_attention_rows_kernel(const __grid_constant__ CUtensorMap map_q,
                            const __grid_constant__ CUtensorMap map_kc,
                            const __grid_constant__ CUtensorMap map_vc,
@@ -218,10 +227,15 @@ tree_attention_rows_kernel(const __grid_constant__ CUtensorMap map_q,
     const int lane = threadIdx.x & 31;
     const int T = p.T;
 
+    const bool pair_cta = rows_pair_cta<RANGE>(p);
     if (threadIdx.x == 0) {
         for (int i = 0; i < Lay::NBAR; ++i) {
             uint32_t count = 1;
             if (i >= Lay::B_PFULL && i < Lay::B_PFULL + 4) count = 4;
+            // both issuers pass every ring position, and both read a single job's Q block
+            if (i >= Lay::B_EMPTY && i < Lay::B_EMPTY + Lay::RS) count = 2;
+            if (!pair_cta && i >= Lay::B_QEMPTY && i < Lay::B_QEMPTY + Lay::QS) count = 2;
+            if (i == Lay::B_DRAIN) count = 2;
             if (i >= Lay::B_OFREE && i < Lay::B_OFREE + 2) count = 8;
             mbar_init(bars + i, count);
         }
@@ -264,7 +278,7 @@ tree_attention_rows_kernel(const __grid_constant__ CUtensorMap map_q,
     const uint32_t tmem_base = *tmem_ptr;
     const WorkRange &wr = *wr_s;
 
-    if (warp == 10) {
+    if (warp == 11) {
         // ------------------------------------------------------------ fused-step side work
         if (p.fused) fused_side_warp<false>(p, wr, lane, abort_flag);
         else if (p.set_status) status_warp(p, lane);
@@ -351,159 +365,169 @@ tree_attention_rows_kernel(const __grid_constant__ CUtensorMap map_q,
                 if (n_q1 > 0) mbar_wait_drain(bars + Lay::B_QFULL + 1, (n_q1 - 1) & 1);
             }
         }
-    } else if (warp == 9) {
-        // ------------------------------------------------------------ MMA issuer
-        // the whole warp walks the jobs and waits; one elected lane issues
+    } else if (warp == 9 || warp == 10) {
+        // ------------------------------------------------------------ MMA issuers
+        // one warp per stream: the whole warp walks the tiles and waits, one elected lane
+        // issues.  (One warp for both left the tensor pipe idle at every wait: its queue
+        // holds two to three products.)  Both warps pass every position of the ring in
+        // order, also those of the other stream's tiles, and a slot is refilled when both
+        // have: a wait on a barrier's parity is then never more than one phase behind.
+        const uint32_t s = (uint32_t)warp - 9u;
         const uint32_t idesc_qk = make_idesc_bf16(128, 128, 0, 0);
         const uint32_t idesc_pv = make_idesc_bf16(128, D, 0, 1);
-        const uint32_t tmem = warp_uniform(tmem_base);
+        const uint32_t t_s = warp_uniform(tmem_base) + Lay::T_S + s * 128u, t_o = warp_uniform(tmem_base) + Lay::T_O + s * D;
         const uint64_t dq0 = make_smem_desc(warp_uniform(smem_addr(smem + Lay::OFF_Q)), 16, 1024);
         const uint64_t dk0 = make_smem_desc(warp_uniform(smem_addr(smem + Lay::OFF_R)), 16, 1024);
         const uint64_t dv0 = make_smem_desc(warp_uniform(smem_addr(smem + Lay::OFF_R)), Lay::GROUP_BYTES, 1024);
-        using a_t = kind_t<0>;
-        using b_t = kind_t<1>;
 
-        Pos pos;                                  // next ring slot to consume
-        Pos p_v[2];                               // pair jobs: the V tile of a stream's pending tile
-        bool pend[2] = {false, false};            // a tile's PV product is still to be issued
-        bool p_first[2] = {false, false}, p_last[2] = {false, false};   // the tile's place in its job
-        bool p_frees[2] = {false, false};         // its PV product is the last reader of the V tile
-        int p_job[2] = {-1, -1};                  // its job, counting those with tiles of the stream
-        uint32_t p_par[2] = {0, 0};
+        Pos pos;                                  // next ring position
+        bool pend = false;                        // a tile's PV product is still to be issued
+        bool p_first = false, p_last = false;     // the tile's place among the stream's of its job
+        int p_job = -1;                           // its job, counting those with tiles of the stream
+        uint32_t p_par = 0;
         bool dead = false;                        // the CTA gave up: keep the control flow, issue nothing
-        bool v_seen = false;                      // the next PV product's V tile is known to have landed
 
-        // O_s += P_hi V + P_lo V for stream s's pending tile, as its halves of 64 keys
-        // arrive.  Per 32 keys the probability columns hold 8 columns of hi pairs for
-        // keys 0..15, 8 for keys 16..31, then the lo pairs in the same order.  A job's
-        // first PV product overwrites O: it waits until the softmax warps have read back
-        // the output of the stream's job before (one phase of the barrier for each job
-        // with tiles of the stream, so the wait is never more than one phase behind).
-        auto issue_pv = [&](auto s_c, bool pair) {
-            constexpr int s = decltype(s_c)::value;
-            const Pos v = pair ? p_v[s] : pos;
-            if (!pair) pos.advance();
-            if (!v_seen) mbar_wait(bars + Lay::B_FULL + v.slot, v.phase, abort_flag);
-            if (p_first[s] && p_job[s] >= 1)
-                mbar_wait(bars + Lay::B_OFREE + s, (uint32_t)(p_job[s] - 1) & 1u, abort_flag);
+        // The streams take turns, a tile's PV and the next scores at a time: A, B, A, ...
+        // (Free-running they fall into step and their softmaxes coincide.)  A warp waits
+        // for everything else first.
+        uint32_t turn = 0;
+        auto take_turn = [&]() {
+            if (s == 1 || turn > 0) mbar_wait(bars + Lay::B_TURN + s, (turn - 1u + s) & 1u, abort_flag);
+            ++turn;
+        };
+
+        // A position that only the other stream's products read.
+        auto pass = [&]() {
+            mbar_wait(bars + Lay::B_FULL + pos.slot, pos.phase, abort_flag);
+            if (elect_one()) mbar_arrive(bars + Lay::B_EMPTY + pos.slot);
+            __syncwarp();
+            pos.advance();
+        };
+
+        // O += P_hi V + P_lo V for the pending tile, as its halves of 64 keys arrive.  Per
+        // 32 keys the probability columns hold 8 columns of hi pairs for keys 0..15, 8 for
+        // keys 16..31, then the lo pairs in the same order.  A job's first PV product
+        // overwrites O: it waits until the softmax warps have read back the output of the
+        // stream's job before (one phase of the barrier for each job with tiles of the
+        // stream, so the wait is never more than one phase behind).
+        auto issue_pv = [&](bool flush) {
+            mbar_wait(bars + Lay::B_FULL + pos.slot, pos.phase, abort_flag);
+            if (p_first && p_job >= 1) mbar_wait(bars + Lay::B_OFREE + s, (uint32_t)(p_job - 1) & 1u, abort_flag);
 #pragma unroll
             for (int half = 0; half < 2; ++half) {
-                mbar_wait(bars + Lay::B_PFULL + 2 * s + half, p_par[s], abort_flag);
+                mbar_wait(bars + Lay::B_PFULL + 2 * s + half, p_par, abort_flag);
+                if (half == 0 && !flush) take_turn();
                 tc_fence_after();
                 if (elect_one()) {
                     if (!dead) {
-                        const uint32_t t_o = tmem + Lay::T_O + s * D;
-                        const uint32_t a0 = tmem + Lay::T_S + s * 128u;
-                        const uint64_t b0 = desc_advance(dv0, v.slot * Lay::TILE_BYTES);
+                        const uint64_t b0 = desc_advance(dv0, pos.slot * Lay::TILE_BYTES);
 #pragma unroll
                         for (int kk = 4 * half; kk < 4 * half + 4; ++kk) {
                             const uint64_t b = desc_advance(b0, kk * 2048);
-                            const uint32_t a_hi = a0 + 32u * (kk >> 1) + 8u * (kk & 1);
-                            umma_bf16_ta(t_o, a_hi, b, idesc_pv, (p_first[s] && kk == 0) ? 0u : 1u);
+                            const uint32_t a_hi = t_s + 32u * (kk >> 1) + 8u * (kk & 1);
+                            umma_bf16_ta(t_o, a_hi, b, idesc_pv, (p_first && kk == 0) ? 0u : 1u);
                             umma_bf16_ta(t_o, a_hi + 16u, b, idesc_pv, 1u);
                         }
                     }
                     if (half == 1) {
-                        if (p_frees[s]) umma_commit(bars + Lay::B_EMPTY + v.slot);
-                        if (p_last[s]) umma_commit(bars + Lay::B_DONE + s);
+                        umma_commit(bars + Lay::B_EMPTY + pos.slot);
+                        if (p_last) umma_commit(bars + Lay::B_DONE + s);
                     }
                 }
                 __syncwarp();
             }
-            p_par[s] ^= 1u;
-            pend[s] = false;
+            pos.advance();
+            p_par ^= 1u;
+            pend = false;
         };
 
-        // S_s = Q K^T of one tile, after the stream's pending PV product (which reads
-        // the probabilities that the new scores replace: one thread's products execute
-        // in the order they are issued).  k_done: no later product reads the K tile;
-        // q_done: the job's last scores from Q slot qs.
-        auto issue_s = [&](auto s_c, int qs, const Pos &kp, const Pos &next_v, bool first, bool last, bool k_done, bool v_done,
-                           bool q_done) {
-            constexpr int s = decltype(s_c)::value;
-            mbar_wait(bars + Lay::B_FULL + kp.slot, kp.phase, abort_flag);
-            // look for the next PV product's V tile now, while the tensor pipe still has
-            // queued work, and not right before that product
-            v_seen = mbar_test(bars + Lay::B_FULL + next_v.slot, next_v.phase);
+        // S = Q K^T of one tile, after the stream's pending PV product (which reads the
+        // probabilities that the new scores replace: one thread's products execute in the
+        // order they are issued).  first, last: the tile among the stream's of the job.
+        auto issue_s = [&](int qs, bool first, bool last) {
+            mbar_wait(bars + Lay::B_FULL + pos.slot, pos.phase, abort_flag);
             tc_fence_after();
             if (elect_one()) {
                 if (!dead) {
                     const uint64_t a0 = desc_advance(dq0, qs * Lay::Q_BYTES);
-                    const uint64_t b0 = desc_advance(dk0, kp.slot * Lay::TILE_BYTES);
-                    const uint32_t d_s = tmem + Lay::T_S + s * 128u;
+                    const uint64_t b0 = desc_advance(dk0, pos.slot * Lay::TILE_BYTES);
 #pragma unroll
                     for (int kk = 0; kk < D / 16; ++kk) {
                         const uint32_t off = (kk >> 2) * Lay::GROUP_BYTES + (kk & 3) * 32;
-                        umma_bf16(d_s, desc_advance(a0, off), desc_advance(b0, off), idesc_qk, kk > 0 ? 1u : 0u);
+                        umma_bf16(t_s, desc_advance(a0, off), desc_advance(b0, off), idesc_qk, kk > 0 ? 1u : 0u);
                     }
                 }
+                mbar_arrive(bars + Lay::B_TURN + (s ^ 1u));   // the turn is over
                 umma_commit(bars + Lay::B_SFULL + s);
-                if (k_done) umma_commit(bars + Lay::B_EMPTY + kp.slot);
-                if (q_done) umma_commit(bars + Lay::B_QEMPTY + qs);
+                umma_commit(bars + Lay::B_EMPTY + pos.slot);
+                if (last) umma_commit(bars + Lay::B_QEMPTY + qs);
             }
             __syncwarp();
-            pend[s] = true;
-            p_first[s] = first;
-            p_last[s] = last;
-            p_frees[s] = v_done;
-            if (first) ++p_job[s];
+            pos.advance();
+            pend = true;
+            p_first = first;
+            p_last = last;
+            if (first) ++p_job;
         };
 
-        int g = 0, k = 0;
         RowsIter<RANGE, RAGGED> it(p, wr);
         const bool pair = it.pair;
+        int g = 0, k = 0;   // tiles and jobs of the CTA so far
         for (RowsJob jb;; ++k) {
             const int n = warp_uniform(it.next(p, jb) ? jb.j1 - jb.j0 : 0);
             if (n == 0) break;
-            if (!pair) {
-                const int qs = k & 1;
-                for (int j = 0; j < n; ++j, ++g) {
-                    auto tile = [&](auto s_c) {
-                        if (pend[decltype(s_c)::value]) issue_pv(s_c, false);
-                        if (j == 0) {
-                            mbar_wait(bars + Lay::B_QFULL + qs, (uint32_t)(k >> 1) & 1u, abort_flag);
-                            dead = warp_uniform(*abort_flag) != 0;
-                        }
-                        const Pos kp = pos;
-                        pos.advance();
-                        // a stream's last tile of the job is one of the job's last two
-                        issue_s(s_c, qs, kp, pos, j < 2, j + 2 >= n, true, true, j == n - 1);
-                    };
-                    if (g & 1) tile(b_t{});
-                    else tile(a_t{});
-                }
-            } else {
+            if (pair) {
                 // K0 V0 K1 V1 ...; the job's last tile holds no key that a query of its first
                 // block may see (n >= 2), so stream A stops one tile earlier
-                for (int j = 0; j < n; ++j) {
-                    const bool first = j == 0, last = j == n - 1;
-                    const Pos kp = pos;
-                    pos.advance();
-                    const Pos vp = pos;
-                    pos.advance();
-                    if (pend[0]) issue_pv(a_t{}, true);
-                    if (!last) {
-                        if (first) {
-                            mbar_wait(bars + Lay::B_QFULL + 0, (uint32_t)k & 1u, abort_flag);
-                            dead = warp_uniform(*abort_flag) != 0;
-                        }
-                        issue_s(a_t{}, 0, kp, p_v[1], first, j == n - 2, false, false, j == n - 2);
-                        p_v[0] = vp;
+                for (int i = 0; i < n; ++i) {
+                    if (pend) issue_pv(false);
+                    else take_turn();
+                    if (s == 0 && i == n - 1) {
+                        if (elect_one()) mbar_arrive(bars + Lay::B_TURN + 1);
+                        __syncwarp();
+                        pass();
+                        pass();
+                        continue;
                     }
-                    if (pend[1]) issue_pv(b_t{}, true);
-                    if (first) mbar_wait(bars + Lay::B_QFULL + 1, (uint32_t)k & 1u, abort_flag);
-                    issue_s(b_t{}, 1, kp, p_v[0], first, last, true, true, last);
-                    p_v[1] = vp;
+                    if (i == 0) {
+                        mbar_wait(bars + Lay::B_QFULL + s, (uint32_t)k & 1u, abort_flag);
+                        dead = warp_uniform(*abort_flag) != 0;
+                    }
+                    issue_s((int)s, i == 0, i == (s == 0 ? n - 2 : n - 1));
                 }
+            } else {
+                // K0 K1 V0 K2 V1 ...: tile e of all jobs is preceded by the V of tile e - 2
+                const int qs = k & 1, i0 = (g ^ (int)s) & 1;
+                auto q_wait = [&]() {
+                    mbar_wait(bars + Lay::B_QFULL + qs, (uint32_t)(k >> 1) & 1u, abort_flag);
+                    dead = warp_uniform(*abort_flag) != 0;
+                };
+                for (int i = 0; i < n; ++i) {
+                    if (((i ^ i0) & 1) == 0) {
+                        if (pend) issue_pv(false);
+                        else take_turn();
+                        if (i == i0) q_wait();
+                        issue_s(qs, i == i0, i + 2 >= n);
+                    } else {
+                        if (g + i >= 2) pass();
+                        pass();
+                    }
+                }
+                if (i0 >= n) {   // none of the job's tiles is this stream's
+                    q_wait();
+                    if (elect_one()) mbar_arrive(bars + Lay::B_QEMPTY + qs);
+                    __syncwarp();
+                }
+                g += n;
             }
         }
-        v_seen = false;
-        if (pair || !(g & 1)) {
-            if (pend[0]) issue_pv(a_t{}, pair);
-            if (pend[1]) issue_pv(b_t{}, pair);
+        if (pair) {
+            if (pend) issue_pv(true);
         } else {
-            if (pend[1]) issue_pv(b_t{}, false);
-            if (pend[0]) issue_pv(a_t{}, false);
+            for (int e = max(0, g - 2); e < g; ++e) {
+                if ((e & 1) == (int)s) issue_pv(true);
+                else pass();
+            }
         }
         if (elect_one()) umma_commit(bars + Lay::B_DRAIN);
         __syncwarp();
@@ -808,8 +832,8 @@ tree_attention_rows_kernel(const __grid_constant__ CUtensorMap map_q,
                         if (tree) bits[c] = anc[4 * (j - ui.n_pref) + c];
                     }
                     // V rows of invisible keys in a partial prefix tile may be NaN: zero them
-                    // (a pair's tile once, by stream A, whose PV product comes first)
-                    if (!tree && (!jb.pair || s == 0)) {
+                    // (each stream of a pair before its own product)
+                    if (!tree) {
                         const int e = g + i;
                         int pos;   // the V tile's place in the ring order
                         if (jb.pair) pos = 2 * e + 1;
@@ -883,15 +907,15 @@ static cudaError_t launch_rows_t(const AttnMaps &m, const AttnParams &p, int num
 {
     static std::atomic<uint64_t> configured[4] = {{0}, {0}, {0}, {0}};
     if (whole_ragged(p))
-        return launch_attention_grid(tree_attention_rows_kernel<D, 3>, RowsLayout<D>::SMEM_BYTES, 352,
+        return launch_attention_grid(tree_attention_rows_kernel<D, 3>, RowsLayout<D>::SMEM_BYTES, 384,
                                      configured[3], m, p, num_sms, programmatic, stream);
     if (p.cluster > 1)
-        return launch_attention_grid(tree_attention_rows_kernel<D, 2>, RowsLayout<D>::SMEM_BYTES, 352,
+        return launch_attention_grid(tree_attention_rows_kernel<D, 2>, RowsLayout<D>::SMEM_BYTES, 384,
                                      configured[2], m, p, num_sms, programmatic, stream);
     if (p.split)
-        return launch_attention_grid(tree_attention_rows_kernel<D, 1>, RowsLayout<D>::SMEM_BYTES, 352,
+        return launch_attention_grid(tree_attention_rows_kernel<D, 1>, RowsLayout<D>::SMEM_BYTES, 384,
                                      configured[1], m, p, num_sms, programmatic, stream);
-    return launch_attention_grid(tree_attention_rows_kernel<D, 0>, RowsLayout<D>::SMEM_BYTES, 352,
+    return launch_attention_grid(tree_attention_rows_kernel<D, 0>, RowsLayout<D>::SMEM_BYTES, 384,
                                  configured[0], m, p, num_sms, programmatic, stream);
 }
 
