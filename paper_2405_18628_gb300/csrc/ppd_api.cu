@@ -527,31 +527,39 @@ static ppd_status verify_step_impl(const void *q, void *k_cache, void *v_cache,
         }
     }
 
-    // large batches: the same steps as separate grids
+    // large batches: the same steps as separate grids, the combine, the acceptance and
+    // (bf16) the attention grid as a chain of programmatic launches: the attention reads
+    // nothing that this step's other grids write, so it does not wait for them and
+    // starts where the first grid's blocks leave the SMs (80 sequences: 250 -> 242 us)
     AcceptArgs a{cand_tokens, parent, prefix_len, accept_len, path, next_token, new_prefix_len,
                  dev_status, T, V, S_max};
     if (ppd::launch_argmax_partials(logits, rows, V, wl.splits, pv, pi, pst, temp, nullptr, 0, s) !=
         cudaSuccess)
         return cuda_failed();
+    cudaError_t e;
     if (typ) {
         float *nl = reinterpret_cast<float *>(ws + wl.node_lse);
         float *ne = reinterpret_cast<float *>(ws + wl.node_ent);
-        if (ppd::launch_node_stats_combine(pv, pi, pst, rows, wl.splits, argmax_out, nl, ne, s) !=
-                cudaSuccess ||
-            ppd::launch_typical_accept(logits, nl, ne, argmax_out, a, B, typ->temperature,
-                                       typ->epsilon, typ->delta, s) != cudaSuccess)
-            return cuda_failed();
+        e = ppd::launch_node_stats_combine(pv, pi, pst, rows, wl.splits, argmax_out, nl, ne, s);
+        if (e == cudaSuccess)
+            e = ppd::launch_typical_accept(logits, nl, ne, argmax_out, a, B, typ->temperature, typ->epsilon,
+                                           typ->delta, s);
     } else {
-        if (ppd::launch_argmax_combine(pv, pi, rows, wl.splits, argmax_out, s) != cudaSuccess ||
-            ppd::launch_accept_path(argmax_out, a, B, s) != cudaSuccess)
-            return cuda_failed();
+        e = ppd::launch_argmax_combine(pv, pi, rows, wl.splits, argmax_out, s);
+        if (e == cudaSuccess) e = ppd::launch_accept_path(argmax_out, a, B, s);
     }
-    ppd_status st = enqueue_attention_any(q, k_cache, v_cache, k_tree, v_tree, prefix_len, parent,
-                                          L, B, H, T, D, S_max, dt, scale, out, lse, dev_status,
-                                          ws, wl, nullptr, s);
+    if (e != cudaSuccess) return cuda_status(e);
+    ppd_status st;
+    if (dt == PPD_BF16)
+        st = enqueue_attention(q, k_cache, v_cache, k_tree, v_tree, prefix_len, parent, L, B, H, T, D, S_max,
+                               scale, out, lse, dev_status, ws, &wl, nullptr, true, false, false, s);
+    else
+        st = enqueue_attention_any(q, k_cache, v_cache, k_tree, v_tree, prefix_len, parent, L, B, H, T, D,
+                                   S_max, dt, scale, out, lse, dev_status, ws, wl, nullptr, s);
     if (st != PPD_OK) return st;
+    // in plain stream order: it needs the acceptance and the attention done
     return cuda_status(ppd::launch_kv_compact(k_cache, v_cache, k_tree, v_tree, path, accept_len,
-                                              prefix_len, L, B, H, T, D, S_max, eb, s));
+                                              prefix_len, L, B, H, T, D, S_max, eb, s, false));
 }
 
 int ppd_verify_step_form(int L, int B, int H, int T, int D, int V, int S_max, ppd_dtype dt)

@@ -298,11 +298,12 @@ cudaError_t launch_typical_accept(const float *logits, const float *lse, const f
                                   float temperature, float epsilon, float delta,
                                   cudaStream_t stream);
 
+// chained: as a programmatic dependent of the stream's previous grid.
 cudaError_t launch_kv_compact(void *k_cache, void *v_cache, const void *k_tree,
                               const void *v_tree, const int32_t *path,
                               const int32_t *accept_len, const int32_t *prefix_len, int L,
                               int B, int H, int T, int D, int S_max, int elem_bytes,
-                              cudaStream_t stream);
+                              cudaStream_t stream, bool chained = true);
 
 // Next-step candidate tree: at most this many guesses per depth.
 constexpr int kNextMaxK = 16;

@@ -127,6 +127,8 @@ argmax_partial_kernel(const float *__restrict__ logits, int V, int splits, int c
 __global__ void argmax_combine_kernel(const float *part_val, const int32_t *part_idx, int64_t rows,
                                       int splits, int32_t *argmax_out)
 {
+    pdl_release();
+    pdl_wait();
     const int64_t row = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (row < rows) argmax_out[row] = combine_partials(part_val, part_idx, row, splits);
 }
@@ -317,9 +319,8 @@ cudaError_t launch_node_argmax(const float *logits, int64_t rows, int V, float t
 cudaError_t launch_argmax_combine(const float *part_val, const int32_t *part_idx, int64_t rows,
                                   int splits, int32_t *argmax_out, cudaStream_t stream)
 {
-    argmax_combine_kernel<<<(unsigned)((rows + 127) / 128), 128, 0, stream>>>(part_val, part_idx, rows,
-                                                                              splits, argmax_out);
-    return cudaGetLastError();
+    return launch_chained(argmax_combine_kernel, dim3((unsigned)((rows + 127) / 128)), dim3(128), dim3(1), stream,
+                          part_val, part_idx, rows, splits, argmax_out);
 }
 
 // ------------------------------------------------------------------ accept
@@ -377,6 +378,8 @@ __global__ void node_stats_combine_kernel(const float *part_val, const int32_t *
                                           const float *part_stats, int64_t rows, int splits,
                                           int32_t *argmax_out, float *lse_out, float *ent_out)
 {
+    pdl_release();
+    pdl_wait();
     const int64_t row = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (row >= rows) return;
     argmax_out[row] = combine_partials(part_val, part_idx, row, splits);
@@ -389,9 +392,8 @@ cudaError_t launch_node_stats_combine(const float *part_val, const int32_t *part
                                       int32_t *argmax_out, float *lse_out, float *ent_out,
                                       cudaStream_t stream)
 {
-    node_stats_combine_kernel<<<(unsigned)((rows + 127) / 128), 128, 0, stream>>>(
-        part_val, part_idx, part_stats, rows, splits, argmax_out, lse_out, ent_out);
-    return cudaGetLastError();
+    return launch_chained(node_stats_combine_kernel, dim3((unsigned)((rows + 127) / 128)), dim3(128), dim3(1), stream,
+                          part_val, part_idx, part_stats, rows, splits, argmax_out, lse_out, ent_out);
 }
 
 // Typical acceptance, one warp per sequence, from the node statistics.
@@ -459,14 +461,18 @@ cudaError_t launch_kv_compact(void *k_cache, void *v_cache, const void *k_tree,
                               const void *v_tree, const int32_t *path,
                               const int32_t *accept_len, const int32_t *prefix_len, int L,
                               int B, int H, int T, int D, int S_max, int elem_bytes,
-                              cudaStream_t stream)
+                              cudaStream_t stream, bool chained)
 {
     const int64_t n_units = (int64_t)L * B * H;
     const int grid = (int)(n_units < 4096 ? n_units : 4096);
-    return launch_chained(kv_compact_kernel, dim3((unsigned)grid), dim3(128), dim3(1), stream,
-                          static_cast<uint8_t *>(k_cache), static_cast<uint8_t *>(v_cache),
-                          static_cast<const uint8_t *>(k_tree), static_cast<const uint8_t *>(v_tree), path,
-                          accept_len, prefix_len, n_units, B, H, T, S_max, D * elem_bytes);
+    uint8_t *kc = static_cast<uint8_t *>(k_cache), *vc = static_cast<uint8_t *>(v_cache);
+    const uint8_t *kt = static_cast<const uint8_t *>(k_tree), *vt = static_cast<const uint8_t *>(v_tree);
+    if (chained)
+        return launch_chained(kv_compact_kernel, dim3((unsigned)grid), dim3(128), dim3(1), stream, kc, vc, kt, vt,
+                              path, accept_len, prefix_len, n_units, B, H, T, S_max, D * elem_bytes);
+    kv_compact_kernel<<<(unsigned)grid, 128, 0, stream>>>(kc, vc, kt, vt, path, accept_len, prefix_len, n_units, B, H,
+                                                          T, S_max, D * elem_bytes);
+    return cudaGetLastError();
 }
 
 // ------------------------------------------------------------------ status reset
