@@ -26,7 +26,7 @@
 // redux) is a lower bound of the K-th best, the largest of those bounds leaves
 // a few dozen candidates, and a candidate's place is the number of better ones.
 // Insertion into per-thread lists, with the merges of lists in grids of their
-// own, took 48.2 us there (one box; 14.1 now).
+// own, took 48.2 us there (one box; 12.2 now).
 #include "ppd.h"
 #include "ppd_accept.cuh"
 #include "ppd_device.cuh"
@@ -124,13 +124,17 @@ PPD_DEV void find_chains(ChainSmem &c, const int32_t *parent, const int32_t *can
     const int cap = n_states - 1;
     const int32_t *par = parent + (size_t)b * T;
     const int32_t *tok = cand + (size_t)b * T;
+    int pa = -1, tk = 0;
+    if (tid < T) {
+        pa = __ldcg(par + tid);
+        tk = __ldcg(tok + tid);
+    }
     const int n = __ldcg(accept_len + b);
     const int e = (n >= 1 && n <= T) ? __ldcg(path + (size_t)b * T + n - 1) : -1;
     for (int i = tid; i < T; i += kTopkThreads) c.fc[i] = INT_MAX;
     __syncthreads();
     bool head = false;
     if (tid < T) {
-        const int pa = __ldcg(par + tid), tk = __ldcg(tok + tid);
         if (tk == -1 && pa >= 0 && pa < tid) atomicMin(c.fc + pa, tid);
         head = tk == -1 && e >= 0 && e < T && pa == e && tid > e;
     }
@@ -235,7 +239,8 @@ next_lse_kernel(const float *__restrict__ logits, const int32_t *parent, const i
 // into topk[(b * (n_states - 1) + d - 1) * K ...]: one cluster, CTA z taking
 // columns [z * chunk, (z + 1) * chunk).  Position 1 also writes the state k of
 // its sequence to kstate[b].  vec: rows may be read as float4 (chunk is then a
-// multiple of 4).
+// multiple of 4).  kChains: ensemble chains whose loads are in flight together.
+template <int kChains>
 __global__ void __launch_bounds__(kTopkThreads)
 next_topk_kernel(const float *__restrict__ logits, const int32_t *parent, const int32_t *cand,
                  const int32_t *path, const int32_t *accept_len, int T, int V, int n_states, int K,
@@ -284,30 +289,40 @@ next_topk_kernel(const float *__restrict__ logits, const int32_t *parent, const 
             for (int q = 0; q < kBatch; ++q) a[q] = make_float4(0.f, 0.f, 0.f, 0.f);
             // the EPT average is summed in chain order, then divided once (IEEE); the
             // probabilities are summed in chain order, a NaN lse_j making every score NaN
-            for (int j = 0; j < n_ept; ++j) {
-                const float *x = row(j);
-                float4 f[kBatch];
+            // (the loads of kChains chains are in flight together)
+            for (int j0 = 0; j0 < n_ept; j0 += kChains) {
+                float4 fj[kChains][kBatch];
 #pragma unroll
-                for (int q = 0; q < kBatch; ++q) {
-                    f[q] = make_float4(0.f, 0.f, 0.f, 0.f);
-                    if (col(4 * q) < c1) f[q] = __ldcs(reinterpret_cast<const float4 *>(x + col(4 * q)));
-                }
-                const float l = probs ? s_lse[j] : 0.f;
+                for (int y = 0; y < kChains; ++y) {
+                    if (j0 + y >= n_ept) break;
+                    const float *x = row(j0 + y);
 #pragma unroll
-                for (int q = 0; q < kBatch; ++q) {
-                    if (probs) {
-                        f[q].x = exp2f((f[q].x - l) * kLog2e);
-                        f[q].y = exp2f((f[q].y - l) * kLog2e);
-                        f[q].z = exp2f((f[q].z - l) * kLog2e);
-                        f[q].w = exp2f((f[q].w - l) * kLog2e);
+                    for (int q = 0; q < kBatch; ++q) {
+                        fj[y][q] = make_float4(0.f, 0.f, 0.f, 0.f);
+                        if (col(4 * q) < c1) fj[y][q] = __ldcs(reinterpret_cast<const float4 *>(x + col(4 * q)));
                     }
-                    if (j == 0) {
-                        a[q] = f[q];
-                    } else {
-                        a[q].x += f[q].x;
-                        a[q].y += f[q].y;
-                        a[q].z += f[q].z;
-                        a[q].w += f[q].w;
+                }
+#pragma unroll
+                for (int y = 0; y < kChains; ++y) {
+                    if (j0 + y >= n_ept) break;
+                    const float l = probs ? s_lse[j0 + y] : 0.f;
+#pragma unroll
+                    for (int q = 0; q < kBatch; ++q) {
+                        float4 f = fj[y][q];
+                        if (probs) {
+                            f.x = exp2f((f.x - l) * kLog2e);
+                            f.y = exp2f((f.y - l) * kLog2e);
+                            f.z = exp2f((f.z - l) * kLog2e);
+                            f.w = exp2f((f.w - l) * kLog2e);
+                        }
+                        if (j0 + y == 0) {
+                            a[q] = f;
+                        } else {
+                            a[q].x += f.x;
+                            a[q].y += f.y;
+                            a[q].z += f.z;
+                            a[q].w += f.w;
+                        }
                     }
                 }
             }
@@ -515,7 +530,14 @@ cudaError_t launch_next_tree(const float *logits, const int32_t *parent, const i
                                n_ept, vec, lse);
             if (e != cudaSuccess) return e;
         }
-        e = launch_chained(next_topk_kernel, dim3((unsigned)B, cap, (unsigned)n_split), dim3(kTopkThreads),
+        // Four chains' loads in flight take 118 registers, one CTA per SM: where the grid
+        // fits that way (clusters of eight find places on about 3/4 of the SMs), it hides
+        // more latency (4 sequences, V 32000, 4 chains: 14.2 -> 12.2 us; 13.4 with two),
+        // beyond that the second CTA is worth more (16 sequences, V 50257: 115 us with
+        // four, 64.7 with two, 65.2 with one).
+        auto *kern = n_ept == 1 ? next_topk_kernel<1>
+                     : 4 * rows * n_split <= 3LL * num_sms ? next_topk_kernel<4> : next_topk_kernel<2>;
+        e = launch_chained(kern, dim3((unsigned)B, cap, (unsigned)n_split), dim3(kTopkThreads),
                            dim3(1, 1, (unsigned)n_split), stream, logits, parent, cand, path, accept_len, T,
                            V, n_states, K, n_ept, ept_mean, vec, chunk, (const float *)lse, topk, kstate);
         if (e != cudaSuccess) return e;

@@ -316,20 +316,21 @@ def test_next_tree_small_vocab_split_rows(cuda_device, V, K):
 @pytest.mark.parametrize("B,V", [(7, 140000),      # several batches of columns in every CTA of a row
                                  (7, 20001),       # the same with scalar loads, an odd last CTA
                                  (160, 9000)])     # a row per CTA
-@pytest.mark.parametrize("n_ept", [1, 2])
+@pytest.mark.parametrize("n_ept", [1, 2, 3, 5])
 def test_next_tree_selection(cuda_device, B, V, n_ept):
     """The selection on rows that crowd its candidates: sorted either way,
     constant, all but a few entries -inf, NaNs and ties at the end, a few
     values repeated everywhere."""
-    T, K = 7, 16
-    parent = np.tile(np.array([-1, 0, 1, 1, 2, 3, 0], np.int32), (B, 1))
-    cand = np.tile(np.array([3, 4, -1, -1, -1, -1, -1], np.int32), (B, 1))
-    path = np.tile(np.array([0, 1, -1, -1, -1, -1, -1], np.int32), (B, 1))
+    ne, K = max(n_ept, 2), 16
+    T = 3 + 2 * ne                    # root, its accepted child with ne chains of two, a head of the root
+    parent = np.tile(np.array([-1, 0] + [1] * ne + list(range(2, 2 + ne)) + [0], np.int32), (B, 1))
+    cand = np.tile(np.array([3, 4] + [-1] * (T - 2), np.int32), (B, 1))
+    path = np.tile(np.array([0, 1] + [-1] * (T - 2), np.int32), (B, 1))
     rng = np.random.default_rng(V + n_ept)
     logits = rng.standard_normal((B, T, V)).astype(np.float32)
     ramp = np.linspace(-3, 3, V).astype(np.float32)
     for b in range(B):
-        for r in range(2, 6):
+        for r in range(2, T - 1):
             x = logits[b, r]
             kind = b % 7
             if kind == 0:
