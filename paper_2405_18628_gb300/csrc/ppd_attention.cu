@@ -688,8 +688,6 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap map_q,
             if (pend_f) {
                 float *st = reinterpret_cast<float *>(smem + Lay::OFF_K);
                 read_o(0, pend_g, [&](int e, float v) { st[(q0 + e) * D + t] = v; });
-            } else if (t < NC) {
-                ml[t] = make_float2(-INFINITY, 0.f);
             }
         } else if (pend_f) {
             named_bar_sync(1 + wg, 128);   // the row sums are in shared memory
@@ -700,13 +698,14 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap map_q,
     if (MODE == 2) {
         __syncwarp();
         cluster_sync();
+        bool unused = false;
         if (warp < Lay::SW) {
             const int u = (int)blockIdx.x / p.cluster;
-            cluster_merge<1>(p, smem_addr(smem) + Lay::OFF_K, D * 4, smem_addr(smem) + Lay::OFF_PMX,
+            unused = cluster_merge<1>(p, wr.parts, smem_addr(smem) + Lay::OFF_K, D * 4, smem_addr(smem) + Lay::OFF_PMX,
                           D, (int)blockIdx.x - u * p.cluster, T, (size_t)u * T, threadIdx.x, Lay::SW * 32);
         }
         __syncwarp();
-        cluster_sync();   // no CTA leaves while a peer reads its shared memory
+        cluster_leave(unused);
     }
     tc_fence_before();
     __syncthreads();

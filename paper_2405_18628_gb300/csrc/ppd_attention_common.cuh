@@ -60,6 +60,7 @@ struct WorkRange {
     long long x_first;       // index of the range's first tile
     long long n_tail;        // tiles shared out by the split
     const uint8_t *seq;      // not null: whole jobs go longest sequence first, in this order
+    int parts;               // cluster split: the CTAs of the cluster with tiles, the first ones
 };
 
 // Whole jobs (n in all, `per` a slice) go to `step` queues round-robin, queue x
@@ -101,8 +102,11 @@ PPD_DEV WorkRange plan_alone(const AttnParams &p)
         const int32_t *P = p.prefix_len + w.u_first / (p.H * p.n_qb) % p.B;
         const int nt = ((min(max(kHint ? ld_relaxed_gpu_s32(P) : __ldg(P), 0), p.S_max) + 127) >> 7) + p.n_tt;
         const int r = c - w.u_first * p.cluster;
-        w.j_first = r * nt / p.cluster;
-        w.n_tiles = (r + 1) * nt / p.cluster - w.j_first;
+        w.parts = min(p.cluster, nt);
+        if (r < w.parts) {
+            w.j_first = r * nt / w.parts;
+            w.n_tiles = (r + 1) * nt / w.parts - w.j_first;
+        }
     }
     return w;
 }
@@ -399,50 +403,68 @@ static __device__ __forceinline__ void split_merge_chunk(const float *split_part
     if (c0 == 0 && lse) lse[out_row0 + r] = (M + lg2(Ls)) * 0.69314718055994530942f;
 }
 
-// The end of a cluster split: every CTA of the cluster has left its partial state
-// in its shared memory -- unnormalised O rows at `o` (`pitch` bytes apart), each
-// row's (maximum, sum) at `ml` (maximum -inf: no key seen, the row of O may hold
-// anything) -- and all threads have passed a cluster_sync().  CTA `rank` merges
-// its share of the n_rows rows, 4 X columns per thread at a time (four of each
-// X-th of the row, so that a warp reads whole lines), every CTA's values loaded
-// before any is used.  X = 2 pays with many rows (the query-row kernel: 16 calls
-// of 64 units, 200 tokens, 343 -> 326 us), X = 1 keeps more threads busy with few.
+// The end of a cluster split: the first `parts` CTAs of the cluster have left their
+// partial states in shared memory -- unnormalised O rows at `o` (`pitch` bytes apart),
+// each row's (maximum, sum) at `ml` (maximum -inf: no key seen, the row of O may hold
+// anything) -- and all threads have passed a cluster_sync().  CTA `rank` merges its
+// share of the n_rows rows, 4 X columns per thread at a time (four of each X-th of the
+// row, so that a warp reads whole lines), every value of kParts parts loaded before
+// any is used.  The code runs once or twice a launch and mostly waits for its own
+// instructions (a first pass takes 1.1 us, a second 0.35), so it is kept short: all
+// kMaxCluster parts in one go took 32 calls of 32 slices, 64 tokens, 433 us instead of
+// 421.  Returns true when a part had weight 0 in a row of this thread's, so that its O
+// values, unused, may still be on their way.  X = 2 pays with many rows (the query-row
+// kernel: 16 calls of 64 units, 200 tokens, 343 -> 326 us), X = 1 keeps more threads
+// busy with few.
 template <int X>
-PPD_DEV void cluster_merge(const AttnParams &p, uint32_t o, uint32_t pitch, uint32_t ml, int D, int rank, int n_rows,
-                           size_t out_row0, int tid, int n_threads)
+PPD_DEV bool cluster_merge(const AttnParams &p, int parts, uint32_t o, uint32_t pitch, uint32_t ml, int D,
+                           int rank, int n_rows, size_t out_row0, int tid, int n_threads)
 {
+    constexpr int kParts = 4;
     const int n = p.cluster, per_row = D / (4 * X);
     const int r0 = rank * n_rows / n, r1 = (rank + 1) * n_rows / n;
     const bool vec_out = (reinterpret_cast<uintptr_t>(p.out) & 15u) == 0;
+    bool unused = false;
     for (int i = tid; i < (r1 - r0) * per_row; i += n_threads) {
         const int row = r0 + i / per_row, col = 4 * (i % per_row);   // and D / X further
-        float2 s[kMaxCluster];
-        float4 v[kMaxCluster][X];
+        float M = -INFINITY, Ls = 0.f, acc[4 * X] = {};
+#pragma unroll 1
+        for (int c0 = 0; c0 < parts; c0 += kParts) {
+            float2 s[kParts];
+            float4 v[kParts][X];
+            float Mn = M;
 #pragma unroll
-        for (int c = 0; c < kMaxCluster; ++c) {
-            s[c] = make_float2(-INFINITY, 0.f);
-            if (c < n) {
-                s[c] = ld_cluster_v2(cluster_map(ml + row * 8, c));
-                const uint32_t a = cluster_map(o + row * pitch + col * 4, c);
+            for (int c = 0; c < kParts; ++c) {
+                s[c] = make_float2(-INFINITY, 0.f);
+                if (c0 + c < parts) {
+                    s[c] = ld_cluster_v2(cluster_map(ml + row * 8, c0 + c));
+                    const uint32_t a = cluster_map(o + row * pitch + col * 4, c0 + c);
 #pragma unroll
-                for (int x = 0; x < X; ++x) v[c][x] = ld_cluster_v4(a + x * (4 * D / X));
+                    for (int x = 0; x < X; ++x) v[c][x] = ld_cluster_v4(a + x * (4 * D / X));
+                }
             }
-        }
-        float M = -INFINITY, Ls = 0.f;
 #pragma unroll
-        for (int c = 0; c < kMaxCluster; ++c) M = fmaxf(M, s[c].x);
-        float acc[4 * X] = {};
+            for (int c = 0; c < kParts; ++c) {
+                Mn = fmaxf(Mn, s[c].x);
+                unused |= c0 + c < parts && s[c].x == -INFINITY;
+            }
+            const float f = M == -INFINITY ? 0.f : ex2(M - Mn);
+            M = Mn;
+            Ls *= f;
 #pragma unroll
-        for (int c = 0; c < kMaxCluster; ++c) {
-            if (c >= n || s[c].x == -INFINITY) continue;
-            const float w = ex2(s[c].x - M);
-            Ls = fmaf(w, s[c].y, Ls);
+            for (int x = 0; x < 4 * X; ++x) acc[x] *= f;
 #pragma unroll
-            for (int x = 0; x < X; ++x) {
-                acc[4 * x] = fmaf(w, v[c][x].x, acc[4 * x]);
-                acc[4 * x + 1] = fmaf(w, v[c][x].y, acc[4 * x + 1]);
-                acc[4 * x + 2] = fmaf(w, v[c][x].z, acc[4 * x + 2]);
-                acc[4 * x + 3] = fmaf(w, v[c][x].w, acc[4 * x + 3]);
+            for (int c = 0; c < kParts; ++c) {
+                if (c0 + c >= parts || s[c].x == -INFINITY) continue;
+                const float w = ex2(s[c].x - M);
+                Ls = fmaf(w, s[c].y, Ls);
+#pragma unroll
+                for (int x = 0; x < X; ++x) {
+                    acc[4 * x] = fmaf(w, v[c][x].x, acc[4 * x]);
+                    acc[4 * x + 1] = fmaf(w, v[c][x].y, acc[4 * x + 1]);
+                    acc[4 * x + 2] = fmaf(w, v[c][x].z, acc[4 * x + 2]);
+                    acc[4 * x + 3] = fmaf(w, v[c][x].w, acc[4 * x + 3]);
+                }
             }
         }
         const float inv = 1.f / Ls;
@@ -458,6 +480,17 @@ PPD_DEV void cluster_merge(const AttnParams &p, uint32_t o, uint32_t pitch, uint
         }
         if (col == 0 && p.lse) p.lse[out_row0 + row] = (M + lg2(Ls)) * 0.69314718055994530942f;
     }
+    return unused;
+}
+
+// The barrier before the cluster's CTAs leave: no shared memory that a peer reads
+// goes away.  A thread that has used every value it loaded has no load under way and
+// arrives without waiting for its output's stores (with a release, 16 calls of four
+// slices, 64 tokens, took 118 us instead of 111); other warps arrive with release.
+PPD_DEV void cluster_leave(bool unused)
+{
+    if (__any_sync(0xffffffffu, unused)) cluster_sync();
+    else cluster_sync_exit();
 }
 
 // The statuses of an attention call that is not part of a fused step, by one

@@ -873,21 +873,21 @@ tree_attention_rows_kernel(const __grid_constant__ CUtensorMap map_q,
             m = -INFINITY;
             l = 0.f;
         }
-        if (MODE == 2 && wr.n_tiles == 0 && s == 0) cs[q] = make_float2(-INFINITY, 0.f);
     }
 
     if (MODE == 2) {
         __syncwarp();
         cluster_sync();
+        bool unused = false;
         if (warp < 8) {
             const int u = (int)blockIdx.x / p.cluster;
             const int lbh = u / p.n_qb, qb = u - lbh * p.n_qb;
-            cluster_merge<2>(p, smem_addr(smem) + Lay::OFF_R, Lay::C_PITCH * 4, smem_addr(cs), D,
+            unused = cluster_merge<2>(p, wr.parts, smem_addr(smem) + Lay::OFF_R, Lay::C_PITCH * 4, smem_addr(cs), D,
                           (int)blockIdx.x - u * p.cluster, min(Lay::M, T - qb * Lay::M),
                           (size_t)lbh * T + (size_t)qb * Lay::M, threadIdx.x, 256);
         }
         __syncwarp();
-        cluster_sync();   // no CTA leaves while a peer reads its shared memory
+        cluster_leave(unused);
     }
     tc_fence_before();
     __syncthreads();

@@ -204,6 +204,14 @@ PPD_DEV void cluster_sync()
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
+// The barrier before the cluster's threads leave, once every value that this thread
+// loads from a peer's shared memory is used (so the load is done): it orders no memory
+// accesses, so nothing waits for this thread's stores to global memory to be performed.
+PPD_DEV void cluster_sync_exit()
+{
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
+}
+
 // The address of the same shared-memory location in the cluster's CTA `rank`.
 PPD_DEV uint32_t cluster_map(uint32_t saddr, uint32_t rank)
 {

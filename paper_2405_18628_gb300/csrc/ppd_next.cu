@@ -26,7 +26,7 @@
 // redux) is a lower bound of the K-th best, the largest of those bounds leaves
 // a few dozen candidates, and a candidate's place is the number of better ones.
 // Insertion into per-thread lists, with the merges of lists in grids of their
-// own, took 48.2 us there (one box; 12.2 now).
+// own, took 48.2 us there (one box; 12.0 now).
 #include "ppd.h"
 #include "ppd_accept.cuh"
 #include "ppd_device.cuh"
@@ -421,7 +421,7 @@ next_topk_kernel(const float *__restrict__ logits, const int32_t *parent, const 
                 topk[((size_t)b * (n_states - 1) + d - 1) * K + place] = entry_index(mine);
         }
     }
-    cluster_sync();   // no CTA leaves while CTA 0 reads its list
+    cluster_sync_exit();   // no CTA leaves while CTA 0 reads its list
 }
 
 // One block per sequence: state, template checks, and the next tree.  The

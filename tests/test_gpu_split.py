@@ -151,6 +151,7 @@ def test_split_status_per_call(cuda_device):
     (10, 128, 64, [900, 513], 1024),      # 20: clusters of 6, query-row kernel
     (7, 300, 64, [400, 129], 600),        # 14 slices of three query blocks
     (1, 64, 128, [1, 900], 4096),         # clusters of 8 with more CTAs than tiles
+    (2, 200, 128, [0, 300], 4096),        # the same in the query-row kernel, rows without keys in a part
 ])
 def test_split_sizes(cuda_device, H, T, D, prefix, S_max):
     """Clusters of every size, and the work split where no cluster size fits."""
