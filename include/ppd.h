@@ -93,12 +93,12 @@ size_t ppd_workspace_bytes(int L, int B, int H, int T, int D, int V, int S_max, 
  *   PPD_ERR_CAPACITY / PPD_ERR_TIMEOUT; outputs of a failed sequence are
  *   unspecified.  Cache rows at or beyond prefix_len[b] are never used and may
  *   hold anything, NaN included.
- * Workspace: ppd_workspace_bytes(...) bytes.  With it (and B <= 64) the
- * (layer, sequence, head) slices left over after full rounds of one slice per
- * SM -- all of them, when there are fewer slices than SMs -- are shared out
- * over every SM by their key tiles, the slices cut between SMs being merged by
- * a second, small grid; a bf16 call may pass none (NULL or fewer bytes) and
- * then runs one whole slice per SM at a time.
+ * Workspace: ppd_workspace_bytes(...) bytes; a bf16 call may pass none (NULL
+ * or fewer bytes).  Launches with fewer (layer, sequence, head) slices than SMs
+ * give each slice a cluster of SMs, which needs no workspace; where the clusters
+ * that fit would be too small, the slices are shared out by their key tiles
+ * (with a workspace and B <= 64; a second, small grid merges the cut ones) or
+ * run whole.
  */
 ppd_status ppd_tree_attention(const void *q, const void *k_cache, const void *v_cache,
                               const void *k_tree, const void *v_tree,
@@ -158,7 +158,8 @@ ppd_status ppd_kv_compact(void *k_cache, void *v_cache, const void *k_tree, cons
  * workspace also holds, so its contents still do not matter); otherwise an
  * argmax grid runs first and the attention grid may start while it runs.
  * If the cooperative launch cannot have every CTA resident, the step falls
- * back to the two-grid form.  Larger batches run the steps as separate grids.
+ * back to the two-grid form.  Larger batches run the steps as separate grids,
+ * the attention grid beside the acceptance.
  * Arguments as in the four entry points above; `out`/`lse` as in
  * ppd_tree_attention, `argmax_out` as in ppd_node_argmax.  Attention reads
  * only prefix rows [0, prefix_len[b]) and compaction writes only rows
@@ -320,18 +321,16 @@ int ppd_verify_step_launches(int L, int B, int H, int T, int D, int V, int S_max
  *   1  an argmax grid, then the attention grid (which accepts and compacts);
  *   2  one attention grid whose spare warp per CTA also computes the argmax
  *      partial maxima while the K/V stream runs (chosen when the logits are
- *      at most 1/64 of the K/V bytes and form 3 does not fit);
- *   3  one attention grid whose softmax warps compute the argmax partial
- *      maxima before their first tile (chosen when the logits are at most
- *      128 KB per CTA of the attention grid).
- * Forms 2 and 3 fall back to form 1 when the cooperative launch cannot have
+ *      at most 1/64 of the K/V bytes and no argmax grid fits on SMs that the
+ *      attention's last round leaves idle).
+ * Form 2 falls back to form 1 when the cooperative launch cannot have
  * every CTA resident.  Returns -1 for sizes the step rejects.
  */
 int ppd_verify_step_form(int L, int B, int H, int T, int D, int V, int S_max, ppd_dtype dt);
 
 /*
- * Force the form of every later fused step of this process (B <= 64): 1, 2
- * or 3 as above, or -1 to return to the automatic choice.  The forms compute
+ * Force the form of every later fused step of this process (B <= 64): 1 or 2
+ * as above, or -1 to return to the automatic choice.  The forms compute
  * the same results; this exists so that tests can cover each one at any size
  * and benchmarks can compare them (no paper counterpart).  Returns the
  * previous setting, or -2 (and changes nothing) for any other value.  Not

@@ -325,6 +325,7 @@ ppd_status enqueue_attention(const void *q, const void *kc, const void *vc, cons
     p.fused = fused != nullptr;
     if (fused) p.fs = *fused;
     p.pdl_wait = chained ? 1 : 0;
+    p.late_wait = programmatic && !chained && !fused ? 1 : 0;
     return cuda_status(ppd::launch_tree_attention(m, p, D, split_grid(), programmatic || chained,
                                                   stream));
 }
@@ -529,8 +530,8 @@ static ppd_status verify_step_impl(const void *q, void *k_cache, void *v_cache,
 
     // large batches: the same steps as separate grids, the combine, the acceptance and
     // (bf16) the attention grid as a chain of programmatic launches: the attention reads
-    // nothing that this step's other grids write, so it does not wait for them and
-    // starts where the first grid's blocks leave the SMs (80 sequences: 250 -> 242 us)
+    // nothing that this step's other grids write, so it starts where the first grid's
+    // blocks leave the SMs (80 sequences: 250 -> 242 us); one of its warps waits for them
     AcceptArgs a{cand_tokens, parent, prefix_len, accept_len, path, next_token, new_prefix_len,
                  dev_status, T, V, S_max};
     if (ppd::launch_argmax_partials(logits, rows, V, wl.splits, pv, pi, pst, temp, nullptr, 0, s) !=
@@ -557,7 +558,7 @@ static ppd_status verify_step_impl(const void *q, void *k_cache, void *v_cache,
         st = enqueue_attention_any(q, k_cache, v_cache, k_tree, v_tree, prefix_len, parent, L, B, H, T, D,
                                    S_max, dt, scale, out, lse, dev_status, ws, wl, nullptr, s);
     if (st != PPD_OK) return st;
-    // in plain stream order: it needs the acceptance and the attention done
+    // in plain stream order: it needs the attention done, which waited for the acceptance
     return cuda_status(ppd::launch_kv_compact(k_cache, v_cache, k_tree, v_tree, path, accept_len,
                                               prefix_len, L, B, H, T, D, S_max, eb, s, false));
 }

@@ -46,9 +46,10 @@
 // and their V rows are zeroed in shared memory before the PV product.  O is
 // double-buffered in TMEM and a unit's output is read back only after the
 // next unit's first tile, so the stream of tiles never waits for a unit's
-// last PV product.  With the work split (ppd_attention_common.cuh) a CTA's
-// tiles are an equal share of the launch's; a unit cut by a share boundary is
-// done in parts whose partial states the last part merges.
+// last PV product.  Launches with fewer units than SMs share units among CTAs
+// (ppd_attention_common.cuh): by clusters, whose CTAs merge their partial states
+// through distributed shared memory, or by the work split, merged by a grid of
+// its own (split_merge_kernel).
 #include "ppd_attention_common.cuh"
 
 #include <cmath>
@@ -199,6 +200,7 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap map_q,
         // ------------------------------------------------------------ fused-step side work
         if (p.fused) fused_side_warp<true>(p, wr, lane, abort_flag);
         else if (p.set_status) status_warp(p, lane);
+        if (p.late_wait) pdl_wait();
     } else if (warp == Lay::SW) {
         // ------------------------------------------------------------ TMA producer
         if (lane == 0) {

@@ -1,7 +1,7 @@
 // ppd_attention_common.cuh -- pieces shared by the two tree-attention kernels
 // (ppd_attention.cu for trees of up to 64 tokens, ppd_attention_rows.cu for
-// 65..512): the work split and unit walk, drain waits, mask kinds and the
-// fused step's side warp.
+// 65..512): the unit walk and the two ways to share a unit among CTAs (work split
+// and clusters) with their merges, drain waits and the fused step's side warp.
 #pragma once
 
 #include "ppd_accept.cuh"
@@ -40,9 +40,10 @@ PPD_DEV UnitInfo unit_info(const AttnParams &p, int u)
 
 // ------------------------------------------------------------------ work split
 //
-// Without p.split, units are taken round-robin (CTA c: units c, c+G, c+2G,
-// ...), whole.  With p.split (launches with fewer units than CTAs, where whole
-// units would leave SMs idle) all units are shared out by their key tiles: the
+// Units are taken round-robin (CTA c: units c, c+G, c+2G, ...), whole, unless there
+// are fewer units than CTAs.  With p.cluster > 1 every unit then has a cluster of
+// CTAs (plan_cluster, cluster_merge).  With p.split (the clusters that fit would be
+// too small) all units are shared out by their key tiles: the
 // tiles (unit u's tiles 0..n_tiles(u)-1, units in order) go to the CTAs in
 // equal contiguous ranges (CTA c: tiles [c*N/G, (c+1)*N/G)).  A unit cut by a
 // range boundary is done in parts, one per CTA; each part leaves its partial
@@ -85,28 +86,20 @@ PPD_DEV int ragged_job(const AttnParams &p, const uint8_t *seq, int i, int step,
 PPD_DEV long long split_start(int c, long long N, int G) { return (long long)c * N / G; }
 PPD_DEV int split_cta_of(long long x, long long N, int G) { return (int)(((x + 1) * G + N - 1) / N) - 1; }
 
-// This CTA's work where any thread can tell by itself: whole units round-robin,
-// or with the cluster split its share of its cluster's unit.  (Every role plans for
-// itself as soon as the inputs are there: no pass through shared memory.)
+// This CTA's share of its cluster's unit (the cluster split): no lane needs another's.
 template <bool kHint = false>
-PPD_DEV WorkRange plan_alone(const AttnParams &p)
+PPD_DEV WorkRange plan_cluster(const AttnParams &p)
 {
     WorkRange w{};
-    w.u_first = p.n_units;
-    w.u_last = -1;
-    w.rr_units = p.n_units;
-    if (p.cluster > 1) {
-        const int c = (int)blockIdx.x;
-        w.rr_units = 0;
-        w.u_first = w.u_last = c / p.cluster;
-        const int32_t *P = p.prefix_len + w.u_first / (p.H * p.n_qb) % p.B;
-        const int nt = ((min(max(kHint ? ld_relaxed_gpu_s32(P) : __ldg(P), 0), p.S_max) + 127) >> 7) + p.n_tt;
-        const int r = c - w.u_first * p.cluster;
-        w.parts = min(p.cluster, nt);
-        if (r < w.parts) {
-            w.j_first = r * nt / w.parts;
-            w.n_tiles = (r + 1) * nt / w.parts - w.j_first;
-        }
+    const int c = (int)blockIdx.x;
+    w.u_first = w.u_last = c / p.cluster;
+    const int32_t *P = p.prefix_len + w.u_first / (p.H * p.n_qb) % p.B;
+    const int nt = ((min(max(kHint ? ld_relaxed_gpu_s32(P) : __ldg(P), 0), p.S_max) + 127) >> 7) + p.n_tt;
+    const int r = c - w.u_first * p.cluster;
+    w.parts = min(p.cluster, nt);
+    if (r < w.parts) {
+        w.j_first = r * nt / w.parts;
+        w.n_tiles = (r + 1) * nt / w.parts - w.j_first;
     }
     return w;
 }
@@ -121,7 +114,7 @@ PPD_DEV WorkRange plan_alone(const AttnParams &p)
 template <bool kHint = false>
 PPD_DEV WorkRange plan_range(const AttnParams &p, int lane, uint8_t *seq = nullptr)
 {
-    if (p.cluster > 1) return plan_alone<kHint>(p);
+    if (p.cluster > 1) return plan_cluster<kHint>(p);
     WorkRange w{};
     const int G = (int)gridDim.x, c = (int)blockIdx.x;
     // no tail range unless one is found below

@@ -21,10 +21,11 @@
 // tile (D = 128), or HBM for trees of up to 128 tokens.  One stream with three
 // score buffers, issued from one lane's branch, kept the pipe 43 % busy: the
 // softmax and its hand-offs took longer than the pipe's work for a tile, and
-// the issue of a tcgen05.mma ~100 cycles.  Steps of 32 x 32 slices, D = 128:
-// 285 tokens over 1500 keys 541 -> 458 us; 96 tokens over 4096 keys (40 x 40
-// slices) 628 -> 575 us, 0.92 of the measured copy rate; eight ragged sequences
-// of up to 16384 keys with 128 tokens (4 x 32 slices each) 1046 -> 935 us.
+// the issue of a tcgen05.mma ~100 cycles.  Steps at D = 128, from that form to this
+// one: 32 x 32 slices, 285 tokens over 1500 keys 541 -> 411 us (its pipe time is 245);
+// 96 tokens over 4096 keys (40 x 40 slices) 628 -> 561 us, 0.94 of the measured copy
+// rate; eight ragged sequences of up to 16384 keys with 128 tokens (4 x 32 slices
+// each) 1046 -> 885 us, the longest queue's share of the bytes taking 870.
 // Measured on the way: probabilities handed over in one piece per tile, 5 %
 // slower on 285 tokens; the softmax unrolled over a tile with its scores in
 // registers, 606 us there (instruction fetch).  What the streams work on:
@@ -54,7 +55,7 @@
 // for single jobs (an SM's copies land roughly in issue order, so a tile
 // queued ahead of its turn would hold back the one needed first).
 //
-// The work split, the fused step's side warp and the merge of a cut unit's
+// The sharing of units among CTAs, the fused step's side warp and the merges of
 // partial states are those of the kernel for trees of up to 64 tokens
 // (ppd_attention.cu).  Warp roles (384 threads): warps 0-7 softmax, 8 TMA producer,
 // 9 and 10 the streams' MMA issuers (9 owns TMEM), 11 the fused step's side work.
@@ -282,6 +283,7 @@ tree_attention_rows_kernel(const __grid_constant__ CUtensorMap map_q,
         // ------------------------------------------------------------ fused-step side work
         if (p.fused) fused_side_warp<false>(p, wr, lane, abort_flag);
         else if (p.set_status) status_warp(p, lane);
+        if (p.late_wait) pdl_wait();
     } else if (warp == 8) {
         // ------------------------------------------------------------ TMA producer
         if (lane == 0) {

@@ -80,20 +80,6 @@ PPD_DEV bool mbar_try_wait(uint32_t bar, uint32_t parity)
     return done != 0;
 }
 
-// Has the phase with the given parity completed?  Never waits.
-PPD_DEV bool mbar_test(uint64_t *bar, uint32_t parity)
-{
-    uint32_t done;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}\n"
-        : "=r"(done)
-        : "r"(smem_addr(bar)), "r"(parity)
-        : "memory");
-    return done != 0;
-}
-
 // Wait for the phase with the given parity to complete.  Gives up (and raises
 // *abort) after kWaitLimitNs, or as soon as *abort is raised by another thread;
 // returns false in both cases.  The caller keeps its control flow unchanged
@@ -269,13 +255,6 @@ PPD_DEV uint64_t l2_policy_evict_normal()
 {
     uint64_t p;
     asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(p));
-    return p;
-}
-
-PPD_DEV uint64_t l2_policy_evict_last()
-{
-    uint64_t p;
-    asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(p));
     return p;
 }
 
@@ -650,9 +629,6 @@ PPD_DEV float warp_transpose_reduce16(float (&v)[16], int lane, Op op)
     return v[0];
 }
 
-struct OpMax {
-    PPD_DEV float operator()(float a, float b) const { return fmaxf(a, b); }
-};
 struct OpAdd {
     PPD_DEV float operator()(float a, float b) const { return a + b; }
 };

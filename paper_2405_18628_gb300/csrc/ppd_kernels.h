@@ -85,8 +85,8 @@ struct AttnParams {
     int pairs;                  // query-row kernel: two blocks of queries of a slice are one job
     int pair_grid;              // with n_qb 3: the CTAs that take the slices' pairs
     float scale_log2;           // softmax scale * log2(e)
-    // Work split: split != 0 shares the units left after the full round-robin
-    // rounds out by their key tiles (B <= kSplitMaxB); units cut by a range
+    // Work split: split != 0 shares all units out by their key tiles (launches with
+    // fewer units than CTAs, B <= kSplitMaxB); units cut by a range
     // boundary leave partial softmax states in split_part, merged afterwards by
     // launch_split_merge from the per-CTA records in split_rec.
     int split;
@@ -103,6 +103,10 @@ struct AttnParams {
     // ppd_tree_attention calls): the setup that reads no input overlaps that
     // grid, then every thread waits for it before reading any input.
     int pdl_wait;
+    // Launched as a programmatic dependent of grids whose results it does not read
+    // (a step of more than 64 sequences): a spare warp waits for them, so that this
+    // grid's completion says that they are complete too.
+    int late_wait;
 };
 
 // Work split limits: batch size (the per-CTA range search holds the batch in
@@ -204,7 +208,7 @@ cudaError_t launch_split_merge(const AttnParams &p, int D, int grid, cudaStream_
 constexpr int kFusedMaxB = 64;
 
 // Dispatches on the padded tree size: up to 64 tokens the key-row kernel
-// (ppd_attention.cu), 65..128 the query-row kernel (ppd_attention_rows.cu).
+// (ppd_attention.cu), 65..512 the query-row kernel (ppd_attention_rows.cu).
 cudaError_t launch_tree_attention(const AttnMaps &m, const AttnParams &p, int D, int num_sms,
                                   bool programmatic, cudaStream_t stream);
 cudaError_t launch_tree_attention_rows(const AttnMaps &m, const AttnParams &p, int D, int num_sms,

@@ -136,7 +136,7 @@ def ppd_verify_step_form(L, B, H, T, D, V, S_max, dtype=PPD_BF16) -> int:
 
 
 def ppd_set_verify_step_form(form: int) -> int:
-    """Force the fused step's form (1, 2 or 3; -1 = automatic); returns the
+    """Force the fused step's form (1 or 2; -1 = automatic); returns the
     previous setting."""
     return int(load().ppd_set_verify_step_form(int(form)))
 
