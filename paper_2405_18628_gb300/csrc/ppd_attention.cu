@@ -17,14 +17,12 @@
 //
 // This kernel serves trees of up to 64 tokens (padded to TP = 32 or 64 columns);
 // larger trees fill the tensor core's M side with queries and run the
-// query-row kernel (ppd_attention_rows.cu).  Warp roles (NWG softmax
-// warpgroups, each owning 1 / NWG of the query columns, then three warps): the
-// TMA producer, the MMA issuer and TMEM owner, and the fused step's argmax /
-// acceptance / compaction.  Two warpgroups, except D = 64 with TP = 64, where
-// four hide more of the latency (8 sequences of 3000 keys: 103.7 against 108.8
-// us) -- with TP = 32 they have too few columns each (80 short sequences: 219.6
-// against 213.1 us), and at D = 128 they gain nothing (HBM) or lose (24 x 16
-// slices of 512 keys: 34.3 against 31.3 us).
+// query-row kernel (ppd_attention_rows.cu).  Warp roles: two softmax warpgroups,
+// each owning half of the query columns, then the TMA producer, the MMA issuer and
+// TMEM owner, and the fused step's argmax / acceptance / compaction.  Four
+// warpgroups of a quarter each gain 3 % on long slices of D = 64 with TP = 64 (8 x 16
+// slices of 8000 keys: 302 against 292 us) but leave 96 registers a thread, too few
+// for the side warp: 30 x 16 slices of 1000 keys, 40 tokens, 439 against 510 us.
 //
 // Bound: HBM for long slices (32 x 32 slices of 2048 keys: 177.6 us for 1.17 GB,
 // 0.97 of the measured copy rate); for short ones the chain of a tile -- scores,
@@ -57,13 +55,13 @@
 
 namespace ppd {
 
-template <int D_, int TP_, int NWG_>
+template <int D_, int TP_>
 struct AttnLayout {
     static constexpr int D = D_;
     static constexpr int TP = TP_;                // query columns (the tree padded to 32 or 64)
     static constexpr int KT = 128;                // keys per tile
     static constexpr int DCH = D / 64;            // 64-column (128-byte) groups along D
-    static constexpr int NWG = NWG_;              // softmax warpgroups
+    static constexpr int NWG = 2;                 // softmax warpgroups
     static constexpr int NC = TP / NWG;           // query columns of each
     static constexpr int SW = 4 * NWG;            // softmax warps; then producer, issuer, side warp
     static constexpr int THREADS = (SW + 3) * 32;
@@ -115,20 +113,20 @@ struct AttnLayout {
     static_assert(SMEM_BYTES <= 232448, "shared memory budget");
     static_assert((OFF_P | OFF_K | OFF_V) % 1024 == 0, "1024-byte aligned operand tiles");
     static_assert((2 + 2 * OB) * TP <= TMEM_COLS, "TMEM budget");
-    static_assert(NC == 8 || NC == 16 || NC == 32, "query columns of a softmax thread");
+    static_assert(NC == 16 || NC == 32, "query columns of a softmax thread");
 };
 
 // MODE: whole units round-robin (0), the work split (1), the cluster split (2),
 // whole units with the longest sequences first (3).
-template <int D, int TP, int NWG, int MODE>
-__global__ void __launch_bounds__((4 * NWG + 3) * 32, 1)
+template <int D, int TP, int MODE>
+__global__ void __launch_bounds__(AttnLayout<D, TP>::THREADS, 1)
 tree_attention_kernel(const __grid_constant__ CUtensorMap map_q,
                       const __grid_constant__ CUtensorMap map_kc,
                       const __grid_constant__ CUtensorMap map_vc,
                       const __grid_constant__ CUtensorMap map_kt,
                       const __grid_constant__ CUtensorMap map_vt, const AttnParams p)
 {
-    using Lay = AttnLayout<D, TP, NWG>;
+    using Lay = AttnLayout<D, TP>;
     using KPos = RingPos<Lay::KS>;
     using VPos = RingPos<Lay::VS>;
     constexpr bool SPLIT = MODE == 1, RANGE = MODE == 1 || MODE == 2, RAGGED = MODE == 3;
@@ -438,8 +436,7 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap map_q,
 
         auto load_cols = [&](uint32_t taddr, Cols &r) {   // then tmem_wait_ld
             if constexpr (NC == 32) tmem_ld32(taddr, r);
-            else if constexpr (NC == 16) tmem_ld16(taddr, r);
-            else tmem_ld8(taddr, r);
+            else tmem_ld16(taddr, r);
         };
 
         // A score jumped past its column's maximum by more than 2^16: the optimistic
@@ -648,12 +645,9 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap map_q,
                 for (int c = 0; c < NC; c += 16) {
                     float v[16];
 #pragma unroll
-                    for (int e = 0; e < 16; e += 2) {
-                        if (c + e < NC) unpack2(lacc[(c + e < NC ? c + e : 0) >> 1], v[e], v[e + 1]);
-                        else v[e] = v[e + 1] = 0.f;
-                    }
+                    for (int e = 0; e < 16; e += 2) unpack2(lacc[(c + e) >> 1], v[e], v[e + 1]);
                     const float s = warp_transpose_reduce16(v, lane, OpAdd());
-                    if (!(lane & 1) && c + (lane >> 1) < NC) red[wq * NC + c + (lane >> 1)] = s;
+                    if (!(lane & 1)) red[wq * NC + c + (lane >> 1)] = s;
                 }
                 named_bar_sync(1 + wg, 128);
                 if (t < NC) {
@@ -760,22 +754,22 @@ cudaError_t launch_split_merge(const AttnParams &p, int D, int grid, cudaStream_
     return cudaLaunchKernelEx(&cfg, split_merge_kernel, p, D);
 }
 
-template <int D, int TP, int NWG>
+template <int D, int TP>
 static cudaError_t launch_tree_attention_t(const AttnMaps &m, const AttnParams &p, int num_sms,
                                            bool programmatic, cudaStream_t stream)
 {
-    using Lay = AttnLayout<D, TP, NWG>;
+    using Lay = AttnLayout<D, TP>;
     static std::atomic<uint64_t> configured[4] = {{0}, {0}, {0}, {0}};
     if (whole_ragged(p))
-        return launch_attention_grid(tree_attention_kernel<D, TP, NWG, 3>, Lay::SMEM_BYTES, Lay::THREADS,
+        return launch_attention_grid(tree_attention_kernel<D, TP, 3>, Lay::SMEM_BYTES, Lay::THREADS,
                                      configured[3], m, p, num_sms, programmatic, stream);
     if (p.cluster > 1)
-        return launch_attention_grid(tree_attention_kernel<D, TP, NWG, 2>, Lay::SMEM_BYTES, Lay::THREADS,
+        return launch_attention_grid(tree_attention_kernel<D, TP, 2>, Lay::SMEM_BYTES, Lay::THREADS,
                                      configured[2], m, p, num_sms, programmatic, stream);
     if (p.split)
-        return launch_attention_grid(tree_attention_kernel<D, TP, NWG, 1>, Lay::SMEM_BYTES, Lay::THREADS,
+        return launch_attention_grid(tree_attention_kernel<D, TP, 1>, Lay::SMEM_BYTES, Lay::THREADS,
                                      configured[1], m, p, num_sms, programmatic, stream);
-    return launch_attention_grid(tree_attention_kernel<D, TP, NWG, 0>, Lay::SMEM_BYTES, Lay::THREADS,
+    return launch_attention_grid(tree_attention_kernel<D, TP, 0>, Lay::SMEM_BYTES, Lay::THREADS,
                                  configured[0], m, p, num_sms, programmatic, stream);
 }
 
@@ -792,8 +786,8 @@ int max_attention_clusters(int size)
     if (dev < 0 || dev >= 64 || size < 1 || size > kMaxCluster) return 0;
     int got = cache[dev][size].load(std::memory_order_relaxed);
     if (got > 0) return got - 1;
-    using Lay = AttnLayout<128, 64, 2>;
-    auto kern = tree_attention_kernel<128, 64, 2, 2>;
+    using Lay = AttnLayout<128, 64>;
+    auto kern = tree_attention_kernel<128, 64, 2>;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)size);
     cfg.blockDim = dim3(Lay::THREADS);
@@ -820,10 +814,10 @@ cudaError_t launch_tree_attention(const AttnMaps &m, const AttnParams &p, int D,
 {
     cudaError_t e;
     if (p.T_pad > 64) e = launch_tree_attention_rows(m, p, D, num_sms, programmatic, stream);
-    else if (D == 128 && p.T_pad == 64) e = launch_tree_attention_t<128, 64, 2>(m, p, num_sms, programmatic, stream);
-    else if (D == 128) e = launch_tree_attention_t<128, 32, 2>(m, p, num_sms, programmatic, stream);
-    else if (p.T_pad == 64) e = launch_tree_attention_t<64, 64, 4>(m, p, num_sms, programmatic, stream);
-    else e = launch_tree_attention_t<64, 32, 2>(m, p, num_sms, programmatic, stream);
+    else if (D == 128 && p.T_pad == 64) e = launch_tree_attention_t<128, 64>(m, p, num_sms, programmatic, stream);
+    else if (D == 128) e = launch_tree_attention_t<128, 32>(m, p, num_sms, programmatic, stream);
+    else if (p.T_pad == 64) e = launch_tree_attention_t<64, 64>(m, p, num_sms, programmatic, stream);
+    else e = launch_tree_attention_t<64, 32>(m, p, num_sms, programmatic, stream);
     if (e != cudaSuccess || !p.split) return e;
     return launch_split_merge(p, D, attention_grid(p, num_sms), stream);
 }
