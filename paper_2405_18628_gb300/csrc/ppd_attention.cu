@@ -28,7 +28,7 @@
 // 0.97 of the measured copy rate); for short ones the chain of a tile -- scores,
 // softmax, hand-over -- and the unit's two ends.  What shortened it, measured
 // together on that case, on 24 x 16 slices of 512 keys and on 4 x 80 x 16 slices
-// of 350-700 keys (D = 64, T = 32): 184.7 -> 177.6, 36.3 -> 31.3, 307 -> 213 us:
+// of 350-700 keys (D = 64, T = 32): 184.7 -> 177.6, 36.3 -> 32, 307 -> 195 us:
 // products issued from warp-uniform code (ppd_device.cuh, elect_one); two fp32
 // operations per instruction; all of a thread's scores in one TMEM load; a
 // unit's first tile without the exact maximum; ancestor sets by shuffles,

@@ -22,7 +22,7 @@
 // score buffers, issued from one lane's branch, kept the pipe 43 % busy: the
 // softmax and its hand-offs took longer than the pipe's work for a tile, and
 // the issue of a tcgen05.mma ~100 cycles.  Steps at D = 128, from that form to this
-// one: 32 x 32 slices, 285 tokens over 1500 keys 541 -> 411 us (its pipe time is 245);
+// one: 32 x 32 slices, 285 tokens over 1500 keys 541 -> 430 us (its pipe time is 245);
 // 96 tokens over 4096 keys (40 x 40 slices) 628 -> 561 us, 0.94 of the measured copy
 // rate; eight ragged sequences of up to 16384 keys with 128 tokens (4 x 32 slices
 // each) 1046 -> 885 us, the longest queue's share of the bytes taking 870.
