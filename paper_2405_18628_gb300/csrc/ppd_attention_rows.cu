@@ -878,7 +878,6 @@ tree_attention_rows_kernel(const __grid_constant__ CUtensorMap map_q,
     }
 
     if (MODE == 2) {
-        __syncwarp();
         cluster_sync();
         bool unused = false;
         if (warp < 8) {

@@ -184,9 +184,11 @@ PPD_DEV void st_global_v8(float *dst, const uint32_t *v, float scale)
 
 // Barrier over every thread of the cluster: what a thread wrote (to its own
 // shared memory, for peers to read) before its arrival is seen by every thread
-// after its wait.
+// after its wait.  The instructions are .aligned (all lanes of a warp at once), and
+// callers come from code whose lanes part ways: the warp converges here first.
 PPD_DEV void cluster_sync()
 {
+    __syncwarp();
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
@@ -195,6 +197,7 @@ PPD_DEV void cluster_sync()
 // accesses, so nothing waits for this thread's stores to global memory to be performed.
 PPD_DEV void cluster_sync_exit()
 {
+    __syncwarp();
     asm volatile("barrier.cluster.arrive.relaxed.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
 }
 
