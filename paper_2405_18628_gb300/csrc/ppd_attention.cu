@@ -484,7 +484,7 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap map_q,
                 for (int part = 0; part < 2; ++part) {
                     uint32_t o[8];
                     tmem_ld8(t_o + part * TP + h, o);
-                    tmem_wait_ld();
+                    tmem_wait_ld(o);
 #pragma unroll
                     for (int e = 0; e < 8; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * a[e]);
                     tmem_st8(t_o + part * TP + h, o);
@@ -504,7 +504,8 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap map_q,
                 Cols rh, rl;
                 load_cols(t_o, rh);
                 load_cols(t_o + TP, rl);
-                tmem_wait_ld();
+                tmem_wait_ld(rh);
+                tmem_wait_ld(rl);
 #pragma unroll
                 for (int e = 0; e < NC; ++e)
                     if (q0 + e < T) put(e, __uint_as_float(rh[e]) + __uint_as_float(rl[e]));
@@ -590,7 +591,7 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap map_q,
                 // a dedicated probability tile is free once the PV product of tile
                 // g - PS is done; a K slot is free as soon as S(g) is (waited above)
                 if constexpr (!Lay::P_IN_K) mbar_wait(bars + Lay::B_PFREE + ps, ((g >> 1) & 1) ^ 1, abort_flag);
-                tmem_wait_ld();
+                tmem_wait_ld(r);
                 if (first) {
                     // a unit starts with the scores of the tile's first key (visible to every
                     // query: a prefix key, or the root) as its maxima: none is above the

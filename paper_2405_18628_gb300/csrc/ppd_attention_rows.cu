@@ -614,7 +614,7 @@ tree_attention_rows_kernel(const __grid_constant__ CUtensorMap map_q,
             float mx = -INFINITY;
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
-                tmem_wait_ld32(r[c]);
+                tmem_wait_ld(r[c]);
                 mx = chunk_max(bits_c, r[c], bits[c], mx);
             }
             mx *= sl2;   // sl2 > 0
@@ -632,7 +632,7 @@ tree_attention_rows_kernel(const __grid_constant__ CUtensorMap map_q,
                 for (int ch = 0; ch < D / 16; ++ch) {
                     uint32_t o[16];
                     tmem_ld16(t_os + ch * 16, o);
-                    tmem_wait_ld();
+                    tmem_wait_ld(o);
 #pragma unroll
                     for (int e = 0; e < 16; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
                     tmem_st16(t_os + ch * 16, o);
@@ -651,8 +651,8 @@ tree_attention_rows_kernel(const __grid_constant__ CUtensorMap map_q,
                 tmem_ld32(t_h, ra);
                 tmem_ld32(t_h + 32, rb);
                 const uint32_t b0 = BITS && half ? bits[2] : bits[0], b1 = BITS && half ? bits[3] : bits[1];
-                tmem_wait_ld32(ra);
-                tmem_wait_ld32(rb);
+                tmem_wait_ld(ra);
+                tmem_wait_ld(rb);
                 emit(bits_c, ra, b0, negm, t_h, sum);
                 emit(bits_c, rb, b1, negm, t_h + 32, sum);
                 p_ready(half);
@@ -700,8 +700,8 @@ tree_attention_rows_kernel(const __grid_constant__ CUtensorMap map_q,
                 uint32_t r0[32], r1[32];
                 tmem_ld32(t_os + c, r0);
                 tmem_ld32(t_os + c + 32, r1);
-                tmem_wait_ld32(r0);
-                tmem_wait_ld32(r1);
+                tmem_wait_ld(r0);
+                tmem_wait_ld(r1);
                 if (c + 64 == D) {
                     tc_fence_before();
                     __syncwarp();
@@ -763,8 +763,8 @@ tree_attention_rows_kernel(const __grid_constant__ CUtensorMap map_q,
                 uint32_t r0[32] = {}, r1[32] = {};
                 if (has_a) tmem_ld32(t_o + c, r0);
                 if (has_b) tmem_ld32(t_o + D + c, r1);
-                tmem_wait_ld32(r0);
-                tmem_wait_ld32(r1);
+                tmem_wait_ld(r0);
+                tmem_wait_ld(r1);
                 if (c + 32 == D / 2) {
                     tc_fence_before();
                     __syncwarp();

@@ -689,7 +689,7 @@ selftest_umma_kernel(const __grid_constant__ CUtensorMap ma, const __grid_consta
     for (int ch = 0; ch < N / 16; ++ch) {
         uint32_t r[16];
         tmem_ld16(tmem + lane_off + ch * 16, r);
-        tmem_wait_ld();
+        tmem_wait_ld(r);
         for (int e = 0; e < 16; ++e)
             d[(size_t)(warp * 32 + lane) * N + ch * 16 + e] =
                 *abort_flag ? NAN : __uint_as_float(r[e]);

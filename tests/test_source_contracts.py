@@ -38,3 +38,20 @@ def test_cluster_barriers_are_reached_by_converged_warps():
     assert set(bodies) == {"cluster_sync", "cluster_sync_exit"}
     for f, body in bodies.items():
         assert 0 <= body.find("__syncwarp()") < body.find("asm"), f
+
+
+def test_tensor_memory_loads_are_waited_for_by_name():
+    """tcgen05.ld fills its registers some time after it issues, and arithmetic on them
+    is free to move across a wait that does not mention them: every wait names the
+    registers (in-out operands), and the waits are issued by those functions only."""
+    src = _sources()
+    for name, text in src.items():
+        if name != "ppd_device.cuh":
+            assert "wait::ld" not in text, name
+    bodies = {f: b for f, b in _bodies(src["ppd_device.cuh"]).items() if "wait::ld" in b}
+    assert bodies
+    for f, body in bodies.items():
+        for stmt in re.findall(r"asm volatile\(\s*\"tcgen05\.wait::ld.*?;\n", body, flags=re.S):
+            outs = len(re.findall(r'"\+r"', stmt))
+            n = int(re.search(r"\(&r\)\[(\d+)\]", body[:body.index(stmt)].rsplit("PPD_DEV", 1)[1]).group(1))
+            assert outs == n, (f, outs, n)
