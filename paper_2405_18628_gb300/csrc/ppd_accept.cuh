@@ -337,7 +337,7 @@ PPD_DEV AcceptResult accept_warp_typical(TopLoad top, const float *x, Lse lse, E
     return accept_warp_pass(
         top,
         [&](int, int pa, int tk) {
-            const float pt = expf(__ldg(x + (size_t)pa * V + tk) * inv_temp - lse(pa));
+            const float pt = expf(ld_input(x + (size_t)pa * V + tk) * inv_temp - lse(pa));
             return pt > fminf(epsilon, delta * expf(-ent(pa)));
         },
         par, tok, P, T, V, S_max, lane, s_par, path);

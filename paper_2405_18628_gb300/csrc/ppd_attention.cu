@@ -548,7 +548,7 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap map_q,
             if (new_tree) {
 #pragma unroll
                 for (int x = 0; x < TP / 32; ++x)
-                    if (lane + 32 * x < T) par[x] = __ldg(p.parent + (size_t)ui.b * T + lane + 32 * x);
+                    if (lane + 32 * x < T) par[x] = ld_input(p.parent + (size_t)ui.b * T + lane + 32 * x);
             }
 
             for (int j = sg.j0; j < sg.j1; ++j, ++g) {

@@ -31,7 +31,7 @@ PPD_DEV UnitInfo unit_info(const AttnParams &p, int u)
     ui.lbh = SKIP && p.n_qb == 1 ? u : u / p.n_qb;
     ui.qb = u - ui.lbh * p.n_qb;
     ui.b = SKIP && p.B == 1 ? 0 : (ui.lbh / p.H) % p.B;
-    ui.P_raw = __ldg(p.prefix_len + ui.b);
+    ui.P_raw = ld_input(p.prefix_len + ui.b);
     ui.P = min(max(ui.P_raw, 0), p.S_max);
     ui.n_pref = (ui.P + 127) >> 7;
     ui.n_tiles = ui.n_pref + p.n_tt;
@@ -94,7 +94,7 @@ PPD_DEV WorkRange plan_cluster(const AttnParams &p)
     const int c = (int)blockIdx.x;
     w.u_first = w.u_last = c / p.cluster;
     const int32_t *P = p.prefix_len + w.u_first / (p.H * p.n_qb) % p.B;
-    const int nt = ((min(max(kHint ? ld_relaxed_gpu_s32(P) : __ldg(P), 0), p.S_max) + 127) >> 7) + p.n_tt;
+    const int nt = ((min(max(kHint ? ld_relaxed_gpu_s32(P) : ld_input(P), 0), p.S_max) + 127) >> 7) + p.n_tt;
     const int r = c - w.u_first * p.cluster;
     w.parts = min(p.cluster, nt);
     if (r < w.parts) {
@@ -126,7 +126,7 @@ PPD_DEV WorkRange plan_range(const AttnParams &p, int lane, uint8_t *seq = nullp
     const unsigned full = 0xffffffffu;
     const int per_b = p.H * p.n_qb;
     auto nt_of = [&](int b) {
-        const int P = min(max(kHint ? ld_relaxed_gpu_s32(p.prefix_len + b) : __ldg(p.prefix_len + b), 0),
+        const int P = min(max(kHint ? ld_relaxed_gpu_s32(p.prefix_len + b) : ld_input(p.prefix_len + b), 0),
                           p.S_max);
         return ((P + 127) >> 7) + p.n_tt;
     };
@@ -496,11 +496,11 @@ PPD_DEV void status_warp(const AttnParams &p, int lane)
     for (int b = blockIdx.x; b < p.B; b += gridDim.x) {
         bool bad = false;
         for (int i = lane; i < p.T; i += 32) {
-            const int pa = __ldg(p.parent + (size_t)b * p.T + i);
+            const int pa = ld_input(p.parent + (size_t)b * p.T + i);
             bad |= i == 0 ? pa != -1 : (pa < 0 || pa >= i);
         }
         bad = __any_sync(0xffffffffu, bad);
-        const int P = __ldg(p.prefix_len + b);
+        const int P = ld_input(p.prefix_len + b);
         if (lane == 0) p.dev_status[b] = bad ? kErrTree : (P < 0 || P > p.S_max ? kErrCapacity : kOk);
     }
 }
@@ -750,7 +750,7 @@ static __device__ __noinline__ void fused_side_warp(const AttnParams &p, const W
         };
         const int32_t *par_b = p.parent + (size_t)b * T;
         const int32_t *tok_b = f.cand_tokens + (size_t)b * T;
-        const int P = __ldg(p.prefix_len + b);
+        const int P = ld_input(p.prefix_len + b);
         AcceptResult res;
         // the accepted path: in registers (lane j % 32, slot j / 32) for trees of up
         // to 64 nodes, else in the scratch
@@ -772,7 +772,7 @@ static __device__ __noinline__ void fused_side_warp(const AttnParams &p, const W
                 res = accept_warp_small(
                     top_r,
                     [&](int, int pa, int tk) {
-                        const float pt = expf(__ldg(x + (size_t)pa * f.V + tk) * f.inv_temp - node_value(lse_r, pa));
+                        const float pt = expf(ld_input(x + (size_t)pa * f.V + tk) * f.inv_temp - node_value(lse_r, pa));
                         return pt > fminf(f.epsilon, f.delta * expf(-node_value(ent_r, pa)));
                     },
                     par_b, tok_b, P, T, f.V, p.S_max, lane, path_r);
@@ -829,8 +829,8 @@ static __device__ __noinline__ void fused_side_warp(const AttnParams &p, const W
                         if (in) {
                             const size_t so = ((size_t)lbh * T + src) * f.row_bytes + (size_t)c * 16;
                             dof[u] = ((size_t)lbh * p.S_max + P + j) * f.row_bytes + (size_t)c * 16;
-                            kx[u] = __ldg(reinterpret_cast<const uint4 *>(f.k_tree + so));
-                            vx[u] = __ldg(reinterpret_cast<const uint4 *>(f.v_tree + so));
+                            kx[u] = ld_input(reinterpret_cast<const uint4 *>(f.k_tree + so));
+                            vx[u] = ld_input(reinterpret_cast<const uint4 *>(f.v_tree + so));
                         }
                     }
 #pragma unroll

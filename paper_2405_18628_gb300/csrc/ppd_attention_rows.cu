@@ -801,7 +801,7 @@ tree_attention_rows_kernel(const __grid_constant__ CUtensorMap map_q,
                     int a = qg;
                     while (true) {
                         anc[a >> 5] |= 1u << (a & 31);
-                        const int pa = __ldg(p.parent + (size_t)ui.b * T + a);
+                        const int pa = ld_input(p.parent + (size_t)ui.b * T + a);
                         if (pa < 0 || pa >= a) break;   // the root, or a malformed tree
                         a = pa;
                     }

@@ -155,6 +155,37 @@ PPD_DEV int ld_relaxed_gpu_s32(const int *p)
     return v;
 }
 
+// Loads of data that another grid may have written while this one was already on the
+// chip (a grid of a programmatic chain waits for the grids before it, then reads).  Not
+// __ldg: ld.global.nc is for data that stays unchanged for as long as the grid exists.
+PPD_DEV int ld_input(const int *p)
+{
+    int v;
+    asm volatile("ld.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+
+PPD_DEV float ld_input(const float *p)
+{
+    float v;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
+    return v;
+}
+
+PPD_DEV float4 ld_input(const float4 *p)
+{
+    float4 v;
+    asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p) : "memory");
+    return v;
+}
+
+PPD_DEV uint4 ld_input(const uint4 *p)
+{
+    uint4 v;
+    asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
+    return v;
+}
+
 PPD_DEV void st_release_gpu(unsigned long long *p, unsigned long long v)
 {
     asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");

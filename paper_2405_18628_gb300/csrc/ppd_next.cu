@@ -182,7 +182,7 @@ PPD_DEV void find_chains(ChainSmem &c, const int32_t *parent, const int32_t *can
 // block; NaN when the row holds a NaN or +inf, or only -inf.  Written to
 // lse[(b * (n_states - 1) + d - 1) * kNextMaxEpt + j].
 __global__ void __launch_bounds__(kTopkThreads)
-next_lse_kernel(const float *__restrict__ logits, const int32_t *parent, const int32_t *cand,
+next_lse_kernel(const float *logits, const int32_t *parent, const int32_t *cand,
                 const int32_t *path, const int32_t *accept_len, int T, int V, int n_states,
                 int n_ept, int vec, float *lse)
 {
@@ -204,7 +204,7 @@ next_lse_kernel(const float *__restrict__ logits, const int32_t *parent, const i
 #pragma unroll
             for (int q = 0; q < kBatch; ++q) {
                 xs[q] = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
-                if (v4 + q * kTopkThreads < V4) xs[q] = __ldg(reinterpret_cast<const float4 *>(x) + v4 + q * kTopkThreads);
+                if (v4 + q * kTopkThreads < V4) xs[q] = ld_input(reinterpret_cast<const float4 *>(x) + v4 + q * kTopkThreads);
             }
 #pragma unroll
             for (int q = 0; q < kBatch; ++q) {
@@ -215,7 +215,7 @@ next_lse_kernel(const float *__restrict__ logits, const int32_t *parent, const i
             }
         }
     } else {
-        for (int v = tid; v < V; v += kTopkThreads) lse_add(acc, __ldg(x + v));
+        for (int v = tid; v < V; v += kTopkThreads) lse_add(acc, ld_input(x + v));
     }
     lse_warp(acc);
     if (lane == 0) {
@@ -242,7 +242,7 @@ next_lse_kernel(const float *__restrict__ logits, const int32_t *parent, const i
 // multiple of 4).  kChains: ensemble chains whose loads are in flight together.
 template <int kChains>
 __global__ void __launch_bounds__(kTopkThreads)
-next_topk_kernel(const float *__restrict__ logits, const int32_t *parent, const int32_t *cand,
+next_topk_kernel(const float *logits, const int32_t *parent, const int32_t *cand,
                  const int32_t *path, const int32_t *accept_len, int T, int V, int n_states, int K,
                  int n_ept, int ept_mean, int vec, int chunk, const float *lse, int32_t *topk,
                  int32_t *kstate)
@@ -441,10 +441,10 @@ next_assemble_kernel(const int32_t *path, const int32_t *accept_len, const int32
     const int total = n_states * T_next;
     const bool all = early && total <= kAsmEntries;
     auto clamp16 = [](int v) { return (int16_t)max(-2, min(v, 32767)); };
-    auto load = [&](int first, int n) {
+    auto load = [&](int first, int n) {   // through L2: ahead of the wait, no earlier line of L1 will do
         for (int i = tid; i < n; i += kAsmThreads) {
-            s_par[i] = clamp16(__ldg(tmpl_parent + first + i));
-            s_rank[i] = clamp16(__ldg(tmpl_rank + first + i));
+            s_par[i] = clamp16(ld_relaxed_gpu_s32(tmpl_parent + first + i));
+            s_rank[i] = clamp16(ld_relaxed_gpu_s32(tmpl_rank + first + i));
         }
     };
     if (!early) pdl_wait();

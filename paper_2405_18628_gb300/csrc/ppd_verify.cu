@@ -33,7 +33,7 @@ namespace ppd {
 // serialization may start right away.
 template <bool kVec, bool kStats>
 __global__ void __launch_bounds__(256)
-argmax_partial_kernel(const float *__restrict__ logits, int V, int splits, int chunk,
+argmax_partial_kernel(const float *logits, int V, int splits, int chunk,
                       float *part_val, int32_t *part_idx, float *part_stats, float stat_k,
                       int32_t *zero_status, int n_zero)
 {
@@ -170,7 +170,7 @@ cudaError_t launch_argmax_partials(const float *logits, int64_t rows, int V, int
 // with programmatic stream serialization may start right away.
 template <bool kStats>
 __global__ void __launch_bounds__(512)
-argmax_narrow_kernel(const float *__restrict__ logits, int V, int splits, int chunk, int vec,
+argmax_narrow_kernel(const float *logits, int V, int splits, int chunk, int vec,
                      int64_t n_chunks, float *part_val, int32_t *part_idx, float *part_stats,
                      float stat_k, int32_t *zero_status, int n_zero)
 {
@@ -229,7 +229,7 @@ cudaError_t launch_argmax_narrow(const float *logits, int64_t rows, int V, int s
 // (host-bound: 64 nodes, 1024 slices, four calls).
 template <bool kStats>
 __global__ void __launch_bounds__(256)
-node_argmax_kernel(const float *__restrict__ logits, int V, int chunk, int vec, int32_t *argmax_out,
+node_argmax_kernel(const float *logits, int V, int chunk, int vec, int32_t *argmax_out,
                    float stat_k, float *lse_out, float *ent_out, int n_cta)
 {
     struct Best {
@@ -333,8 +333,6 @@ PPD_DEV void write_accept(const AcceptArgs &a, int b, const AcceptResult &r)
     a.dev_status[b] = r.status;
 }
 
-// (Grids of a programmatic chain start before the one that writes their inputs is
-// done, so what other grids write is read through L2.)
 // One warp per sequence; trees of up to 64 nodes in registers, whose walks cost
 // shuffles instead of dependent loads.
 __global__ void __launch_bounds__(128)
@@ -430,10 +428,9 @@ cudaError_t launch_typical_accept(const float *logits, const float *lse, const f
 // ------------------------------------------------------------------ compaction
 
 __global__ void __launch_bounds__(128)
-kv_compact_kernel(uint8_t *kc, uint8_t *vc, const uint8_t *__restrict__ kt,
-                  const uint8_t *__restrict__ vt, const int32_t *path, const int32_t *accept_len,
-                  const int32_t *prefix_len, int64_t n_units, int B, int H, int T, int S_max,
-                  int row_bytes)
+kv_compact_kernel(uint8_t *kc, uint8_t *vc, const uint8_t *kt, const uint8_t *vt, const int32_t *path,
+                  const int32_t *accept_len, const int32_t *prefix_len, int64_t n_units, int B, int H,
+                  int T, int S_max, int row_bytes)
 {
     const int chunks = row_bytes >> 4;
     pdl_release();
@@ -449,8 +446,8 @@ kv_compact_kernel(uint8_t *kc, uint8_t *vc, const uint8_t *__restrict__ kt,
             if (src < 0 || src >= T) continue;
             const size_t so = ((size_t)u * T + src) * row_bytes + (size_t)c * 16;
             const size_t dof = ((size_t)u * S_max + P + j) * row_bytes + (size_t)c * 16;
-            const uint4 kx = __ldg(reinterpret_cast<const uint4 *>(kt + so));
-            const uint4 vx = __ldg(reinterpret_cast<const uint4 *>(vt + so));
+            const uint4 kx = ld_input(reinterpret_cast<const uint4 *>(kt + so));
+            const uint4 vx = ld_input(reinterpret_cast<const uint4 *>(vt + so));
             *reinterpret_cast<uint4 *>(kc + dof) = kx;
             *reinterpret_cast<uint4 *>(vc + dof) = vx;
         }
@@ -524,7 +521,7 @@ __global__ void __launch_bounds__(256) round_bf16_kernel(const RoundArgs r, int6
     if (i == r.n) return;
     const RoundArgs::Tensor t = r.t[i];
     int rows = t.rows;
-    if (t.cache) rows = min(max(__ldg(r.prefix_len + (lbh / r.H) % r.B), 0), rows);
+    if (t.cache) rows = min(max(ld_input(r.prefix_len + (lbh / r.H) % r.B), 0), rows);
     const int per_row = r.D / 8;
     const int first = blk * kRoundRows, n = min(kRoundRows, rows - first) * per_row;   // 8-element pieces
     const float4 *src = reinterpret_cast<const float4 *>(t.src + ((size_t)lbh * t.rows + first) * r.D);
@@ -536,8 +533,8 @@ __global__ void __launch_bounds__(256) round_bf16_kernel(const RoundArgs r, int6
         for (int u = 0; u < U; ++u) {
             const int x = x0 + u * 256;
             if (x < n) {
-                v[u][0] = __ldg(src + 2 * x);
-                v[u][1] = __ldg(src + 2 * x + 1);
+                v[u][0] = ld_input(src + 2 * x);
+                v[u][1] = ld_input(src + 2 * x + 1);
             }
         }
 #pragma unroll

@@ -55,3 +55,13 @@ def test_tensor_memory_loads_are_waited_for_by_name():
             outs = len(re.findall(r'"\+r"', stmt))
             n = int(re.search(r"\(&r\)\[(\d+)\]", body[:body.index(stmt)].rsplit("PPD_DEV", 1)[1]).group(1))
             assert outs == n, (f, outs, n)
+
+
+def test_no_load_assumes_that_its_data_never_changes():
+    """A grid of a programmatic chain is on the chip while the grids before it still
+    write its inputs; it waits for them and then reads.  ld.global.nc (__ldg, or a plain
+    load through a const __restrict__ pointer) wants data that stays unchanged for as long
+    as the grid exists, so no kernel uses it."""
+    for name, text in _sources().items():
+        for word in ("__ldg", "global.nc", "__restrict__"):
+            assert word not in text, (name, word)
