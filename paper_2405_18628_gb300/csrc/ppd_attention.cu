@@ -777,36 +777,35 @@ static cudaError_t launch_tree_attention_t(const AttnMaps &m, const AttnParams &
 // answer only depends on how the device groups its SMs.
 int max_attention_clusters(int size)
 {
-    static std::atomic<int> cache[64][kMaxCluster + 1];   // the answer + 1
+    static std::atomic<int> cache[64][kMaxCluster + 1];
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) {
         (void)cudaGetLastError();
         return 0;
     }
     if (dev < 0 || dev >= 64 || size < 1 || size > kMaxCluster) return 0;
-    int got = cache[dev][size].load(std::memory_order_relaxed);
-    if (got > 0) return got - 1;
-    using Lay = AttnLayout<128, 64>;
-    auto kern = tree_attention_kernel<128, 64, 2>;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)size);
-    cfg.blockDim = dim3(Lay::THREADS);
-    cfg.dynamicSmemBytes = Lay::SMEM_BYTES;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)size;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    int n = 0;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Lay::SMEM_BYTES) != cudaSuccess ||
-        cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) {
-        (void)cudaGetLastError();
-        n = 0;
-    }
-    cache[dev][size].store(n + 1, std::memory_order_relaxed);
-    return n;
+    return asked_once(cache[dev][size], [&] {
+        using Lay = AttnLayout<128, 64>;
+        auto kern = tree_attention_kernel<128, 64, 2>;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)size);
+        cfg.blockDim = dim3(Lay::THREADS);
+        cfg.dynamicSmemBytes = Lay::SMEM_BYTES;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = (unsigned)size;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        int n = 0;
+        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Lay::SMEM_BYTES) != cudaSuccess ||
+            cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) {
+            (void)cudaGetLastError();
+            return -1;
+        }
+        return n;
+    });
 }
 
 cudaError_t launch_tree_attention(const AttnMaps &m, const AttnParams &p, int D, int num_sms,

@@ -4,6 +4,8 @@
 
 #include <cuda.h>
 #include <cuda_runtime.h>
+
+#include <atomic>
 #include <cstdint>
 
 namespace ppd {
@@ -121,6 +123,19 @@ constexpr int kMaxCluster = 8;
 // Clusters of `size` attention CTAs (one per SM) the current device can hold at
 // once; 0 when it cannot be asked.
 int max_attention_clusters(int size);
+
+// A number >= 0 asked for once: kept in `slot` (plus one; 0: not known yet).  An `ask`
+// that fails (a negative answer) counts as 0 this time and is asked again the next.
+template <class Ask>
+inline int asked_once(std::atomic<int> &slot, Ask ask)
+{
+    const int got = slot.load(std::memory_order_relaxed);
+    if (got > 0) return got - 1;
+    const int n = ask();
+    if (n < 0) return 0;
+    slot.store(n + 1, std::memory_order_relaxed);
+    return n;
+}
 
 // The unit a CTA has to have merged: it holds the unit's first tile and its
 // range ends inside the unit (u = -1: none).  off: the unit's tile 0 among
