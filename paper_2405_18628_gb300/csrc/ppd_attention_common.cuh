@@ -209,12 +209,16 @@ PPD_DEV WorkRange plan_range(const AttnParams &p, int lane, uint8_t *seq = nullp
 }
 
 // Before the wait of a chained launch (one warp, all lanes): ask L2 for the
-// first `n` K and V prefix tiles this CTA will stream, from a plan made with
+// first `n` K and V prefix tiles of this CTA's work, from a plan made with
 // prefix lengths that may still be changing.  Only a hint -- nothing is
 // written to shared memory and nothing waits on it; the real loads follow the
 // wait with the plan remade -- so the preceding grid's work overlaps the
 // first tiles' trip from HBM.  Tree tiles are skipped (in a model the
-// preceding grids write them).
+// preceding grids write them).  Whole units go in index order here, also where
+// the work then takes the longest sequences first: L2 serves every CTA, so a tile
+// helps whichever CTA streams it, and working that order out costs time before the
+// hint (calls of 8 sequences of up to 4096 keys, 32 heads, 64 tokens: 76.5 us like
+// this, 77.4 in the order of the work, 78.4 without the hint).
 template <bool SPLIT>
 PPD_DEV void prefetch_first_tiles(const AttnParams &p, int lane, const CUtensorMap *kc,
                                   const CUtensorMap *vc, int dch, int n)

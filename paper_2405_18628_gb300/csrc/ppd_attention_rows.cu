@@ -176,7 +176,8 @@ struct RowsIter {
     }
 };
 
-// prefetch_first_tiles for whole jobs: this CTA's first `n` prefix tiles.
+// prefetch_first_tiles for whole jobs: the first `n` prefix tiles of this CTA's first
+// job in round-robin order.
 template <bool RANGE>
 PPD_DEV void rows_prefetch(const AttnParams &p, int lane, const CUtensorMap *kc, const CUtensorMap *vc,
                            int dch, int n)
@@ -287,7 +288,9 @@ tree_attention_rows_kernel(const __grid_constant__ CUtensorMap map_q,
     } else if (warp == 8) {
         // ------------------------------------------------------------ TMA producer
         if (lane == 0) {
-            // slices read by more than one CTA stay in L2 for the second reader
+            // slices of three or four blocks stay in L2 for their later readers; two single
+            // blocks of a slice are read side by side (with the normal policy too: 32 slices
+            // of 2048 keys, 200 tokens, 18.8 us a call either way, 40 of 4096 38.9 -> 39.6)
             const uint64_t pol = p.n_qb > 2 ? l2_policy_evict_normal() : l2_policy_evict_first();
             Pos pos;
             int n_tiles = 0, n_q0 = 0, n_q1 = 0;   // copies issued: ring tiles, Q blocks per slot
