@@ -670,11 +670,11 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap map_q,
                 pend_g = g - 1;
                 pend_f = 1 | (ob << 3);
                 if (SPLIT && !seg_whole(sg)) {
-                    // a part: slot 2c for the tail range's first segment, 2c + 1 for its last
+                    // a part: slot 2c for the range's first segment, 2c + 1 for its last
                     pend_f |= 2 | (sg.u == wr.u_first ? 4 : 0);
                     // the part holding the unit's first tile records it for the merge
                     if (sg.j0 == 0 && threadIdx.x == 0)
-                        p.split_rec[blockIdx.x] = SplitRecord{wr.x_first + (wr.n_tiles - it.left) - sg.j1, wr.n_tail, u, ui.n_tiles};
+                        p.split_rec[blockIdx.x] = SplitRecord{wr.x_first + (wr.n_tiles - it.left) - sg.j1, wr.n_shared, u, ui.n_tiles};
                 }
             }
         }
@@ -733,8 +733,8 @@ __global__ void __launch_bounds__(256) split_merge_kernel(const AttnParams p, in
     const int n_rows = min(kSplitRows, p.T - qb * kSplitRows);
     const int row = (int)blockIdx.y * rows_per_block + (int)threadIdx.x / per_row;
     if (row >= n_rows) return;
-    const SplitParts sp = split_parts(r.n_tail, r.off, r.n_tiles);
-    split_merge_chunk(p.split_part, p.out, p.lse, sp, r.n_tail, (int)gridDim.x,
+    const SplitParts sp = split_parts(r.n_shared, r.off, r.n_tiles);
+    split_merge_chunk(p.split_part, p.out, p.lse, sp, r.n_shared, (int)gridDim.x,
                       (size_t)lbh * p.T + (size_t)qb * kSplitRows, row, ((int)threadIdx.x % per_row) * 8, D);
 }
 

@@ -59,7 +59,7 @@ struct WorkRange {
     int n_tiles;             // tiles in the range (0: none)
     int u_last;              // last unit the range touches
     long long x_first;       // index of the range's first tile
-    long long n_tail;        // tiles shared out by the split
+    long long n_shared;        // tiles shared out by the split
     const uint8_t *seq;      // not null: whole jobs go longest sequence first, in this order
     int parts;               // cluster split: the CTAs of the cluster with tiles, the first ones
 };
@@ -82,7 +82,7 @@ PPD_DEV int ragged_job(const AttnParams &p, const uint8_t *seq, int i, int step,
     return (rest / per_layer * p.B + b) * per_layer + rest % per_layer;
 }
 
-// First tail tile of CTA c, and the CTA holding tail tile x.
+// First shared tile of CTA c, and the CTA holding shared tile x.
 PPD_DEV long long split_start(int c, long long N, int G) { return (long long)c * N / G; }
 PPD_DEV int split_cta_of(long long x, long long N, int G) { return (int)(((x + 1) * G + N - 1) / N) - 1; }
 
@@ -117,7 +117,7 @@ PPD_DEV WorkRange plan_range(const AttnParams &p, int lane, uint8_t *seq = nullp
     if (p.cluster > 1) return plan_cluster<kHint>(p);
     WorkRange w{};
     const int G = (int)gridDim.x, c = (int)blockIdx.x;
-    // no tail range unless one is found below
+    // no range of tiles unless one is found below
     w.u_first = p.n_units;
     w.u_last = -1;
     w.n_tiles = 0;
@@ -163,15 +163,6 @@ PPD_DEV WorkRange plan_range(const AttnParams &p, int lane, uint8_t *seq = nullp
     s1 += __shfl_sync(full, s0, 31);
     const long long per_layer = __shfl_sync(full, s1, 31);
     const long long N = per_layer * p.L;
-    // global tile index of unit u's tile 0
-    auto origin = [&](int u) {
-        const int l = u / (p.B * per_b);
-        const int rem = u - l * p.B * per_b;
-        const int b = rem / per_b, idx = rem - b * per_b;
-        const int incl = b < 32 ? __shfl_sync(full, s0, b & 31) : __shfl_sync(full, s1, b & 31);
-        const int wt = b < 32 ? __shfl_sync(full, w0, b & 31) : __shfl_sync(full, w1, b & 31);
-        return (long long)l * per_layer + (incl - wt) + (long long)idx * (wt / per_b);
-    };
     // unit and tile of global tile x (0 <= x < N)
     auto locate = [&](long long x, int &u, int &j) {
         const int l = (int)(x / per_layer);
@@ -195,15 +186,14 @@ PPD_DEV WorkRange plan_range(const AttnParams &p, int lane, uint8_t *seq = nullp
         j = rb - idx * nt;
         u = (l * p.B + b) * per_b + idx;
     };
-    const long long base = origin(w.rr_units);
-    w.n_tail = N - base;
-    const long long gs = split_start(c, w.n_tail, G), ge = split_start(c + 1, w.n_tail, G);
+    w.n_shared = N;
+    const long long gs = split_start(c, w.n_shared, G), ge = split_start(c + 1, w.n_shared, G);
     w.x_first = gs;
     w.n_tiles = (int)(ge - gs);
     if (ge > gs) {
         int jl;
-        locate(base + gs, w.u_first, w.j_first);
-        locate(base + ge - 1, w.u_last, jl);
+        locate(gs, w.u_first, w.j_first);
+        locate(ge - 1, w.u_last, jl);
     }
     return w;
 }
@@ -687,7 +677,7 @@ static __device__ __noinline__ void fused_side_warp(const AttnParams &p, const W
         have_all = true;
     }
     // the units whose first tile this CTA streams (its round-robin units and the
-    // tail units starting in its range) compact their slices here
+    // units starting in its range) compact their slices here
     const int t_lo = wr.u_first + (wr.j_first > 0 ? 1 : 0), t_hi = wr.n_tiles > 0 ? wr.u_last : -1;
     auto owns_first_tile = [&](auto fn) {
         for (int u = (int)blockIdx.x; u < wr.rr_units; u += (int)gridDim.x)

@@ -871,7 +871,7 @@ tree_attention_rows_kernel(const __grid_constant__ CUtensorMap map_q,
                     // the part holding the unit's first tile records it for the merge
                     if (jb.j0 == 0 && threadIdx.x == 0)
                         p.split_rec[blockIdx.x] =
-                            SplitRecord{wr.x_first + (wr.n_tiles - it.seg.left) - jb.j1, wr.n_tail, u, ui.n_tiles};
+                            SplitRecord{wr.x_first + (wr.n_tiles - it.seg.left) - jb.j1, wr.n_shared, u, ui.n_tiles};
                 }
                 finish_single(jb, st0, n >= 2, slot);
             }

@@ -139,9 +139,9 @@ inline int asked_once(std::atomic<int> &slot, Ask ask)
 
 // The unit a CTA has to have merged: it holds the unit's first tile and its
 // range ends inside the unit (u = -1: none).  off: the unit's tile 0 among
-// the tail's tiles; n_tail: the tail's tile count.
+// the launch's tiles; n_shared: their number.
 struct SplitRecord {
-    long long off, n_tail;
+    long long off, n_shared;
     int u, n_tiles;
 };
 
