@@ -308,7 +308,9 @@ ppd_status ppd_node_argmax_noalloc(const float *logits, int B, int T, int V, int
  * ppd_verify_step_typical call (typical != 0) enqueues for these sizes, with
  * a workspace of ppd_workspace_bytes(...) bytes and the whole GPU available.
  * No paper counterpart: it lets a caller or benchmark count the kernels of a
- * step without a profiler.  Returns -1 for sizes the step rejects.
+ * step without a profiler.  It depends on the current device (its SMs and the clusters
+ * it can hold; without one, 148 SMs and no clusters are assumed).  Returns -1 for
+ * sizes the step rejects.
  */
 int ppd_verify_step_launches(int L, int B, int H, int T, int D, int V, int S_max, ppd_dtype dt,
                              int typical);
@@ -327,6 +329,18 @@ int ppd_verify_step_launches(int L, int B, int H, int T, int D, int V, int S_max
  * every CTA resident.  Returns -1 for sizes the step rejects.
  */
 int ppd_verify_step_form(int L, int B, int H, int T, int D, int V, int S_max, ppd_dtype dt);
+
+/*
+ * How an attention launch of these sizes shares its work out (no paper
+ * counterpart; for tests and benchmarks): 0 whole slices (or blocks of 128
+ * queries), in rounds of one per SM; 2..8 a cluster of that many SMs each; 1
+ * the work split; plus 16 where trees of more than 64 tokens run as pairs of
+ * query blocks.  workspace: whether the call gets a full one; one_grid: whether it
+ * is the attention of a step of form 2.  Like the two functions above it depends on
+ * the current device: without one no clusters are planned.  Returns -1 for sizes
+ * that are rejected.
+ */
+int ppd_attention_plan(int L, int B, int H, int T, int D, int S_max, int workspace, int one_grid);
 
 /*
  * Force the form of every later fused step of this process (B <= 64): 1 or 2

@@ -379,6 +379,18 @@ ppd_status enqueue_attention_any(const void *q, const void *kc, const void *vc, 
                              scale, out, lse, dev_status, ws, &wl, fused, false, chained, chained, stream);
 }
 
+// The jobs of an attention launch without a split: its units, with plan_rows' choice.
+AttnParams row_plan(int L, int B, int H, int T, int S_max)
+{
+    AttnParams p{};
+    p.T_pad = (T + 31) & ~31;
+    p.n_qb = p.T_pad > 64 ? (T + 127) / 128 : 1;
+    p.n_units = (int)((long long)L * B * H) * p.n_qb;
+    p.S_max = S_max;
+    ppd::plan_rows(p, split_grid());
+    return p;
+}
+
 // Blocks of the fused step's narrow argmax grid (0: use the wide grid).  When
 // the attention grid's jobs do not fill whole rounds, the CTAs of the last,
 // partial round that hold one job fewer -- grid - (jobs mod grid) of
@@ -392,12 +404,7 @@ int narrow_argmax_grid(int L, int B, int H, int T, int D, int V, int S_max)
 {
     const AttnPlan plan = plan_attention(L, B, H, T, S_max, true, true);
     if (plan.split || plan.cluster > 1) return 0;
-    AttnParams p{};
-    p.T_pad = (T + 31) & ~31;
-    p.n_qb = p.T_pad > 64 ? (T + 127) / 128 : 1;
-    p.n_units = (int)((long long)L * B * H) * p.n_qb;
-    p.S_max = S_max;
-    ppd::plan_rows(p, split_grid());
+    const AttnParams p = row_plan(L, B, H, T, S_max);
     // two groups of CTAs with queues of their own: none is known to have time to spare
     if (p.pairs && p.n_qb == 3) return 0;
     const long long n_jobs = ppd::whole_jobs(p);
@@ -568,6 +575,14 @@ int ppd_verify_step_form(int L, int B, int H, int T, int D, int V, int S_max, pp
     if (!attn_dims_ok(L, B, H, T, D, S_max, dt) || V < 1) return -1;
     if (B > ppd::kFusedMaxB) return kFormGrids;
     return choose_form(L, B, H, T, D, V, S_max);
+}
+
+int ppd_attention_plan(int L, int B, int H, int T, int D, int S_max, int workspace, int one_grid)
+{
+    if (!attn_dims_ok(L, B, H, T, D, S_max, PPD_BF16)) return -1;
+    const AttnPlan plan = plan_attention(L, B, H, T, S_max, workspace != 0, one_grid == 0);
+    if (plan.split || plan.cluster > 1) return plan.split ? 1 : plan.cluster;
+    return row_plan(L, B, H, T, S_max).pairs ? 16 : 0;
 }
 
 ppd_status ppd_debug_grid_wait(unsigned long long limit_ns, int withhold_cta)

@@ -51,7 +51,7 @@ def load() -> ctypes.CDLL:
             "ppd_debug_grid_wait": ([ctypes.c_ulonglong, i32], i32),
             "ppd_status_string": ([i32], ctypes.c_char_p),
             "ppd_last_cuda_error": ([], ctypes.c_char_p),
-            "ppd_last_cuda_error": ([], ctypes.c_char_p),
+            "ppd_attention_plan": ([i32] * 8, i32),
             "ppd_tree_attention": ([vp] * 7 + [i32] * 7 + [f32, vp, vp, vp, vp, sz, vp], i32),
             "ppd_node_argmax": ([vp, i32, i32, i32, vp, vp, sz, vp], i32),
             "ppd_accept_path": ([vp] * 4 + [i32] * 4 + [vp] * 5 + [vp], i32),
@@ -130,9 +130,14 @@ def ppd_verify_step_launches(L, B, H, T, D, V, S_max, dtype=PPD_BF16, typical=Fa
 
 def ppd_verify_step_form(L, B, H, T, D, V, S_max, dtype=PPD_BF16) -> int:
     """Form of the fused step for these sizes: 0 separate grids, 1 argmax grid
-    then attention grid, 2 one grid with the argmax in the side warps, 3 one
-    grid with the argmax in the CTAs of the last, partial round."""
+    then attention grid, 2 one grid with the argmax in the side warps."""
     return int(load().ppd_verify_step_form(L, B, H, T, D, V, S_max, dtype))
+
+
+def ppd_attention_plan(L, B, H, T, D, S_max, workspace=True, one_grid=False) -> int:
+    """How an attention launch shares its work out: 0 whole slices, 2..8 clusters of
+    that many SMs, 1 the work split, + 16 with pairs of query blocks."""
+    return int(load().ppd_attention_plan(L, B, H, T, D, S_max, int(workspace), int(one_grid)))
 
 
 def ppd_set_verify_step_form(form: int) -> int:
