@@ -36,7 +36,8 @@ def _wl(name, seed, **kw):
 
 
 CASES = {
-    # key-row kernel, work split (24 slices), scalar logits loads (V % 4 != 0)
+    # key-row kernel, 24 slices (work split in form 2, clusters in form 1), scalar logits
+    # loads (V % 4 != 0)
     "keyrow_split_v301": (_wl("a", 501, L=2, B=3, H=4, D=64, P=1500, T=40, V=301),
                           [1500, 700, 3]),
     # key-row kernel, whole slices round-robin (256 slices)
@@ -312,7 +313,7 @@ def test_in_grid_reports_bad_sequences(cuda_device, case, form):
 def test_argmax_grid_form(cuda_device, case, typical):
     """Form 1 (an argmax grid, then the attention grid) against the oracle: on
     the idle SMs of a partial round of slices the step runs a narrow argmax
-    grid (the first three cases), under the work split the wide one (the
+    grid (the first three cases), with slices on clusters the wide one (the
     last).  Exact matching and typical acceptance."""
     w, pl = CASES[case]
     s, t = _inputs(w, pl)

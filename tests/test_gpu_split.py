@@ -1,13 +1,12 @@
-"""The attention work split against the oracle.  Launches with fewer slices
-than SMs share all key tiles out over every SM, and the slices cut between
-SMs are merged by a second grid.
+"""The attention of launches with fewer slices than SMs against the oracle: each
+slice on a cluster of SMs, or (where only clusters too small to pay would fit) all key
+tiles shared out over every SM, the slices cut between SMs merged by a second grid.
 
-Cases: calls with few slices and long prefixes (many parts per slice);
-prefixes far shorter than the cache (fewer tiles than SMs, so some SMs get
-none); both kernels, including trees over 128 tokens; launches with more
-slices than SMs (whole slices, with a workspace).  Also: the unsplit path (no
-workspace), repeated calls on one workspace, and a workspace full of junk
-(any contents must do)."""
+Cases: calls with few slices and long prefixes; prefixes far shorter than the
+cache (SMs of a cluster without tiles); both kernels, including trees over 128
+tokens; launches with more slices than SMs (whole slices).  With a workspace and
+without one (which only the work split needs), repeated calls on one workspace,
+and a workspace full of junk (any contents must do)."""
 import numpy as np
 import pytest
 import torch
@@ -46,11 +45,11 @@ def _attend(t_dev, pl, parent, dev, ws):
 
 
 CASES = [
-    # L, B, H, T, D, prefix, S_max: what it exercises (all split but the last two)
-    (1, 1, 2, 64, 128, [3000], 3072),          # 2 slices x 25 tiles over 50 SMs: 25 parts each
+    # L, B, H, T, D, prefix, S_max: what it exercises (clusters but for the last two)
+    (1, 1, 2, 64, 128, [3000], 3072),          # 2 slices x 25 tiles
     (2, 3, 5, 48, 64, [0, 129, 2000], 2048),   # mixed prefixes, empty prefix, D = 64
-    (1, 2, 3, 40, 128, [100, 5], 4096),        # 12 tiles for 152 SMs: empty ranges
-    (1, 1, 2, 96, 128, [2500], 2560),          # query-row kernel, slices cut many times
+    (1, 2, 3, 40, 128, [100, 5], 4096),        # fewer tiles than SMs of a cluster
+    (1, 1, 2, 96, 128, [2500], 2560),          # query-row kernel
     (1, 2, 1, 200, 128, [900, 33], 1024),      # two query blocks and two tree tiles per slice
     (1, 1, 1, 512, 64, [300], 1024),           # four query blocks, tree tiles alone in a part
     (2, 1, 32, 64, 128, [2048], 2112),         # Vicuna-7B shapes, two layers
@@ -72,14 +71,13 @@ def test_split_matches_oracle(cuda_device, L, B, H, T, D, prefix, S_max):
         assert (st == 0).all(), st
         assert_attn_close(out.reshape(ref.shape), ref, f"split, call {rep}")
         np.testing.assert_allclose(lse.reshape(ref_lse.shape), ref_lse, rtol=0, atol=1e-3)
-    # the unsplit path: one whole slice per SM at a time
     out, lse, st = _attend(t_dev, pl, parent, cuda_device, None)
     assert (st == 0).all()
-    assert_attn_close(out.reshape(ref.shape), ref, "unsplit")
+    assert_attn_close(out.reshape(ref.shape), ref, "no workspace")
 
 
 def test_split_in_fused_step(cuda_device):
-    """The fused verification step with slices cut between SMs: attention
+    """The fused verification step with slices on clusters of SMs: attention
     within tolerance, indices and compacted KV bit for bit."""
     w = W.scaled(W.WORKLOADS["mobilellama"], L=2, H=3)
     s = W.make_step_inputs(w)
@@ -121,7 +119,7 @@ def test_workspace_contents_do_not_matter(cuda_device):
 
 
 def test_split_status_per_call(cuda_device):
-    """Per-sequence status on the split path: a malformed tree and a prefix
+    """Per-sequence status with slices on clusters: a malformed tree and a prefix
     beyond the cache are reported over a status array holding junk, and the
     next call on the same workspace, with clean inputs, reports neither and
     matches the oracle."""
@@ -148,13 +146,13 @@ def test_split_status_per_call(cuda_device):
     (40, 100, 64, [4000, 10], 4096),      # 80 slices: the work split of the query-row kernel
     (20, 33, 64, [1000, 127], 1024),      # 40 slices: clusters of 3
     (14, 17, 128, [700, 0], 1024),        # 28: clusters of 5, one of a single tile
-    (10, 128, 64, [900, 513], 1024),      # 20: clusters of 6, query-row kernel
-    (7, 300, 64, [400, 129], 600),        # 14 slices of three query blocks
-    (1, 64, 128, [1, 900], 4096),         # clusters of 8 with more CTAs than tiles
+    (10, 128, 64, [900, 513], 1024),      # 20: clusters of 5, query-row kernel
+    (7, 300, 64, [400, 129], 600),        # 14 slices of three query blocks: clusters of 3
+    (1, 64, 128, [1, 900], 4096),         # clusters of 7 with more CTAs than tiles
     (2, 200, 128, [0, 300], 4096),        # the same in the query-row kernel, rows without keys in a part
 ])
 def test_split_sizes(cuda_device, H, T, D, prefix, S_max):
-    """Clusters of every size, and the work split where no cluster size fits."""
+    """Clusters of several sizes, and the work split where no cluster size fits."""
     L, B = 1, 2
     t, pl, parent = _case(L, B, H, T, D, prefix, S_max, seed=H + T)
     t_dev = {k: v.to(cuda_device) for k, v in t.items()}

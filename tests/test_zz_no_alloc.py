@@ -1,13 +1,12 @@
 """ppd_node_argmax_noalloc: the node argmax for callers that cannot allocate
 device memory (a plugin handed only its input and output tensors, a loop that
-forbids allocation after start-up, a fixed memory budget).  Its partial maxima
-live in a fixed array inside the library instead of a caller workspace.
+forbids allocation after start-up, a fixed memory budget).  Its grid needs no
+scratch at all.
 
 The results must equal the fp64 oracle's argmax and ppd_node_argmax's bit for
-bit, on consecutive calls that reuse the shared array with different shapes
-(up to the largest request the array holds, B*T = 65,536 node rows, with
-16-byte and scalar loads), and oversized requests must be refused before any
-work is enqueued.  This file is collected last on purpose.
+bit, on consecutive calls of different shapes (up to the largest request,
+B*T = 65,536 node rows, with 16-byte and scalar loads), and oversized requests
+must be refused before any work is enqueued.  This file is collected last on purpose.
 """
 import ctypes
 
