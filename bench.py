@@ -578,40 +578,38 @@ def next_tree_ept(w, dev, stream, K, n_ept=4, chain=3, B=4):
 def per_layer_attention(w, t, prefix, parent, out, dev, reps, windows):
     """Attention as a model runs it: L ppd_tree_attention calls of one layer
     each, captured in a CUDA graph and replayed `reps` times (CUDA events on the
-    replay stream, median).  With a workspace the library shares each call's
-    key tiles over all SMs when the layer has fewer slices than SMs; without,
-    one whole slice per SM."""
+    replay stream, median).  "plan": how each call shares its slices out, as
+    ppd_attention_plan has it (2..8: a cluster of that many SMs each, 1: the
+    work split, 0: one whole slice per SM at a time)."""
     import torch
 
     from paper_2405_18628_gb300 import ppd
 
     st = torch.zeros(w.B, dtype=torch.int32, device=dev)
     ws = ppd.workspace(1, w.B, w.H, w.T, w.D, 1, w.S_max, device=dev)
-    res = {}
-    for mode, wsx in (("split", ws), ("unsplit", None)):
-        def layers():
-            for l in range(w.L):
-                ppd.ppd_tree_attention(t["q"][l:l + 1], t["k_cache"][l:l + 1], t["v_cache"][l:l + 1],
-                                       t["k_tree"][l:l + 1], t["v_tree"][l:l + 1], prefix, parent,
-                                       out[l:l + 1], st, workspace=wsx)
-        layers()
-        torch.cuda.synchronize()
-        g = torch.cuda.CUDAGraph()
-        cap = torch.cuda.Stream()
-        cap.wait_stream(torch.cuda.current_stream())
-        with torch.cuda.stream(cap):
-            with torch.cuda.graph(g, stream=cap):
-                layers()
-        torch.cuda.current_stream().wait_stream(cap)
-        s = torch.cuda.current_stream()
-        ms, _ = time_loop(g.replay, reps, 5, s, None, windows)
-        if (st.cpu().numpy() != 0).any():
-            raise SystemExit(f"per-layer attention reported device status {st.cpu().tolist()}")
-        us = statistics.median(ms) * 1e3
-        res[mode] = {"us_per_step": us, "us_per_layer": us / w.L,
-                     "gbs": attention_bytes(w) / (us * 1e-6) / 1e9}
-        del g
-    return {"graph": True, "layers": w.L, "slices_per_layer": w.B * w.H, **res}
+
+    def layers():
+        for l in range(w.L):
+            ppd.ppd_tree_attention(t["q"][l:l + 1], t["k_cache"][l:l + 1], t["v_cache"][l:l + 1],
+                                   t["k_tree"][l:l + 1], t["v_tree"][l:l + 1], prefix, parent,
+                                   out[l:l + 1], st, workspace=ws)
+    layers()
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    cap = torch.cuda.Stream()
+    cap.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(cap):
+        with torch.cuda.graph(g, stream=cap):
+            layers()
+    torch.cuda.current_stream().wait_stream(cap)
+    s = torch.cuda.current_stream()
+    ms, _ = time_loop(g.replay, reps, 5, s, None, windows)
+    if (st.cpu().numpy() != 0).any():
+        raise SystemExit(f"per-layer attention reported device status {st.cpu().tolist()}")
+    us = statistics.median(ms) * 1e3
+    return {"graph": True, "layers": w.L, "slices_per_layer": w.B * w.H,
+            "plan": ppd.ppd_attention_plan(1, w.B, w.H, w.T, w.D, w.S_max),
+            "us_per_step": us, "us_per_layer": us / w.L, "gbs": attention_bytes(w) / (us * 1e-6) / 1e9}
 
 
 def copy_bandwidth(n_bytes, dev, reps=20):
