@@ -151,10 +151,10 @@ ppd_status ppd_kv_compact(void *k_cache, void *v_cache, const void *k_tree, cons
  * accepted rows, enqueued on `stream` with no host synchronisation.  For
  * B <= 64 the attention grid does the other steps with one spare warp per CTA
  * while its other warps stream K/V: that warp combines the argmax, decides
- * acceptance and compacts.  When every SM has a slice (or block of 128 queries) and
- * the logits are at most 1/100 of the K/V bytes (counted over S_max + T rows), those
- * warps also compute the argmax partial maxima themselves and the step is a single
- * cooperative grid behind a one-block status reset (the CTAs exchange flags in the workspace, tagged with a per-call epoch that the
+ * acceptance and compacts.  When the logits are at most 1/64 of the K/V bytes
+ * (counted over S_max + T rows), those warps also compute the argmax partial
+ * maxima themselves and the step is a single cooperative grid (the CTAs
+ * exchange flags in the workspace, tagged with a per-call epoch that the
  * workspace also holds, so its contents still do not matter); otherwise an
  * argmax grid runs first and the attention grid may start while it runs.
  * If the cooperative launch cannot have every CTA resident, the step falls
@@ -322,9 +322,9 @@ int ppd_verify_step_launches(int L, int B, int H, int T, int D, int V, int S_max
  *   0  B > 64: argmax, acceptance, attention and compaction as separate grids;
  *   1  an argmax grid, then the attention grid (which accepts and compacts);
  *   2  one attention grid whose spare warp per CTA also computes the argmax
- *      partial maxima while the K/V stream runs (chosen when every SM
- *      has a slice, the logits are at most 1/100 of the K/V bytes and no argmax grid
- *      fits on SMs that the attention's last round leaves idle).
+ *      partial maxima while the K/V stream runs (chosen when the logits are
+ *      at most 1/64 of the K/V bytes and no argmax grid fits on SMs that the
+ *      attention's last round leaves idle).
  * Form 2 falls back to form 1 when the cooperative launch cannot have
  * every CTA resident.  Returns -1 for sizes the step rejects.
  */

@@ -70,26 +70,23 @@ int argmax_vec(const float *logits, int V)
 }
 
 // The fused step computes the node argmax inside the attention grid (one
-// side warp per CTA, while the other warps stream K/V) when every SM has a slice
-// and the logits are at most 1/kInGridRatio of the bytes the attention streams.  A
-// side warp keeps 2 KB in flight (deeper bursts slow the attention more than they
-// gain) and, with the HBM saturated by the K/V stream, reads about 1 GB/s against its
-// CTA's ~42 GB/s of K/V.  Otherwise a separate argmax grid runs first.  S_max bounds
-// the prefix lengths, which only the device knows.  Measured, argmax grid / in-grid:
-//   608 slices of 2048 keys, 64 tokens: logits 1/1000 of the K/V bytes 106.3 / 104.2 us,
-//     1/150 107.3 / 104.2, 1/100 107.3 / 105.3, 1/64 107.3 / 116.0, 1/20 111.2 / 197.9
-//   1216 slices of 4096 keys, 128 tokens: 1/150 357.9 / 356.4, 1/100 359.0 / 360.5,
-//     1/64 360.5 / 399.2
-// With fewer slices than SMs the in-grid form's status reset, cooperative launch and
-// want of clusters cost more at any ratio: 32 slices of 2048 keys, 1/1000, 17.2 / 25.1;
-// 100 of 2048 (D = 64) 19.2 / 21.3; 150 of 2048 33.1 / 33.8.
-constexpr double kInGridRatio = 100;
+// side warp per CTA, while the other warps stream K/V) when the logits are a
+// small share of the bytes the attention streams.  A side warp keeps 2 KB in
+// flight (deeper bursts slow the attention more than they gain) and, with the
+// HBM saturated by the K/V stream, reads about 1 GB/s against its CTA's
+// ~42 GB/s of K/V.  Measured at Vicuna-7B shapes with a growing vocabulary:
+// in-grid beats the two-grid form while the logits are at most 1/70 of the
+// K/V bytes, and the side warps become the bottleneck at 1/35.  Otherwise a
+// separate argmax grid runs first.  S_max bounds the prefix lengths, which
+// only the device knows.
+#ifndef PPD_IN_GRID_MIN_RATIO
+#define PPD_IN_GRID_MIN_RATIO 64
+#endif
 bool in_grid_argmax_pays(int L, int B, int H, int T, int D, int V, int S_max)
 {
-    const double slices = (double)L * B * H * (T > 64 ? (T + 127) / 128 : 1);
     const double kv = 4.0 * L * B * H * ((double)S_max + T) * D;
     const double logits = 4.0 * B * (double)T * V;
-    return slices >= split_grid() && logits * kInGridRatio <= kv;
+    return logits * PPD_IN_GRID_MIN_RATIO <= kv;
 }
 
 // Forms of the fused step (ppd_verify_step_form): separate grids for large

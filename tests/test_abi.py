@@ -70,8 +70,8 @@ def test_verify_step_launch_counts(lib):
 
 def test_verify_step_forms(lib):
     """The fused step's form: separate grids above 64 sequences, an argmax grid
-    first when slices do not reach every SM or the logits weigh more than 1/100 of
-    the K/V bytes (the tiny shapes) or when a narrow argmax grid fits the SMs left idle by the last
+    first when the logits weigh more than 1/64 of the K/V bytes (the tiny
+    shapes) or when a narrow argmax grid fits the SMs left idle by the last
     round of slices (the Vicuna-7B shapes on 152 SMs), the argmax in the
     attention grid's side warps otherwise, -1 for rejected sizes.  The
     side-warp case uses 171 layers of the Vicuna-7B shapes: 5472 slices leave

@@ -1,7 +1,6 @@
-"""The plan of an attention launch with fewer slices than SMs, and the form of a fused
-step, are the ones that were measured to be the shorter.  Without a GPU (148 SMs, no
-clusters are assumed): whole slices against the work split, and an argmax grid against the
-argmax in the attention grid."""
+"""The plan of an attention launch with fewer slices than SMs is the one that was measured
+to be the shorter.  Without a GPU (148 SMs, no clusters are assumed): whole slices against
+the work split."""
 import pytest
 
 
@@ -26,24 +25,3 @@ def test_whole_slices_or_the_work_split(slices, T, D, prefix, plan):
     build.build()
     assert ppd.ppd_attention_plan(1, 1, slices, T, D, prefix + T) == plan
     assert ppd.ppd_attention_plan(1, 1, slices, T, D, prefix + T, workspace=False) == 0
-
-
-@pytest.mark.parametrize("L,B,H,T,D,prefix,ratio,form", [
-    # slices in whole rounds of SMs: no narrow argmax grid
-    (4, 1, 37, 64, 128, 2048, 1000, 2),     # 106.3 us with an argmax grid, 104.2 without (608 slices)
-    (4, 1, 37, 64, 128, 2048, 150, 2),      # 107.3, 104.2
-    (4, 1, 37, 64, 128, 2048, 64, 1),       # 107.3, 116.0
-    (4, 1, 37, 64, 128, 2048, 20, 1),       # 111.2, 197.9
-    (4, 8, 37, 128, 128, 4096, 64, 1),      # 360.5, 399.2 (1216 slices)
-    # fewer slices than SMs
-    (1, 1, 32, 64, 128, 2048, 1000, 1),     # 17.2, 25.1
-    (1, 1, 100, 32, 64, 2048, 300, 1),      # 19.2, 22.8
-])
-def test_argmax_grid_or_in_the_attention_grid(L, B, H, T, D, prefix, ratio, form):
-    torch = pytest.importorskip("torch")
-    if torch.cuda.is_available():
-        pytest.skip("148 SMs assumed")
-    from paper_2405_18628_gb300 import build, ppd
-    build.build()
-    V = 4 * L * B * H * (prefix + 2 * T) * D // ratio // (4 * B * T)
-    assert ppd.ppd_verify_step_form(L, B, H, T, D, V, prefix + T) == form

@@ -23,6 +23,12 @@ from test_gpu_typical import DELTA, EPS, TEMP, _margins_clear
 pytestmark = pytest.mark.gpu
 
 
+def in_grid(w):
+    """The library's choice of mode (in_grid_argmax_pays in ppd_api.cu): in-grid
+    when 64 x the logits bytes are at most the K/V bytes over S_max + T rows."""
+    return 4 * w.B * w.T * w.V * 64 <= 4 * w.L * w.B * w.H * (w.S_max + w.T) * w.D
+
+
 def _wl(name, seed, **kw):
     base = dict(n_cand=12, max_depth=4, chains="fill3", match_rate=0.7, seed=seed)
     base.update(kw)
