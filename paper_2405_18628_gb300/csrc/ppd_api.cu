@@ -247,40 +247,31 @@ bool attn_dims_ok(int L, int B, int H, int T, int D, int S_max, ppd_dtype dt)
 // with fewer units than SMs can gain from either: with more, the last round's
 // idle SMs cost less than the merge (measured on the Vicuna-7B/13B and
 // MobileLlama shapes).  Counted in tiles of 128 keys, S_max standing in for the
-// (device-side) prefix lengths: whole units take t_u tiles of 0.9 us (D = 128) or 0.6
-// (D = 64).  A cluster takes its share and 2.3 us for the merge through distributed
-// shared memory; where more than 3/5 of the SMs stream at D = 128, HBM makes every
-// tile longer, about one more in all.  The work split takes its share of all tiles,
-// which is smaller, 10 us for the range planning and the merge grid, and, with every SM
-// streaming, longer tiles.  Measured per call, 64 tokens, whole / split / cluster:
-//   D = 128:  20 units of 4 tiles  8.6 /    - /  8.1 us   32 of 4   8.7 /    - /  8.8
-//             60 of 7             11.9 / 18.1 / 12.7      48 of 25 28.0 / 25.5 / 21.5
-//             80 of 25            31.3 / 33.5             80 of 64 69.0 / 63.1
-//             100 of 25           32.8 / 39.0             20 of 64 61.5 / 27.0 / 21.0
-//   D = 64, 32 tokens:  60 of 7 8.1 / 13.3 / 8.7          48 of 64 43.8 / 25.4 / 26.1
+// (device-side) prefix lengths: whole units take t_u tiles; a cluster of c takes
+// its share and about kClusterCostTiles for the merge through distributed
+// shared memory; the work split takes its share of all tiles, which is smaller,
+// and about kSplitCostTiles for the range planning and the merge grid.
 struct AttnPlan {
     int split, cluster;
 };
+constexpr long long kClusterCostTiles = 2, kSplitCostTiles = 6;
 
-AttnPlan plan_attention(int L, int B, int H, int T, int D, int S_max, bool workspace, bool clusters)
+AttnPlan plan_attention(int L, int B, int H, int T, int S_max, bool workspace, bool clusters)
 {
     AttnPlan plan{0, 1};
     const int n_tt = T > 64 ? (T + 127) / 128 : 1;
     const long long units = (long long)L * B * H * n_tt, sms = split_grid();
     if (units >= sms) return plan;
     const long long t_u = (S_max + 127) / 128 + n_tt;
-    auto share = [&](int c) { return (t_u + c - 1) / c; };
-    int size = 1;
-    for (int c = 2; clusters && c <= ppd::kMaxCluster && c <= t_u && units * c <= sms; ++c)
-        if (share(c) < share(size) && units <= ppd::max_attention_clusters(c)) size = c;
-    const long long merge = D == 64 ? 4 : 5 * units * size > 3 * sms ? 3 : 2;
     long long best = t_u;
-    if (size > 1 && share(size) + merge < best) {
-        best = share(size) + merge;
-        plan.cluster = size;
+    for (int c = 2; clusters && c <= ppd::kMaxCluster && c <= t_u && units * c <= sms; ++c) {
+        const long long cost = (t_u + c - 1) / c + kClusterCostTiles;
+        if (cost < best && units <= ppd::max_attention_clusters(c)) {
+            best = cost;
+            plan.cluster = c;
+        }
     }
-    const long long split = (units * t_u + sms - 1) / sms + (D == 64 ? 14 : 16);
-    if (workspace && B <= ppd::kSplitMaxB && split < best) plan = {1, 1};
+    if (workspace && B <= ppd::kSplitMaxB && (units * t_u + sms - 1) / sms + kSplitCostTiles < best) plan = {1, 1};
     return plan;
 }
 
@@ -323,7 +314,7 @@ ppd_status enqueue_attention(const void *q, const void *kc, const void *vc, cons
     const float sc = scale > 0.f ? scale : 1.0f / std::sqrt((float)D);
     p.scale_log2 = sc * 1.4426950408889634f;
     ppd::plan_rows(p, split_grid());
-    const AttnPlan plan = plan_attention(L, B, H, T, D, S_max, ws && wl, !(fused && fused->in_grid));
+    const AttnPlan plan = plan_attention(L, B, H, T, S_max, ws && wl, !(fused && fused->in_grid));
     p.cluster = plan.cluster;
     p.set_status = set_status;
     if (plan.split) {
@@ -411,7 +402,7 @@ AttnParams row_plan(int L, int B, int H, int T, int S_max)
 // no CTA with time to spare.
 int narrow_argmax_grid(int L, int B, int H, int T, int D, int V, int S_max)
 {
-    const AttnPlan plan = plan_attention(L, B, H, T, D, S_max, true, true);
+    const AttnPlan plan = plan_attention(L, B, H, T, S_max, true, true);
     if (plan.split || plan.cluster > 1) return 0;
     const AttnParams p = row_plan(L, B, H, T, S_max);
     // two groups of CTAs with queues of their own: none is known to have time to spare
@@ -589,7 +580,7 @@ int ppd_verify_step_form(int L, int B, int H, int T, int D, int V, int S_max, pp
 int ppd_attention_plan(int L, int B, int H, int T, int D, int S_max, int workspace, int one_grid)
 {
     if (!attn_dims_ok(L, B, H, T, D, S_max, PPD_BF16)) return -1;
-    const AttnPlan plan = plan_attention(L, B, H, T, D, S_max, workspace != 0, one_grid == 0);
+    const AttnPlan plan = plan_attention(L, B, H, T, S_max, workspace != 0, one_grid == 0);
     if (plan.split || plan.cluster > 1) return plan.split ? 1 : plan.cluster;
     return row_plan(L, B, H, T, S_max).pairs ? 16 : 0;
 }
@@ -615,7 +606,7 @@ int ppd_verify_step_launches(int L, int B, int H, int T, int D, int V, int S_max
     const int form = ppd_verify_step_form(L, B, H, T, D, V, S_max, dt);
     if (form < 0) return -1;
     const int round = dt == PPD_F32 ? 5 : 0;   // fp32 -> bf16 copies of Q, K/V tree, K/V cache
-    const int attn = plan_attention(L, B, H, T, D, S_max, true, form != kFormSide).split ? 2 : 1;   // + the merge grid
+    const int attn = plan_attention(L, B, H, T, S_max, true, form != kFormSide).split ? 2 : 1;   // + the merge grid
     if (form == kFormTwoGrids) return 1 + round + attn;
     if (form == kFormSide) return 1 + round + attn;   // the status reset, then one grid
     // partial maxima, combine (or statistics), acceptance, attention, compaction

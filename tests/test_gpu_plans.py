@@ -36,16 +36,16 @@ def _wl(seed, L, B, H, D, P, T, V, **kw):
 # in the attention grid (form 2, which rules clusters out)
 FUSED = {
     # 80 slices: no cluster fits, the key tiles are shared out and merged by a grid
-    "split_keyrow": (_wl(601, 1, 2, 40, 64, 4500, 40, 301), [4500, 1900], SPLIT, SPLIT),
-    "split_rows": (_wl(602, 1, 2, 40, 64, 4500, 100, 248), [4500, 1411], SPLIT, SPLIT),
+    "split_keyrow": (_wl(601, 1, 2, 40, 64, 2000, 40, 301), [2000, 1900], SPLIT, SPLIT),
+    "split_rows": (_wl(602, 1, 2, 40, 64, 3000, 100, 248), [3000, 1411], SPLIT, SPLIT),
     # few slices: clusters; without them 25 parts a slice, fewer tiles than SMs (SMs with
     # none), several query blocks and parts of tree tiles alone
     "cluster_keyrow": (_wl(603, 1, 1, 30, 128, 832, 64, 1000), [787], 4, WHOLE),
-    "cluster_rows": (_wl(604, 1, 2, 9, 128, 1308, 100, 248), [1308, 513], 6, WHOLE),
+    "cluster_rows": (_wl(604, 1, 2, 9, 128, 1308, 100, 248), [1308, 513], 6, SPLIT),
     "two_slices": (_wl(610, 1, 1, 2, 128, 3000, 64, 500), [3000], 7, SPLIT),
     "few_tiles": (_wl(611, 1, 2, 3, 128, 4056, 40, 300), [100, 5], 7, SPLIT),
-    "few_tiles_t200": (_wl(612, 1, 2, 1, 128, 2400, 200, 120), [900, 33], 8, SPLIT),
-    "few_tiles_t512": (_wl(613, 1, 1, 1, 64, 2000, 512, 100), [300], 8, SPLIT),
+    "few_tiles_t200": (_wl(612, 1, 2, 1, 128, 900, 200, 120), [900, 33], 6, SPLIT),
+    "few_tiles_t512": (_wl(613, 1, 1, 1, 64, 300, 512, 100), [300], 6, SPLIT),
     # one sequence, more slices than SMs: pairs of query blocks; 285 tokens run pairs and
     # third blocks in two groups of SMs
     "pairs_t200": (_wl(605, 1, 1, 160, 64, 300, 200, 248), [300], PAIRS, PAIRS),
@@ -81,7 +81,7 @@ def test_fused_step_of_every_plan(cuda_device, case, fused_form):
 # ----------------------------------------------------------------------------- clusters of every size
 
 @pytest.mark.parametrize("T,D", [(40, 64), (64, 128), (100, 64), (128, 128)])
-@pytest.mark.parametrize("size,slices,tiles", [(2, 60, 12), (3, 40, 9), (4, 30, 8), (5, 24, 10), (6, 18, 12),
+@pytest.mark.parametrize("size,slices,tiles", [(2, 60, 9), (3, 40, 9), (4, 30, 8), (5, 24, 10), (6, 18, 12),
                                                (7, 12, 14), (8, 10, 16)])
 def test_clusters_of_every_size(cuda_device, size, slices, tiles, T, D):
     """One call of `slices` slices whose cache holds `tiles` tiles with the tree's, both
@@ -313,8 +313,8 @@ def _bf16(bits):
 @pytest.mark.parametrize("L,B,H,T,D,prefix,plan", [
     (1, 1, 10, 64, 128, [1856], 8),                  # clusters, key-row kernel
     (1, 2, 9, 100, 64, [1308, 513], 6),              # clusters, query-row kernel
-    (1, 2, 40, 40, 64, [4500, 1900], SPLIT),         # the merge grid
-    (1, 2, 40, 100, 64, [4500, 1411], SPLIT),        # the query-row kernel's
+    (1, 2, 40, 40, 64, [2000, 1900], SPLIT),         # the merge grid
+    (1, 2, 40, 100, 64, [3000, 1411], SPLIT),        # the query-row kernel's
     (1, 1, 160, 33, 64, [129], WHOLE),               # key-row kernel
     (1, 1, 160, 100, 128, [300], WHOLE),             # single jobs
     (1, 1, 160, 200, 128, [129], PAIRS),             # pair jobs

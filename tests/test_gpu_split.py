@@ -141,11 +141,9 @@ def test_split_status_per_call(cuda_device):
 
 
 @pytest.mark.parametrize("H,T,D,prefix,S_max", [
-    (40, 64, 64, [2000, 2048], 2048),     # 80 slices: whole, on half of the SMs
+    (40, 64, 64, [2000, 2048], 2048),     # 80 slices: the work split of the key-row kernel
     (38, 96, 128, [1900, 1500], 4096),    # 76 slices: clusters of 2
-    (40, 100, 64, [4000, 10], 4096),      # 80 slices in the query-row kernel: whole
-    (40, 64, 64, [5000, 4990], 5120),     # 80 slices of more tiles: the work split of the key-row kernel
-    (40, 100, 64, [5000, 10], 5120),      # and of the query-row kernel
+    (40, 100, 64, [4000, 10], 4096),      # 80 slices: the work split of the query-row kernel
     (20, 33, 64, [1000, 127], 1024),      # 40 slices: clusters of 3
     (14, 17, 128, [700, 0], 1024),        # 28: clusters of 5, one of a single tile
     (10, 128, 64, [900, 513], 1024),      # 20: clusters of 5, query-row kernel
@@ -154,8 +152,7 @@ def test_split_status_per_call(cuda_device):
     (2, 200, 128, [0, 300], 4096),        # the same in the query-row kernel, rows without keys in a part
 ])
 def test_split_sizes(cuda_device, H, T, D, prefix, S_max):
-    """Clusters of several sizes, and whole slices or the work split where no cluster
-    size fits."""
+    """Clusters of several sizes, and the work split where no cluster size fits."""
     L, B = 1, 2
     t, pl, parent = _case(L, B, H, T, D, prefix, S_max, seed=H + T)
     t_dev = {k: v.to(cuda_device) for k, v in t.items()}
