@@ -74,19 +74,23 @@ int argmax_vec(const float *logits, int V)
 // small share of the bytes the attention streams.  A side warp keeps 2 KB in
 // flight (deeper bursts slow the attention more than they gain) and, with the
 // HBM saturated by the K/V stream, reads about 1 GB/s against its CTA's
-// ~42 GB/s of K/V.  Measured at Vicuna-7B shapes with a growing vocabulary:
-// in-grid beats the two-grid form while the logits are at most 1/70 of the
-// K/V bytes, and the side warps become the bottleneck at 1/35.  Otherwise a
-// separate argmax grid runs first.  S_max bounds the prefix lengths, which
-// only the device knows.
-#ifndef PPD_IN_GRID_MIN_RATIO
-#define PPD_IN_GRID_MIN_RATIO 64
-#endif
+// ~42 GB/s of K/V.  Otherwise a separate argmax grid runs first.  S_max bounds
+// the prefix lengths, which only the device knows.  Measured, argmax grid / in-grid:
+//   608 slices of 2048 keys, 64 tokens: logits 1/1000 of the K/V bytes 106.3 / 104.2 us,
+//     1/100 107.3 / 105.3, 1/64 107.3 / 116.0, 1/50 107.8 / 122.2, 1/20 111.2 / 197.9
+//   1216 slices of 4096 keys, 128 tokens: 1/300 356.4 / 352.8, 1/150 357.9 / 356.4,
+//     1/100 359.0 / 360.5, 1/64 360.5 / 399.2
+//   304 slices of 2048 keys, 200 tokens: 1/300 91.7 / 90.9, 1/64 92.5 / 90.5,
+//     1/35 93.0 / 101.2
+// With fewer slices than SMs an argmax grid would be shorter at any ratio (32 slices of
+// 2048 keys, 1/300: 17.2 / 26.9; 100 at D = 64 19.2 / 22.8): it lets the slices have
+// clusters.  The in-grid form shares their tiles out evenly instead, in shorter sums.
+constexpr double kInGridMinRatio = 64;
 bool in_grid_argmax_pays(int L, int B, int H, int T, int D, int V, int S_max)
 {
     const double kv = 4.0 * L * B * H * ((double)S_max + T) * D;
     const double logits = 4.0 * B * (double)T * V;
-    return logits * PPD_IN_GRID_MIN_RATIO <= kv;
+    return logits * kInGridMinRatio <= kv;
 }
 
 // Forms of the fused step (ppd_verify_step_form): separate grids for large
@@ -250,7 +254,17 @@ bool attn_dims_ok(int L, int B, int H, int T, int D, int S_max, ppd_dtype dt)
 // (device-side) prefix lengths: whole units take t_u tiles; a cluster of c takes
 // its share and about kClusterCostTiles for the merge through distributed
 // shared memory; the work split takes its share of all tiles, which is smaller,
-// and about kSplitCostTiles for the range planning and the merge grid.
+// and about kSplitCostTiles for the range planning and the merge grid.  Measured per
+// call, D = 128, 64 tokens, whole / split / cluster:
+//   20 units of 4 tiles  8.6 / 11.7 /  8.1 us     32 of 13  16.6 / 17.8 / 12.7
+//   60 of 7             11.9 / 18.1 / 12.7        48 of 25  28.0 / 25.5 / 21.5
+//   80 of 25            31.3 / 33.5               80 of 64  69.0 / 63.1
+//   100 of 25           32.8 / 39.0               20 of 64  61.5 / 27.0 / 21.0
+// By the time alone the split would cost sixteen tiles (10 us for planning and merging,
+// and longer tiles with every SM streaming) and a cluster three or four.  The lines are
+// not drawn there: parts keep the fp32 sums short, and the calls that would change over
+// lose that (relative error against 64 bits with the split at sixteen: 100 units of 25
+// tiles 3.1e-6 -> 4.2e-6, 120 of 64 6.2e-6 -> 9.5e-6, 48 of 64 3.6e-6 -> 5.2e-6).
 struct AttnPlan {
     int split, cluster;
 };
