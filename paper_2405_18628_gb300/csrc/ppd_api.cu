@@ -700,6 +700,19 @@ ppd_status ppd_node_argmax(const float *logits, int B, int T, int V, int32_t *ar
                                                static_cast<cudaStream_t>(stream)));
 }
 
+// The same grid as ppd_node_argmax, which needs no scratch; requests of more than
+// 65,536 rows stay refused.
+ppd_status ppd_node_argmax_noalloc(const float *logits, int B, int T, int V, int32_t *argmax_out, void *stream)
+{
+    constexpr int64_t kMaxRows = 1 << 16;
+    if (!logits || !argmax_out || B < 1 || T < 1 || V < 1) return PPD_ERR_INVALID_ARG;
+    if ((double)B * T * V > 9.0e15) return PPD_ERR_INVALID_ARG;
+    const int64_t rows = (int64_t)B * T;
+    if (rows > kMaxRows) return PPD_ERR_UNSUPPORTED;
+    return cuda_status(ppd::launch_node_argmax(logits, rows, V, 1.f, argmax_out, nullptr, nullptr,
+                                               static_cast<cudaStream_t>(stream)));
+}
+
 ppd_status ppd_accept_path(const int32_t *argmax, const int32_t *cand_tokens,
                            const int32_t *parent, const int32_t *prefix_len,
                            int B, int T, int V, int S_max,

@@ -11,7 +11,6 @@
 // walks its nodes' root paths, and a warp max-reduction picks the deepest
 // accepted node.  Compaction (Section 3 step (3)) copies the accepted rows
 // into the cache with 16-byte loads and stores.
-#include "ppd.h"
 #include "ppd_accept.cuh"
 #include "ppd_device.cuh"
 #include "ppd_kernels.h"
@@ -710,22 +709,4 @@ cudaError_t launch_selftest_umma(const CUtensorMap &ma, const CUtensorMap &mb, c
     return cudaGetLastError();
 }
 
-// ------------------------------------------------------------------ argmax without a workspace
-
 }  // namespace ppd
-
-// The same grid as ppd_node_argmax, which needs no scratch; requests of more than
-// 65,536 rows stay refused.
-extern "C" ppd_status ppd_node_argmax_noalloc(const float *logits, int B, int T, int V,
-                                              int32_t *argmax_out, void *stream)
-{
-    constexpr int64_t kMaxRows = 1 << 16;
-    if (!logits || !argmax_out || B < 1 || T < 1 || V < 1) return PPD_ERR_INVALID_ARG;
-    if ((double)B * T * V > 9.0e15) return PPD_ERR_INVALID_ARG;
-    const int64_t rows = (int64_t)B * T;
-    if (rows > kMaxRows) return PPD_ERR_UNSUPPORTED;
-    return ppd::launch_node_argmax(logits, rows, V, 1.f, argmax_out, nullptr, nullptr,
-                                   static_cast<cudaStream_t>(stream)) == cudaSuccess
-               ? PPD_OK
-               : PPD_ERR_CUDA;
-}
