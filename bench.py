@@ -324,9 +324,9 @@ def parse(argv=None):
                     help="time the per-layer attention even when extras are off")
     ap.add_argument("--layers", type=int, default=0,
                     help="run the workload with this many layers (profiling captures)")
-    ap.add_argument("--form", type=int, default=None, choices=[1, 2, 3],
+    ap.add_argument("--form", type=int, default=None, choices=[1, 2],
                     help="force the fused step's form (1: argmax grid first; 2: argmax in the "
-                         "side warps; 3: argmax in the softmax warps before their first tile)")
+                         "side warps)")
     ap.add_argument("--l2", default="auto", choices=["auto", "flush", "none"],
                     help="auto: flush L2 before each step unless the step's inputs exceed 4x L2")
     return ap.parse_args(argv)

@@ -111,10 +111,10 @@ int narrow_argmax_grid(int L, int B, int H, int T, int D, int V, int S_max);
 
 // The form of a fused step (B <= kFusedMaxB) of these sizes: an argmax grid
 // first when it fits on the idle SMs of the attention grid's last, partial
-// round (measured at Vicuna-7B shapes: 181.9 us against 183.2 us with the
-// side warps; equal at Vicuna-13B and on the batch-8 sweep), else the side
-// warps when the logits are a small enough share of the K/V bytes, else an
-// argmax grid over every SM.
+// round (measured, us, against the side warps: Vicuna-7B shapes 173.0 / 173.2,
+// Vicuna-13B 534.5 / 540.2, MobileLlama 41.3 / 89.9, the batch-8 sweep at 16 tokens
+// 9390 / 9397), else the side warps when the logits are a small enough share of the
+// K/V bytes, else an argmax grid over every SM.
 int choose_form(int L, int B, int H, int T, int D, int V, int S_max)
 {
     const int forced = g_forced_form.load(std::memory_order_relaxed);
